@@ -440,7 +440,7 @@ vmo_status vmo_finegrain_coords(vmo_hg hg, const float* bipartite_coords, float*
  *   small_step_threads: layout step launches of at most this many threads
  *     use the step-kernel variant with two far-field rows in flight per lane
  *     (latency hiding for small levels); default 19,456 (4 warps per SM);
- *   radix_max_bits: widest digit of the binning sort's LSD passes, 8, 9 or
+ *   radix_max_bits: widest digit of the LSD radix sorts, 8, 9 or
  *     10 (default 10: fewest passes);
  *   assign_items: positions per thread of the Lloyd assignment, 1, 2, 4 or
  *     8 (default 4; fewer are used when the blocks would not fill the GPU);

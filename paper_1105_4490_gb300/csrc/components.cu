@@ -91,7 +91,7 @@ vmo_status group_components(const vmo_hg_s* h, ComponentGroups& g, cudaStream_t 
   if (k == 0) return VMO_OK;
   VMO_TRY(components(h, lab, s));
   launch(k_iota_u32, grid_for(k, 256), 256, 0, s, ids, k);
-  VMO_TRY(radix_sort_u32((uint32_t*)lab, ids, slab, g.cperm, k, bits_for((uint64_t)k), nullptr, s, sc));
+  VMO_TRY(radix_sort_u32((uint32_t*)lab, ids, slab, g.cperm, k, bits_for((uint64_t)k), s, sc));
   launch(k_run_starts, grid_for(k, 256), 256, 0, s, slab, k, flag);
   VMO_LAUNCHED("run_starts");
   VMO_TRY(scan_exclusive<int32_t>(flag, pos, k, total, s, sc));

@@ -17,6 +17,8 @@
 #include <algorithm>
 #include <cmath>
 
+#include <cooperative_groups.h>
+
 #include "blocksort.cuh"
 #include "layout.cuh"
 
@@ -175,6 +177,22 @@ __global__ void k_step0(const uint32_t* __restrict__ bb, const ProbDev* __restri
   s0[p] = (k > 0) ? (float)(sigma * Lbox / pow((double)k, 1.0 / D)) : 0.0f;
 }
 
+// Binning of a level, device-wide: a counting sort by cell.  A step's cells
+// are at most 8 points each on average, so instead of sorting (key, vertex)
+// by digits (two passes of three kernels), every point takes a number in its
+// cell, a scan of the cell counts gives the cell start table directly, and
+// the points of a cell are then put into vertex order by counting the smaller
+// ids among them:
+//   k_keys      cell key of every point, its arrival number in the cell
+//   k_cell_scan cell counts -> first sorted position of every cell
+//   k_slots     vertex ids to their cells in arrival order
+//   k_place     vertex order within the cell; sorted copies of the points
+//   k_cells     cell sums and charges of every grid level
+// The sorted order is that of a stable sort of (key, vertex), so nothing
+// depends on the arrival order.  Five launches; the two-pass digit sort with
+// its gather and per-level sums took eleven or more of about 4 us each, all
+// bound by latency on the levels of a hierarchy.
+
 // Cell keys of the points.  Each thread takes U points, strided by the block
 // so that every load is coalesced, and issues all their loads before the
 // arithmetic (U = 4 on large levels: more bytes in flight per SM; U = 1 on
@@ -185,9 +203,10 @@ constexpr int64_t kKeyItemsMin = int64_t(1) << 20;  // points of a level that ta
 template <int D, int U>
 __global__ void __launch_bounds__(kBlock) k_keys(const float4* __restrict__ x, int64_t K, const int32_t* __restrict__ vprob,
                                                  const ProbDev* __restrict__ prob, const uint32_t* __restrict__ bb,
-                                                 uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                                                 uint32_t* __restrict__ bb_next, int nreset, int32_t* __restrict__ tctr) {
-  pdl_wait();
+                                                 uint32_t* __restrict__ keys, uint32_t* __restrict__ arrival,
+                                                 int32_t* __restrict__ cnt, uint32_t* __restrict__ bb_next, int nreset,
+                                                 int32_t* __restrict__ tctr) {
+  pdl_enter();
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (gt == 0) ++*tctr;  // the level's step (read by the step kernel of this step)
   for (int64_t r = gt; r < nreset; r += (int64_t)gridDim.x * blockDim.x) bb_next[r] = ((r & 7) < 4) ? 0xFFFFFFFFu : 0u;
@@ -209,9 +228,140 @@ __global__ void __launch_bounds__(kBlock) k_keys(const float4* __restrict__ x, i
     grid_frame<D>(bb, pb[u], L, lo, &s);
     int32_t c[D];
     cell_of<D>(xv[u], lo, s, L, c);
-    keys[v] = (uint32_t)rowmajor<D>(c, 1 << L);
-    vals[v] = (uint32_t)v;
+    // the key indexes the count table: kept inside it whatever the coordinates are
+    const uint32_t key = min((uint32_t)rowmajor<D>(c, 1 << L), (uint32_t)((int64_t(1) << (D * L)) - 1));
+    keys[v] = key;
+    arrival[v] = (uint32_t)atomicAdd(&cnt[prob[pb[u]].fbase + pb[u] + key], 1);
   }
+}
+
+// Cell counts -> cell start table: the exclusive scan of cnt (every problem's
+// finest cells and one empty end entry, problem after problem, as the
+// problems' points are) is the first sorted position of every cell, of the
+// end entry the problem's end.  One cluster scans a tile of
+// kCellScanTile entries at a time; its blocks exchange their totals through
+// distributed shared memory.
+constexpr int kCellScanCtas = 8;
+constexpr int kCellScanThreads = 1024;
+constexpr int kCellScanItems = 16;
+constexpr int64_t kCellScanTile = (int64_t)kCellScanCtas * kCellScanThreads * kCellScanItems;
+constexpr int64_t kCellScanMax = 4 * kCellScanTile;  // larger tables: two launches over every SM
+
+__device__ __forceinline__ void load_items(const int32_t* __restrict__ a, int64_t i0, int64_t n, int32_t* v) {
+  if (i0 + kCellScanItems <= n) {
+#pragma unroll
+    for (int j = 0; j < kCellScanItems / 4; ++j) {
+      const int4 q = *reinterpret_cast<const int4*>(a + i0 + 4 * j);
+      v[4 * j] = q.x;
+      v[4 * j + 1] = q.y;
+      v[4 * j + 2] = q.z;
+      v[4 * j + 3] = q.w;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < kCellScanItems; ++j) v[j] = i0 + j < n ? a[i0 + j] : 0;
+  }
+}
+
+__device__ __forceinline__ void store_prefix(int32_t* __restrict__ a, int64_t i0, int64_t n, const int32_t* v,
+                                             int32_t run) {
+  int32_t e[kCellScanItems];
+#pragma unroll
+  for (int j = 0; j < kCellScanItems; ++j) {
+    e[j] = run;
+    run += v[j];
+  }
+  if (i0 + kCellScanItems <= n) {
+#pragma unroll
+    for (int j = 0; j < kCellScanItems / 4; ++j)
+      *reinterpret_cast<int4*>(a + i0 + 4 * j) = make_int4(e[4 * j], e[4 * j + 1], e[4 * j + 2], e[4 * j + 3]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < kCellScanItems; ++j)
+      if (i0 + j < n) a[i0 + j] = e[j];
+  }
+}
+
+__global__ void __cluster_dims__(kCellScanCtas, 1, 1) __launch_bounds__(kCellScanThreads)
+    k_cell_scan(const int32_t* __restrict__ cnt, int32_t* __restrict__ cst, int64_t n) {
+  pdl_enter();
+  __shared__ int32_t ws[33];
+  __shared__ int32_t tot[2];             // this block's total, by parity of the tile
+  __shared__ int32_t peer[kCellScanCtas];
+  auto cluster = cooperative_groups::this_cluster();
+  const unsigned r = cluster.block_rank();
+  int32_t carry = 0;
+  int par = 0;
+  for (int64_t base = 0; base < n; base += kCellScanTile, par ^= 1) {
+    const int64_t i0 = base + ((int64_t)r * kCellScanThreads + threadIdx.x) * kCellScanItems;
+    int32_t v[kCellScanItems];
+    load_items(cnt, i0, n, v);
+    int32_t sum = 0;
+#pragma unroll
+    for (int j = 0; j < kCellScanItems; ++j) sum += v[j];
+    int32_t total;
+    const int32_t ex = block_exclusive<int32_t>(sum, ws, &total);
+    if (threadIdx.x == 0) tot[par] = total;
+    cluster.sync();
+    if (threadIdx.x < kCellScanCtas) peer[threadIdx.x] = *cluster.map_shared_rank(&tot[par], threadIdx.x);
+    __syncthreads();
+    int32_t before = carry;
+#pragma unroll
+    for (unsigned q = 0; q < kCellScanCtas; ++q) {
+      before += q < r ? peer[q] : 0;
+      carry += peer[q];
+    }
+    store_prefix(cst, i0, n, v, before + ex);
+    __syncthreads();  // peer is rewritten by the next tile
+  }
+  cluster.sync();  // no block leaves while another may still read its total
+}
+
+// The same scan for larger tables in two launches: block totals, then every
+// block adds up the totals before its own and scans its part.
+__global__ void __launch_bounds__(kCellScanThreads) k_cell_totals(const int32_t* __restrict__ cnt, int64_t n,
+                                                                  int32_t* __restrict__ tot) {
+  pdl_enter();
+  __shared__ int32_t ws[33];
+  int32_t v[kCellScanItems];
+  load_items(cnt, ((int64_t)blockIdx.x * kCellScanThreads + threadIdx.x) * kCellScanItems, n, v);
+  int32_t sum = 0;
+#pragma unroll
+  for (int j = 0; j < kCellScanItems; ++j) sum += v[j];
+  int32_t total;
+  block_exclusive<int32_t>(sum, ws, &total);
+  if (threadIdx.x == 0) tot[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(kCellScanThreads) k_cell_starts(const int32_t* __restrict__ cnt, int64_t n,
+                                                                  const int32_t* __restrict__ tot,
+                                                                  int32_t* __restrict__ cst) {
+  pdl_enter();
+  __shared__ int32_t ws[33];
+  int32_t v[kCellScanItems];
+  const int64_t i0 = ((int64_t)blockIdx.x * kCellScanThreads + threadIdx.x) * kCellScanItems;
+  load_items(cnt, i0, n, v);
+  int32_t part = 0;
+  for (unsigned b = threadIdx.x; b < blockIdx.x; b += kCellScanThreads) part += tot[b];
+  int32_t before;
+  block_exclusive<int32_t>(part, ws, &before);
+  int32_t sum = 0;
+#pragma unroll
+  for (int j = 0; j < kCellScanItems; ++j) sum += v[j];
+  const int32_t ex = block_exclusive<int32_t>(sum, ws, nullptr);
+  store_prefix(cst, i0, n, v, before + ex);
+}
+
+// Vertex ids to their cells, in arrival order.
+__global__ void __launch_bounds__(kBlock) k_slots(const uint32_t* __restrict__ keys,
+                                                  const uint32_t* __restrict__ arrival, int64_t K,
+                                                  const int32_t* __restrict__ vprob, const ProbDev* __restrict__ prob,
+                                                  const int32_t* __restrict__ cst, uint32_t* __restrict__ slot) {
+  pdl_enter();
+  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= K) return;
+  const int pb = vprob[v];
+  slot[cst[prob[pb].fbase + pb + keys[v]] + arrival[v]] = (uint32_t)v;
 }
 
 // a[lo..hi) = v, with 16-byte stores over the aligned middle of the range
@@ -223,29 +373,39 @@ __device__ inline void fill_i32(int32_t* __restrict__ a, int64_t lo, int64_t hi,
   while (lo < hi) a[lo++] = v;
 }
 
-// Sorted positions: coordinates and weights in sorted order (plain and in
-// the paired table XP), the packed cell of every point, and the cell start
-// table.  cst[fbase + pb + c] is the first
-// sorted position of problem pb whose key is >= c (so empty cells get the
-// start of the next occupied one and a row of cells is one contiguous range),
-// with one extra entry per problem holding its end.  Every position writes the
-// entries of the cells between its predecessor's key and its own; the last
-// position of a problem also writes the cells after its key and the end entry.
+// Sorted positions: the points of a cell by ascending vertex (a point's place
+// is the number of smaller ids in its cell: as many comparisons as the cell
+// has points, against 3^d cells of interactions per point in the step
+// kernel), coordinates and weights in sorted order (plain and in the paired
+// table XP) and the packed cell of every point.  The counts are cleared for
+// the next step.
 template <int D>
-__global__ void __launch_bounds__(kBlock) k_gather(const uint32_t* __restrict__ svals,
-                                                   const uint32_t* __restrict__ skeys, int64_t K,
-                                                   const float4* __restrict__ x, const float* __restrict__ w,
-                                                   const int32_t* __restrict__ vprob, const ProbDev* __restrict__ prob,
-                                                   const uint32_t* __restrict__ bb, float4* __restrict__ xs,
-                                                   float* __restrict__ ws, uint32_t* __restrict__ scell,
-                                                   int32_t* __restrict__ cst, float4* __restrict__ XP) {
-  pdl_wait();
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= K) return;
-  uint32_t v = svals[p];
-  int pb = vprob[p];
-  ProbDev pr = prob[pb];
-  float4 xv = x[v];
+__global__ void __launch_bounds__(kBlock) k_place(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ keys,
+                                                  int64_t K, const float4* __restrict__ x, const float* __restrict__ w,
+                                                  const int32_t* __restrict__ vprob, const ProbDev* __restrict__ prob,
+                                                  const int32_t* __restrict__ cst, int32_t* __restrict__ cnt,
+                                                  int64_t ncnt, uint32_t* __restrict__ svals, float4* __restrict__ xs,
+                                                  float* __restrict__ ws, uint32_t* __restrict__ scell,
+                                                  float4* __restrict__ XP) {
+  pdl_enter();
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (int64_t i = t; i < ncnt; i += (int64_t)gridDim.x * blockDim.x) cnt[i] = 0;
+  if (t >= K) return;
+  const uint32_t v = slot[t];
+  const int pb = vprob[v];
+  const ProbDev pr = prob[pb];
+  const float4 xv = x[v];
+  const uint32_t key = keys[v];
+  const int32_t* cs = cst + pr.fbase + pb;
+  const int32_t q0 = cs[key], q1 = cs[key + 1];
+  int64_t p = q0;
+  int32_t q = q0;
+  for (; q + 4 <= q1; q += 4) {
+    const uint32_t a = slot[q], b = slot[q + 1], c = slot[q + 2], e = slot[q + 3];
+    p += (a < v) + (b < v) + (c < v) + (e < v);
+  }
+  for (; q < q1; ++q) p += slot[q] < v;
+  svals[p] = v;
   xs[p] = xv;
   const float wv = w ? w[v] : 1.0f;
   if (ws) ws[p] = wv;
@@ -258,26 +418,17 @@ __global__ void __launch_bounds__(kBlock) k_gather(const uint32_t* __restrict__ 
     const float zero[4] = {0.f, 0.f, 0.f, 0.f};
     pair_store<D>(XP, e + pr.k, zero, 0.0f);
   }
-  float lo[D], s;
-  grid_frame<D>(bb, pb, pr.L, lo, &s);
-  int32_t c[D];
-  cell_of<D>(xv, lo, s, pr.L, c);
   uint32_t packed = 0;
 #pragma unroll
-  for (int m = 0; m < D; ++m) packed |= (uint32_t)c[m] << (m * field_bits(D));
+  for (int m = 0; m < D; ++m) packed |= ((key >> (m * pr.L)) & ((1u << pr.L) - 1u)) << (m * field_bits(D));
   scell[p] = packed;
-  int32_t* cs = cst + pr.fbase + pb;
-  const int64_t key = skeys[p];
-  const int64_t prev = p == pr.vbase ? -1 : (int64_t)skeys[p - 1];
-  fill_i32(cs, prev + 1, key + 1, (int32_t)p);
-  if (p == pr.vbase + pr.k - 1) fill_i32(cs, key + 1, (int64_t(1) << (D * pr.L)) + 1, (int32_t)(pr.vbase + pr.k));
 }
 
 // Cell sums (St, Wt) at cell index idx, and the cell's charge (weighted mean
 // and weight) at index pidx of the paired cell table.
 template <int D>
-__device__ inline void store_cell(int64_t idx, int64_t pidx, const float* S, float W, float4* __restrict__ St,
-                                  float* __restrict__ Wt, float4* __restrict__ CP) {
+__device__ inline void store_cell(int64_t idx, int64_t pidx, const float* S, float W, float4* St, float* Wt,
+                                  float4* CP) {
   St[idx] = make_float4(S[0], D > 1 ? S[1] : 0.f, D > 2 ? S[2] : 0.f, D > 3 ? S[3] : 0.f);
   Wt[idx] = W;
   float c[4] = {0.f, 0.f, 0.f, 0.f};
@@ -289,12 +440,10 @@ __device__ inline void store_cell(int64_t idx, int64_t pidx, const float* S, flo
   pair_store<D>(CP, pidx, c, W);
 }
 
-// Finest cells: the charge of every cell from its points (the range comes
-// from the cell start table written by k_gather; a problem without points
-// writes its table here).  A cell of at most kCellSerial points is summed by
-// its own thread in point order; a larger cell (dense clusters of the layout)
-// by the whole warp: lane-strided partial sums from the cell's first point,
-// then a fixed xor tree.  Either way the sums depend only on the cell.
+// A finest cell of at most kCellSerial points is summed by one thread in point
+// order; a larger cell (dense clusters of the layout) by a whole warp:
+// lane-strided partial sums from the cell's first point, then a fixed xor
+// tree.  Either way the sums depend only on the cell.
 constexpr int kCellSerial = 32;
 
 template <int D>
@@ -326,61 +475,22 @@ __device__ __forceinline__ void cell_sum(const float4* xs, const float* ws, int6
   for (; q < q1; q += stride) cell_add<D>(xs[q], ws ? ws[q] : 1.0f, S, W);
 }
 
+// Sum of the points [q0, q1) of a large cell by a whole warp (every lane gets it).
 template <int D>
-__global__ void __launch_bounds__(kBlock) k_agg_finest(int64_t ncells, const int64_t* __restrict__ fbase, int P,
-                                                       const ProbDev* __restrict__ prob, const float4* __restrict__ xs,
-                                                       const float* __restrict__ ws, int32_t* __restrict__ cst,
-                                                       float4* __restrict__ St, float* __restrict__ Wt,
-                                                       float4* __restrict__ CP) {
-  pdl_wait();
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool valid = i < ncells;
-  int64_t q0 = 0, q1 = 0, idx = 0, pidx = 0;
-  if (valid) {
-    const int pb = find_problem(fbase, P, i);
-    const ProbDev pr = prob[pb];
-    const int64_t c = i - pr.fbase;
-    int32_t* cs = cst + pr.fbase + pb;
-    if (pr.k == 0) {
-      cs[c] = (int32_t)pr.vbase;
-      if (c == (int64_t(1) << (D * pr.L)) - 1) cs[c + 1] = (int32_t)pr.vbase;
-    } else {
-      q0 = cs[c];
-      q1 = cs[c + 1];
-    }
-    idx = pr.cbase + lvl_off(D, pr.L) + c;
-    pidx = idx + pb + 1;
-  }
-  const bool big = valid && q1 - q0 > kCellSerial;
-  if (valid && !big) {
-    float S[4] = {0.f, 0.f, 0.f, 0.f};
-    float W = 0.f;
-    cell_sum<D>(xs, ws, q0, q1, 1, S, W);
-    store_cell<D>(idx, pidx, S, W, St, Wt, CP);
-  }
-  const int lane = lane_id();
-  unsigned todo = __ballot_sync(0xffffffffu, big);
-  while (todo) {
-    const int src = __ffs(todo) - 1;
-    todo &= todo - 1;
-    const int64_t b0 = __shfl_sync(0xffffffffu, q0, src), b1 = __shfl_sync(0xffffffffu, q1, src);
-    float S[4] = {0.f, 0.f, 0.f, 0.f};
-    float W = 0.f;
-    cell_sum<D>(xs, ws, b0 + lane, b1, 32, S, W);
+__device__ __forceinline__ void cell_sum_warp(const float4* xs, const float* ws, int64_t q0, int64_t q1, float* S,
+                                              float& W) {
+  cell_sum<D>(xs, ws, q0 + lane_id(), q1, 32, S, W);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+  for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-      for (int m = 0; m < D; ++m) S[m] += __shfl_xor_sync(0xffffffffu, S[m], o);
-      W += __shfl_xor_sync(0xffffffffu, W, o);
-    }
-    if (lane == src) store_cell<D>(idx, pidx, S, W, St, Wt, CP);
+    for (int m = 0; m < D; ++m) S[m] += __shfl_xor_sync(0xffffffffu, S[m], o);
+    W += __shfl_xor_sync(0xffffffffu, W, o);
   }
 }
 
 // Coarse cells: sums of the 2^d children (fixed order), charge at the mean.
 template <int D>
-__device__ inline void agg_cell(const ProbDev& pr, int pb, int l, int64_t c, float4* __restrict__ St,
-                                float* __restrict__ Wt, float4* __restrict__ CP) {
+__device__ inline void agg_cell(const ProbDev& pr, int pb, int l, int64_t c, float4* St, float* Wt, float4* CP) {
   const int side = 1 << l;
   int32_t cc[D];
   int64_t rem = c;
@@ -398,43 +508,141 @@ __device__ inline void agg_cell(const ProbDev& pr, int pb, int l, int64_t c, flo
 #pragma unroll
     for (int m = 0; m < D; ++m) q[m] = 2 * cc[m] + ((ch >> m) & 1);
     const int64_t idx = child_base + rowmajor<D>(q, 2 * side);
-    const float4 s4 = St[idx];
+    const float4 s4 = __ldcg(St + idx);  // written by other threads of this launch
     S[0] += s4.x;
     if (D > 1) S[1] += s4.y;
     if (D > 2) S[2] += s4.z;
     if (D > 3) S[3] += s4.w;
-    W += Wt[idx];
+    W += __ldcg(Wt + idx);
   }
   const int64_t idx = pr.cbase + lvl_off(D, l) + c;
   store_cell<D>(idx, idx + pb + 1, S, W, St, Wt, CP);
 }
 
-// Levels of at most 512 cells are aggregated by one block per problem (all of
-// them in one launch, a block barrier between levels); the larger coarse
-// levels by one launch per level over all problems.
-__host__ __device__ constexpr int small_level_max(int d) { return d == 2 ? 4 : (d == 3 ? 3 : 2); }
+// Cell sums and charges of every grid level (k_cells): one block per brick of
+// 2^(d B) finest cells, B = kBrick(d) (the whole grid when L < B).  The block
+// sums its finest cells from their points, then the B coarser levels from
+// their children in shared memory; the problem's last block to arrive sums
+// the levels above the bricks' roots from the roots' sums in global memory.
+// Small bricks, so that the large cells of a dense cluster spread over many
+// blocks (a warp took up to 32 of them in turn when a warp owned 32
+// consecutive cells: 17 us on the 64^3 grid's finest level).
+__host__ __device__ constexpr int brick_log2(int d) { return d == 2 ? 3 : 2; }
 
 template <int D>
-__global__ void __launch_bounds__(kBlock) k_agg_level(int step, const int64_t* __restrict__ off, int P, int64_t ncells,
-                                                      const ProbDev* __restrict__ prob, float4* __restrict__ St,
-                                                      float* __restrict__ Wt, float4* __restrict__ CP) {
-  pdl_wait();
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= ncells) return;
-  int pb = find_problem(off, P, i);
-  ProbDev pr = prob[pb];
-  agg_cell<D>(pr, pb, pr.L - step, i - off[pb], St, Wt, CP);
-}
-
-template <int D>
-__global__ void __launch_bounds__(kBlock) k_agg_small(const ProbDev* __restrict__ prob, float4* __restrict__ St,
-                                                      float* __restrict__ Wt, float4* __restrict__ CP) {
-  pdl_wait();
-  const int pb = blockIdx.x;
+__global__ void __launch_bounds__(kBlock) k_cells(const int64_t* __restrict__ bbase, int P,
+                                                  const ProbDev* __restrict__ prob, const float4* __restrict__ xs,
+                                                  const float* __restrict__ ws, const int32_t* __restrict__ cst,
+                                                  float4* St, float* Wt, float4* CP, int32_t* __restrict__ done) {
+  pdl_enter();
+  constexpr int B = brick_log2(D), NC = 1 << (D * B);
+  constexpr int NT = ((1 << (D * (B + 1))) - 1) / ((1 << D) - 1);  // cells of a brick on its B + 1 levels
+  __shared__ float sS[D][NT], sW[NT];  // finest level first
+  __shared__ int32_t big[NC], bq0[NC], bq1[NC];
+  __shared__ int nbig;
+  __shared__ bool last;
+  const int pb = find_problem(bbase, P, blockIdx.x);
   const ProbDev pr = prob[pb];
-  for (int l = min(pr.L - 1, small_level_max(D)); l >= 2; --l) {
+  const int L = pr.L, lb = min(L, B), Lb = L - lb;
+  const int64_t brick = (int64_t)blockIdx.x - bbase[pb];
+  int32_t bc[D];
+#pragma unroll
+  for (int m = 0; m < D; ++m) bc[m] = (int32_t)((brick >> (m * Lb)) & ((1 << Lb) - 1));
+  if (threadIdx.x == 0) nbig = 0;
+  __syncthreads();
+  // cell i of the brick on level l = L - j: row-major index in the level's grid
+  auto cell_index = [&](int i, int j) {
+    const int bits = lb - j;
+    int32_t c[D];
+#pragma unroll
+    for (int m = 0; m < D; ++m) c[m] = (bc[m] << bits) | ((i >> (m * bits)) & ((1 << bits) - 1));
+    return rowmajor<D>(c, 1 << (L - j));
+  };
+  auto store_charge = [&](int64_t c, int l, const float* S, float W) {
+    float z[4] = {0.f, 0.f, 0.f, 0.f};
+    if (W > 0.0f) {
+      const float iw = 1.0f / W;
+#pragma unroll
+      for (int m = 0; m < D; ++m) z[m] = S[m] * iw;
+    }
+    pair_store<D>(CP, pr.cbase + lvl_off(D, l) + c + pb + 1, z, W);
+  };
+  const int nc = 1 << (D * lb);
+  const int32_t* cs = cst + pr.fbase + pb;
+  for (int i = threadIdx.x; i < nc; i += kBlock) {
+    const int64_t c = cell_index(i, 0);
+    const int32_t q0 = cs[c], q1 = cs[c + 1];
+    if (q1 - q0 > kCellSerial) {
+      const int b = atomicAdd(&nbig, 1);
+      big[b] = i;
+      bq0[b] = q0;
+      bq1[b] = q1;
+      continue;
+    }
+    float S[4] = {0.f, 0.f, 0.f, 0.f};
+    float W = 0.f;
+    cell_sum<D>(xs, ws, q0, q1, 1, S, W);
+#pragma unroll
+    for (int m = 0; m < D; ++m) sS[m][i] = S[m];
+    sW[i] = W;
+    store_charge(c, L, S, W);
+  }
+  __syncthreads();
+  for (int b = threadIdx.x >> 5; b < nbig; b += kBlock / 32) {
+    float S[4] = {0.f, 0.f, 0.f, 0.f};
+    float W = 0.f;
+    cell_sum_warp<D>(xs, ws, bq0[b], bq1[b], S, W);
+    if (lane_id() == 0) {
+      const int i = big[b];
+#pragma unroll
+      for (int m = 0; m < D; ++m) sS[m][i] = S[m];
+      sW[i] = W;
+      store_charge(cell_index(i, 0), L, S, W);
+    }
+  }
+  int off = 0;  // first cell of level L - j + 1 in the shared sums
+  for (int j = 1; j <= lb && L - j >= 2; ++j) {
+    __syncthreads();
+    const int bits = lb - j, n = 1 << (D * bits), next = off + (1 << (D * (bits + 1)));
+    for (int i = threadIdx.x; i < n; i += kBlock) {
+      float S[4] = {0.f, 0.f, 0.f, 0.f};
+      float W = 0.f;
+#pragma unroll
+      for (int ch = 0; ch < (1 << D); ++ch) {
+        int q = 0;
+#pragma unroll
+        for (int m = 0; m < D; ++m)
+          q |= (2 * ((i >> (m * bits)) & ((1 << bits) - 1)) + ((ch >> m) & 1)) << (m * (bits + 1));
+#pragma unroll
+        for (int m = 0; m < D; ++m) S[m] += sS[m][off + q];
+        W += sW[off + q];
+      }
+#pragma unroll
+      for (int m = 0; m < D; ++m) sS[m][next + i] = S[m];
+      sW[next + i] = W;
+      store_charge(cell_index(i, j), L - j, S, W);
+    }
+    off = next;
+  }
+  if (Lb <= 2) return;  // every level down to 2 lies inside the bricks
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int64_t idx = pr.cbase + lvl_off(D, Lb) + brick;  // the brick's root is cell `brick` of level Lb
+    St[idx] = make_float4(sS[0][off], sS[1][off], D > 2 ? sS[D > 2 ? 2 : 0][off] : 0.f,
+                          D > 3 ? sS[D > 3 ? 3 : 0][off] : 0.f);
+    Wt[idx] = sW[off];
+    __threadfence();
+    last = atomicAdd(&done[pb], 1) == (1 << (D * Lb)) - 1;
+    if (last) {
+      done[pb] = 0;  // for the next step
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  if (!last) return;
+  for (int l = Lb - 1; l >= 2; --l) {
     const int64_t n = int64_t(1) << (D * l);
-    for (int64_t c = threadIdx.x; c < n; c += blockDim.x) agg_cell<D>(pr, pb, l, c, St, Wt, CP);
+    for (int64_t c = threadIdx.x; c < n; c += kBlock) agg_cell<D>(pr, pb, l, c, St, Wt, CP);
     __syncthreads();
   }
 }
@@ -467,7 +675,7 @@ __global__ void __launch_bounds__(kSortThreads) k_bin_small(
     uint32_t* __restrict__ keys, uint32_t* __restrict__ svals, float4* __restrict__ xs, float* __restrict__ ws,
     uint32_t* __restrict__ scell, int32_t* __restrict__ cst, float4* __restrict__ XP, float4* St, float* Wt,
     float4* CP) {
-  pdl_wait();
+  pdl_enter();
   extern __shared__ __align__(16) unsigned char bin_raw[];
   BinSmem& sm = *reinterpret_cast<BinSmem*>(bin_raw);
   const int pb = blockIdx.x;
@@ -631,7 +839,7 @@ __device__ __forceinline__ void pull_range(float* a, const float4& xv, const int
 __global__ void __launch_bounds__(kBlock) k_attract(const int32_t* __restrict__ adj_ptr, const int32_t* __restrict__ adj,
                                                     const float* __restrict__ acost, const float4* __restrict__ x,
                                                     int64_t K, float4* __restrict__ y) {
-  pdl_wait();
+  pdl_enter();
   int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= K) return;
   int32_t t0 = adj_ptr[v], t1 = adj_ptr[v + 1];
@@ -646,7 +854,7 @@ __global__ void __launch_bounds__(kBlock) k_attract_warp(const int32_t* __restri
                                                          const int32_t* __restrict__ adj_ptr,
                                                          const int32_t* __restrict__ adj, const float* __restrict__ acost,
                                                          const float4* __restrict__ x, float4* __restrict__ y) {
-  pdl_wait();
+  pdl_enter();
   int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= n) return;
   const int lane = lane_id();
@@ -666,7 +874,7 @@ __global__ void __launch_bounds__(kBlock) k_attract_block(const int32_t* __restr
                                                           const int32_t* __restrict__ adj,
                                                           const float* __restrict__ acost,
                                                           const float4* __restrict__ x, float4* __restrict__ y) {
-  pdl_wait();
+  pdl_enter();
   __shared__ float part[kBlock / 32][4];
   const int lane = lane_id(), warp = threadIdx.x >> 5;
   int32_t v = list[blockIdx.x];
@@ -706,7 +914,7 @@ __global__ void k_compact_flags(const int32_t* __restrict__ flag, const int32_t*
 // Net centres z_j of general nets (Algorithm 4).
 __global__ void k_net_center(const int32_t* __restrict__ net_ptr, const int32_t* __restrict__ pins, int64_t l,
                              const float4* __restrict__ x, float4* __restrict__ z) {
-  pdl_wait();
+  pdl_enter();
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= l) return;
   int32_t a = net_ptr[j], b = net_ptr[j + 1];
@@ -722,7 +930,7 @@ __global__ void k_net_center(const int32_t* __restrict__ net_ptr, const int32_t*
 __global__ void k_attract_hyper(const int32_t* __restrict__ vtx_ptr, const int32_t* __restrict__ vnets,
                                 const float4* __restrict__ x, const float4* __restrict__ z, int64_t K,
                                 float4* __restrict__ y) {
-  pdl_wait();
+  pdl_enter();
   int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= K) return;
   float4 xv = x[v];
@@ -1122,7 +1330,7 @@ __global__ void __launch_bounds__(kStepBlock, MLP ? 3 : VMO_STEP_MINBLOCKS) k_re
     const float* __restrict__ scale_tab, const int32_t* __restrict__ tctr,
     float step_override, float4* __restrict__ x, float4* __restrict__ y_out, uint32_t* __restrict__ bb_next,
     unsigned long long* __restrict__ icount) {
-  pdl_wait();
+  pdl_enter();
   constexpr int N = Pair<D>::N;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int pb = find_problem(tbase, P, t < T ? t : T - 1);
@@ -1625,7 +1833,7 @@ vmo_status level_setup(LevelBatch& lb, int d, int occ, cudaStream_t s) {
   lb.cbase.assign(P + 1, 0);
   lb.fbase.assign(P + 1, 0);
   std::vector<ProbDev> pd(P);
-  std::vector<int64_t> tb(P + 1, 0);
+  std::vector<int64_t> tb(P + 1, 0), bk(P + 1, 0);
   lb.maxL = 1;
   for (int p = 0; p < P; ++p) {
     int64_t k = lb.vbase[p + 1] - lb.vbase[p];
@@ -1643,26 +1851,17 @@ vmo_status level_setup(LevelBatch& lb, int d, int occ, cudaStream_t s) {
     pd[p].group = group_size(k);
     pd[p].tbase = tb[p];
     tb[p + 1] = tb[p] + ((k * pd[p].group + 31) / 32) * 32;
+    bk[p + 1] = bk[p] + (int64_t(1) << (d * std::max(L - brick_log2(d), 0)));
   }
   lb.threads = tb[P];
-  // prefix tables of the coarse-level aggregation steps: step s covers level L_p - s >= 2
-  int nsteps = std::max(lb.maxL - 2, 0);
-  std::vector<int64_t> off((size_t)(nsteps + 1) * (P + 1), 0);
-  for (int st = 1; st <= nsteps; ++st)
-    for (int p = 0; p < P; ++p) {
-      int l = lb.L[p] - st;
-      int64_t cnt = l > small_level_max(d) ? (int64_t(1) << (d * l)) : 0;
-      off[(size_t)st * (P + 1) + p + 1] = off[(size_t)st * (P + 1) + p] + cnt;
-    }
+  lb.bricks = bk[P];
   VMO_TRY(lb.prob.resize(std::max(P, 1)));
-  VMO_TRY(lb.aggoff.resize(off.size()));
   VMO_TRY(lb.vprob.resize((size_t)std::max<int64_t>(lb.K, 1)));
   VMO_CUDA(cudaMemcpyAsync(lb.prob.ptr, pd.data(), P * sizeof(ProbDev), cudaMemcpyHostToDevice, s));
-  VMO_CUDA(cudaMemcpyAsync(lb.aggoff.ptr, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s));
   VMO_TRY(lb.tbase.resize(P + 1));
   VMO_CUDA(cudaMemcpyAsync(lb.tbase.ptr, tb.data(), (P + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-  VMO_TRY(lb.fbase_dev.resize(P + 1));
-  VMO_CUDA(cudaMemcpyAsync(lb.fbase_dev.ptr, lb.fbase.data(), (P + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+  VMO_TRY(lb.bbase.resize(P + 1));
+  VMO_CUDA(cudaMemcpyAsync(lb.bbase.ptr, bk.data(), (P + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
   int64_t* vb;
   VMO_CUDA(cudaMallocAsync((void**)&vb, (P + 1) * sizeof(int64_t), s));
   g_device_allocs.fetch_add(1, std::memory_order_relaxed);
@@ -1734,15 +1933,12 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   const int d = o.d;
   if (K == 0 || iters <= 0) return VMO_OK;
   ScratchFrame frame(sc);
-  uint32_t *keys, *vals, *skeys, *svals, *scell, *bb;
+  uint32_t *keys, *arrival = nullptr, *slot = nullptr, *svals, *scell, *bb;
   float4 *xs, *XP, *yatt, *St, *CP, *z = nullptr;
   float *ws = nullptr, *Wt, *s0;
-  int32_t* cst;
-  int64_t *fb;
+  int32_t *cst, *cnt = nullptr, *tot = nullptr, *done = nullptr;
   const int64_t ncell = lb.cbase[P], nfine = lb.fbase[P];
   VMO_TRY(sc.alloc(&keys, K));
-  VMO_TRY(sc.alloc(&vals, K));
-  VMO_TRY(sc.alloc(&skeys, K));
   VMO_TRY(sc.alloc(&svals, K));
   VMO_TRY(sc.alloc(&scell, K));
   VMO_TRY(sc.alloc(&xs, K));
@@ -1756,7 +1952,6 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   VMO_TRY(sc.alloc(&bb, (size_t)2 * 8 * P));
   VMO_TRY(sc.alloc(&s0, P));
   if (lb.net_ptr) VMO_TRY(sc.alloc(&z, std::max<int64_t>(lb.nnets, 1)));
-  fb = lb.fbase_dev.ptr;
   // levels whose problems all fit one sort tile are binned by one block per
   // problem (k_bin_small) when the tuning allows it
   int64_t kmax = 0;
@@ -1772,9 +1967,18 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
         bin1 = false;  // the device-wide sequence then
       }
     });
-  SortSegments segs;
-  bool segmented = P > 1;
-  if (segmented && !bin1) VMO_TRY(make_sort_segments(lb.vbase, &segs, s, sc));
+  const int64_t ncnt = nfine + P;  // entries of the cell start table
+  const bool one_cluster = ncnt <= kCellScanMax;
+  const unsigned scan_blocks = grid_for(ncnt, kCellScanThreads * kCellScanItems);
+  if (!bin1) {
+    VMO_TRY(sc.alloc(&arrival, K));
+    VMO_TRY(sc.alloc(&slot, K));
+    VMO_TRY(sc.alloc(&cnt, ncnt));
+    VMO_TRY(sc.alloc(&done, P));
+    if (!one_cluster) VMO_TRY(sc.alloc(&tot, scan_blocks));
+    VMO_CUDA(cudaMemsetAsync(cnt, 0, ncnt * sizeof(int32_t), s));
+    VMO_CUDA(cudaMemsetAsync(done, 0, P * sizeof(int32_t), s));
+  }
   const int nreset = 8 * P;
   launch(k_bbox_reset, grid_for(16 * P, kBlock), kBlock, 0, s, bb, 16 * P);
   VMO_LAUNCHED("bbox_reset");
@@ -1832,35 +2036,21 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
                keys_out && t == 0 ? keys : nullptr, svals, xs, ws, scell, cst, XP, St, Wt, CP);
         if (keys_out && t == 0) cudaMemcpyAsync(keys_out, keys, K * 4, cudaMemcpyDeviceToDevice, ms);
       } else {
-        if (K >= kKeyItemsMin)
-          launch(k_keys<D, 4>, grid_for((K + 3) / 4, kBlock), kBlock, 0, ms, x, K, lb.vprob.ptr, lb.prob.ptr, cur, keys,
-                 vals, nxt, nreset, tctr);
-        else
-          launch(k_keys<D, 1>, grid_for(K, kBlock), kBlock, 0, ms, x, K, lb.vprob.ptr, lb.prob.ptr, cur, keys, vals, nxt,
-                 nreset, tctr);
+        auto keys_kernel = K >= kKeyItemsMin ? k_keys<D, 4> : k_keys<D, 1>;
+        launch(keys_kernel, grid_for(K >= kKeyItemsMin ? (K + 3) / 4 : K, kBlock), kBlock, 0, ms, x, K, lb.vprob.ptr,
+               lb.prob.ptr, cur, keys, arrival, cnt, nxt, nreset, tctr);
         if (keys_out && t == 0) cudaMemcpyAsync(keys_out, keys, K * 4, cudaMemcpyDeviceToDevice, ms);
-        bool in_b = false;
-        VMO_TRY(radix_sort_u32_pingpong(keys, vals, skeys, svals, K, D * lb.maxL, segmented ? &segs : nullptr, &in_b,
-                                        ms, sc));
-        if (!in_b) {  // sorted pairs are in (keys, vals): use them as (skeys, svals) from here on
-          std::swap(keys, skeys);
-          std::swap(vals, svals);
+        if (one_cluster) {
+          launch(k_cell_scan, kCellScanCtas, kCellScanThreads, 0, ms, cnt, cst, ncnt);
+        } else {
+          launch(k_cell_totals, scan_blocks, kCellScanThreads, 0, ms, cnt, ncnt, tot);
+          launch(k_cell_starts, scan_blocks, kCellScanThreads, 0, ms, cnt, ncnt, tot, cst);
         }
-        launch(k_gather<D>, grid_for(K, kBlock), kBlock, 0, ms, svals, skeys, K, x, lb.w, lb.vprob.ptr, lb.prob.ptr,
-               cur, xs, ws, scell, cst, XP);
-        launch(k_agg_finest<D>, grid_for(nfine, kBlock), kBlock, 0, ms, nfine, fb, P, lb.prob.ptr, xs, ws, cst, St, Wt,
-               CP);
-        for (int stp = 1; stp <= lb.maxL - 2; ++stp) {
-          const int64_t* off = lb.aggoff.ptr + (size_t)stp * (P + 1);
-          int64_t n = 0;
-          for (int p = 0; p < P; ++p) {
-            int l = lb.L[p] - stp;
-            n += l > small_level_max(D) ? (int64_t(1) << (D * l)) : 0;
-          }
-          if (n == 0) continue;
-          launch(k_agg_level<D>, grid_for(n, kBlock), kBlock, 0, ms, stp, off, P, n, lb.prob.ptr, St, Wt, CP);
-        }
-        if (lb.maxL >= 3) launch(k_agg_small<D>, (unsigned)P, kBlock, 0, ms, lb.prob.ptr, St, Wt, CP);
+        launch(k_slots, grid_for(K, kBlock), kBlock, 0, ms, keys, arrival, K, lb.vprob.ptr, lb.prob.ptr, cst, slot);
+        launch(k_place<D>, grid_for(K, kBlock), kBlock, 0, ms, slot, keys, K, x, lb.w, lb.vprob.ptr, lb.prob.ptr, cst,
+               cnt, ncnt, svals, xs, ws, scell, XP);
+        launch(k_cells<D>, (unsigned)lb.bricks, kBlock, 0, ms, lb.bbase.ptr, P, lb.prob.ptr, xs, ws, cst, St, Wt, CP,
+               done);
       }
       if (side) cudaStreamWaitEvent(ms, ev_join, 0);
       const bool timed = stats_timing();

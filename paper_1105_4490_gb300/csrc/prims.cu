@@ -5,11 +5,9 @@
 // and stores are coalesced).
 //
 // Radix sort: 8-bit digits, one histogram kernel and one scatter kernel per
-// pass plus a scan of the (segment, digit, tile)-ordered histogram.  The
-// scatter ranks keys stably inside a warp with __match_any_sync, so equal keys
-// keep their input order.  Tiles never straddle a segment, so with the
-// histogram laid out segment-major the same kernels sort many independent
-// segments (one per problem of a batch) in one launch sequence.
+// pass plus a scan of the (digit, tile)-ordered histogram.  The scatter ranks
+// keys stably inside a warp with __match_any_sync, so equal keys keep their
+// input order.
 #include <algorithm>
 
 #include <type_traits>
@@ -108,102 +106,29 @@ vmo_status scan_impl(const T* in, T* out, int64_t n, T* total, cudaStream_t s, S
 // 2 passes of 9 bits).
 constexpr int kMaxRadixBits = 10;
 
-struct TileInfo {
-  int64_t start;
-  int32_t count;
-  int64_t hist_base;  // index of (digit 0, this tile) in the histogram
-  int32_t stride;     // distance between digits (tiles in the segment)
-};
-
-__device__ inline TileInfo tile_info(const SortSegments& sg, int64_t n, int64_t t, int radix) {
-  TileInfo ti;
-  if (sg.tile_seg == nullptr) {
-    ti.start = t * kSortTile;
-    int64_t c = n - ti.start;
-    ti.count = (int32_t)(c < kSortTile ? c : kSortTile);
-    ti.hist_base = t;
-    ti.stride = (int32_t)sg.ntiles;
-  } else {
-    int32_t seg = sg.tile_seg[t];
-    int32_t t0 = sg.seg_tile0[seg], nt = sg.seg_tile0[seg + 1] - t0;
-    ti.start = sg.tile_start[t];
-    ti.count = sg.tile_count[t];
-    ti.hist_base = (int64_t)t0 * radix + (t - t0);
-    ti.stride = nt;
-  }
-  return ti;
-}
-
 template <class K, int BITS>
-__global__ void radix_hist_kernel(const K* __restrict__ keys, int64_t n, int shift, SortSegments sg,
-                                  uint32_t* __restrict__ hist) {
-  pdl_wait();
+__global__ void radix_hist_kernel(const K* __restrict__ keys, int64_t n, int shift, uint32_t* __restrict__ hist) {
   constexpr int R = 1 << BITS;
   __shared__ uint32_t h[R];
   for (int i = threadIdx.x; i < R; i += blockDim.x) h[i] = 0;
   __syncthreads();
-  TileInfo ti = tile_info(sg, n, blockIdx.x, R);
-  for (int i = threadIdx.x; i < ti.count; i += blockDim.x) {
-    uint32_t dg = (uint32_t)(keys[ti.start + i] >> shift) & (R - 1);
+  const int64_t start = (int64_t)blockIdx.x * kSortTile;
+  const int count = (int)min((int64_t)kSortTile, n - start);
+  for (int i = threadIdx.x; i < count; i += blockDim.x) {
+    uint32_t dg = (uint32_t)(keys[start + i] >> shift) & (R - 1);
     atomicAdd(&h[dg], 1u);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < R; i += blockDim.x) hist[ti.hist_base + (int64_t)i * ti.stride] = h[i];
+  for (int i = threadIdx.x; i < R; i += blockDim.x) hist[(int64_t)i * gridDim.x + blockIdx.x] = h[i];
 }
 
-// Row prefix of the tile histograms: one thread per (segment, digit) row
-// (the counts of that digit in the segment's tiles, contiguous): exclusive
-// prefix in place, row total to rowtot.
-__global__ void radix_rowscan(uint32_t* __restrict__ hist, SortSegments sg, int R, int64_t nrows,
-                              uint32_t* __restrict__ rowtot) {
-  pdl_wait();
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrows) return;
-  const int seg = (int)(r / R), d = (int)(r % R);
-  int64_t t0 = 0, nt = sg.ntiles;
-  if (sg.tile_seg) {
-    t0 = sg.seg_tile0[seg];
-    nt = sg.seg_tile0[seg + 1] - t0;
-  }
-  if (nt > kLongSegTiles || nt <= 1) return;  // long: radix_rowscan_warp; single tile: the scatter's own counts
-  uint32_t* row = hist + t0 * R + (int64_t)d * nt;
-  uint32_t run = 0;
-  int64_t t = 0;
-  for (; t + 4 <= nt; t += 4) {
-    const uint32_t c0 = row[t], c1 = row[t + 1], c2 = row[t + 2], c3 = row[t + 3];
-    row[t] = run;
-    run += c0;
-    row[t + 1] = run;
-    run += c1;
-    row[t + 2] = run;
-    run += c2;
-    row[t + 3] = run;
-    run += c3;
-  }
-  for (; t < nt; ++t) {
-    const uint32_t c = row[t];
-    row[t] = run;
-    run += c;
-  }
-  rowtot[r] = run;
-}
-
-// Same for the rows of long segments (more than kLongSegTiles tiles), one
-// warp per row; nrows = R x the long segments (all rows when unsegmented).
-__global__ void radix_rowscan_warp(uint32_t* __restrict__ hist, SortSegments sg, int R, int64_t nrows,
-                                   uint32_t* __restrict__ rowtot) {
-  pdl_wait();
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= nrows) return;
+// Row prefix of the tile histograms: one warp per digit (its counts in the nt
+// tiles, contiguous): exclusive prefix in place, row total to rowtot.
+__global__ void radix_rowscan(uint32_t* __restrict__ hist, int64_t nt, int R, uint32_t* __restrict__ rowtot) {
+  const int64_t d = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (d >= R) return;
   const int lane = lane_id();
-  const int seg = sg.tile_seg ? sg.long_seg[w / R] : 0, d = (int)(w % R);
-  const int64_t r = (int64_t)seg * R + d;
-  int64_t t0 = 0, nt = sg.ntiles;
-  if (sg.tile_seg) {
-    t0 = sg.seg_tile0[seg];
-    nt = sg.seg_tile0[seg + 1] - t0;
-  }
-  uint32_t* row = hist + t0 * R + (int64_t)d * nt;
+  uint32_t* row = hist + d * nt;
   uint32_t carry = 0;
   for (int64_t b = 0; b < nt; b += 32) {
     const int64_t t = b + lane;
@@ -212,15 +137,14 @@ __global__ void radix_rowscan_warp(uint32_t* __restrict__ hist, SortSegments sg,
     if (t < nt) row[t] = carry + inc - c;
     carry += __shfl_sync(0xffffffffu, inc, 31);
   }
-  if (lane == 0) rowtot[r] = carry;
+  if (lane == 0) rowtot[d] = carry;
 }
 
 template <class K, bool HasVal, int BITS>
 __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(
     const K* __restrict__ keys, const uint32_t* __restrict__ vals, K* __restrict__ keys_out,
-    uint32_t* __restrict__ vals_out, int64_t n, int shift, SortSegments sg, const uint32_t* __restrict__ offs,
+    uint32_t* __restrict__ vals_out, int64_t n, int shift, const uint32_t* __restrict__ offs,
     const uint32_t* __restrict__ rowtot) {
-  pdl_wait();
   constexpr int R = 1 << BITS;
   constexpr int PER = (R + kSortThreads - 1) / kSortThreads;
   // the per-warp digit counts, then (once every element knows its place) the
@@ -237,28 +161,25 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(
   __shared__ uint32_t ws[33];
   const int lane = lane_id(), warp = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < kSortWarps * R; i += blockDim.x) (&wcnt[0][0])[i] = 0;
-  TileInfo ti = tile_info(sg, n, blockIdx.x, R);
-  const int seg = sg.tile_seg ? sg.tile_seg[blockIdx.x] : 0;
-  const int64_t seg_start = sg.seg_base ? sg.seg_base[seg] : 0;
-  const int64_t seg_tiles = sg.tile_seg ? sg.seg_tile0[seg + 1] - sg.seg_tile0[seg] : sg.ntiles;
-  const bool single = seg_tiles == 1;  // the tile is its whole segment: bases from its own counts
-  // destination of digit d in this tile: segment start + keys of the segment
-  // with a smaller digit (scan of the row totals) + keys of digit d in the
-  // segment's earlier tiles (row prefix)
+  const int64_t start = (int64_t)blockIdx.x * kSortTile;
+  const int count = (int)min((int64_t)kSortTile, n - start);
+  const bool single = gridDim.x == 1;  // one tile: bases from its own counts
+  // destination of digit d in this tile: keys with a smaller digit (scan of
+  // the row totals) + keys of digit d in the earlier tiles (row prefix)
   if (!single) {
     uint32_t v[PER];
     uint32_t sum = 0;
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
       const int d = threadIdx.x * PER + j;
-      v[j] = d < R ? rowtot[(int64_t)seg * R + d] : 0u;
+      v[j] = d < R ? rowtot[d] : 0u;
       sum += v[j];
     }
-    uint32_t ex = block_exclusive<uint32_t>(sum, ws, nullptr) + (uint32_t)seg_start;
+    uint32_t ex = block_exclusive<uint32_t>(sum, ws, nullptr);
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
       const int d = threadIdx.x * PER + j;
-      if (d < R) tbase[d] = ex + offs[ti.hist_base + (int64_t)d * ti.stride];
+      if (d < R) tbase[d] = ex + offs[(int64_t)d * gridDim.x + blockIdx.x];
       ex += v[j];
     }
   }
@@ -271,9 +192,9 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(
 #pragma unroll
   for (int j = 0; j < kSortItems; ++j) {
     int idx = warp * (32 * kSortItems) + j * 32 + lane;
-    bool valid = idx < ti.count;
-    key[j] = valid ? keys[ti.start + idx] : K(0);
-    if (HasVal) val[j] = valid ? vals[ti.start + idx] : 0u;
+    bool valid = idx < count;
+    key[j] = valid ? keys[start + idx] : K(0);
+    if (HasVal) val[j] = valid ? vals[start + idx] : 0u;
     uint32_t dg = valid ? ((uint32_t)(key[j] >> shift) & (R - 1)) : (uint32_t)R;
     dig[j] = dg;
     unsigned peers = __match_any_sync(0xffffffffu, dg);
@@ -311,7 +232,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(
       const int d = threadIdx.x * PER + j;
       if (d < R) {
         lbase[d] = ex;
-        if (single) tbase[d] = ex + (uint32_t)seg_start;
+        if (single) tbase[d] = ex;
       }
       ex += v[j];
     }
@@ -331,7 +252,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(
     if (HasVal) sval[lpos[j]] = val[j];
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < ti.count; e += blockDim.x) {
+  for (int e = threadIdx.x; e < count; e += blockDim.x) {
     const K k = skey[e];
     const uint32_t d = (uint32_t)(k >> shift) & (R - 1);
     const uint32_t dst = tbase[d] + ((uint32_t)e - lbase[d]);
@@ -340,26 +261,23 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(
   }
 }
 
-// Whole sort of one tile that is its own segment (at most 2,048 keys), all
-// passes of 8-bit digits in shared memory, by one block: the sort of the
-// small levels of a layout (one launch instead of three per pass).  Ranks
+// Whole sort of at most one tile (2,048 keys), all passes of 8-bit digits in
+// shared memory, by one block (one launch instead of three per pass).  Ranks
 // within a digit follow the input order exactly as in radix_scatter_kernel.
 __global__ void __launch_bounds__(kSortThreads) radix_tile_sort_kernel(const uint32_t* __restrict__ keys,
                                                                        const uint32_t* __restrict__ vals,
                                                                        uint32_t* __restrict__ keys_out,
-                                                                       uint32_t* __restrict__ vals_out, int64_t n,
-                                                                       int bits, SortSegments sg) {
-  pdl_wait();
+                                                                       uint32_t* __restrict__ vals_out, int n,
+                                                                       int bits) {
   __shared__ TileSortSmem sm;
-  const TileInfo ti = tile_info(sg, n, blockIdx.x, 256);
-  for (int i = threadIdx.x; i < ti.count; i += blockDim.x) {
-    sm.key[0][i] = keys[ti.start + i];
-    sm.val[0][i] = vals[ti.start + i];
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    sm.key[0][i] = keys[i];
+    sm.val[0][i] = vals[i];
   }
-  const int cur = tile_sort_smem(sm, ti.count, bits);
-  for (int i = threadIdx.x; i < ti.count; i += blockDim.x) {
-    keys_out[ti.start + i] = sm.key[cur][i];
-    vals_out[ti.start + i] = sm.val[cur][i];
+  const int cur = tile_sort_smem(sm, n, bits);
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    keys_out[i] = sm.key[cur][i];
+    vals_out[i] = sm.val[cur][i];
   }
 }
 
@@ -372,54 +290,41 @@ inline int digit_bits(int bits, int* passes) {
 }
 
 template <class K, int BITS>
-void radix_pass(const K* ka, const uint32_t* va, K* kb, uint32_t* vb, int64_t n, int shift, const SortSegments& sg,
+void radix_pass(const K* ka, const uint32_t* va, K* kb, uint32_t* vb, int64_t n, int shift, int64_t ntiles,
                 uint32_t* hist, uint32_t* rowtot, cudaStream_t s) {
   constexpr int R = 1 << BITS;
-  const int64_t nrows = (int64_t)(sg.tile_seg ? sg.nseg : 1) * R;
-  launch(radix_hist_kernel<K, BITS>, (unsigned)sg.ntiles, 256, 0, s, ka, n, shift, sg, hist);
-  const int64_t nlong = sg.tile_seg ? sg.nlong : (sg.ntiles > kLongSegTiles ? 1 : 0);
-  if (nlong > 0)
-    launch(radix_rowscan_warp, (unsigned)((nlong * R * 32 + 255) / 256), 256, 0, s, hist, sg, R, nlong * R, rowtot);
-  if (sg.tile_seg ? sg.nmid > 0 : (sg.ntiles > 1 && nlong == 0))
-    launch(radix_rowscan, (unsigned)((nrows + 255) / 256), 256, 0, s, hist, sg, R, nrows, rowtot);
+  launch(radix_hist_kernel<K, BITS>, (unsigned)ntiles, 256, 0, s, ka, n, shift, hist);
+  if (ntiles > 1) launch(radix_rowscan, (unsigned)((R * 32 + 255) / 256), 256, 0, s, hist, ntiles, R, rowtot);
   if (va)
-    launch(radix_scatter_kernel<K, true, BITS>, (unsigned)sg.ntiles, kSortThreads, 0, s, ka, va, kb, vb, n, shift, sg,
-           hist, rowtot);
+    launch(radix_scatter_kernel<K, true, BITS>, (unsigned)ntiles, kSortThreads, 0, s, ka, va, kb, vb, n, shift, hist,
+           rowtot);
   else
-    launch(radix_scatter_kernel<K, false, BITS>, (unsigned)sg.ntiles, kSortThreads, 0, s, ka, nullptr, kb, nullptr, n,
-           shift, sg, hist, rowtot);
+    launch(radix_scatter_kernel<K, false, BITS>, (unsigned)ntiles, kSortThreads, 0, s, ka, nullptr, kb, nullptr, n,
+           shift, hist, rowtot);
 }
 
 template <class K>
 vmo_status radix_sort_impl(K* keys_in, uint32_t* vals_in, K* keys_out, uint32_t* vals_out, int64_t n, int bits,
-                           const SortSegments* segs, cudaStream_t s, Scratch& sc, bool* in_b = nullptr) {
-  if (in_b) *in_b = false;
+                           cudaStream_t s, Scratch& sc) {
   if (n <= 0) return VMO_OK;
-  SortSegments sg;
-  if (segs) sg = *segs;
-  if (sg.tile_seg == nullptr) sg.ntiles = (n + kSortTile - 1) / kSortTile;
+  const int64_t ntiles = (n + kSortTile - 1) / kSortTile;
   int passes = 0;
   const int B = bits > 0 ? digit_bits(bits, &passes) : 8;
   if (passes == 0) {
-    if (in_b) return VMO_OK;  // already sorted, left in place
     VMO_CUDA(cudaMemcpyAsync(keys_out, keys_in, n * sizeof(K), cudaMemcpyDeviceToDevice, s));
     if (vals_in) VMO_CUDA(cudaMemcpyAsync(vals_out, vals_in, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
     return VMO_OK;
   }
   if constexpr (std::is_same<K, uint32_t>::value) {
-    // every segment one tile: the whole sort of each tile in one block
-    const bool one_tile = sg.tile_seg ? (sg.nlong == 0 && sg.nmid == 0) : (sg.ntiles == 1);
-    if (one_tile && vals_in && bits <= 32) {
-      launch(radix_tile_sort_kernel, (unsigned)sg.ntiles, kSortThreads, 0, s, keys_in, vals_in, keys_out, vals_out, n,
-             bits, sg);
+    if (ntiles == 1 && vals_in && bits <= 32) {
+      launch(radix_tile_sort_kernel, 1, kSortThreads, 0, s, keys_in, vals_in, keys_out, vals_out, (int)n, bits);
       VMO_LAUNCHED("radix_tile_sort");
-      if (in_b) *in_b = true;
       return VMO_OK;
     }
   }
   uint32_t *hist, *rowtot;
-  VMO_TRY(sc.alloc(&hist, (size_t)(sg.ntiles << B)));
-  VMO_TRY(sc.alloc(&rowtot, (size_t)(sg.tile_seg ? sg.nseg : 1) << B));
+  VMO_TRY(sc.alloc(&hist, (size_t)(ntiles << B)));
+  VMO_TRY(sc.alloc(&rowtot, (size_t)1 << B));
   K* ka = keys_in;
   K* kb = keys_out;
   uint32_t* va = vals_in;
@@ -427,18 +332,14 @@ vmo_status radix_sort_impl(K* keys_in, uint32_t* vals_in, K* keys_out, uint32_t*
   for (int p = 0; p < passes; ++p) {
     const int shift = p * B;
     switch (B) {
-      case 6: radix_pass<K, 6>(ka, va, kb, vb, n, shift, sg, hist, rowtot, s); break;
-      case 8: radix_pass<K, 8>(ka, va, kb, vb, n, shift, sg, hist, rowtot, s); break;
-      case 9: radix_pass<K, 9>(ka, va, kb, vb, n, shift, sg, hist, rowtot, s); break;
-      default: radix_pass<K, 10>(ka, va, kb, vb, n, shift, sg, hist, rowtot, s); break;
+      case 6: radix_pass<K, 6>(ka, va, kb, vb, n, shift, ntiles, hist, rowtot, s); break;
+      case 8: radix_pass<K, 8>(ka, va, kb, vb, n, shift, ntiles, hist, rowtot, s); break;
+      case 9: radix_pass<K, 9>(ka, va, kb, vb, n, shift, ntiles, hist, rowtot, s); break;
+      default: radix_pass<K, 10>(ka, va, kb, vb, n, shift, ntiles, hist, rowtot, s); break;
     }
     VMO_LAUNCHED("radix_sort");
     K* tk = ka; ka = kb; kb = tk;
     uint32_t* tv = va; va = vb; vb = tv;
-  }
-  if (in_b) {
-    *in_b = ka == keys_out;
-    return VMO_OK;
   }
   if (ka != keys_out) {
     VMO_CUDA(cudaMemcpyAsync(keys_out, ka, n * sizeof(K), cudaMemcpyDeviceToDevice, s));
@@ -481,79 +382,13 @@ vmo_status scan_inclusive_u64_into(const uint64_t* in, uint64_t* out, int64_t n,
 int64_t scan_partials_needed(int64_t n) { return (n + kScanTile - 1) / kScanTile; }
 
 vmo_status radix_sort_u32(uint32_t* keys_in, uint32_t* vals_in, uint32_t* keys_out, uint32_t* vals_out, int64_t n,
-                          int bits, const SortSegments* segs, cudaStream_t s, Scratch& sc) {
-  return radix_sort_impl<uint32_t>(keys_in, vals_in, keys_out, vals_out, n, bits, segs, s, sc);
-}
-
-vmo_status radix_sort_u32_pingpong(uint32_t* keys_a, uint32_t* vals_a, uint32_t* keys_b, uint32_t* vals_b, int64_t n,
-                                  int bits, const SortSegments* segs, bool* in_b, cudaStream_t s, Scratch& sc) {
-  return radix_sort_impl<uint32_t>(keys_a, vals_a, keys_b, vals_b, n, bits, segs, s, sc, in_b);
+                          int bits, cudaStream_t s, Scratch& sc) {
+  return radix_sort_impl<uint32_t>(keys_in, vals_in, keys_out, vals_out, n, bits, s, sc);
 }
 
 vmo_status radix_sort_u64(uint64_t* keys_in, uint32_t* vals_in, uint64_t* keys_out, uint32_t* vals_out, int64_t n,
                           int bits, cudaStream_t s, Scratch& sc) {
-  return radix_sort_impl<uint64_t>(keys_in, vals_in, keys_out, vals_out, n, bits, nullptr, s, sc);
-}
-
-vmo_status make_sort_segments(const std::vector<int64_t>& base, SortSegments* out, cudaStream_t s, Scratch& sc) {
-  int32_t nseg = (int32_t)base.size() - 1;
-  std::vector<int32_t> tseg, tcount, t0(nseg + 1);
-  std::vector<int64_t> tstart;
-  for (int32_t g = 0; g < nseg; ++g) {
-    t0[g] = (int32_t)tseg.size();
-    int64_t a = base[g], b = base[g + 1];
-    for (int64_t x = a; x < b; x += kSortTile) {
-      tseg.push_back(g);
-      tstart.push_back(x);
-      tcount.push_back((int32_t)std::min<int64_t>(kSortTile, b - x));
-    }
-  }
-  t0[nseg] = (int32_t)tseg.size();
-  int64_t nt = (int64_t)tseg.size();
-  if (nt == 0) {  // all segments empty: one empty tile keeps the kernels well-formed
-    tseg.push_back(0); tstart.push_back(0); tcount.push_back(0);
-    t0[nseg] = 1;
-    for (int32_t g = 1; g < nseg; ++g) t0[g] = 1;
-    nt = 1;
-  }
-  int32_t *d_tseg, *d_tcount, *d_t0;
-  int64_t *d_tstart, *d_base;
-  VMO_TRY(sc.alloc(&d_tseg, nt));
-  VMO_TRY(sc.alloc(&d_tcount, nt));
-  VMO_TRY(sc.alloc(&d_tstart, nt));
-  VMO_TRY(sc.alloc(&d_t0, nseg + 1));
-  VMO_TRY(sc.alloc(&d_base, nseg + 1));
-  VMO_CUDA(cudaMemcpyAsync(d_tseg, tseg.data(), nt * 4, cudaMemcpyHostToDevice, s));
-  VMO_CUDA(cudaMemcpyAsync(d_tcount, tcount.data(), nt * 4, cudaMemcpyHostToDevice, s));
-  VMO_CUDA(cudaMemcpyAsync(d_tstart, tstart.data(), nt * 8, cudaMemcpyHostToDevice, s));
-  VMO_CUDA(cudaMemcpyAsync(d_t0, t0.data(), (nseg + 1) * 4, cudaMemcpyHostToDevice, s));
-  VMO_CUDA(cudaMemcpyAsync(d_base, base.data(), (nseg + 1) * 8, cudaMemcpyHostToDevice, s));
-  // host vectors must outlive the asynchronous copies
-  VMO_CUDA(cudaStreamSynchronize(s));
-  out->nseg = nseg;
-  out->seg_base = d_base;
-  out->tile_seg = d_tseg;
-  out->tile_start = d_tstart;
-  out->tile_count = d_tcount;
-  out->seg_tile0 = d_t0;
-  out->ntiles = nt;
-  std::vector<int32_t> lg;
-  int32_t nmid = 0;
-  for (int32_t g = 0; g < nseg; ++g) {
-    const int32_t tiles = t0[g + 1] - t0[g];
-    if (tiles > kLongSegTiles) lg.push_back(g);
-    else if (tiles > 1) ++nmid;
-  }
-  out->nlong = (int32_t)lg.size();
-  out->nmid = nmid;
-  if (!lg.empty()) {
-    int32_t* d_lg;
-    VMO_TRY(sc.alloc(&d_lg, lg.size()));
-    VMO_CUDA(cudaMemcpyAsync(d_lg, lg.data(), lg.size() * 4, cudaMemcpyHostToDevice, s));
-    VMO_CUDA(cudaStreamSynchronize(s));  // lg must outlive the copy
-    out->long_seg = d_lg;
-  }
-  return VMO_OK;
+  return radix_sort_impl<uint64_t>(keys_in, vals_in, keys_out, vals_out, n, bits, s, sc);
 }
 
 }  // namespace vmo

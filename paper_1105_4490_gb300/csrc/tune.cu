@@ -1,6 +1,6 @@
 // Autotuner of the launch shapes that never change a result: the largest
 // step launch that takes the two-rows-in-flight variant of the step kernel,
-// the widest radix digit of the binning sort, the positions per thread of
+// the widest radix digit, the positions per thread of
 // the Lloyd assignment, and the largest problem whose level is binned by one
 // block per problem.  Every candidate orders the caller's matrices
 // through vmo_batch_order; the fastest (median of the repetitions, CUDA

@@ -188,38 +188,15 @@ vmo_status scan_inclusive(const T* in, T* out, int64_t n, cudaStream_t s, Scratc
 vmo_status scan_inclusive_u64_into(const uint64_t* in, uint64_t* out, int64_t n, uint64_t* partial, cudaStream_t s);
 int64_t scan_partials_needed(int64_t n);
 
-// Segment map for the radix sort: tiles never straddle segments.
-struct SortSegments {
-  int32_t nseg = 1;               // number of segments
-  const int64_t* seg_base = nullptr;  // device, nseg+1 element offsets (null: one segment [0, n))
-  const int32_t* tile_seg = nullptr;  // device, per tile: segment
-  const int64_t* tile_start = nullptr;// device, per tile: first element
-  const int32_t* tile_count = nullptr;// device, per tile: elements
-  const int32_t* seg_tile0 = nullptr; // device, per segment: first tile (nseg+1)
-  int64_t ntiles = 0;
-  const int32_t* long_seg = nullptr;  // device, segments of more than kLongSegTiles tiles
-  int32_t nlong = 0;
-  int32_t nmid = 0;                   // segments of 2..kLongSegTiles tiles
-};
-constexpr int kLongSegTiles = 16;
 constexpr int kSortTile = 2048;  // 256 threads x 8 keys
 
-// Stable LSD radix sort of (key, value) pairs on bits [0, bits).  Keys are
-// sorted within each segment.  Buffers are ping-ponged; the sorted result ends
-// in (keys_out, vals_out).  vals may be null (keys only).
+// Stable LSD radix sort of (key, value) pairs on bits [0, bits).  Buffers are
+// ping-ponged; the sorted result ends in (keys_out, vals_out).  vals may be
+// null (keys only).
 vmo_status radix_sort_u32(uint32_t* keys_in, uint32_t* vals_in, uint32_t* keys_out, uint32_t* vals_out,
-                          int64_t n, int bits, const SortSegments* segs, cudaStream_t s, Scratch& sc);
-// Same sort without the final copy: the sorted keys and values are left in
-// (keys_b, vals_b) if *in_b, else in (keys_a, vals_a); the other pair is
-// overwritten.
-vmo_status radix_sort_u32_pingpong(uint32_t* keys_a, uint32_t* vals_a, uint32_t* keys_b, uint32_t* vals_b, int64_t n,
-                                  int bits, const SortSegments* segs, bool* in_b, cudaStream_t s, Scratch& sc);
+                          int64_t n, int bits, cudaStream_t s, Scratch& sc);
 vmo_status radix_sort_u64(uint64_t* keys_in, uint32_t* vals_in, uint64_t* keys_out, uint32_t* vals_out,
                           int64_t n, int bits, cudaStream_t s, Scratch& sc);
-
-// Build SortSegments for segments given by host base offsets.
-vmo_status make_sort_segments(const std::vector<int64_t>& seg_base_host, SortSegments* out, cudaStream_t s,
-                              Scratch& sc);
 
 // ---------------------------------------------------------------------------
 // Instrumentation: every kernel launch of the library goes through launch(),
@@ -258,6 +235,13 @@ struct PdlScope {
 };
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// pdl_wait(), then lets the next kernel of the stream be placed as soon as
+// every block of this one has started (it waits in its own pdl_wait until this
+// kernel has completed, so its launch overlaps this kernel's last wave).
+__device__ __forceinline__ void pdl_enter() {
+  pdl_wait();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 template <class... KArgs, class... Args>
 inline void launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {

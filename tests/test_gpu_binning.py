@@ -1,0 +1,77 @@
+"""Device-wide binning of a layout step (cell counts, scan, vertex order within
+the cell, cell sums by bricks) at the sizes where it can go wrong: grids of
+fewer levels than a brick, one and several levels above the bricks, tables of
+one scan tile, of several and of more than one cluster takes, cells of one
+point, of just over the serial limit and of thousands, and, with all points in
+one problem of at most 2,048 vertices, the same bits as the one-block binning."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-4  # normwise, the stated tolerance of one layout step
+
+
+@pytest.fixture(scope="module")
+def V():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1105_4490_gb300 as P
+    assert torch.cuda.is_available()
+    t0 = P.get_tuning()
+    yield P
+    P.set_tuning(**t0)
+
+
+@pytest.fixture(scope="module")
+def O():
+    import oracle
+    oracle.build()
+    return oracle
+
+
+def _clustered(k, d, seed, share):
+    """`share` of the points in three tight clusters, the others uniform."""
+    rng = np.random.default_rng(seed)
+    x = np.zeros((k, 4), dtype=np.float32)
+    side = float(k) ** (1.0 / d)
+    x[:, :d] = rng.random((k, d)) * side
+    n = int(share * k)
+    x[:n, :d] = side * (0.2 + 0.3 * rng.integers(0, 3, n)[:, None]) + 0.02 * side * rng.standard_normal((n, d))
+    return x[rng.permutation(k)]
+
+
+@pytest.mark.parametrize("d,k,occ,share", [
+    (2, 3, 8, 0.0), (2, 33, 8, 0.0), (2, 2049, 8, 0.3), (2, 9000, 1, 0.5),
+    (3, 17, 8, 0.0), (3, 65, 8, 0.0), (3, 2600, 8, 0.9), (3, 30000, 8, 0.2), (3, 40000, 1, 0.1),
+    (4, 40, 8, 0.0), (4, 5000, 8, 0.5), (4, 70000, 1, 0.02)])
+def test_device_wide_binning(V, O, d, k, occ, share):
+    A = W.random_symmetric(k, 6, seed=k)
+    hg, ref = V.Hypergraph.from_matrix(A), O.build_from_matrix("symmetric", A)
+    x = _clustered(k, d, k + d, share)
+    p = V.Params(d=d, occupancy=occ)
+    V.set_tuning(19456, 10, 4, 0)
+    xg, yg, kg, L = hg.layout_step(torch.as_tensor(x).cuda(), 0.25, p)
+    xo, yo, ko, Lo = O.layout_step(ref, d, x.astype(np.float64), 0.25, occ=occ)
+    assert L == Lo
+    assert np.array_equal(kg.cpu().numpy().view(np.uint32), ko)
+    yg = yg.cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(yg[:, :d] - yo[:, :d]) <= TOL * np.linalg.norm(yo[:, :d])
+    if k <= 2048:
+        V.set_tuning(19456, 10, 4, 2048)
+        xs, ys, ks, _ = hg.layout_step(torch.as_tensor(x).cuda(), 0.25, p)
+        assert np.array_equal(ys.cpu().numpy().view(np.uint32), yg.astype(np.float32).view(np.uint32))
+        assert np.array_equal(xs.cpu().numpy(), xg.cpu().numpy()) and np.array_equal(ks.cpu().numpy(), kg.cpu().numpy())
+
+
+def test_device_wide_binning_many_problems(V):
+    """A batch of matrices with isolated vertices: the two binnings agree."""
+    mats = W.batch_mix(12, 5, nmin=200, nmax=1800)
+    for d in (2, 3):
+        out = []
+        for small in (0, 2048):
+            V.set_tuning(19456, 10, 4, small)
+            out.append(V.batch_layout(mats, V.Params(d=d, iters=9, seed=4))[0].cpu().numpy())
+        assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
