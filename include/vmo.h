@@ -438,8 +438,10 @@ vmo_status vmo_finegrain_coords(vmo_hg hg, const float* bipartite_coords, float*
  * implementation).  None of these settings changes any result, bit for bit;
  * they only change how the work is split into launches:
  *   small_step_threads: layout step launches of at most this many threads
- *     use the step-kernel variant with two far-field rows in flight per lane
- *     (latency hiding for small levels); default 19,456 (4 warps per SM);
+ *     (d = 2; five eighths of it for d = 3 and 4) use the step kernel for
+ *     small levels, which hides latency (two far-field rows in flight, d = 2)
+ *     or gives every target more threads (d = 3 and 4); default 19,456 (4
+ *     warps per SM);
  *   radix_max_bits: widest digit of the LSD radix sorts, 8, 9 or
  *     10 (default 10: fewest passes);
  *   assign_items: positions per thread of the Lloyd assignment, 1, 2, 4 or

@@ -56,6 +56,27 @@ struct Pair {
   static constexpr int WO = D == 4 ? 0 : 2; // float offset of the weights in it
 };
 
+// Pair j of a table (read-only during the launch): one 32-byte load for
+// d <= 3, where a pair starts on a 32-byte boundary.
+template <int D>
+__device__ __forceinline__ void pair_load(const float4* __restrict__ tab, int64_t j, float4* P) {
+  const float4* p = tab + j * Pair<D>::N;
+  if (Pair<D>::N == 2) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(P[0].x), "=f"(P[0].y), "=f"(P[0].z), "=f"(P[0].w), "=f"(P[1].x), "=f"(P[1].y), "=f"(P[1].z),
+          "=f"(P[1].w)
+        : "l"(p));
+  } else {
+#pragma unroll
+    for (int i = 0; i < Pair<D>::N; ++i) P[i] = p[i];
+  }
+}
+template <int D>
+__device__ __forceinline__ void pair_zero(float4* P) {
+#pragma unroll
+  for (int i = 0; i < Pair<D>::N; ++i) P[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 template <int D>
 __device__ __forceinline__ void pair_store(float4* __restrict__ tab, int64_t i, const float* c, float w) {
   float* f = reinterpret_cast<float*>(tab + (i >> 1) * Pair<D>::N);
@@ -204,11 +225,14 @@ template <int D, int U>
 __global__ void __launch_bounds__(kBlock) k_keys(const float4* __restrict__ x, int64_t K, const int32_t* __restrict__ vprob,
                                                  const ProbDev* __restrict__ prob, const uint32_t* __restrict__ bb,
                                                  uint32_t* __restrict__ keys, uint32_t* __restrict__ arrival,
-                                                 int32_t* __restrict__ cnt, uint32_t* __restrict__ bb_next, int nreset,
-                                                 int32_t* __restrict__ tctr) {
+                                                 int32_t* __restrict__ cnt, int32_t* __restrict__ nchunk, int P,
+                                                 uint32_t* __restrict__ bb_next, int32_t* __restrict__ tctr) {
   pdl_enter();
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (gt == 0) ++*tctr;  // the level's step (read by the step kernel of this step)
+  const int64_t nreset = 8 * (int64_t)P;
+  if (nchunk)
+    for (int64_t r = gt; r < P; r += (int64_t)gridDim.x * blockDim.x) nchunk[r] = 0;
   for (int64_t r = gt; r < nreset; r += (int64_t)gridDim.x * blockDim.x) bb_next[r] = ((r & 7) < 4) ? 0xFFFFFFFFu : 0u;
   const int64_t v0 = (int64_t)blockIdx.x * blockDim.x * U + threadIdx.x;
   float4 xv[U];
@@ -245,7 +269,7 @@ constexpr int kCellScanCtas = 8;
 constexpr int kCellScanThreads = 1024;
 constexpr int kCellScanItems = 16;
 constexpr int64_t kCellScanTile = (int64_t)kCellScanCtas * kCellScanThreads * kCellScanItems;
-constexpr int64_t kCellScanMax = 4 * kCellScanTile;  // larger tables: two launches over every SM
+constexpr int64_t kCellScanMax = kCellScanTile;  // larger tables: two launches over every SM
 
 __device__ __forceinline__ void load_items(const int32_t* __restrict__ a, int64_t i0, int64_t n, int32_t* v) {
   if (i0 + kCellScanItems <= n) {
@@ -530,10 +554,11 @@ __device__ inline void agg_cell(const ProbDev& pr, int pb, int l, int64_t c, flo
 __host__ __device__ constexpr int brick_log2(int d) { return d == 2 ? 3 : 2; }
 
 template <int D>
-__global__ void __launch_bounds__(kBlock) k_cells(const int64_t* __restrict__ bbase, int P,
-                                                  const ProbDev* __restrict__ prob, const float4* __restrict__ xs,
-                                                  const float* __restrict__ ws, const int32_t* __restrict__ cst,
-                                                  float4* St, float* Wt, float4* CP, int32_t* __restrict__ done) {
+__global__ void __launch_bounds__(kBlock) k_cells(const int32_t* __restrict__ bprob, const ProbDev* __restrict__ prob,
+                                                  const float4* __restrict__ xs, const float* __restrict__ ws,
+                                                  const int32_t* __restrict__ cst, float4* St, float* Wt, float4* CP,
+                                                  int32_t* __restrict__ done, int32_t* __restrict__ chunk,
+                                                  int32_t* __restrict__ nchunk) {
   pdl_enter();
   constexpr int B = brick_log2(D), NC = 1 << (D * B);
   constexpr int NT = ((1 << (D * (B + 1))) - 1) / ((1 << D) - 1);  // cells of a brick on its B + 1 levels
@@ -541,10 +566,11 @@ __global__ void __launch_bounds__(kBlock) k_cells(const int64_t* __restrict__ bb
   __shared__ int32_t big[NC], bq0[NC], bq1[NC];
   __shared__ int nbig;
   __shared__ bool last;
-  const int pb = find_problem(bbase, P, blockIdx.x);
+  __shared__ int32_t cws[33], cbase;
+  const int pb = bprob[blockIdx.x];
   const ProbDev pr = prob[pb];
   const int L = pr.L, lb = min(L, B), Lb = L - lb;
-  const int64_t brick = (int64_t)blockIdx.x - bbase[pb];
+  const int64_t brick = (int64_t)blockIdx.x - pr.bbase;
   int32_t bc[D];
 #pragma unroll
   for (int m = 0; m < D; ++m) bc[m] = (int32_t)((brick >> (m * Lb)) & ((1 << Lb) - 1));
@@ -567,8 +593,31 @@ __global__ void __launch_bounds__(kBlock) k_cells(const int64_t* __restrict__ bb
     }
     pair_store<D>(CP, pr.cbase + lvl_off(D, l) + c + pb + 1, z, W);
   };
-  const int nc = 1 << (D * lb);
+  const int nc = 1 << (D * lb);  // at most kBlock
   const int32_t* cs = cst + pr.fbase + pb;
+  if (chunk) {  // the brick's chunks of at most two points of a cell, into the problem's list
+    int32_t q0 = 0, n = 0;
+    if (threadIdx.x < nc) {
+      const int64_t c = cell_index(threadIdx.x, 0);
+      q0 = cs[c];
+      n = cs[c + 1] - q0;
+    }
+    int32_t total;
+    const int32_t ex = block_exclusive<int32_t>((n + 1) >> 1, cws, &total);
+    if (threadIdx.x == 0) cbase = atomicAdd(&nchunk[pb], total);
+    __syncthreads();
+    int32_t* out = chunk + pr.lbase + cbase;
+    if (n <= kCellSerial)
+      for (int32_t h = 0; 2 * h < n; ++h) out[ex + h] = q0 + 2 * h;
+    unsigned todo = __ballot_sync(0xffffffffu, n > kCellSerial);
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int32_t e = __shfl_sync(0xffffffffu, ex, src), a = __shfl_sync(0xffffffffu, q0, src);
+      const int32_t m = (__shfl_sync(0xffffffffu, n, src) + 1) >> 1;
+      for (int32_t h = lane_id(); h < m; h += 32) out[e + h] = a + 2 * h;
+    }
+  }
   for (int i = threadIdx.x; i < nc; i += kBlock) {
     const int64_t c = cell_index(i, 0);
     const int32_t q0 = cs[c], q1 = cs[c + 1];
@@ -964,17 +1013,9 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
 // layout (mean point spacing ~1).
 constexpr float kR2Floor = 1e-15f;
 
-// F += w r^-d (src - xn) for the two sources of a pair; nx holds -xn twice
-// per coordinate, w the (masked) weights.  UNIT: both weights are 1 (the
-// multiply by w is left out; a half is masked by giving it the target's own
-// coordinates instead, so that its dx = 0 contributes 0).
-template <int D, bool UNIT = false>
-__device__ __forceinline__ void pair_charge(float2* F, const float4* P, const float2* nx, float2 w) {
-  float2 dx[D];
-  dx[0] = __fadd2_rn(make_float2(P[0].x, P[0].y), nx[0]);
-  if (D > 1) dx[1] = __fadd2_rn(make_float2(P[0].z, P[0].w), nx[1]);
-  if (D > 2) dx[2] = __fadd2_rn(make_float2(P[1].x, P[1].y), nx[2]);
-  if (D > 3) dx[3] = __fadd2_rn(make_float2(P[1].z, P[1].w), nx[3]);
+// w r^-d of the two sources of a pair at the differences dx.
+template <int D, bool UNIT>
+__device__ __forceinline__ float2 pair_factor(const float2* dx, float2 w) {
   float2 r2 = make_float2(kR2Floor, kR2Floor);  // offset: a source at the target's position gives 0 * finite
 #pragma unroll
   for (int m = 0; m < D; ++m) r2 = __ffma2_rn(dx[m], dx[m], r2);
@@ -989,6 +1030,21 @@ __device__ __forceinline__ void pair_charge(float2* F, const float4* P, const fl
     const float2 i2 = make_float2(rcp_approx(r2.x), rcp_approx(r2.y));
     g = UNIT ? __fmul2_rn(i2, i2) : __fmul2_rn(__fmul2_rn(w, i2), i2);
   }
+  return g;
+}
+
+// F += w r^-d (src - xn) for the two sources of a pair; nx holds -xn twice
+// per coordinate, w the (masked) weights.  UNIT: both weights are 1 (the
+// multiply by w is left out; a half is masked by giving it the target's own
+// coordinates instead, so that its dx = 0 contributes 0).
+template <int D, bool UNIT = false>
+__device__ __forceinline__ void pair_charge(float2* F, const float4* P, const float2* nx, float2 w) {
+  float2 dx[D];
+  dx[0] = __fadd2_rn(make_float2(P[0].x, P[0].y), nx[0]);
+  if (D > 1) dx[1] = __fadd2_rn(make_float2(P[0].z, P[0].w), nx[1]);
+  if (D > 2) dx[2] = __fadd2_rn(make_float2(P[1].x, P[1].y), nx[2]);
+  if (D > 3) dx[3] = __fadd2_rn(make_float2(P[1].z, P[1].w), nx[3]);
+  const float2 g = pair_factor<D, UNIT>(dx, w);
 #pragma unroll
   for (int m = 0; m < D; ++m) F[m] = __ffma2_rn(g, dx[m], F[m]);
 }
@@ -1011,195 +1067,181 @@ __device__ __forceinline__ float2 pair_weight(const float4* P) {
   return Pair<D>::WO == 0 ? make_float2(q.x, q.y) : make_float2(q.z, q.w);
 }
 
-// Far-field charges of one level for a target in cell `me` (level l): the
-// cells of the 6^d box spanned by the children of the cells around the
-// target's parent cell, minus the 3^d cells adjacent to the target's cell.
-// One row of the box along coordinate 0 starts at an even cell and holds 4 or
-// 6 cells, i.e. 2 or 3 pairs: all loads are issued first, then the pairs are
-// accumulated without branches (a pair beyond the row is loaded as zeros and
-// weighs 0).  A cell counts if it holds weight and is not adjacent to the
-// target's cell.
-template <int D, bool COUNT>
-__device__ inline void far_row(const float4* __restrict__ CP, int64_t cell0, int lo0, int hi0, bool incore, int me0,
-                               const float2* nx, float2* F, unsigned long long& nint) {
-  constexpr int N = Pair<D>::N;
-  float4 P[3][N];
-  const int npairs = (hi0 - lo0 + 1) >> 1;
-  const float4* row = CP + (cell0 >> 1) * N;
-  // a row holds 2 or 3 pairs: only the third is conditional
+// The targets of one thread: T points of one finest cell, so that every
+// loaded source pair serves all of them (T = 2 halves the L1 bandwidth per
+// interaction).  nx holds -x twice per coordinate, F the force sums of the
+// even and the odd sources.  A target's sums take the same sources in the same
+// order whatever T is.
+template <int D, int T>
+struct Targets {
+  float2 nx[T][D], F[T][D];
+};
+
+template <int D, bool UNIT, int T>
+__device__ __forceinline__ void charge_all(Targets<D, T>& g, const float4* P, float2 w) {
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
+  for (int t = 0; t < T; ++t) pair_charge<D, UNIT>(g.F[t], P, g.nx[t], w);
+}
+
+// Far field.  Of level l the cells of the 6^d box spanned by the children of
+// the cells around the target's parent cell act as charges, minus the 3^d
+// cells adjacent to the target's cell.  One row of the box along coordinate 0
+// starts at an even cell and holds 4 or 6 cells, i.e. 2 or 3 pairs.  The rows
+// (row-major, coordinate 1 fastest) go round-robin to the G lanes of the
+// target's group: FarRows steps through one lane's rows of every level
+// l = 2..L in that order.
+template <int D>
+struct FarRows {
+  int64_t cell0;  // table index of the problem's level-0 cell (lvl_off(0) = 0), odd
+  int l, L, G, lane_g;
+  int32_t c[D];   // the target's finest cell
+  int32_t me[D], lo[D], hi[D];
+  int q[D];       // current row: q[1..D-1]
+  int half;       // pairs per row of the level's grid
+  int64_t base;   // first pair of the level plus lo[0] / 2
+
+  __device__ __forceinline__ void init(int64_t cell, const int32_t* cc, int LL, int GG, int lg) {
+    cell0 = cell;
+    L = LL;
+    G = GG;
+    lane_g = lg;
 #pragma unroll
-    for (int j = 0; j < N; ++j) P[i][j] = (i < 2 || npairs > 2) ? row[i * N + j] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int m = 0; m < D; ++m) c[m] = cc[m];
+    l = 1;
+    next_level();
+  }
+  __device__ __forceinline__ bool done() const { return l > L; }
+  __device__ __forceinline__ void next_level() {
+    do {
+      ++l;
+      if (l > L) return;
+      const int sl = 1 << l;
+#pragma unroll
+      for (int m = 0; m < D; ++m) {
+        me[m] = c[m] >> (L - l);
+        const int par = me[m] >> 1;
+        lo[m] = max(2 * par - 2, 0);
+        hi[m] = min(2 * par + 3, sl - 1);
+        q[m] = lo[m];
+      }
+      half = sl >> 1;
+      base = ((cell0 + lvl_off(D, l)) >> 1) + (lo[0] >> 1);
+      q[1] += lane_g;
+      carry();
+    } while (q[D - 1] > hi[D - 1]);  // fewer rows than lanes
+  }
+  __device__ __forceinline__ void carry() {
+#pragma unroll
+    for (int m = 1; m + 1 < D; ++m) {
+      const int e = hi[m] - lo[m] + 1;
+      while (q[m] > hi[m]) {
+        q[m] -= e;
+        ++q[m + 1];
+      }
+    }
+  }
+  __device__ __forceinline__ void advance() {
+    q[1] += G;
+    carry();
+    if (q[D - 1] > hi[D - 1]) next_level();
+  }
+  // first pair of the row, whether it has a third pair, and the mask of its
+  // cells (bit i: cell lo[0] + i) that are adjacent to the target's cell
+  __device__ __forceinline__ int64_t row(bool& third, unsigned& mask) const {
+    int64_t idx = 0;
+    bool in = true;
+#pragma unroll
+    for (int m = D - 1; m >= 1; --m) {
+      idx = (idx << l) + q[m];
+      in = in && q[m] >= me[m] - 1 && q[m] <= me[m] + 1;
+    }
+    third = hi[0] - lo[0] > 4;
+    const int o = me[0] - lo[0];  // 0, 1, 2 or 3
+    mask = in ? (o > 0 ? 7u << (o - 1) : 3u) : 0u;
+    return base + idx * half;
+  }
+};
+
+// Loads of a row: all issued together; a pair beyond the row reads as zeros
+// and weighs 0.
+template <int D>
+__device__ __forceinline__ void row_load(const float4* __restrict__ CP, int64_t row, bool third,
+                                         float4 (*P)[Pair<D>::N]) {
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    float2 w = pair_weight<D>(P[i]);
-    if (incore) {
-      const int xa = lo0 + 2 * i;
-      w.x = (xa >= me0 - 1 && xa <= me0 + 1) ? 0.0f : w.x;
-      w.y = (xa + 1 >= me0 - 1 && xa + 1 <= me0 + 1) ? 0.0f : w.y;
-    }
-    pair_charge<D>(F, P[i], nx, w);
-    if (COUNT) nint += (w.x > 0.0f) + (w.y > 0.0f);
+    if (i < 2 || third) pair_load<D>(CP, row + i, P[i]);
+    else pair_zero<D>(P[i]);
   }
 }
 
-// Far field of one level for one lane of the target's group: the rows of the
-// box (row-major order) go round-robin to the G lanes of the group, each lane
-// visiting only its own rows.  `cell` is the paired-table index of the
-// level's cell 0 (even).
-template <int D, bool COUNT>
-__device__ inline void far_level_lane(const float4* __restrict__ CP, int64_t cell, const int32_t* me, int l,
-                                      const float2* nx, float2* F, int G, int lane_g, unsigned long long& nint) {
-  const int sl = 1 << l;
-  int lo[D], hi[D];
+template <int D, bool COUNT, int T>
+__device__ __forceinline__ void row_apply(float4 (*P)[Pair<D>::N], unsigned mask, Targets<D, T>& g,
+                                          unsigned long long& nint) {
+  float2 w[3];
 #pragma unroll
-  for (int m = 0; m < D; ++m) {
-    int par = me[m] >> 1;
-    lo[m] = max(2 * par - 2, 0);
-    hi[m] = min(2 * par + 3, sl - 1);
+  for (int i = 0; i < 3; ++i) w[i] = pair_weight<D>(P[i]);
+  if (mask) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      w[i].x = (mask >> (2 * i)) & 1u ? 0.0f : w[i].x;
+      w[i].y = (mask >> (2 * i + 1)) & 1u ? 0.0f : w[i].y;
+    }
   }
-  if (G > 1) {
-    // several lanes: the lane's own rows lane_g, lane_g + G, ... (row-major,
-    // coordinate 1 fastest), stepped with carries instead of walking the others
-    const int e1 = hi[1] - lo[1] + 1, e2 = D > 2 ? hi[2] - lo[2] + 1 : 1;
-    int y = lo[1] + lane_g, z = D > 2 ? lo[2] : 0, w = D > 3 ? lo[3] : 0;
-    auto carry = [&]() {
-      while (y > hi[1]) {
-        y -= e1;
-        ++z;
-        if (D > 3 && z > hi[2]) {
-          z -= e2;
-          ++w;
-        }
-      }
-    };
-    if (D > 2) carry();
-    for (;;) {
-      if (D == 2 && y > hi[1]) break;
-      if (D == 3 && z > hi[2]) break;
-      if (D == 4 && w > hi[3]) break;
-      bool in = y >= me[1] - 1 && y <= me[1] + 1;
-      int64_t idx = y;
-      if (D > 2) {
-        in = in && z >= me[2] - 1 && z <= me[2] + 1;
-        idx = (int64_t)z * sl + y;
-      }
-      if (D > 3) {
-        in = in && w >= me[3] - 1 && w <= me[3] + 1;
-        idx = ((int64_t)w * sl + z) * sl + y;
-      }
-      far_row<D, COUNT>(CP, cell + idx * sl + lo[0], lo[0], hi[0], in, me[0], nx, F, nint);
-      y += G;
-      if (D > 2) carry();
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    charge_all<D, false, T>(g, P[i], w[i]);
+    if (COUNT) nint += (w[i].x > 0.0f) + (w[i].y > 0.0f);
+  }
+}
+
+// PIPE: the next two rows are loaded before the current two are accumulated
+// (launches with too few warps to hide a load behind other warps); else one
+// row at a time.
+template <int D, bool COUNT, int T, bool PIPE>
+__device__ __forceinline__ void far_field(const float4* CP, int64_t cell0, const int32_t* c, int L, int G, int lane_g,
+                                          Targets<D, T>& g, unsigned long long& nint) {
+  constexpr int N = Pair<D>::N;
+  FarRows<D> it;
+  it.init(cell0, c, L, G, lane_g);
+  if (!PIPE) {
+    while (!it.done()) {
+      float4 P[3][N];
+      bool third;
+      unsigned mask;
+      const int64_t r = it.row(third, mask);
+      row_load<D>(CP, r, third, P);
+      it.advance();
+      row_apply<D, COUNT, T>(P, mask, g, nint);
     }
     return;
   }
-  if (D == 2) {
-    for (int y = lo[1]; y <= hi[1]; ++y) {
-      const bool iny = y >= me[1] - 1 && y <= me[1] + 1;
-      far_row<D, COUNT>(CP, cell + (int64_t)y * sl + lo[0], lo[0], hi[0], iny, me[0], nx, F, nint);
-    }
-  } else if (D == 3) {
-    for (int z = lo[2]; z <= hi[2]; ++z) {
-      const bool inz = z >= me[2] - 1 && z <= me[2] + 1;
-      for (int y = lo[1]; y <= hi[1]; ++y) {
-        const bool iny = inz && y >= me[1] - 1 && y <= me[1] + 1;
-        far_row<D, COUNT>(CP, cell + ((int64_t)z * sl + y) * sl + lo[0], lo[0], hi[0], iny, me[0], nx, F, nint);
-      }
-    }
-  } else {
-    for (int w = lo[3]; w <= hi[3]; ++w) {
-      const bool inw = w >= me[3] - 1 && w <= me[3] + 1;
-      for (int z = lo[2]; z <= hi[2]; ++z) {
-        const bool inz = inw && z >= me[2] - 1 && z <= me[2] + 1;
-        for (int y = lo[1]; y <= hi[1]; ++y) {
-          const bool iny = inz && y >= me[1] - 1 && y <= me[1] + 1;
-          far_row<D, COUNT>(CP, cell + (((int64_t)w * sl + z) * sl + y) * sl + lo[0], lo[0], hi[0], iny, me[0], nx,
-                            F, nint);
-        }
-      }
-    }
-  }
-}
-
-// The same far field with two of the lane's rows in flight: both rows' pairs
-// are loaded before either is accumulated, rows taken in the same order (so
-// the sums are bit-identical to far_level_lane).  Used for launches too small
-// to hide load latency with other warps (the small levels of a hierarchy).
-template <int D, bool COUNT>
-__device__ inline void far_level_lane2(const float4* __restrict__ CP, int64_t cell, const int32_t* me, int l,
-                                       const float2* nx, float2* F, int G, int lane_g, unsigned long long& nint) {
-  constexpr int N = Pair<D>::N;
-  const int sl = 1 << l;
-  int lo[D], hi[D], ext[D];
+  float4 A[2][3][N], B[2][3][N];
+  unsigned ma[2] = {0u, 0u}, mb[2] = {0u, 0u};
+  int na = 0, nb = 0;
+  auto fetch = [&](float4 (*P)[3][N], unsigned* m, int& n) {
+    n = 0;
 #pragma unroll
-  for (int m = 0; m < D; ++m) {
-    int par = me[m] >> 1;
-    lo[m] = max(2 * par - 2, 0);
-    hi[m] = min(2 * par + 3, sl - 1);
-    ext[m] = hi[m] - lo[m] + 1;
-  }
-  int nrows = 1;
-#pragma unroll
-  for (int m = 1; m < D; ++m) nrows *= ext[m];
-  const int npairs = ext[0] >> 1;
-  // row r (row-major over coordinates 1..D-1, coordinate 1 fastest): its
-  // first cell and whether it is adjacent to the target's cell in 1..D-1
-  auto row_at = [&](int r, int64_t& c0, bool& in) {
-    int64_t idx = 0;
-    bool adj = true;
-    int q[D];
-#pragma unroll
-    for (int m = 1; m < D; ++m) {
-      q[m] = lo[m] + r % ext[m];
-      r /= ext[m];
-      adj = adj && q[m] >= me[m] - 1 && q[m] <= me[m] + 1;
-    }
-#pragma unroll
-    for (int m = D - 1; m >= 1; --m) idx = idx * sl + q[m];
-    c0 = cell + idx * sl + lo[0];
-    in = adj;
-  };
-  auto load = [&](int64_t c0, float4 (*P)[N]) {
-    const float4* row = CP + (c0 >> 1) * N;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < N; ++j) P[i][j] = (i < 2 || npairs > 2) ? row[i * N + j] : make_float4(0.f, 0.f, 0.f, 0.f);
-  };
-  auto apply = [&](float4 (*P)[N], bool incore) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      float2 w = pair_weight<D>(P[i]);
-      if (incore) {
-        const int xa = lo[0] + 2 * i;
-        w.x = (xa >= me[0] - 1 && xa <= me[0] + 1) ? 0.0f : w.x;
-        w.y = (xa + 1 >= me[0] - 1 && xa + 1 <= me[0] + 1) ? 0.0f : w.y;
-      }
-      pair_charge<D>(F, P[i], nx, w);
-      if (COUNT) nint += (w.x > 0.0f) + (w.y > 0.0f);
+    for (int u = 0; u < 2; ++u) {
+      if (it.done()) break;
+      bool third;
+      const int64_t r = it.row(third, m[u]);
+      row_load<D>(CP, r, third, P[u]);
+      it.advance();
+      ++n;
     }
   };
-  int r = lane_g;
-  for (; r + G < nrows; r += 2 * G) {
-    int64_t ca, cb;
-    bool ia, ib;
-    row_at(r, ca, ia);
-    row_at(r + G, cb, ib);
-    float4 A[3][N], B[3][N];
-    load(ca, A);
-    load(cb, B);
-    apply(A, ia);
-    apply(B, ib);
-  }
-  if (r < nrows) {
-    int64_t ca;
-    bool ia;
-    row_at(r, ca, ia);
-    float4 A[3][N];
-    load(ca, A);
-    apply(A, ia);
+  auto apply = [&](float4 (*P)[3][N], unsigned* m, int n) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (u < n) row_apply<D, COUNT, T>(P[u], m[u], g, nint);
+  };
+  fetch(A, ma, na);
+  while (na > 0) {
+    fetch(B, mb, nb);
+    apply(A, ma, na);
+    if (nb == 0) break;
+    fetch(A, ma, na);
+    apply(B, mb, nb);
   }
 }
 
@@ -1208,14 +1250,21 @@ __device__ inline void far_level_lane2(const float4* __restrict__ CP, int64_t ce
 // order-preserving integer images of its lanes' new coordinates to the
 // problem's box, which k_keys reset earlier in the step.  Min and max are
 // exact, so the order of the atomics does not matter.
-template <int D>
-__device__ inline void bbox_warp_fold(const float4& v, bool valid, uint32_t* __restrict__ box) {
+template <int D, int T>
+__device__ inline void bbox_warp_fold(const float4* v, const bool* valid, uint32_t* __restrict__ box) {
   uint32_t mn[4], mx[4];
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
-    uint32_t o = (valid && m < D) ? f2ord(comp(v, m)) : 0u;
-    mn[m] = __reduce_min_sync(0xffffffffu, (valid && m < D) ? o : 0xFFFFFFFFu);
-    mx[m] = __reduce_max_sync(0xffffffffu, o);
+    uint32_t a = 0xFFFFFFFFu, b = 0u;
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+      if (valid[t] && m < D) {
+        const uint32_t o = f2ord(comp(v[t], m));
+        a = min(a, o);
+        b = max(b, o);
+      }
+    mn[m] = __reduce_min_sync(0xffffffffu, a);
+    mx[m] = __reduce_max_sync(0xffffffffu, b);
   }
   if (lane_id() == 0 && mn[0] != 0xFFFFFFFFu) {
 #pragma unroll
@@ -1227,76 +1276,79 @@ __device__ inline void bbox_warp_fold(const float4& v, bool valid, uint32_t* __r
 }
 
 // Near field of one row range [qa, qb) of problem-local sorted positions for
-// one lane of the target's group: source pairs j = qa/2 + lane_g, + G, ...,
-// four pairs per trip (all loads issued before the arithmetic; the order of
-// the pairs in the sums is the same as one pair per trip).  Only the first
+// one lane of the targets' group: source pairs j = qa/2 + lane_g, + G, ...,
+// U pairs per trip (all loads issued before the arithmetic).  Only the first
 // pair can start before qa and only the last can end at or after qb; those
 // halves are masked (weight 0, or the target's own coordinates when UNIT).
-template <int D, bool COUNT, bool UNIT>
-__device__ __forceinline__ void near_range(const float4* __restrict__ xp, int qa, int qb, int G, int lane_g,
-                                           int64_t tgt, const float2* nx, float2* F, unsigned long long& nint) {
+template <int D, bool COUNT, bool UNIT, int T, int U, bool GUARD>
+__device__ __forceinline__ void near_trip(const float4* __restrict__ xp, int j, int qa, int qb, int G, int64_t tgt,
+                                          Targets<D, T>& g, unsigned long long& nint) {
   constexpr int N = Pair<D>::N;
-  int j = (qa >> 1) + lane_g;
-  for (; 2 * (j + 7 * G) < qb; j += 8 * G) {
-    float4 Q[8][N];
+  float4 Q[U][N];
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-#pragma unroll
-      for (int i = 0; i < N; ++i) Q[u][i] = xp[(int64_t)(j + u * G) * N + i];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int h0 = 2 * (j + u * G);
-      float2 w = make_float2(1.0f, 1.0f);
-      if (UNIT) {
-        if (u == 0) pair_mask_half<D>(Q[u], 0, h0 < qa, nx);
-        if (u == 7) pair_mask_half<D>(Q[u], 1, h0 + 1 >= qb, nx);
-      } else {
-        w = pair_weight<D>(Q[u]);
-        if (u == 0) w.x = h0 >= qa ? w.x : 0.0f;
-        if (u == 7) w.y = h0 + 1 < qb ? w.y : 0.0f;
-      }
-      pair_charge<D, UNIT>(F, Q[u], nx, w);
-      if (COUNT) nint += (h0 >= qa && h0 != tgt) + (h0 + 1 < qb && h0 + 1 != tgt);
-    }
+  for (int u = 0; u < U; ++u) {
+    if (!GUARD || u == 0 || 2 * (j + u * G) < qb) pair_load<D>(xp, j + u * G, Q[u]);
+    else pair_zero<D>(Q[u]);
   }
-  for (; 2 * (j + 3 * G) < qb; j += 4 * G) {
-    float4 Q[4][N];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int i = 0; i < N; ++i) Q[u][i] = xp[(int64_t)(j + u * G) * N + i];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int h0 = 2 * (j + u * G);
-      float2 w = make_float2(1.0f, 1.0f);
-      if (UNIT) {
-        if (u == 0) pair_mask_half<D>(Q[u], 0, h0 < qa, nx);
-        if (u == 3) pair_mask_half<D>(Q[u], 1, h0 + 1 >= qb, nx);
-      } else {
-        w = pair_weight<D>(Q[u]);
-        if (u == 0) w.x = h0 >= qa ? w.x : 0.0f;
-        if (u == 3) w.y = h0 + 1 < qb ? w.y : 0.0f;
-      }
-      pair_charge<D, UNIT>(F, Q[u], nx, w);
-      if (COUNT) nint += (h0 >= qa && h0 != tgt) + (h0 + 1 < qb && h0 + 1 != tgt);
-    }
-  }
-  for (; 2 * j < qb; j += G) {
-    float4 Q[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) Q[i] = xp[(int64_t)j * N + i];
-    float2 w = make_float2(1.0f, 1.0f);
+  for (int u = 0; u < U; ++u) {
+    const int h0 = 2 * (j + u * G);
+    if (GUARD && u > 0 && h0 >= qb) break;
+    const bool m0 = u == 0 && h0 < qa, m1 = (GUARD || u == U - 1) && h0 + 1 >= qb;
     if (UNIT) {
-      pair_mask_half<D>(Q, 0, 2 * j < qa, nx);
-      pair_mask_half<D>(Q, 1, 2 * j + 1 >= qb, nx);
+#pragma unroll
+      for (int t = 0; t < T; ++t) {
+        float4 R[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) R[i] = Q[u][i];
+        if (u == 0) pair_mask_half<D>(R, 0, m0, g.nx[t]);
+        if (GUARD || u == U - 1) pair_mask_half<D>(R, 1, m1, g.nx[t]);
+        pair_charge<D, true>(g.F[t], R, g.nx[t], make_float2(1.0f, 1.0f));
+      }
     } else {
-      w = pair_weight<D>(Q);
-      w.x = 2 * j >= qa ? w.x : 0.0f;
-      w.y = 2 * j + 1 < qb ? w.y : 0.0f;
+      float2 w = pair_weight<D>(Q[u]);
+      w.x = m0 ? 0.0f : w.x;
+      w.y = m1 ? 0.0f : w.y;
+      charge_all<D, false, T>(g, Q[u], w);
     }
-    pair_charge<D, UNIT>(F, Q, nx, w);
-    if (COUNT) nint += (2 * j >= qa && 2 * j != tgt) + (2 * j + 1 < qb && 2 * j + 1 != tgt);
+    if (COUNT) nint += (h0 >= qa && h0 != tgt) + (h0 + 1 < qb && h0 + 1 != tgt);
   }
+}
+
+template <int D, bool COUNT, bool UNIT, int T, int BIG>
+__device__ __forceinline__ void near_range(const float4* __restrict__ xp, int qa, int qb, int G, int lane_g,
+                                           int64_t tgt, Targets<D, T>& g, unsigned long long& nint) {
+  int j = (qa >> 1) + lane_g;
+  if (BIG > 4)
+    for (; 2 * (j + (BIG - 1) * G) < qb; j += BIG * G)
+      near_trip<D, COUNT, UNIT, T, BIG, false>(xp, j, qa, qb, G, tgt, g, nint);
+  for (; 2 * (j + 3 * G) < qb; j += 4 * G)
+    near_trip<D, COUNT, UNIT, T, 4, false>(xp, j, qa, qb, G, tgt, g, nint);
+  if (2 * j < qb) near_trip<D, COUNT, UNIT, T, 3, true>(xp, j, qa, qb, G, tgt, g, nint);
+}
+
+// Gradient and step of the point at sorted position p from its repulsion sums.
+template <int D>
+__device__ __forceinline__ float4 step_target(int64_t p, const float4& xn, const float* Fs, const float* __restrict__ ws,
+                                              const uint32_t* __restrict__ svals, const float4* __restrict__ yatt,
+                                              float kappa, float step_override, const float* __restrict__ s0, int pb,
+                                              const float* __restrict__ scale_tab, const int32_t* __restrict__ tctr,
+                                              float4* __restrict__ x, float4* __restrict__ y_out) {
+  const float wn = ws ? ws[p] : 1.0f;
+  const uint32_t v = svals[p];
+  float4 ya = yatt[v];
+  float y0 = kappa * wn * Fs[0] + ya.x;
+  float y1 = D > 1 ? kappa * wn * Fs[1] + ya.y : 0.f;
+  float y2 = D > 2 ? kappa * wn * Fs[2] + ya.z : 0.f;
+  float y3 = D > 3 ? kappa * wn * Fs[3] + ya.w : 0.f;
+  if (y_out) y_out[v] = make_float4(y0, y1, y2, y3);
+  float ny = sqrtf(y0 * y0 + y1 * y1 + y2 * y2 + y3 * y3);
+  float step = step_override > 0.0f ? step_override : s0[pb] * scale_tab[*tctr];
+  float a = ny > 0.0f ? step / ny : 0.0f;
+  const float4 xnew = make_float4(xn.x - a * y0, D > 1 ? xn.y - a * y1 : 0.f, D > 2 ? xn.z - a * y2 : 0.f,
+                                  D > 3 ? xn.w - a * y3 : 0.f);
+  x[v] = xnew;
+  return xnew;
 }
 
 // Gradient (eq. graphenergygradientsimple with the grid pyramid) and step of
@@ -1311,48 +1363,89 @@ __device__ __forceinline__ void near_range(const float4* __restrict__ xp, int qa
 // (vbase + pb + 1) & ~1; the halves outside the range weigh 0).  Far field:
 // the paired cell table CP, whose index of (problem pb, level l, cell c) is
 // cbase + pb + lvl_off(l) + 1 + c (even for even c).
-#ifndef VMO_STEP_BLOCK
-#define VMO_STEP_BLOCK 128
-#endif
-#ifndef VMO_STEP_MINBLOCKS
-#define VMO_STEP_MINBLOCKS 6
-#endif
-constexpr int kStepBlock = VMO_STEP_BLOCK;
-// step launches of at most g_tuning.small_step_threads threads (default
-// about 4 warps per SM) take the far-field variant with two rows in flight
+//
+// T = 1: a group handles the point at its own sorted position.  T = 2: a
+// group handles a chunk of one or two consecutive points of one finest cell;
+// the chunks of a problem (first positions, in any order) are listed by the
+// binning, nchunk[pb] of them, and its threads are numbered from tbase2.
+// One target per thread is bound by the 32 bytes a pair costs every lane of
+// L1 bandwidth (65% busy, FMA pipe 59%, 500,000 clustered points, d = 3, 587
+// us); two per thread halve that (36%) and leave the FMA pipe (66%): 568 us,
+// 405 against 461 us in that level's later steps.  Measured and not kept:
+// leaving out the middle pair of a row where every lane of the warp has it
+// masked (8% of the far field's work, 1% slower), other block sizes and
+// register limits (within 2%).
+constexpr int kStepBlock = 128;
 
-template <int D, bool COUNT, bool MLP>
-__global__ void __launch_bounds__(kStepBlock, MLP ? 3 : VMO_STEP_MINBLOCKS) k_repulse_update(
+// Which step kernel a level takes, by d and by the threads of one target lane
+// each (per step, one level, GB300):
+//  - d >= 3, at most 5/8 of g_tuning.small_step_threads (12,160): the split
+//    kernel; 3-D grids of 1,728 / 8,000 / 13,824 points 25.2 / 34.9 / 50.2 us
+//    against 29.7 / 45.0 / 48.5 us with one thread per lane.
+//  - d = 2, at most g_tuning.small_step_threads (4 warps per SM): two far-field
+//    rows in flight; 2-D grids of 1,024 / 4,096 points 16.4 / 20.5 us against
+//    17.4 / 21.5 us (a target's sums are too short there for the split: 17.6 /
+//    22.3 us).
+//  - at least kPairThreadsMin: two targets per thread; 110,592 / 262,144 grid
+//    points and 500,000 clustered ones 104 / 186 / 489 us against 95 / 196 /
+//    538 us with one.
+//  - else one target per thread.
+constexpr int64_t kPairThreadsMin = 196608;
+
+enum StepMode { kStepPlain = 0, kStepPipe = 1, kStepPair = 2 };
+__host__ __device__ constexpr int step_min_blocks(int mode) { return mode == kStepPlain ? 6 : (mode == kStepPipe ? 3 : 4); }
+
+template <int D, bool COUNT, int MODE>
+__global__ void __launch_bounds__(kStepBlock, step_min_blocks(MODE)) k_repulse_update(
     const float4* __restrict__ xs, const float* __restrict__ ws, const float4* __restrict__ XP,
     const uint32_t* __restrict__ svals, const uint32_t* __restrict__ scell, const int32_t* __restrict__ cst,
-    const float4* __restrict__ CP, const float4* __restrict__ yatt, const int64_t* __restrict__ tbase, int P,
-    const ProbDev* __restrict__ prob, int64_t T, float kappa, const float* __restrict__ s0,
+    const float4* __restrict__ CP, const float4* __restrict__ yatt, const int32_t* __restrict__ wprob,
+    const ProbDev* __restrict__ prob, int64_t nthreads, const int32_t* __restrict__ chunk,
+    const int32_t* __restrict__ nchunk, float kappa, const float* __restrict__ s0,
     const float* __restrict__ scale_tab, const int32_t* __restrict__ tctr,
     float step_override, float4* __restrict__ x, float4* __restrict__ y_out, uint32_t* __restrict__ bb_next,
     unsigned long long* __restrict__ icount) {
   pdl_enter();
   constexpr int N = Pair<D>::N;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int pb = find_problem(tbase, P, t < T ? t : T - 1);
+  constexpr int T = MODE == kStepPair ? 2 : 1;
+  constexpr bool PIPE = MODE == kStepPipe;
+  constexpr int BIG = MODE == kStepPair ? 4 : 8;
+  const int64_t th = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int pb = wprob[(th < nthreads ? th : nthreads - 1) >> 5];  // a warp never straddles two problems
   const ProbDev pr = prob[pb];
   const int G = pr.group;
-  const int64_t rel = t - pr.tbase;
-  const int64_t tgt = rel / G;
+  const int64_t rel = th - (T == 2 ? pr.tbase2 : pr.tbase);
   const int lane_g = (int)(rel & (G - 1));
-  const bool valid = t < T && tgt < pr.k;
+  int64_t tgt = rel / G;  // problem-local sorted position of the first target
+  bool valid = th < nthreads && tgt < (T == 2 ? nchunk[pb] : pr.k);
+  int64_t p = pr.vbase + tgt;
+  if (T == 2 && valid) {
+    p = chunk[pr.lbase + tgt];
+    tgt = p - pr.vbase;
+  }
   unsigned long long nint = 0;
-  float2 F[D];
+  Targets<D, T> g;
+  float4 xn[T];
+  bool ok[T];
 #pragma unroll
-  for (int m = 0; m < D; ++m) F[m] = make_float2(0.f, 0.f);
-  const int64_t p = pr.vbase + tgt;
-  float4 xn = make_float4(0, 0, 0, 0);
+  for (int t = 0; t < T; ++t) {
+    ok[t] = valid && t == 0;
+    xn[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int m = 0; m < D; ++m) g.F[t][m] = make_float2(0.f, 0.f);
+  }
   if (valid) {
     const int L = pr.L, side = 1 << L;
-    xn = xs[p];
-    float2 nx[D];
-#pragma unroll
-    for (int m = 0; m < D; ++m) nx[m] = make_float2(-comp(xn, m), -comp(xn, m));
     const uint32_t packed = scell[p];
+    xn[0] = xs[p];
+    if (T == 2) {  // the second target (the first again when the chunk has one)
+      ok[T - 1] = tgt + 1 < pr.k && scell[p + (tgt + 1 < pr.k)] == packed;
+      xn[T - 1] = xs[p + ok[T - 1]];
+    }
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+#pragma unroll
+      for (int m = 0; m < D; ++m) g.nx[t][m] = make_float2(-comp(xn[t], m), -comp(xn[t], m));
     int32_t c[D];
 #pragma unroll
     for (int m = 0; m < D; ++m) c[m] = (int32_t)((packed >> (m * field_bits(D))) & ((1u << field_bits(D)) - 1));
@@ -1382,11 +1475,11 @@ __global__ void __launch_bounds__(kStepBlock, MLP ? 3 : VMO_STEP_MINBLOCKS) k_re
     auto near_row = [&](int qa, int qb) {
       if (qa >= qb) return;
       if (ws)
-        near_range<D, COUNT, false>(xp, qa, qb, G, lane_g, tgt, nx, F, nint);
+        near_range<D, COUNT, false, T, BIG>(xp, qa, qb, G, lane_g, tgt, g, nint);
       else
-        near_range<D, COUNT, true>(xp, qa, qb, G, lane_g, tgt, nx, F, nint);
+        near_range<D, COUNT, true, T, BIG>(xp, qa, qb, G, lane_g, tgt, g, nint);
     };
-    if (MLP && D <= 3) {
+    if (PIPE) {
       // small launches: all rows' ranges loaded before the first row is used
       int qa[NR], qb[NR];
 #pragma unroll
@@ -1400,41 +1493,23 @@ __global__ void __launch_bounds__(kStepBlock, MLP ? 3 : VMO_STEP_MINBLOCKS) k_re
         near_row(qa, qb);
       }
     }
-    // far field, levels 2..L
-    for (int l = 2; l <= L; ++l) {
-      int32_t me[D];
-#pragma unroll
-      for (int m = 0; m < D; ++m) me[m] = c[m] >> (L - l);
-      if (MLP)
-        far_level_lane2<D, COUNT>(CP, pr.cbase + pb + lvl_off(D, l) + 1, me, l, nx, F, G, lane_g, nint);
-      else
-        far_level_lane<D, COUNT>(CP, pr.cbase + pb + lvl_off(D, l) + 1, me, l, nx, F, G, lane_g, nint);
-    }
+    far_field<D, COUNT, T, PIPE>(CP, pr.cbase + pb + 1, c, L, G, lane_g, g, nint);
   }
-  float Fs[4] = {0.f, 0.f, 0.f, 0.f};
+  float4 xnew[T];
+  bool leader[T];
 #pragma unroll
-  for (int m = 0; m < D; ++m) Fs[m] = F[m].x + F[m].y;
-  // combine the lanes of the group (groups never straddle a warp)
-  for (int o = G >> 1; o > 0; o >>= 1)
+  for (int t = 0; t < T; ++t) {
+    float Fs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int m = 0; m < D; ++m) Fs[m] += __shfl_xor_sync(0xffffffffu, Fs[m], o);
-  const bool leader = valid && lane_g == 0;
-  float4 xnew = make_float4(0, 0, 0, 0);
-  if (leader) {
-    const float wn = ws ? ws[p] : 1.0f;
-    const uint32_t v = svals[p];
-    float4 ya = yatt[v];
-    float y0 = kappa * wn * Fs[0] + ya.x;
-    float y1 = D > 1 ? kappa * wn * Fs[1] + ya.y : 0.f;
-    float y2 = D > 2 ? kappa * wn * Fs[2] + ya.z : 0.f;
-    float y3 = D > 3 ? kappa * wn * Fs[3] + ya.w : 0.f;
-    if (y_out) y_out[v] = make_float4(y0, y1, y2, y3);
-    float ny = sqrtf(y0 * y0 + y1 * y1 + y2 * y2 + y3 * y3);
-    float step = step_override > 0.0f ? step_override : s0[pb] * scale_tab[*tctr];
-    float a = ny > 0.0f ? step / ny : 0.0f;
-    xnew = make_float4(xn.x - a * y0, D > 1 ? xn.y - a * y1 : 0.f, D > 2 ? xn.z - a * y2 : 0.f,
-                       D > 3 ? xn.w - a * y3 : 0.f);
-    x[v] = xnew;
+    for (int m = 0; m < D; ++m) Fs[m] = g.F[t][m].x + g.F[t][m].y;
+    // combine the lanes of the group (groups never straddle a warp)
+    for (int o = G >> 1; o > 0; o >>= 1)
+#pragma unroll
+      for (int m = 0; m < D; ++m) Fs[m] += __shfl_xor_sync(0xffffffffu, Fs[m], o);
+    leader[t] = ok[t] && lane_g == 0;
+    xnew[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (leader[t])
+      xnew[t] = step_target<D>(p + t, xn[t], Fs, ws, svals, yatt, kappa, step_override, s0, pb, scale_tab, tctr, x, y_out);
   }
   if (COUNT) {
     unsigned long long tot = nint;
@@ -1442,7 +1517,339 @@ __global__ void __launch_bounds__(kStepBlock, MLP ? 3 : VMO_STEP_MINBLOCKS) k_re
     for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
     if (lane_id() == 0 && tot) atomicAdd(icount, tot);
   }
-  bbox_warp_fold<D>(xnew, leader, bb_next + (int64_t)pb * 8);
+  bbox_warp_fold<D, T>(xnew, leader, bb_next + (int64_t)pb * 8);
+}
+
+// The same step for launches that leave most of the GPU idle at one thread
+// per target lane.  The force sums of a lane are chains of additions whose
+// order is part of the result, so they cannot be split; but only the
+// additions are serial.  kSplitR threads of the producer warps work for each
+// target lane: each evaluates the terms (factor g and difference dx of each
+// half) of its own source pairs of the lane's sequence, a round of up to
+// kSplitS pairs at a time, and leaves them in shared memory; meanwhile the
+// block's last warp, one thread per target lane and half, adds the round
+// before in sequence order with the same fused operations.  The sums are those
+// of k_repulse_update bit for bit.
+constexpr int kSplitR = 8;                          // threads per target lane
+constexpr int kSplitS = 4 * kSplitR;                // pairs of a round
+constexpr int kSplitWarps = 4;                      // producer warps
+constexpr int kSplitLanes = kSplitWarps * 32 / kSplitR;  // target lanes of a block: 16, two threads each of the last warp
+constexpr int kSplitBlock = 32 * (kSplitWarps + 1);
+constexpr int kSplitPitch = kSplitS + 1;            // terms between two halves: 16-byte reads of 8 threads miss no bank twice
+
+// Far-field rows of a target lane as one sequence over the levels (the rows
+// and the order of FarRows), visited by one of R threads: rows first, first + R, ...
+template <int D, int R>
+struct FarSeq {
+  int l, L, G, lane_g;
+  int32_t c[D], me[D], lo[D], hi[D];
+  int i, n;      // the lane's row of the level and how many it has there
+  int64_t base;  // first pair of the level plus lo[0] / 2
+  int64_t cell0;
+
+  __device__ __forceinline__ void level() {
+    if (l > L) return;
+    const int sl = 1 << l;
+    int rows = 1;
+#pragma unroll
+    for (int m = 0; m < D; ++m) {
+      me[m] = c[m] >> (L - l);
+      const int par = me[m] >> 1;
+      lo[m] = max(2 * par - 2, 0);
+      hi[m] = min(2 * par + 3, sl - 1);
+      if (m > 0) rows *= hi[m] - lo[m] + 1;
+    }
+    n = rows > lane_g ? (rows - lane_g + G - 1) / G : 0;
+    base = ((cell0 + lvl_off(D, l)) >> 1) + (lo[0] >> 1);
+  }
+  __device__ __forceinline__ void init(int64_t cell, const int32_t* cc, int LL, int GG, int lg, int first) {
+    cell0 = cell;
+    L = LL;
+    G = GG;
+    lane_g = lg;
+#pragma unroll
+    for (int m = 0; m < D; ++m) c[m] = cc[m];
+    l = 2;
+    n = 0;
+    level();
+    i = first;
+    settle();
+  }
+  __device__ __forceinline__ void settle() {
+    while (l <= L && i >= n) {
+      i -= n;
+      ++l;
+      level();
+    }
+  }
+  __device__ __forceinline__ bool done() const { return l > L; }
+  // rows of the lane on all levels
+  __device__ __forceinline__ int count(int64_t cell, const int32_t* cc, int LL, int GG, int lg) const {
+    FarSeq<D, R> s;
+    s.init(cell, cc, LL, GG, lg, 0);
+    int sum = 0;
+    for (s.l = 2; s.l <= LL; ++s.l) {
+      s.level();
+      sum += s.n;
+    }
+    return sum;
+  }
+  __device__ __forceinline__ void advance() {
+    i += R;
+    settle();
+  }
+  __device__ __forceinline__ int64_t row(bool& third, unsigned& mask) const {
+    int rr = lane_g + G * i;
+    int q[D];
+    bool in = true;
+#pragma unroll
+    for (int m = 1; m < D; ++m) {
+      const int e = hi[m] - lo[m] + 1;  // 4 or 6 cells
+      const int t = m + 1 < D ? (e == 4 ? rr >> 2 : (rr * 10923) >> 16) : 0;
+      q[m] = lo[m] + rr - t * e;
+      rr = t;
+      in = in && q[m] >= me[m] - 1 && q[m] <= me[m] + 1;
+    }
+    int64_t idx = 0;
+#pragma unroll
+    for (int m = D - 1; m >= 1; --m) idx = (idx << l) + q[m];
+    third = hi[0] - lo[0] > 4;
+    const int o = me[0] - lo[0];
+    mask = in ? (o > 0 ? 7u << (o - 1) : 3u) : 0u;
+    return base + idx * (int64_t(1) << (l - 1));
+  }
+};
+
+// Terms of one pair, with pair_charge's operations: (g, dx0, dx1, dx2) of the
+// even and the odd source to slot `at` of their halves (dx3 beside them).
+template <int D, bool UNIT>
+__device__ __forceinline__ void pair_terms(const float4* P, const float2* nx, float2 w, float4* terms, float* dx3,
+                                           int at) {
+  float2 dx[4];
+  dx[0] = __fadd2_rn(make_float2(P[0].x, P[0].y), nx[0]);
+  dx[1] = __fadd2_rn(make_float2(P[0].z, P[0].w), nx[1]);
+  dx[2] = dx[3] = make_float2(0.f, 0.f);
+  if (D > 2) dx[2] = __fadd2_rn(make_float2(P[1].x, P[1].y), nx[D > 2 ? 2 : 0]);
+  if (D > 3) dx[3] = __fadd2_rn(make_float2(P[1].z, P[1].w), nx[D > 3 ? 3 : 0]);
+  const float2 g = pair_factor<D, UNIT>(dx, w);
+  terms[at] = make_float4(g.x, dx[0].x, dx[1].x, dx[2].x);
+  terms[kSplitPitch + at] = make_float4(g.y, dx[0].y, dx[1].y, dx[2].y);
+  if (D > 3) {
+    dx3[at] = dx[3].x;
+    dx3[kSplitPitch + at] = dx[3].y;
+  }
+}
+
+template <int D>
+__global__ void __launch_bounds__(kSplitBlock, 4) k_repulse_split(
+    const float4* __restrict__ xs, const float* __restrict__ ws, const float4* __restrict__ XP,
+    const uint32_t* __restrict__ svals, const uint32_t* __restrict__ scell, const int32_t* __restrict__ cst,
+    const float4* __restrict__ CP, const float4* __restrict__ yatt, const int32_t* __restrict__ wprob,
+    const ProbDev* __restrict__ prob, float kappa, const float* __restrict__ s0,
+    const float* __restrict__ scale_tab, const int32_t* __restrict__ tctr, float step_override,
+    float4* __restrict__ x, float4* __restrict__ y_out, uint32_t* __restrict__ bb_next) {
+  pdl_enter();
+  constexpr int N = Pair<D>::N, R = kSplitR, S = kSplitS, PITCH = kSplitPitch, LN = kSplitLanes;
+  constexpr int NR = D == 2 ? 3 : (D == 3 ? 9 : 27);  // near-field rows
+  __shared__ float4 terms[2][LN * 2 * PITCH];
+  __shared__ float terms3[2][D > 3 ? LN * 2 * PITCH : 1];
+  __shared__ int32_t rq[LN][NR][2];     // near rows: [qa, qb)
+  __shared__ int32_t rpre[LN][NR + 1];  // pairs of the lane before each row
+  __shared__ int rounds[2];             // near, far
+  const bool producer = threadIdx.x < 32 * kSplitWarps;
+  const int grp = producer ? threadIdx.x / R : (threadIdx.x & 31) >> 1;  // target lane of the block
+  const int r = threadIdx.x & (R - 1);
+  const int64_t vl = (int64_t)blockIdx.x * LN + grp;  // a block's target lanes lie in one problem
+  const int pb = wprob[((int64_t)blockIdx.x * LN) >> 5];
+  const ProbDev pr = prob[pb];
+  const int G = pr.group;
+  const int64_t rel = vl - pr.tbase;
+  const int lane_g = (int)(rel & (G - 1));
+  const int64_t tgt = rel / G;
+  const bool valid = tgt < pr.k;
+  const int64_t p = valid ? pr.vbase + tgt : pr.vbase;
+  const int L = pr.L, side = 1 << L;
+  float4 xn = make_float4(0.f, 0.f, 0.f, 0.f);
+  uint32_t packed = 0;
+  if (valid) {
+    xn = xs[p];
+    packed = scell[p];
+  }
+  int32_t c[D];
+#pragma unroll
+  for (int m = 0; m < D; ++m) c[m] = (int32_t)((packed >> (m * field_bits(D))) & ((1u << field_bits(D)) - 1));
+  if (threadIdx.x < 2) rounds[threadIdx.x] = 0;
+  if (producer) {  // near field: the lane's pairs of the 3^(d-1) rows as one sequence
+    for (int o = r; o < NR; o += R) {
+      int32_t cc[D];
+      int oo = o;
+      bool inside = valid;
+      cc[0] = max(c[0] - 1, 0);
+#pragma unroll
+      for (int m = 1; m < D; ++m) {
+        cc[m] = c[m] + (oo % 3) - 1;
+        oo /= 3;
+        inside = inside && cc[m] >= 0 && cc[m] < side;
+      }
+      int qa = 0, qb = 0, np = 0;
+      if (inside) {
+        const int32_t* cs = cst + pr.fbase + pb;
+        const int64_t r0 = rowmajor<D>(cc, side);
+        qa = cs[r0] - (int)pr.vbase;  // problem-local
+        qb = cs[r0 + min(c[0] + 1, side - 1) - cc[0] + 1] - (int)pr.vbase;
+        if (qb > qa) np = max(((qb + 1) >> 1) - (qa >> 1) - lane_g, 0);
+      }
+      rq[grp][o][0] = qa;
+      rq[grp][o][1] = qb;
+      rpre[grp][o + 1] = (np + G - 1) / G;
+    }
+  }
+  __syncthreads();
+  FarSeq<D, R> it;
+  it.init(pr.cbase + pb + 1, c, valid ? L : 1, G, lane_g, r);
+  if (producer && r == 0) {
+    int run = 0;
+    rpre[grp][0] = 0;
+    for (int o = 1; o <= NR; ++o) rpre[grp][o] = run += rpre[grp][o];
+    atomicMax(&rounds[0], (run + S - 1) / S);
+    atomicMax(&rounds[1], valid ? (it.count(pr.cbase + pb + 1, c, L, G, lane_g) + R - 1) / R : 0);
+  }
+  __syncthreads();
+  const int near = rounds[0], all = near + rounds[1];
+  if (producer) {
+    float2 nx[D];
+#pragma unroll
+    for (int m = 0; m < D; ++m) nx[m] = make_float2(-comp(xn, m), -comp(xn, m));
+    const int total = rpre[grp][NR];
+    const float4* xp = XP + ((pr.vbase + pb + 1) >> 1) * N;  // the problem's first pair
+    float4* out = nullptr;
+    float* out3 = nullptr;
+    int o = 0, h0[4], qa[4], qb[4];
+    float4 Q[4][N];
+    // the thread's pairs of a near round: r, r + R, ... of the round's part of
+    // the sequence, so that the R threads read consecutive pairs
+    auto load_near = [&](int rd) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int f = rd * S + u * R + r;
+        h0[u] = -1;
+        if (f < total) {
+          while (f >= rpre[grp][o + 1]) ++o;
+          qa[u] = rq[grp][o][0];
+          qb[u] = rq[grp][o][1];
+          const int j = (qa[u] >> 1) + lane_g + G * (f - rpre[grp][o]);
+          h0[u] = 2 * j;
+          pair_load<D>(xp, j, Q[u]);
+        }
+      }
+    };
+    // its pairs of a far round: thread r steps through row r of the round's R
+    // rows, and the R threads share out the rows' 3 R pairs in order (three
+    // neighbours read one row; a row each would scatter every load over R lines)
+    unsigned mask[3] = {0u, 0u, 0u};
+    bool have[3] = {false, false, false};
+    auto load_far = [&]() {
+      bool third = false;
+      unsigned m = 0u;
+      const bool live = !it.done();
+      const int row = live ? (int)it.row(third, m) : -1;
+      m |= third ? 64u : 0u;
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        const int f = u * R + r, q = (f * 11) >> 5, i = f - 3 * q;  // f / 3 for f < 24
+        const int rq_ = __shfl_sync(0xffffffffu, row, (threadIdx.x & 31 & ~(R - 1)) + q);
+        const unsigned mq = __shfl_sync(0xffffffffu, m, (threadIdx.x & 31 & ~(R - 1)) + q);
+        have[u] = rq_ >= 0 && (i < 2 || (mq & 64u));
+        mask[u] = mq >> (2 * i);
+        if (have[u]) pair_load<D>(CP, (int64_t)rq_ + i, Q[u]);
+      }
+      it.advance();
+    };
+    auto put_zero = [&](int at) {
+      out[at] = out[PITCH + at] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (D > 3) out3[at] = out3[PITCH + at] = 0.f;
+    };
+    if (near > 0) load_near(0);
+    else if (all > 0) load_far();
+    for (int t = 0; t < all; ++t) {
+      out = &terms[t & 1][grp * 2 * PITCH];
+      out3 = &terms3[t & 1][D > 3 ? grp * 2 * PITCH : 0];
+      if (t < near) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int at = u * R + r;  // 16-byte writes of the R threads side by side
+          if (h0[u] < 0) {
+            put_zero(at);
+            continue;
+          }
+          const bool m0 = h0[u] < qa[u], m1 = h0[u] + 1 >= qb[u];
+          if (ws) {
+            float2 w = pair_weight<D>(Q[u]);
+            w.x = m0 ? 0.0f : w.x;
+            w.y = m1 ? 0.0f : w.y;
+            pair_terms<D, false>(Q[u], nx, w, out, out3, at);
+          } else {
+            pair_mask_half<D>(Q[u], 0, m0, nx);
+            pair_mask_half<D>(Q[u], 1, m1, nx);
+            pair_terms<D, true>(Q[u], nx, make_float2(1.0f, 1.0f), out, out3, at);
+          }
+        }
+        if (t + 1 < near) load_near(t + 1);
+        else if (t + 1 < all) load_far();
+      } else {
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+          if (!have[u]) {
+            put_zero(u * R + r);
+            continue;
+          }
+          float2 w = pair_weight<D>(Q[u]);
+          w.x = mask[u] & 1u ? 0.0f : w.x;
+          w.y = mask[u] & 2u ? 0.0f : w.y;
+          pair_terms<D, false>(Q[u], nx, w, out, out3, u * R + r);
+        }
+        if (t + 1 < all) load_far();
+      }
+      __syncthreads();
+    }
+    return;
+  }
+  // the adding warp: thread = target lane and half
+  float F[D];
+#pragma unroll
+  for (int m = 0; m < D; ++m) F[m] = 0.f;
+  const int half = (threadIdx.x & 31) * PITCH;
+  auto add = [&](const float4* in, const float* in3, auto U) {
+#pragma unroll
+    for (int f = 0; f < R * decltype(U)::value; ++f) {
+      const float4 v = in[half + f];
+      F[0] = __fmaf_rn(v.x, v.y, F[0]);
+      F[1] = __fmaf_rn(v.x, v.z, F[1]);
+      if (D > 2) F[D > 2 ? 2 : 0] = __fmaf_rn(v.x, v.w, F[D > 2 ? 2 : 0]);
+      if (D > 3) F[D > 3 ? 3 : 0] = __fmaf_rn(v.x, in3[half + f], F[D > 3 ? 3 : 0]);
+    }
+  };
+  auto add_round = [&](int t) {
+    if (t < near) add(terms[t & 1], terms3[t & 1], std::integral_constant<int, 4>());
+    else add(terms[t & 1], terms3[t & 1], std::integral_constant<int, 3>());
+  };
+  for (int t = 0; t < all; ++t) {
+    if (t > 0) add_round(t - 1);
+    __syncthreads();
+  }
+  if (all > 0) add_round(all - 1);
+  // even + odd sources, then the G lanes of the target with the same xor tree
+  float Fs[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int m = 0; m < D; ++m) Fs[m] = F[m] + __shfl_xor_sync(0xffffffffu, F[m], 1);
+  for (int o = G >> 1; o > 0; o >>= 1)
+#pragma unroll
+    for (int m = 0; m < D; ++m) Fs[m] += __shfl_xor_sync(0xffffffffu, Fs[m], 2 * o);
+  const bool leader = valid && lane_g == 0 && (threadIdx.x & 1) == 0;
+  float4 xnew = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (leader)
+    xnew = step_target<D>(p, xn, Fs, ws, svals, yatt, kappa, step_override, s0, pb, scale_tab, tctr, x, y_out);
+  bbox_warp_fold<D, 1>(&xnew, &leader, bb_next + (int64_t)pb * 8);
 }
 
 // Step-length factors decay^t, t < iters: the running double product, each
@@ -1748,10 +2155,11 @@ __global__ void k_round_w(const double* __restrict__ wd, int64_t n, float* __res
   if (i < n) w[i] = (float)wd[i];
 }
 
-__global__ void k_fill_vprob(const int64_t* __restrict__ vb, int P, int64_t K, int32_t* __restrict__ vprob) {
+// Problem of every item of a table whose problems start at base.
+__global__ void k_fill_prob(const int64_t* __restrict__ base, int P, int64_t n, int32_t* __restrict__ out) {
   int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= K) return;
-  vprob[v] = find_problem(vb, P, v);
+  if (v >= n) return;
+  out[v] = find_problem(base, P, v);
 }
 
 __global__ void k_set_last(int32_t* ptr, int64_t n, const int32_t* total) { ptr[n] = *total; }
@@ -1833,7 +2241,11 @@ vmo_status level_setup(LevelBatch& lb, int d, int occ, cudaStream_t s) {
   lb.cbase.assign(P + 1, 0);
   lb.fbase.assign(P + 1, 0);
   std::vector<ProbDev> pd(P);
-  std::vector<int64_t> tb(P + 1, 0), bk(P + 1, 0);
+  // per problem: vertices, warps of the step kernel (one and two targets per
+  // thread), bricks; each with the map from the item to its problem
+  std::vector<int64_t> base((size_t)4 * (P + 1), 0);
+  int64_t *vb = base.data(), *wb = vb + P + 1, *wb2 = wb + P + 1, *bk = wb2 + P + 1;
+  int64_t chunks = 0;
   lb.maxL = 1;
   for (int p = 0; p < P; ++p) {
     int64_t k = lb.vbase[p + 1] - lb.vbase[p];
@@ -1849,28 +2261,39 @@ vmo_status level_setup(LevelBatch& lb, int d, int occ, cudaStream_t s) {
     pd[p].L = L;
     pd[p].side = init_side(std::max<int64_t>(k, 1), d);
     pd[p].group = group_size(k);
-    pd[p].tbase = tb[p];
-    tb[p + 1] = tb[p] + ((k * pd[p].group + 31) / 32) * 32;
+    pd[p].tbase = 32 * wb[p];
+    pd[p].tbase2 = 32 * wb2[p];
+    pd[p].bbase = bk[p];
+    pd[p].lbase = chunks;
+    // at most one chunk of a single point per cell
+    const int64_t ch = (k + std::min<int64_t>(k, int64_t(1) << (d * L))) / 2;
+    chunks += ch;
+    vb[p + 1] = lb.vbase[p + 1];
+    wb[p + 1] = wb[p] + (k * pd[p].group + 31) / 32;
+    wb2[p + 1] = wb2[p] + (ch * pd[p].group + 31) / 32;
     bk[p + 1] = bk[p] + (int64_t(1) << (d * std::max(L - brick_log2(d), 0)));
   }
-  lb.threads = tb[P];
+  lb.threads = 32 * wb[P];
+  lb.threads2 = 32 * wb2[P];
   lb.bricks = bk[P];
+  lb.chunks = chunks;
   VMO_TRY(lb.prob.resize(std::max(P, 1)));
   VMO_TRY(lb.vprob.resize((size_t)std::max<int64_t>(lb.K, 1)));
   VMO_CUDA(cudaMemcpyAsync(lb.prob.ptr, pd.data(), P * sizeof(ProbDev), cudaMemcpyHostToDevice, s));
-  VMO_TRY(lb.tbase.resize(P + 1));
-  VMO_CUDA(cudaMemcpyAsync(lb.tbase.ptr, tb.data(), (P + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-  VMO_TRY(lb.bbase.resize(P + 1));
-  VMO_CUDA(cudaMemcpyAsync(lb.bbase.ptr, bk.data(), (P + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-  int64_t* vb;
-  VMO_CUDA(cudaMallocAsync((void**)&vb, (P + 1) * sizeof(int64_t), s));
+  VMO_TRY(lb.wprob.resize((size_t)std::max<int64_t>(wb[P], 1)));
+  VMO_TRY(lb.wprob2.resize((size_t)std::max<int64_t>(wb2[P], 1)));
+  VMO_TRY(lb.bprob.resize((size_t)std::max<int64_t>(bk[P], 1)));
+  int64_t* db;
+  VMO_CUDA(cudaMallocAsync((void**)&db, base.size() * sizeof(int64_t), s));
   g_device_allocs.fetch_add(1, std::memory_order_relaxed);
-  VMO_CUDA(cudaMemcpyAsync(vb, lb.vbase.data(), (P + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-  if (lb.K > 0) {
-    launch(k_fill_vprob, grid_for(lb.K, kBlock), kBlock, 0, s, vb, P, lb.K, lb.vprob.ptr);
-    VMO_LAUNCHED("fill_vprob");
+  VMO_CUDA(cudaMemcpyAsync(db, base.data(), base.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+  int32_t* maps[4] = {lb.vprob.ptr, lb.wprob.ptr, lb.wprob2.ptr, lb.bprob.ptr};
+  for (int q = 0; q < 4; ++q) {
+    const int64_t n = base[(size_t)q * (P + 1) + P];
+    if (n > 0) launch(k_fill_prob, grid_for(n, kBlock), kBlock, 0, s, db + (size_t)q * (P + 1), P, n, maps[q]);
   }
-  VMO_CUDA(cudaFreeAsync(vb, s));
+  VMO_LAUNCHED("fill_prob");
+  VMO_CUDA(cudaFreeAsync(db, s));
 
   // host vectors must outlive the copies
   VMO_CUDA(cudaStreamSynchronize(s));
@@ -1936,7 +2359,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   uint32_t *keys, *arrival = nullptr, *slot = nullptr, *svals, *scell, *bb;
   float4 *xs, *XP, *yatt, *St, *CP, *z = nullptr;
   float *ws = nullptr, *Wt, *s0;
-  int32_t *cst, *cnt = nullptr, *tot = nullptr, *done = nullptr;
+  int32_t *cst, *cnt = nullptr, *tot = nullptr, *done = nullptr, *chunk = nullptr, *nchunk = nullptr;
   const int64_t ncell = lb.cbase[P], nfine = lb.fbase[P];
   VMO_TRY(sc.alloc(&keys, K));
   VMO_TRY(sc.alloc(&svals, K));
@@ -1967,6 +2390,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
         bin1 = false;  // the device-wide sequence then
       }
     });
+  const bool pair = !bin1 && lb.threads >= kPairThreadsMin;
   const int64_t ncnt = nfine + P;  // entries of the cell start table
   const bool one_cluster = ncnt <= kCellScanMax;
   const unsigned scan_blocks = grid_for(ncnt, kCellScanThreads * kCellScanItems);
@@ -1976,10 +2400,13 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
     VMO_TRY(sc.alloc(&cnt, ncnt));
     VMO_TRY(sc.alloc(&done, P));
     if (!one_cluster) VMO_TRY(sc.alloc(&tot, scan_blocks));
+    if (pair) {
+      VMO_TRY(sc.alloc(&chunk, std::max<int64_t>(lb.chunks, 1)));
+      VMO_TRY(sc.alloc(&nchunk, P));
+    }
     VMO_CUDA(cudaMemsetAsync(cnt, 0, ncnt * sizeof(int32_t), s));
     VMO_CUDA(cudaMemsetAsync(done, 0, P * sizeof(int32_t), s));
   }
-  const int nreset = 8 * P;
   launch(k_bbox_reset, grid_for(16 * P, kBlock), kBlock, 0, s, bb, 16 * P);
   VMO_LAUNCHED("bbox_reset");
   const float kappa = d == 2 ? 1.0f : (float)(d - 2);
@@ -2038,7 +2465,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
       } else {
         auto keys_kernel = K >= kKeyItemsMin ? k_keys<D, 4> : k_keys<D, 1>;
         launch(keys_kernel, grid_for(K >= kKeyItemsMin ? (K + 3) / 4 : K, kBlock), kBlock, 0, ms, x, K, lb.vprob.ptr,
-               lb.prob.ptr, cur, keys, arrival, cnt, nxt, nreset, tctr);
+               lb.prob.ptr, cur, keys, arrival, cnt, nchunk, P, nxt, tctr);
         if (keys_out && t == 0) cudaMemcpyAsync(keys_out, keys, K * 4, cudaMemcpyDeviceToDevice, ms);
         if (one_cluster) {
           launch(k_cell_scan, kCellScanCtas, kCellScanThreads, 0, ms, cnt, cst, ncnt);
@@ -2049,20 +2476,29 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
         launch(k_slots, grid_for(K, kBlock), kBlock, 0, ms, keys, arrival, K, lb.vprob.ptr, lb.prob.ptr, cst, slot);
         launch(k_place<D>, grid_for(K, kBlock), kBlock, 0, ms, slot, keys, K, x, lb.w, lb.vprob.ptr, lb.prob.ptr, cst,
                cnt, ncnt, svals, xs, ws, scell, XP);
-        launch(k_cells<D>, (unsigned)lb.bricks, kBlock, 0, ms, lb.bbase.ptr, P, lb.prob.ptr, xs, ws, cst, St, Wt, CP,
-               done);
+        launch(k_cells<D>, (unsigned)lb.bricks, kBlock, 0, ms, lb.bprob.ptr, lb.prob.ptr, xs, ws, cst, St, Wt, CP,
+               done, chunk, nchunk);
       }
       if (side) cudaStreamWaitEvent(ms, ev_join, 0);
       const bool timed = stats_timing();
       if (timed) stats_time_begin(ms);
       unsigned long long* icount = stats_interaction_counter();
-      // few warps per SM: the far-field variant with two rows in flight
-      const bool mlp = lb.threads <= g_tuning.small_step_threads.load(std::memory_order_relaxed);
-      auto step_kernel = icount ? (mlp ? k_repulse_update<D, true, true> : k_repulse_update<D, true, false>)
-                                : (mlp ? k_repulse_update<D, false, true> : k_repulse_update<D, false, false>);
-      launch(step_kernel, grid_for(lb.threads, kStepBlock), kStepBlock, 0, ms, xs, ws, XP, svals, scell, cst, CP,
-             yatt, lb.tbase.ptr, P, lb.prob.ptr, lb.threads, kappa, s0, scale_tab, tctr, step_override, x, y_out, nxt,
-             icount);
+      const int64_t small = g_tuning.small_step_threads.load(std::memory_order_relaxed);
+      auto step_launch = [&](auto kernel, int64_t nth, const int32_t* wprob) {
+        launch(kernel, grid_for(nth, kStepBlock), kStepBlock, 0, ms, xs, ws, XP, svals, scell, cst, CP, yatt, wprob,
+               lb.prob.ptr, nth, chunk, nchunk, kappa, s0, scale_tab, tctr, step_override, x, y_out, nxt, icount);
+      };
+      if (icount)
+        step_launch(k_repulse_update<D, true, kStepPlain>, lb.threads, lb.wprob.ptr);
+      else if (pair)
+        step_launch(k_repulse_update<D, false, kStepPair>, lb.threads2, lb.wprob2.ptr);
+      else if (D > 2 && lb.threads <= small / 8 * 5)
+        launch(k_repulse_split<D>, (unsigned)(lb.threads / kSplitLanes), kSplitBlock, 0, ms, xs, ws, XP, svals, scell,
+               cst, CP, yatt, lb.wprob.ptr, lb.prob.ptr, kappa, s0, scale_tab, tctr, step_override, x, y_out, nxt);
+      else if (D == 2 && lb.threads <= small)
+        step_launch(k_repulse_update<2, false, kStepPipe>, lb.threads, lb.wprob.ptr);
+      else
+        step_launch(k_repulse_update<D, false, kStepPlain>, lb.threads, lb.wprob.ptr);
       if (timed) stats_time_end(ms, (uint64_t)K);
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return cuda_fail(e, "layout step", __FILE__, __LINE__);
