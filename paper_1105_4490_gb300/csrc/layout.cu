@@ -225,14 +225,12 @@ template <int D, int U>
 __global__ void __launch_bounds__(kBlock) k_keys(const float4* __restrict__ x, int64_t K, const int32_t* __restrict__ vprob,
                                                  const ProbDev* __restrict__ prob, const uint32_t* __restrict__ bb,
                                                  uint32_t* __restrict__ keys, uint32_t* __restrict__ arrival,
-                                                 int32_t* __restrict__ cnt, int32_t* __restrict__ nchunk, int P,
-                                                 uint32_t* __restrict__ bb_next, int32_t* __restrict__ tctr) {
+                                                 int32_t* __restrict__ cnt, int P, uint32_t* __restrict__ bb_next,
+                                                 int32_t* __restrict__ tctr) {
   pdl_enter();
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (gt == 0) ++*tctr;  // the level's step (read by the step kernel of this step)
   const int64_t nreset = 8 * (int64_t)P;
-  if (nchunk)
-    for (int64_t r = gt; r < P; r += (int64_t)gridDim.x * blockDim.x) nchunk[r] = 0;
   for (int64_t r = gt; r < nreset; r += (int64_t)gridDim.x * blockDim.x) bb_next[r] = ((r & 7) < 4) ? 0xFFFFFFFFu : 0u;
   const int64_t v0 = (int64_t)blockIdx.x * blockDim.x * U + threadIdx.x;
   float4 xv[U];
@@ -262,14 +260,14 @@ __global__ void __launch_bounds__(kBlock) k_keys(const float4* __restrict__ x, i
 // Cell counts -> cell start table: the exclusive scan of cnt (every problem's
 // finest cells and one empty end entry, problem after problem, as the
 // problems' points are) is the first sorted position of every cell, of the
-// end entry the problem's end.  One cluster scans a tile of
-// kCellScanTile entries at a time; its blocks exchange their totals through
-// distributed shared memory.
+// end entry the problem's end.  With two targets per thread the scan of
+// ceil(cnt / 2) next to it (cch) numbers the cells' chunks of two points.  One
+// cluster scans a table of up to kCellScanTile entries; its blocks exchange
+// their totals through distributed shared memory.
 constexpr int kCellScanCtas = 8;
 constexpr int kCellScanThreads = 1024;
 constexpr int kCellScanItems = 16;
 constexpr int64_t kCellScanTile = (int64_t)kCellScanCtas * kCellScanThreads * kCellScanItems;
-constexpr int64_t kCellScanMax = kCellScanTile;  // larger tables: two launches over every SM
 
 __device__ __forceinline__ void load_items(const int32_t* __restrict__ a, int64_t i0, int64_t n, int32_t* v) {
   if (i0 + kCellScanItems <= n) {
@@ -287,14 +285,7 @@ __device__ __forceinline__ void load_items(const int32_t* __restrict__ a, int64_
   }
 }
 
-__device__ __forceinline__ void store_prefix(int32_t* __restrict__ a, int64_t i0, int64_t n, const int32_t* v,
-                                             int32_t run) {
-  int32_t e[kCellScanItems];
-#pragma unroll
-  for (int j = 0; j < kCellScanItems; ++j) {
-    e[j] = run;
-    run += v[j];
-  }
+__device__ __forceinline__ void store_items(int32_t* __restrict__ a, int64_t i0, int64_t n, const int32_t* e) {
   if (i0 + kCellScanItems <= n) {
 #pragma unroll
     for (int j = 0; j < kCellScanItems / 4; ++j)
@@ -306,74 +297,87 @@ __device__ __forceinline__ void store_prefix(int32_t* __restrict__ a, int64_t i0
   }
 }
 
+// Sum of a thread's items: points in the low, chunks in the high word (both
+// below 2^31, so the words of a sum never mix).
+__device__ __forceinline__ uint64_t items_sum(const int32_t* v) {
+  uint64_t s = 0;
+#pragma unroll
+  for (int j = 0; j < kCellScanItems; ++j) s += ((uint64_t)(uint32_t)((v[j] + 1) >> 1) << 32) | (uint32_t)v[j];
+  return s;
+}
+
+// The starts of a thread's items from the sums before it.
+__device__ __forceinline__ void store_starts(int32_t* __restrict__ cst, int32_t* __restrict__ cch, int64_t i0, int64_t n,
+                                             const int32_t* v, uint64_t before) {
+  int32_t e[kCellScanItems];
+  int32_t run = (int32_t)(uint32_t)before;
+#pragma unroll
+  for (int j = 0; j < kCellScanItems; ++j) {
+    e[j] = run;
+    run += v[j];
+  }
+  store_items(cst, i0, n, e);
+  if (!cch) return;
+  run = (int32_t)(before >> 32);
+#pragma unroll
+  for (int j = 0; j < kCellScanItems; ++j) {
+    e[j] = run;
+    run += (v[j] + 1) >> 1;
+  }
+  store_items(cch, i0, n, e);
+}
+
 __global__ void __cluster_dims__(kCellScanCtas, 1, 1) __launch_bounds__(kCellScanThreads)
-    k_cell_scan(const int32_t* __restrict__ cnt, int32_t* __restrict__ cst, int64_t n) {
+    k_cell_scan(const int32_t* __restrict__ cnt, int32_t* __restrict__ cst, int32_t* __restrict__ cch, int64_t n) {
   pdl_enter();
-  __shared__ int32_t ws[33];
-  __shared__ int32_t tot[2];             // this block's total, by parity of the tile
-  __shared__ int32_t peer[kCellScanCtas];
+  __shared__ uint64_t ws[33];
+  __shared__ uint64_t tot;
+  __shared__ uint64_t peer[kCellScanCtas];
   auto cluster = cooperative_groups::this_cluster();
   const unsigned r = cluster.block_rank();
-  int32_t carry = 0;
-  int par = 0;
-  for (int64_t base = 0; base < n; base += kCellScanTile, par ^= 1) {
-    const int64_t i0 = base + ((int64_t)r * kCellScanThreads + threadIdx.x) * kCellScanItems;
-    int32_t v[kCellScanItems];
-    load_items(cnt, i0, n, v);
-    int32_t sum = 0;
+  const int64_t i0 = ((int64_t)r * kCellScanThreads + threadIdx.x) * kCellScanItems;
+  int32_t v[kCellScanItems];
+  load_items(cnt, i0, n, v);
+  uint64_t total;
+  const uint64_t ex = block_exclusive<uint64_t>(items_sum(v), ws, &total);
+  if (threadIdx.x == 0) tot = total;
+  cluster.sync();
+  if (threadIdx.x < kCellScanCtas) peer[threadIdx.x] = *cluster.map_shared_rank(&tot, threadIdx.x);
+  cluster.sync();  // also: no block leaves while another may still read its total
+  uint64_t before = ex;
 #pragma unroll
-    for (int j = 0; j < kCellScanItems; ++j) sum += v[j];
-    int32_t total;
-    const int32_t ex = block_exclusive<int32_t>(sum, ws, &total);
-    if (threadIdx.x == 0) tot[par] = total;
-    cluster.sync();
-    if (threadIdx.x < kCellScanCtas) peer[threadIdx.x] = *cluster.map_shared_rank(&tot[par], threadIdx.x);
-    __syncthreads();
-    int32_t before = carry;
-#pragma unroll
-    for (unsigned q = 0; q < kCellScanCtas; ++q) {
-      before += q < r ? peer[q] : 0;
-      carry += peer[q];
-    }
-    store_prefix(cst, i0, n, v, before + ex);
-    __syncthreads();  // peer is rewritten by the next tile
-  }
-  cluster.sync();  // no block leaves while another may still read its total
+  for (unsigned q = 0; q < kCellScanCtas; ++q) before += q < r ? peer[q] : 0;
+  store_starts(cst, cch, i0, n, v, before);
 }
 
 // The same scan for larger tables in two launches: block totals, then every
-// block adds up the totals before its own and scans its part.
+// block adds up the totals before its own and scans its part (one cluster
+// taking several tiles in turn needs 14 us for three, the two launches 9 us).
 __global__ void __launch_bounds__(kCellScanThreads) k_cell_totals(const int32_t* __restrict__ cnt, int64_t n,
-                                                                  int32_t* __restrict__ tot) {
+                                                                  uint64_t* __restrict__ tot) {
   pdl_enter();
-  __shared__ int32_t ws[33];
+  __shared__ uint64_t ws[33];
   int32_t v[kCellScanItems];
   load_items(cnt, ((int64_t)blockIdx.x * kCellScanThreads + threadIdx.x) * kCellScanItems, n, v);
-  int32_t sum = 0;
-#pragma unroll
-  for (int j = 0; j < kCellScanItems; ++j) sum += v[j];
-  int32_t total;
-  block_exclusive<int32_t>(sum, ws, &total);
+  uint64_t total;
+  block_exclusive<uint64_t>(items_sum(v), ws, &total);
   if (threadIdx.x == 0) tot[blockIdx.x] = total;
 }
 
 __global__ void __launch_bounds__(kCellScanThreads) k_cell_starts(const int32_t* __restrict__ cnt, int64_t n,
-                                                                  const int32_t* __restrict__ tot,
-                                                                  int32_t* __restrict__ cst) {
+                                                                  const uint64_t* __restrict__ tot,
+                                                                  int32_t* __restrict__ cst, int32_t* __restrict__ cch) {
   pdl_enter();
-  __shared__ int32_t ws[33];
+  __shared__ uint64_t ws[33];
   int32_t v[kCellScanItems];
   const int64_t i0 = ((int64_t)blockIdx.x * kCellScanThreads + threadIdx.x) * kCellScanItems;
   load_items(cnt, i0, n, v);
-  int32_t part = 0;
+  uint64_t part = 0;
   for (unsigned b = threadIdx.x; b < blockIdx.x; b += kCellScanThreads) part += tot[b];
-  int32_t before;
-  block_exclusive<int32_t>(part, ws, &before);
-  int32_t sum = 0;
-#pragma unroll
-  for (int j = 0; j < kCellScanItems; ++j) sum += v[j];
-  const int32_t ex = block_exclusive<int32_t>(sum, ws, nullptr);
-  store_prefix(cst, i0, n, v, before + ex);
+  uint64_t before;
+  block_exclusive<uint64_t>(part, ws, &before);
+  const uint64_t ex = block_exclusive<uint64_t>(items_sum(v), ws, nullptr);
+  store_starts(cst, cch, i0, n, v, before + ex);
 }
 
 // Vertex ids to their cells, in arrival order.
@@ -408,9 +412,10 @@ __global__ void __launch_bounds__(kBlock) k_place(const uint32_t* __restrict__ s
                                                   int64_t K, const float4* __restrict__ x, const float* __restrict__ w,
                                                   const int32_t* __restrict__ vprob, const ProbDev* __restrict__ prob,
                                                   const int32_t* __restrict__ cst, int32_t* __restrict__ cnt,
-                                                  int64_t ncnt, uint32_t* __restrict__ svals, float4* __restrict__ xs,
-                                                  float* __restrict__ ws, uint32_t* __restrict__ scell,
-                                                  float4* __restrict__ XP) {
+                                                  int64_t ncnt, const int32_t* __restrict__ cch,
+                                                  int32_t* __restrict__ chunk, uint32_t* __restrict__ svals,
+                                                  float4* __restrict__ xs, float* __restrict__ ws,
+                                                  uint32_t* __restrict__ scell, float4* __restrict__ XP) {
   pdl_enter();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (int64_t i = t; i < ncnt; i += (int64_t)gridDim.x * blockDim.x) cnt[i] = 0;
@@ -422,13 +427,16 @@ __global__ void __launch_bounds__(kBlock) k_place(const uint32_t* __restrict__ s
   const uint32_t key = keys[v];
   const int32_t* cs = cst + pr.fbase + pb;
   const int32_t q0 = cs[key], q1 = cs[key + 1];
-  int64_t p = q0;
+  int32_t less = 0;
   int32_t q = q0;
-  for (; q + 4 <= q1; q += 4) {
-    const uint32_t a = slot[q], b = slot[q + 1], c = slot[q + 2], e = slot[q + 3];
-    p += (a < v) + (b < v) + (c < v) + (e < v);
+  for (; q < q1 && (q & 3); ++q) less += slot[q] < v;
+  for (; q + 8 <= q1; q += 8) {  // 16-byte reads, two in flight
+    const uint4 a = *reinterpret_cast<const uint4*>(slot + q), b = *reinterpret_cast<const uint4*>(slot + q + 4);
+    less += (a.x < v) + (a.y < v) + (a.z < v) + (a.w < v) + (b.x < v) + (b.y < v) + (b.z < v) + (b.w < v);
   }
-  for (; q < q1; ++q) p += slot[q] < v;
+  for (; q < q1; ++q) less += slot[q] < v;
+  const int64_t p = (int64_t)q0 + less;
+  if (cch && !(less & 1)) chunk[cch[pr.fbase + pb + key] + (less >> 1)] = (int32_t)p;
   svals[p] = v;
   xs[p] = xv;
   const float wv = w ? w[v] : 1.0f;
@@ -469,6 +477,7 @@ __device__ inline void store_cell(int64_t idx, int64_t pidx, const float* S, flo
 // lane-strided partial sums from the cell's first point, then a fixed xor
 // tree.  Either way the sums depend only on the cell.
 constexpr int kCellSerial = 32;
+constexpr int kCellHuge = 512;  // points of a cell from which a whole warp sums it
 
 template <int D>
 __device__ __forceinline__ void cell_add(const float4& p, float wq, float* S, float& W) {
@@ -479,33 +488,73 @@ __device__ __forceinline__ void cell_add(const float4& p, float wq, float* S, fl
   W += wq;
 }
 
-// Points q0, q0 + stride, ... < q1 added in that order; four loads issued
-// before their additions.
-template <int D>
+// Points q0, q0 + stride, ... < q1 added in that order; U loads issued before
+// their additions (the last of them guarded).
+template <int D, int U>
 __device__ __forceinline__ void cell_sum(const float4* xs, const float* ws, int64_t q0, int64_t q1, int64_t stride,
                                          float* S, float& W) {
-  int64_t q = q0;
-  for (; q + 3 * stride < q1; q += 4 * stride) {
-    float4 p[4];
-    float wq[4];
+  for (int64_t q = q0; q < q1; q += U * stride) {
+    float4 p[U];
+    float wq[U];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      p[u] = xs[q + u * stride];
-      wq[u] = ws ? ws[q + u * stride] : 1.0f;
+    for (int u = 0; u < U; ++u) {
+      const bool in = q + u * stride < q1;
+      p[u] = in ? xs[q + u * stride] : make_float4(0.f, 0.f, 0.f, 0.f);
+      wq[u] = in && ws ? ws[q + u * stride] : 1.0f;
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) cell_add<D>(p[u], wq[u], S, W);
+    for (int u = 0; u < U; ++u)
+      if (q + u * stride < q1) cell_add<D>(p[u], wq[u], S, W);
   }
-  for (; q < q1; q += stride) cell_add<D>(xs[q], ws ? ws[q] : 1.0f, S, W);
 }
 
-// Sum of the points [q0, q1) of a large cell by a whole warp (every lane gets it).
+// Sum of the points [q0, q1) of a large cell (every lane gets it): 32 partial
+// sums of every 32nd point, then the xor tree, by a whole warp ...
 template <int D>
 __device__ __forceinline__ void cell_sum_warp(const float4* xs, const float* ws, int64_t q0, int64_t q1, float* S,
                                               float& W) {
-  cell_sum<D>(xs, ws, q0 + lane_id(), q1, 32, S, W);
+  cell_sum<D, 8>(xs, ws, q0 + lane_id(), q1, 32, S, W);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int m = 0; m < D; ++m) S[m] += __shfl_xor_sync(0xffffffffu, S[m], o);
+    W += __shfl_xor_sync(0xffffffffu, W, o);
+  }
+}
+
+// ... or by kCellLanes lanes that hold four of the partial sums each (the same
+// sums; four cells per warp, so a brick of large cells takes a quarter of the
+// turns).  Every lane of the warp calls it; an empty range gives zeros.
+constexpr int kCellLanes = 8;
+
+template <int D>
+__device__ __forceinline__ void cell_sum_quarter(const float4* xs, const float* ws, int64_t q0, int64_t q1, float* S,
+                                                 float& W) {
+  float P[4][4], V[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    V[j] = 0.f;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) P[j][m] = 0.f;
+  }
+  for (int64_t q = q0 + (lane_id() & (kCellLanes - 1)); q < q1; q += 64) {
+    float4 p[8];
+    float wq[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const bool in = q + 8 * u < q1;
+      p[u] = in ? xs[q + 8 * u] : make_float4(0.f, 0.f, 0.f, 0.f);
+      wq[u] = in && ws ? ws[q + 8 * u] : 1.0f;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (q + 8 * u < q1) cell_add<D>(p[u], wq[u], P[u & 3], V[u & 3]);
+  }
+  W = (V[0] + V[2]) + (V[1] + V[3]);
+#pragma unroll
+  for (int m = 0; m < D; ++m) S[m] = (P[0][m] + P[2][m]) + (P[1][m] + P[3][m]);
+#pragma unroll
+  for (int o = kCellLanes / 2; o > 0; o >>= 1) {
 #pragma unroll
     for (int m = 0; m < D; ++m) S[m] += __shfl_xor_sync(0xffffffffu, S[m], o);
     W += __shfl_xor_sync(0xffffffffu, W, o);
@@ -550,15 +599,21 @@ __device__ inline void agg_cell(const ProbDev& pr, int pb, int l, int64_t c, flo
 // the levels above the bricks' roots from the roots' sums in global memory.
 // Small bricks, so that the large cells of a dense cluster spread over many
 // blocks (a warp took up to 32 of them in turn when a warp owned 32
-// consecutive cells: 17 us on the 64^3 grid's finest level).
+// consecutive cells: 17 us on the 64^3 grid's finest level).  A problem of one
+// grid level has no far field and so no bricks (the isolated vertices of a
+// power-law pattern are thousands of such problems).
 __host__ __device__ constexpr int brick_log2(int d) { return d == 2 ? 3 : 2; }
+// A block's time is mostly its chain of dependent loads (9.5 us for 512 bricks, 36 us
+// for 4,096 of clustered points); 64 threads are slower (large cells want
+// threads), 256 equal. Finest cells first in a launch that spreads the cells
+// of a cluster over all blocks was no faster (493 against 480 us a step).
+constexpr int kCellsBlock = 128;
 
 template <int D>
-__global__ void __launch_bounds__(kBlock) k_cells(const int32_t* __restrict__ bprob, const ProbDev* __restrict__ prob,
+__global__ void __launch_bounds__(kCellsBlock) k_cells(const int32_t* __restrict__ bprob, const ProbDev* __restrict__ prob,
                                                   const float4* __restrict__ xs, const float* __restrict__ ws,
                                                   const int32_t* __restrict__ cst, float4* St, float* Wt, float4* CP,
-                                                  int32_t* __restrict__ done, int32_t* __restrict__ chunk,
-                                                  int32_t* __restrict__ nchunk) {
+                                                  int32_t* __restrict__ done) {
   pdl_enter();
   constexpr int B = brick_log2(D), NC = 1 << (D * B);
   constexpr int NT = ((1 << (D * (B + 1))) - 1) / ((1 << D) - 1);  // cells of a brick on its B + 1 levels
@@ -566,7 +621,6 @@ __global__ void __launch_bounds__(kBlock) k_cells(const int32_t* __restrict__ bp
   __shared__ int32_t big[NC], bq0[NC], bq1[NC];
   __shared__ int nbig;
   __shared__ bool last;
-  __shared__ int32_t cws[33], cbase;
   const int pb = bprob[blockIdx.x];
   const ProbDev pr = prob[pb];
   const int L = pr.L, lb = min(L, B), Lb = L - lb;
@@ -593,32 +647,9 @@ __global__ void __launch_bounds__(kBlock) k_cells(const int32_t* __restrict__ bp
     }
     pair_store<D>(CP, pr.cbase + lvl_off(D, l) + c + pb + 1, z, W);
   };
-  const int nc = 1 << (D * lb);  // at most kBlock
+  const int nc = 1 << (D * lb);  // at most kCellsBlock
   const int32_t* cs = cst + pr.fbase + pb;
-  if (chunk) {  // the brick's chunks of at most two points of a cell, into the problem's list
-    int32_t q0 = 0, n = 0;
-    if (threadIdx.x < nc) {
-      const int64_t c = cell_index(threadIdx.x, 0);
-      q0 = cs[c];
-      n = cs[c + 1] - q0;
-    }
-    int32_t total;
-    const int32_t ex = block_exclusive<int32_t>((n + 1) >> 1, cws, &total);
-    if (threadIdx.x == 0) cbase = atomicAdd(&nchunk[pb], total);
-    __syncthreads();
-    int32_t* out = chunk + pr.lbase + cbase;
-    if (n <= kCellSerial)
-      for (int32_t h = 0; 2 * h < n; ++h) out[ex + h] = q0 + 2 * h;
-    unsigned todo = __ballot_sync(0xffffffffu, n > kCellSerial);
-    while (todo) {
-      const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const int32_t e = __shfl_sync(0xffffffffu, ex, src), a = __shfl_sync(0xffffffffu, q0, src);
-      const int32_t m = (__shfl_sync(0xffffffffu, n, src) + 1) >> 1;
-      for (int32_t h = lane_id(); h < m; h += 32) out[e + h] = a + 2 * h;
-    }
-  }
-  for (int i = threadIdx.x; i < nc; i += kBlock) {
+  for (int i = threadIdx.x; i < nc; i += kCellsBlock) {
     const int64_t c = cell_index(i, 0);
     const int32_t q0 = cs[c], q1 = cs[c + 1];
     if (q1 - q0 > kCellSerial) {
@@ -630,30 +661,39 @@ __global__ void __launch_bounds__(kBlock) k_cells(const int32_t* __restrict__ bp
     }
     float S[4] = {0.f, 0.f, 0.f, 0.f};
     float W = 0.f;
-    cell_sum<D>(xs, ws, q0, q1, 1, S, W);
+    cell_sum<D, 8>(xs, ws, q0, q1, 1, S, W);
 #pragma unroll
     for (int m = 0; m < D; ++m) sS[m][i] = S[m];
     sW[i] = W;
     store_charge(c, L, S, W);
   }
   __syncthreads();
-  for (int b = threadIdx.x >> 5; b < nbig; b += kBlock / 32) {
+  auto keep = [&](int i, const float* S, float W) {
+#pragma unroll
+    for (int m = 0; m < D; ++m) sS[m][i] = S[m];
+    sW[i] = W;
+    store_charge(cell_index(i, 0), L, S, W);
+  };
+  for (int b0 = 0; b0 < nbig; b0 += kCellsBlock / kCellLanes) {  // large cells, four to a warp
+    const int b = b0 + threadIdx.x / kCellLanes;
+    const bool mine = b < nbig && bq1[b] - bq0[b] <= kCellHuge;
+    float S[4] = {0.f, 0.f, 0.f, 0.f};
+    float W = 0.f;
+    cell_sum_quarter<D>(xs, ws, mine ? bq0[b] : 0, mine ? bq1[b] : 0, S, W);
+    if (mine && (threadIdx.x & (kCellLanes - 1)) == 0) keep(big[b], S, W);
+  }
+  for (int b = threadIdx.x >> 5; b < nbig; b += kCellsBlock / 32) {  // the largest, a warp each
+    if (bq1[b] - bq0[b] <= kCellHuge) continue;
     float S[4] = {0.f, 0.f, 0.f, 0.f};
     float W = 0.f;
     cell_sum_warp<D>(xs, ws, bq0[b], bq1[b], S, W);
-    if (lane_id() == 0) {
-      const int i = big[b];
-#pragma unroll
-      for (int m = 0; m < D; ++m) sS[m][i] = S[m];
-      sW[i] = W;
-      store_charge(cell_index(i, 0), L, S, W);
-    }
+    if (lane_id() == 0) keep(big[b], S, W);
   }
   int off = 0;  // first cell of level L - j + 1 in the shared sums
   for (int j = 1; j <= lb && L - j >= 2; ++j) {
     __syncthreads();
     const int bits = lb - j, n = 1 << (D * bits), next = off + (1 << (D * (bits + 1)));
-    for (int i = threadIdx.x; i < n; i += kBlock) {
+    for (int i = threadIdx.x; i < n; i += kCellsBlock) {
       float S[4] = {0.f, 0.f, 0.f, 0.f};
       float W = 0.f;
 #pragma unroll
@@ -691,7 +731,7 @@ __global__ void __launch_bounds__(kBlock) k_cells(const int32_t* __restrict__ bp
   if (!last) return;
   for (int l = Lb - 1; l >= 2; --l) {
     const int64_t n = int64_t(1) << (D * l);
-    for (int64_t c = threadIdx.x; c < n; c += kBlock) agg_cell<D>(pr, pb, l, c, St, Wt, CP);
+    for (int64_t c = threadIdx.x; c < n; c += kCellsBlock) agg_cell<D>(pr, pb, l, c, St, Wt, CP);
     __syncthreads();
   }
 }
@@ -849,7 +889,7 @@ __global__ void __launch_bounds__(kSortThreads) k_bin_small(
 
 // Rubber bands of 2-pin nets: y_v = sum_u c_vu (x_v - x_u) / 2.  Rows are
 // split by degree: light rows (<= kLightMax) take one thread, medium rows a
-// warp and heavy rows a block; each class sums in a fixed order (sequential,
+// quarter warp and heavy rows a block; each class sums in a fixed order (sequential,
 // lane-strided + xor tree, thread-strided + fixed tree), so the result of a
 // vertex depends only on its own row.
 constexpr int kLightMax = 32;
@@ -863,86 +903,132 @@ __device__ inline void add_pull(float* a, const float4& xv, const float4& xu, fl
 }
 
 // a += sum over t = t0, t0 + stride, ... < t1 of c_t (xv - x[adj[t]]), in that
-// order; four neighbours per trip with all their loads issued first.
+// order; U neighbours per trip with all their loads issued first.
+template <int U>
 __device__ __forceinline__ void pull_range(float* a, const float4& xv, const int32_t* __restrict__ adj,
                                            const float* __restrict__ acost, const float4* __restrict__ x, int32_t t,
                                            int32_t t1, int32_t stride) {
-  constexpr int U = 4;
-  for (; t + (U - 1) * stride < t1; t += U * stride) {
+  for (; t < t1; t += U * stride) {
     int32_t u[U];
     float c[U];
     float4 q[U];
 #pragma unroll
     for (int i = 0; i < U; ++i) {
-      u[i] = adj[t + i * stride];
-      c[i] = acost ? acost[t + i * stride] : 1.0f;
+      const bool in = t + i * stride < t1;
+      u[i] = in ? adj[t + i * stride] : -1;
+      c[i] = in && acost ? acost[t + i * stride] : 1.0f;
     }
 #pragma unroll
-    for (int i = 0; i < U; ++i) q[i] = x[u[i]];
+    for (int i = 0; i < U; ++i) q[i] = u[i] >= 0 ? x[u[i]] : xv;
 #pragma unroll
-    for (int i = 0; i < U; ++i) add_pull(a, xv, q[i], c[i]);
+    for (int i = 0; i < U; ++i)
+      if (u[i] >= 0) add_pull(a, xv, q[i], c[i]);
   }
-  for (; t < t1; t += stride) add_pull(a, xv, x[adj[t]], acost ? acost[t] : 1.0f);
 }
+
+// All rows in one launch: first the blocks of the heavy rows (one each), then
+// the blocks of medium rows, then the light rows' (a thread each, by vertex).
+// A medium row's 32 partial sums (entries t0 + l, t0 + l + 32, ...; then the xor
+// tree) are held four to a lane by kMidLanes = 8 lanes: four rows per warp, so
+// that a row of 33 to 100 entries has all its gathers in flight at once and
+// the tree's first two levels need no shuffle; rows longer than kMidMax take
+// the whole warp with 16 entries of a lane in flight.  500,000-row power-law
+// matrix, per step: 31 us, against 46 us of three launches (a thread, a warp
+// and a block per row).
+constexpr int kMidLanes = 8;
+constexpr int kMidMax = 512;  // entries of a row from which the whole warp takes it
 
 __global__ void __launch_bounds__(kBlock) k_attract(const int32_t* __restrict__ adj_ptr, const int32_t* __restrict__ adj,
                                                     const float* __restrict__ acost, const float4* __restrict__ x,
-                                                    int64_t K, float4* __restrict__ y) {
-  pdl_enter();
-  int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= K) return;
-  int32_t t0 = adj_ptr[v], t1 = adj_ptr[v + 1];
-  if (t1 - t0 > kLightMax) return;  // medium and heavy rows: k_attract_warp / k_attract_block
-  float4 xv = x[v];
-  float a[4] = {0.f, 0.f, 0.f, 0.f};
-  pull_range(a, xv, adj, acost, x, t0, t1, 1);
-  y[v] = make_float4(0.5f * a[0], 0.5f * a[1], 0.5f * a[2], 0.5f * a[3]);
-}
-
-__global__ void __launch_bounds__(kBlock) k_attract_warp(const int32_t* __restrict__ list, int64_t n,
-                                                         const int32_t* __restrict__ adj_ptr,
-                                                         const int32_t* __restrict__ adj, const float* __restrict__ acost,
-                                                         const float4* __restrict__ x, float4* __restrict__ y) {
-  pdl_enter();
-  int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= n) return;
-  const int lane = lane_id();
-  int32_t v = list[w];
-  float4 xv = x[v];
-  float a[4] = {0.f, 0.f, 0.f, 0.f};
-  pull_range(a, xv, adj, acost, x, adj_ptr[v] + lane, adj_ptr[v + 1], 32);
-#pragma unroll
-  for (int m = 0; m < 4; ++m)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a[m] += __shfl_xor_sync(0xffffffffu, a[m], o);
-  if (lane == 0) y[v] = make_float4(0.5f * a[0], 0.5f * a[1], 0.5f * a[2], 0.5f * a[3]);
-}
-
-__global__ void __launch_bounds__(kBlock) k_attract_block(const int32_t* __restrict__ list,
-                                                          const int32_t* __restrict__ adj_ptr,
-                                                          const int32_t* __restrict__ adj,
-                                                          const float* __restrict__ acost,
-                                                          const float4* __restrict__ x, float4* __restrict__ y) {
+                                                    int64_t K, const int32_t* __restrict__ heavy, int64_t n_heavy,
+                                                    const int32_t* __restrict__ mid, int64_t n_mid, int64_t mid_blocks,
+                                                    float4* __restrict__ y) {
   pdl_enter();
   __shared__ float part[kBlock / 32][4];
   const int lane = lane_id(), warp = threadIdx.x >> 5;
-  int32_t v = list[blockIdx.x];
-  float4 xv = x[v];
-  float a[4] = {0.f, 0.f, 0.f, 0.f};
-  pull_range(a, xv, adj, acost, x, adj_ptr[v] + threadIdx.x, adj_ptr[v + 1], blockDim.x);
+  int64_t b = blockIdx.x;
+  if (b < n_heavy) {
+    const int32_t v = heavy[b];
+    const float4 xv = x[v];
+    float a[4] = {0.f, 0.f, 0.f, 0.f};
+    pull_range<16>(a, xv, adj, acost, x, adj_ptr[v] + threadIdx.x, adj_ptr[v + 1], blockDim.x);
 #pragma unroll
-  for (int m = 0; m < 4; ++m)
+    for (int m = 0; m < 4; ++m)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a[m] += __shfl_xor_sync(0xffffffffu, a[m], o);
-  if (lane == 0)
-    for (int m = 0; m < 4; ++m) part[warp][m] = a[m];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float b[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-      for (int m = 0; m < 4; ++m) b[m] += part[w][m];
-    y[v] = make_float4(0.5f * b[0], 0.5f * b[1], 0.5f * b[2], 0.5f * b[3]);
+      for (int o = 16; o > 0; o >>= 1) a[m] += __shfl_xor_sync(0xffffffffu, a[m], o);
+    if (lane == 0)
+      for (int m = 0; m < 4; ++m) part[warp][m] = a[m];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float s[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+        for (int m = 0; m < 4; ++m) s[m] += part[w][m];
+      y[v] = make_float4(0.5f * s[0], 0.5f * s[1], 0.5f * s[2], 0.5f * s[3]);
+    }
+    return;
   }
+  b -= n_heavy;
+  if (b < mid_blocks) {
+    const int64_t i = (b * kBlock + threadIdx.x) / kMidLanes;
+    const int l = threadIdx.x & (kMidLanes - 1);
+    const bool in = i < n_mid;
+    const int32_t v = in ? mid[i] : 0;
+    const int32_t t0 = in ? adj_ptr[v] : 0, t1 = in ? adj_ptr[v + 1] : 0;
+    const bool quarter = in && t1 - t0 <= kMidMax;
+    const float4 xv = x[v];
+    float a[4][4];  // [partial sum l + 8 j][coordinate]
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) a[j][m] = 0.f;
+    for (int32_t t = t0 + l; quarter && t < t1; t += 64) {  // two entries of every partial sum
+      int32_t u[8];
+      float c[8];
+      float4 q[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const bool ok = t + 8 * j < t1;
+        u[j] = ok ? adj[t + 8 * j] : v;
+        c[j] = ok && acost ? acost[t + 8 * j] : 1.0f;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) q[j] = x[u[j]];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (t + 8 * j < t1) add_pull(a[j & 3], xv, q[j], c[j]);
+    }
+    float s[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {  // the xor tree of 32 partial sums: distances 16, 8 here, 4, 2, 1 across lanes
+      s[m] = (a[0][m] + a[2][m]) + (a[1][m] + a[3][m]);
+#pragma unroll
+      for (int o = kMidLanes / 2; o > 0; o >>= 1) s[m] += __shfl_xor_sync(0xffffffffu, s[m], o);
+    }
+    if (quarter && l == 0) y[v] = make_float4(0.5f * s[0], 0.5f * s[1], 0.5f * s[2], 0.5f * s[3]);
+    unsigned todo = __ballot_sync(0xffffffffu, in && !quarter && l == 0);  // longer rows: the whole warp
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int32_t w = __shfl_sync(0xffffffffu, v, src);
+      const float4 xw = x[w];
+      float g[4] = {0.f, 0.f, 0.f, 0.f};
+      pull_range<16>(g, xw, adj, acost, x, adj_ptr[w] + lane, adj_ptr[w + 1], 32);
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) g[m] += __shfl_xor_sync(0xffffffffu, g[m], o);
+      if (lane == 0) y[w] = make_float4(0.5f * g[0], 0.5f * g[1], 0.5f * g[2], 0.5f * g[3]);
+    }
+    return;
+  }
+  const int64_t v = (b - mid_blocks) * kBlock + threadIdx.x;
+  if (v >= K) return;
+  const int32_t t0 = adj_ptr[v], t1 = adj_ptr[v + 1];
+  if (t1 - t0 > kLightMax) return;  // a medium or heavy row
+  const float4 xv = x[v];
+  float a[4] = {0.f, 0.f, 0.f, 0.f};
+  pull_range<4>(a, xv, adj, acost, x, t0, t1, 1);
+  y[v] = make_float4(0.5f * a[0], 0.5f * a[1], 0.5f * a[2], 0.5f * a[3]);
 }
 
 __global__ void k_degree_class(const int32_t* __restrict__ adj_ptr, int64_t K, int32_t* __restrict__ mid,
@@ -1366,12 +1452,13 @@ __device__ __forceinline__ float4 step_target(int64_t p, const float4& xn, const
 //
 // T = 1: a group handles the point at its own sorted position.  T = 2: a
 // group handles a chunk of one or two consecutive points of one finest cell;
-// the chunks of a problem (first positions, in any order) are listed by the
-// binning, nchunk[pb] of them, and its threads are numbered from tbase2.
+// the binning lists the chunks' first positions in cell order (cch[c]: first
+// chunk of cell c, as cst[c] is its first point), and the problem's threads are
+// numbered from tbase2.
 // One target per thread is bound by the 32 bytes a pair costs every lane of
 // L1 bandwidth (65% busy, FMA pipe 59%, 500,000 clustered points, d = 3, 587
 // us); two per thread halve that (36%) and leave the FMA pipe (66%): 568 us,
-// 405 against 461 us in that level's later steps.  Measured and not kept:
+// 400 against 461 us in that level's later steps.  Measured and not kept:
 // leaving out the middle pair of a row where every lane of the warp has it
 // masked (8% of the far field's work, 1% slower), other block sizes and
 // register limits (within 2%).
@@ -1387,7 +1474,7 @@ constexpr int kStepBlock = 128;
 //    17.4 / 21.5 us (a target's sums are too short there for the split: 17.6 /
 //    22.3 us).
 //  - at least kPairThreadsMin: two targets per thread; 110,592 / 262,144 grid
-//    points and 500,000 clustered ones 104 / 186 / 489 us against 95 / 196 /
+//    points and 500,000 clustered ones 104 / 176 / 480 us against 95 / 196 /
 //    538 us with one.
 //  - else one target per thread.
 constexpr int64_t kPairThreadsMin = 196608;
@@ -1401,7 +1488,7 @@ __global__ void __launch_bounds__(kStepBlock, step_min_blocks(MODE)) k_repulse_u
     const uint32_t* __restrict__ svals, const uint32_t* __restrict__ scell, const int32_t* __restrict__ cst,
     const float4* __restrict__ CP, const float4* __restrict__ yatt, const int32_t* __restrict__ wprob,
     const ProbDev* __restrict__ prob, int64_t nthreads, const int32_t* __restrict__ chunk,
-    const int32_t* __restrict__ nchunk, float kappa, const float* __restrict__ s0,
+    const int32_t* __restrict__ cch, float kappa, const float* __restrict__ s0,
     const float* __restrict__ scale_tab, const int32_t* __restrict__ tctr,
     float step_override, float4* __restrict__ x, float4* __restrict__ y_out, uint32_t* __restrict__ bb_next,
     unsigned long long* __restrict__ icount) {
@@ -1417,10 +1504,15 @@ __global__ void __launch_bounds__(kStepBlock, step_min_blocks(MODE)) k_repulse_u
   const int64_t rel = th - (T == 2 ? pr.tbase2 : pr.tbase);
   const int lane_g = (int)(rel & (G - 1));
   int64_t tgt = rel / G;  // problem-local sorted position of the first target
-  bool valid = th < nthreads && tgt < (T == 2 ? nchunk[pb] : pr.k);
+  int first = 0, ntgt = pr.k;  // chunks of the problem, or points
+  if (T == 2) {
+    first = cch[pr.fbase + pb];
+    ntgt = cch[pr.fbase + pb + (int64_t(1) << (D * pr.L))] - first;
+  }
+  const bool valid = th < nthreads && tgt < ntgt;
   int64_t p = pr.vbase + tgt;
   if (T == 2 && valid) {
-    p = chunk[pr.lbase + tgt];
+    p = chunk[first + tgt];
     tgt = p - pr.vbase;
   }
   unsigned long long nint = 0;
@@ -2264,14 +2356,13 @@ vmo_status level_setup(LevelBatch& lb, int d, int occ, cudaStream_t s) {
     pd[p].tbase = 32 * wb[p];
     pd[p].tbase2 = 32 * wb2[p];
     pd[p].bbase = bk[p];
-    pd[p].lbase = chunks;
     // at most one chunk of a single point per cell
     const int64_t ch = (k + std::min<int64_t>(k, int64_t(1) << (d * L))) / 2;
     chunks += ch;
     vb[p + 1] = lb.vbase[p + 1];
     wb[p + 1] = wb[p] + (k * pd[p].group + 31) / 32;
     wb2[p + 1] = wb2[p] + (ch * pd[p].group + 31) / 32;
-    bk[p + 1] = bk[p] + (int64_t(1) << (d * std::max(L - brick_log2(d), 0)));
+    bk[p + 1] = bk[p] + (L > 1 ? int64_t(1) << (d * std::max(L - brick_log2(d), 0)) : 0);
   }
   lb.threads = 32 * wb[P];
   lb.threads2 = 32 * wb2[P];
@@ -2359,7 +2450,8 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   uint32_t *keys, *arrival = nullptr, *slot = nullptr, *svals, *scell, *bb;
   float4 *xs, *XP, *yatt, *St, *CP, *z = nullptr;
   float *ws = nullptr, *Wt, *s0;
-  int32_t *cst, *cnt = nullptr, *tot = nullptr, *done = nullptr, *chunk = nullptr, *nchunk = nullptr;
+  int32_t *cst, *cnt = nullptr, *done = nullptr, *chunk = nullptr, *cch = nullptr;
+  uint64_t* tot = nullptr;
   const int64_t ncell = lb.cbase[P], nfine = lb.fbase[P];
   VMO_TRY(sc.alloc(&keys, K));
   VMO_TRY(sc.alloc(&svals, K));
@@ -2392,7 +2484,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
     });
   const bool pair = !bin1 && lb.threads >= kPairThreadsMin;
   const int64_t ncnt = nfine + P;  // entries of the cell start table
-  const bool one_cluster = ncnt <= kCellScanMax;
+  const bool one_cluster = ncnt <= kCellScanTile;
   const unsigned scan_blocks = grid_for(ncnt, kCellScanThreads * kCellScanItems);
   if (!bin1) {
     VMO_TRY(sc.alloc(&arrival, K));
@@ -2402,7 +2494,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
     if (!one_cluster) VMO_TRY(sc.alloc(&tot, scan_blocks));
     if (pair) {
       VMO_TRY(sc.alloc(&chunk, std::max<int64_t>(lb.chunks, 1)));
-      VMO_TRY(sc.alloc(&nchunk, P));
+      VMO_TRY(sc.alloc(&cch, ncnt));
     }
     VMO_CUDA(cudaMemsetAsync(cnt, 0, ncnt * sizeof(int32_t), s));
     VMO_CUDA(cudaMemsetAsync(done, 0, P * sizeof(int32_t), s));
@@ -2444,13 +2536,9 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
         cudaStreamWaitEvent(side, ev_fork, 0);
       }
       if (lb.adj_ptr) {
-        launch(k_attract, grid_for(K, kBlock), kBlock, 0, as, lb.adj_ptr, lb.adj, lb.acost, x, K, yatt);
-        if (lb.n_mid)
-          launch(k_attract_warp, grid_for(lb.n_mid * 32, kBlock), kBlock, 0, as, lb.mid_list.ptr, lb.n_mid, lb.adj_ptr,
-                 lb.adj, lb.acost, x, yatt);
-        if (lb.n_heavy)
-          launch(k_attract_block, (unsigned)lb.n_heavy, kBlock, 0, as, lb.heavy_list.ptr, lb.adj_ptr, lb.adj, lb.acost,
-                 x, yatt);
+        const int64_t mid_blocks = (lb.n_mid * kMidLanes + kBlock - 1) / kBlock;
+        launch(k_attract, (unsigned)(lb.n_heavy + mid_blocks + grid_for(K, kBlock)), kBlock, 0, as, lb.adj_ptr, lb.adj,
+               lb.acost, x, K, lb.heavy_list.ptr, lb.n_heavy, lb.mid_list.ptr, lb.n_mid, mid_blocks, yatt);
       } else if (lb.net_ptr) {
         if (lb.nnets > 0) launch(k_net_center, grid_for(lb.nnets, kBlock), kBlock, 0, as, lb.net_ptr, lb.pins, lb.nnets, x, z);
         launch(k_attract_hyper, grid_for(K, kBlock), kBlock, 0, as, lb.vtx_ptr, lb.vnets, x, z, K, yatt);
@@ -2465,19 +2553,20 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
       } else {
         auto keys_kernel = K >= kKeyItemsMin ? k_keys<D, 4> : k_keys<D, 1>;
         launch(keys_kernel, grid_for(K >= kKeyItemsMin ? (K + 3) / 4 : K, kBlock), kBlock, 0, ms, x, K, lb.vprob.ptr,
-               lb.prob.ptr, cur, keys, arrival, cnt, nchunk, P, nxt, tctr);
+               lb.prob.ptr, cur, keys, arrival, cnt, P, nxt, tctr);
         if (keys_out && t == 0) cudaMemcpyAsync(keys_out, keys, K * 4, cudaMemcpyDeviceToDevice, ms);
         if (one_cluster) {
-          launch(k_cell_scan, kCellScanCtas, kCellScanThreads, 0, ms, cnt, cst, ncnt);
+          launch(k_cell_scan, kCellScanCtas, kCellScanThreads, 0, ms, cnt, cst, cch, ncnt);
         } else {
           launch(k_cell_totals, scan_blocks, kCellScanThreads, 0, ms, cnt, ncnt, tot);
-          launch(k_cell_starts, scan_blocks, kCellScanThreads, 0, ms, cnt, ncnt, tot, cst);
+          launch(k_cell_starts, scan_blocks, kCellScanThreads, 0, ms, cnt, ncnt, tot, cst, cch);
         }
         launch(k_slots, grid_for(K, kBlock), kBlock, 0, ms, keys, arrival, K, lb.vprob.ptr, lb.prob.ptr, cst, slot);
         launch(k_place<D>, grid_for(K, kBlock), kBlock, 0, ms, slot, keys, K, x, lb.w, lb.vprob.ptr, lb.prob.ptr, cst,
-               cnt, ncnt, svals, xs, ws, scell, XP);
-        launch(k_cells<D>, (unsigned)lb.bricks, kBlock, 0, ms, lb.bprob.ptr, lb.prob.ptr, xs, ws, cst, St, Wt, CP,
-               done, chunk, nchunk);
+               cnt, ncnt, cch, chunk, svals, xs, ws, scell, XP);
+        if (lb.bricks > 0)
+          launch(k_cells<D>, (unsigned)lb.bricks, kCellsBlock, 0, ms, lb.bprob.ptr, lb.prob.ptr, xs, ws, cst, St, Wt,
+                 CP, done);
       }
       if (side) cudaStreamWaitEvent(ms, ev_join, 0);
       const bool timed = stats_timing();
@@ -2486,7 +2575,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
       const int64_t small = g_tuning.small_step_threads.load(std::memory_order_relaxed);
       auto step_launch = [&](auto kernel, int64_t nth, const int32_t* wprob) {
         launch(kernel, grid_for(nth, kStepBlock), kStepBlock, 0, ms, xs, ws, XP, svals, scell, cst, CP, yatt, wprob,
-               lb.prob.ptr, nth, chunk, nchunk, kappa, s0, scale_tab, tctr, step_override, x, y_out, nxt, icount);
+               lb.prob.ptr, nth, chunk, cch, kappa, s0, scale_tab, tctr, step_override, x, y_out, nxt, icount);
       };
       if (icount)
         step_launch(k_repulse_update<D, true, kStepPlain>, lb.threads, lb.wprob.ptr);

@@ -15,7 +15,6 @@ struct ProbDev {
   int64_t tbase;   // first thread of its targets in the step kernel (multiple of 32)
   int64_t tbase2;  // the same with two targets per thread
   int64_t bbase;   // first brick of its cell sums
-  int64_t lbase;   // first entry of its chunk list
   int32_t k;       // vertices
   int32_t L;       // finest grid level
   int32_t side;    // side of the random initial box
@@ -52,8 +51,8 @@ struct LevelBatch {
   DevArray<int32_t> wprob, wprob2, bprob;  // problem of every warp of the step kernel (one and two targets
                                            // per thread) and of every brick of the cell sums
   int64_t threads = 0, threads2 = 0;       // threads of the step kernel
-  int64_t bricks = 0;                      // bricks of every problem
-  int64_t chunks = 0;                      // entries of the chunk lists
+  int64_t bricks = 0;                      // bricks of every problem with far-field levels
+  int64_t chunks = 0;                      // most chunks of two points of a cell that the level can have
   // vertices by degree class (graph models): medium and heavy rows get a warp
   // or a block each in the gather kernels
   DevArray<int32_t> mid_list, heavy_list;
