@@ -618,7 +618,7 @@ vmo_status vmo_bisect(vmo_hg hg, int32_t d, const float* coords, const int32_t* 
     nd.size = nverts;
     VMO_CUDA(cudaMemcpyAsync(st.nodes, &nd, sizeof(nd), cudaMemcpyHostToDevice, s));
     VMO_TRY(gather_coords((const float4*)coords, st.ord, nverts, st.xo, s));
-    VMO_TRY(two_means(st, 1, d, km_iters, s, sc));
+    VMO_TRY(two_means(st, 1, nverts, d, km_iters, s, sc));
     VMO_CUDA(cudaMemcpyAsync(&nd, st.nodes, sizeof(nd), cudaMemcpyDeviceToHost, s));
     VMO_CUDA(cudaStreamSynchronize(s));
     if (nd.state == 2) {

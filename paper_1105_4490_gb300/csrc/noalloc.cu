@@ -21,16 +21,11 @@ constexpr int64_t kNoAllocMaxPoints = 131072;
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t kOffXo = 0;
-constexpr size_t kOffDval = align256(kOffXo + kNoAllocMaxPoints * sizeof(float4));
-constexpr size_t kOffDpre = align256(kOffDval + kNoAllocMaxPoints * sizeof(unsigned long long));
-constexpr size_t kOffOrd = align256(kOffDpre + kNoAllocMaxPoints * sizeof(unsigned long long));
-constexpr size_t kOffSeg = align256(kOffOrd + kNoAllocMaxPoints * sizeof(int32_t));
-constexpr size_t kOffLab = align256(kOffSeg + kNoAllocMaxPoints * sizeof(int32_t));
-constexpr size_t kOffPart = align256(kOffLab + kNoAllocMaxPoints);
-constexpr size_t kOffNode = align256(kOffPart + ((kNoAllocMaxPoints + 2047) / 2048) * sizeof(uint64_t));
+constexpr size_t kOffOrd = align256(kOffXo + kNoAllocMaxPoints * sizeof(float4));
+constexpr size_t kOffLab = align256(kOffOrd + kNoAllocMaxPoints * sizeof(int32_t));
+constexpr size_t kOffNode = align256(kOffLab + kNoAllocMaxPoints);
 constexpr size_t kOffSeed = align256(kOffNode + sizeof(NodeDev));
-constexpr size_t kOffCnt = align256(kOffSeed + sizeof(uint64_t));
-constexpr size_t kScratchBytes = align256(kOffCnt + sizeof(int));
+constexpr size_t kScratchBytes = align256(kOffSeed + sizeof(uint64_t));
 
 static __device__ __align__(256) unsigned char g_bisect_scratch[kScratchBytes];
 
@@ -58,8 +53,6 @@ vmo_status bisect_noalloc(int32_t d, const float* coords, const int32_t* verts, 
                    std::to_string(kNoAllocMaxPoints) + " points (use vmo_bisect)");
   if (nverts > 0 && (!coords || !verts || !labels || ((uintptr_t)coords & 15u)))
     return invalid("null or unaligned argument");
-  if (scan_partials_needed(nverts) * (int64_t)sizeof(uint64_t) > (int64_t)(kOffNode - kOffPart))
-    return invalid("vmo_bisect_noalloc: scan partials exceed their slot");
   unsigned char* base;
   VMO_TRY(scratch_address(&base));
   float zh[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -69,12 +62,10 @@ vmo_status bisect_noalloc(int32_t d, const float* coords, const int32_t* verts, 
     st.n = nverts;
     st.xo = reinterpret_cast<float4*>(base + kOffXo);
     st.ord = reinterpret_cast<int32_t*>(base + kOffOrd);
-    st.seg = reinterpret_cast<int32_t*>(base + kOffSeg);
     st.lab = base + kOffLab;
     st.nodes = reinterpret_cast<NodeDev*>(base + kOffNode);
     st.seeds = reinterpret_cast<uint64_t*>(base + kOffSeed);
     VMO_CUDA(cudaMemcpyAsync(st.ord, verts, nverts * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-    VMO_CUDA(cudaMemsetAsync(st.seg, 0, nverts * sizeof(int32_t), s));  // every point in node 0
     VMO_CUDA(cudaMemcpyAsync(st.seeds, &seed, sizeof(seed), cudaMemcpyHostToDevice, s));
     NodeDev nd;
     memset(&nd, 0, sizeof(nd));
@@ -82,9 +73,7 @@ vmo_status bisect_noalloc(int32_t d, const float* coords, const int32_t* verts, 
     nd.size = nverts;
     VMO_CUDA(cudaMemcpyAsync(st.nodes, &nd, sizeof(nd), cudaMemcpyHostToDevice, s));
     VMO_TRY(gather_coords(reinterpret_cast<const float4*>(coords), st.ord, nverts, st.xo, s));
-    VMO_TRY(two_means_into(st, 1, d, km_iters, reinterpret_cast<unsigned long long*>(base + kOffDval),
-                           reinterpret_cast<unsigned long long*>(base + kOffDpre), reinterpret_cast<int*>(base + kOffCnt),
-                           reinterpret_cast<uint64_t*>(base + kOffPart), s));
+    VMO_TRY(two_means_one(st, d, km_iters, s));
     VMO_CUDA(cudaMemcpyAsync(&nd, st.nodes, sizeof(nd), cudaMemcpyDeviceToHost, s));
     VMO_CUDA(cudaStreamSynchronize(s));
     zh[0] = nd.z1.x; zh[1] = nd.z1.y; zh[2] = nd.z1.z; zh[3] = nd.z1.w;

@@ -16,6 +16,8 @@
 // implementation of the same arithmetic.
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
 #include "order.cuh"
 
 namespace vmo {
@@ -834,7 +836,8 @@ __global__ void k_scatter(const int32_t* __restrict__ ord, const float4* __restr
 // with separator recursion V3 too (keys 2h + side, or 3h - 1 + side).
 __global__ void k_children(NodeDev* __restrict__ nodes, int N, const int64_t* __restrict__ pbase, int min_part,
                            int max_depth, int sbd, int sep_rec, NodeDev* __restrict__ next,
-                           int* __restrict__ next_count, int next_cap, TreeDev tree, int* __restrict__ err) {
+                           int* __restrict__ next_count, int* __restrict__ next_max, int next_cap, TreeDev tree,
+                           int* __restrict__ err) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= N) return;
   NodeDev& nd = nodes[s];
@@ -859,6 +862,7 @@ __global__ void k_children(NodeDev* __restrict__ nodes, int N, const int64_t* __
     if (size > min_part && depth < max_depth) {
       int c = atomicAdd(next_count, 1);
       if (c >= next_cap) { atomicOr(err, 2); continue; }
+      atomicMax(next_max, size);
       NodeDev& ch = next[c];
       ch.heap = heap; ch.off = off; ch.size = size; ch.depth = depth; ch.prob = nd.prob;
       if (side == 0) nd.child1 = c; else if (side == 1) nd.child2 = c; else nd.child3 = c;
@@ -1048,10 +1052,345 @@ __global__ void k_cut_scatter(const uint64_t* __restrict__ keys, const uint32_t*
   ord2[cr[i].a + (j - gstart[i])] = ord[vals[j]];
 }
 
+// ----- 2-means of a node by one thread block cluster -----
+// The whole of Algorithm 5 for one node in one launch: largest coordinate,
+// k-means++ seeds, Lloyd rounds, final labels and the separator phase's vertex
+// records.  The cluster's blocks hold the node's points in shared memory for
+// all rounds (or stream them from L2 when the node is too large), add exact
+// fixed-point sums, exchange them through distributed shared memory and each
+// compute the new centres; a node stops when its own labels settle.  The
+// arithmetic of every decision is that of the kernels above, and the sums are
+// integers, so the results are the same to the bit.  As a launch sequence a
+// level took up to 45 launches and five host waits, about 0.45 ms whatever
+// its size; here a round is three block barriers and one cluster barrier.
+// Ordering of given coordinates: 64^3 grid to depth 10 5.8 -> 2.0 ms, 400k x
+// 300k bipartite pattern to 64 parts 6.9 -> 3.3 ms.
+struct TwoMeansSums {           // one block's sums of a round, read by the cluster
+  unsigned long long v[6];      // S1[0..3], n1 | labels changed << 40, weights
+};
+
+template <int D, int T>
+__global__ void __launch_bounds__(T) k_two_means(const float4* __restrict__ xo, const int32_t* __restrict__ ord,
+                                                 NodeDev* __restrict__ nodes, const uint64_t* __restrict__ seeds,
+                                                 int km_iters, uint8_t* __restrict__ lab, uint64_t* __restrict__ vrec,
+                                                 int cap, int stream) {
+  namespace cg = cooperative_groups;
+  constexpr int W = T / 32;
+  extern __shared__ __align__(16) unsigned char tm_raw[];
+  __shared__ TwoMeansSums tot[2];
+  __shared__ unsigned long long red[W][D + 1];
+  __shared__ float s_z1[4], s_z2[4];
+  __shared__ unsigned long long s_val[2];
+  __shared__ uint32_t s_max;
+  __shared__ int s_flag;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int s = blockIdx.x / C;
+  NodeDev& nd = nodes[s];
+  const int64_t off = nd.off;
+  const int size = nd.size;
+  const int share = (size + C - 1) / C;
+  const int64_t p0 = off + (int64_t)rank * share;
+  const int cnt = max(0, min(share, size - rank * share));
+  float* xs = reinterpret_cast<float*>(tm_raw);                          // [D][cap] unless streamed
+  uint8_t* sl = tm_raw + (stream ? 0 : (size_t)cap * D * sizeof(float));  // labels of the last round
+  const int lane = lane_id(), warp = threadIdx.x >> 5;
+  const uint64_t seed = seeds[nd.prob] ^ kTagKmeans, heap = nd.heap;
+  auto point = [&](int i) {
+    if (stream) return xo[p0 + i];
+    return make_float4(xs[i], xs[cap + i], D > 2 ? xs[(D > 2 ? 2 : 0) * cap + i] : 0.f,
+                       D > 3 ? xs[(D > 3 ? 3 : 0) * cap + i] : 0.f);
+  };
+  if (threadIdx.x == 0) s_max = 0u;
+  __syncthreads();
+  {
+    uint32_t mx = 0;
+    for (int i = threadIdx.x; i < cnt; i += T) {
+      const float4 x = xo[p0 + i];
+#pragma unroll
+      for (int m = 0; m < D; ++m) {
+        if (!stream) xs[m * cap + i] = comp(x, m);
+        mx = max(mx, __float_as_uint(fabsf(comp(x, m))));
+      }
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) atomicMax(&s_max, mx);
+  }
+  cluster.sync();
+  uint32_t maxbits = 0;
+  for (int q = 0; q < C; ++q) maxbits = max(maxbits, *cluster.map_shared_rank(&s_max, q));
+  const int e = exponent_of(maxbits);
+  float4 z1 = xo[off + (int64_t)scale_draw((uint64_t)size, rand64(seed, heap, 0))];
+  float4 z2 = z1;
+  // k-means++: the point whose prefix of the integer D^2 weights passes the draw
+  auto weight = [&](int i) -> unsigned long long {
+    return (unsigned long long)floorf(__fmul_rn(sqdist32<D>(point(i), z1), exp2i_f(34 - 2 * e)));
+  };
+  {
+    unsigned long long w = 0;
+    for (int i = threadIdx.x; i < cnt; i += T) w += weight(i);
+    w = warp_sum64(w);
+    if (lane == 0) red[warp][0] = w;
+    __syncthreads();
+    if (warp == 0) {
+      w = warp_sum64(lane < W ? red[lane][0] : 0ull);
+      if (lane == 0) tot[0].v[5] = w;
+    }
+    cluster.sync();
+  }
+  unsigned long long total = 0, before = 0;
+  for (int q = 0; q < C; ++q) {
+    const unsigned long long w = cluster.map_shared_rank(&tot[0], q)->v[5];
+    before += q < rank ? w : 0ull;
+    total += w;
+  }
+  int state = 0;
+  long long n1 = 0;
+  if (total == 0) {
+    state = 2;  // every point on the first centre
+    cluster.sync();
+  } else {
+    const unsigned long long thr = scale_draw(total, rand64(seed, heap, 1));
+    if (thr >= before && thr - before < tot[0].v[5]) {  // this block holds it: contiguous parts of the warps
+      const int part = (cnt + W - 1) / W, a = min(warp * part, cnt), b = min(a + part, cnt);
+      unsigned long long w = 0;
+      for (int i = a + lane; i < b; i += 32) w += weight(i);
+      w = warp_sum64(w);
+      if (lane == 0) red[warp][0] = w;
+      __syncthreads();
+      unsigned long long run = before;
+      for (int q = 0; q < warp; ++q) run += red[q][0];
+      if (thr >= run && thr - run < w) {
+        for (int i0 = a; i0 < b; i0 += 32) {
+          const int i = i0 + lane;
+          const unsigned long long v = i < b ? weight(i) : 0ull;
+          unsigned long long inc = v;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
+          }
+          if (i < b && run + inc - v <= thr && thr < run + inc) {
+            const float4 x = xo[p0 + i];
+            for (int q = 0; q < C; ++q) {
+              float* z = cluster.map_shared_rank(s_z2, q);
+              z[0] = x.x;
+              z[1] = x.y;
+              z[2] = x.z;
+              z[3] = x.w;
+            }
+          }
+          run += __shfl_sync(0xffffffffu, inc, 31);
+          if (run > thr) break;
+        }
+      }
+    }
+    cluster.sync();
+    z2 = make_float4(s_z2[0], s_z2[1], s_z2[2], s_z2[3]);
+  }
+  // the node's sums of all points (the second cluster's are their difference to
+  // the first's), then the rounds: labels, sums of the first cluster, centres
+  const float sc = exp2i_f(30 - e);
+  const double inv = __longlong_as_double((long long)(1023 - (30 - e)) << 52);  // 2^-(30 - e)
+  long long all[D];
+  // sums over the cluster of this block's per-thread values (D fixed-point sums
+  // and the packed counts) into every thread of warps 0..D-1: warp m gets sum m and
+  // the counts
+  int par = 0;
+  auto reduce = [&](const long long* v, int c1, bool chg, long long& sum, unsigned long long& counts) {
+#pragma unroll
+    for (int m = 0; m < D; ++m) {  // 16 + 48 bits: two 32-bit warp sums
+      const int lo = __reduce_add_sync(0xffffffffu, (int)(v[m] & 0xffff));
+      const int hi = __reduce_add_sync(0xffffffffu, (int)(v[m] >> 16));
+      if (lane == 0) red[warp][m] = (unsigned long long)(((long long)hi << 16) + lo);
+    }
+    const int c = __reduce_add_sync(0xffffffffu, c1);
+    const bool any = __any_sync(0xffffffffu, chg);
+    if (lane == 0) red[warp][D] = (unsigned long long)c | ((unsigned long long)any << 40);
+    __syncthreads();
+    for (int m = warp; m <= D; m += W) {
+      const unsigned long long w = warp_sum64(lane < W ? red[lane][m] : 0ull);
+      if (lane == 0) tot[par].v[m] = w;
+    }
+    cluster.sync();
+    sum = 0;
+    counts = 0;
+    if (warp < D || warp == 0) {
+      unsigned long long a = 0, b = 0;
+      if (lane < C) {
+        const TwoMeansSums* t = cluster.map_shared_rank(&tot[par], lane);
+        a = t->v[warp];
+        b = t->v[D];
+      }
+      sum = (long long)warp_sum64(a);
+      counts = warp_sum64(b);
+    }
+    par ^= 1;
+  };
+  if (state == 0 && km_iters > 0) {
+    long long T_[D];
+#pragma unroll
+    for (int m = 0; m < D; ++m) T_[m] = 0;
+    for (int i = threadIdx.x; i < cnt; i += T) {
+      const float4 x = point(i);
+#pragma unroll
+      for (int m = 0; m < D; ++m) T_[m] += __float2int_rn(__fmul_rn(comp(x, m), sc));
+    }
+    long long mine;
+    unsigned long long counts;
+    reduce(T_, 0, false, mine, counts);
+    all[0] = mine;  // warp m holds coordinate m
+  }
+  for (int it = 0; state == 0 && it < km_iters; ++it) {
+    long long S[D];
+#pragma unroll
+    for (int m = 0; m < D; ++m) S[m] = 0;
+    int c1 = 0;
+    bool chg = false;
+    for (int i = threadIdx.x; i < cnt; i += T) {
+      const float4 x = point(i);
+      const uint8_t l = (sqdist32<D>(x, z1) <= sqdist32<D>(x, z2)) ? 1 : 2;
+      if (it > 0 && l != sl[i]) chg = true;
+      sl[i] = l;
+      const bool first = l == 1;
+      c1 += first ? 1 : 0;
+#pragma unroll
+      for (int m = 0; m < D; ++m) S[m] += first ? __float2int_rn(__fmul_rn(comp(x, m), sc)) : 0;
+    }
+    long long mine;
+    unsigned long long counts;
+    reduce(S, c1, chg, mine, counts);
+    if (warp < D) {
+      const bool done = it > 0 && (counts >> 40) == 0;
+      const long long k1 = (long long)(counts & ((1ull << 40) - 1)), k2 = size - k1;
+      if (lane < 2 && !done) {
+        const long long k = lane == 0 ? k1 : k2, sum = lane == 0 ? mine : all[0] - mine;
+        float* z = lane == 0 ? s_z1 : s_z2;
+        const float old = comp(lane == 0 ? z1 : z2, warp);
+        z[warp] = k > 0 ? __double2float_rn(__dmul_rn(__ddiv_rn(__ll2double_rn(sum), (double)k), inv)) : old;
+      }
+      if (threadIdx.x == 0) s_flag = done;
+    }
+    __syncthreads();
+    if (s_flag) {
+      state = 1;
+    } else {
+      z1 = make_float4(s_z1[0], s_z1[1], D > 2 ? s_z1[2] : z1.z, D > 3 ? s_z1[3] : z1.w);
+      z2 = make_float4(s_z2[0], s_z2[1], D > 2 ? s_z2[2] : z2.z, D > 3 ? s_z2[3] : z2.w);
+    }
+    __syncthreads();  // s_flag, s_z1 and s_z2 are rewritten by the next round
+  }
+  // final labels from the final centres, their counts, the vertex records
+  if (state != 2) {
+    int c1 = 0;
+    for (int i = threadIdx.x; i < cnt; i += T) {
+      const float4 x = point(i);
+      const uint8_t l = (sqdist32<D>(x, z1) <= sqdist32<D>(x, z2)) ? 1 : 2;
+      sl[i] = l;
+      lab[p0 + i] = l;
+      c1 += l == 1 ? 1 : 0;
+    }
+    c1 = __reduce_add_sync(0xffffffffu, c1);
+    if (lane == 0) red[warp][0] = (unsigned long long)c1;
+    __syncthreads();
+    if (warp == 0) {
+      const unsigned long long w = warp_sum64(lane < W ? red[lane][0] : 0ull);
+      if (lane == 0) s_val[0] = w;
+    }
+    cluster.sync();
+    for (int q = 0; q < C; ++q) n1 += (long long)*cluster.map_shared_rank(&s_val[0], q);
+  }
+  const long long n2 = state != 2 ? size - n1 : 0;
+  if (vrec) {
+    const bool split = state != 2 && n1 > 0 && n2 > 0;
+    float4 r;
+    float delta;
+    plane_of<D>(z1, z2, &r, &delta);
+    for (int i = threadIdx.x; i < cnt; i += T)
+      vrec[ord[p0 + i]] = vrec_make(s, split ? sl[i] : 0u, plane_dist<D>(point(i), r, delta));
+  }
+  if (rank == 0 && threadIdx.x == 0) {
+    nd.e = e;
+    nd.z1 = z1;
+    nd.z2 = z2;
+    nd.state = state;
+    nd.n1 = n1;
+    nd.n2 = n2;
+    nd.c1 = nd.c2 = nd.c3 = 0;
+    nd.child1 = nd.child2 = nd.child3 = -1;
+  }
+  cluster.sync();  // no block leaves while another may still read its shared memory
+}
+
 }  // namespace
 
 // 2-means of every node of the table (Algorithm 5), leaving the final labels
-// in lab (position order) and the node fields z1, z2, n1, n2, state.  The
+// in lab (position order), the node fields z1, z2, n1, n2, state and, when
+// st.vrec is set, the vertex records of the separator phase.  One cluster per
+// node; false: a node of more than kClusterNodeMax points (max_size is the
+// largest; a cluster of 8 holds the labels of that many), to be done by the
+// launch sequence below.  At that size a round of one cluster streams 28 MB
+// from L2 through 16 SMs, about what the launch sequence needs for it.
+constexpr int kClusterSmem = 220 * 1024;
+constexpr int64_t kClusterNodeMax = 8 * (int64_t)(kClusterSmem - 16);
+
+template <int D, int T>
+static cudaError_t launch_two_means(const OrderState& st, int N, int km_iters, int C, int share, cudaStream_t s) {
+  auto kernel = k_two_means<D, T>;
+  const int cap = (share + 15) / 16 * 16;
+  const bool stream = (size_t)cap * (4 * D + 1) > (size_t)kClusterSmem;
+  const size_t smem = (size_t)cap * (stream ? 1 : 4 * D + 1);
+  cudaError_t e = cudaSuccess;
+  if (smem > 32 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kClusterSmem);
+  if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)N * C);
+  cfg.blockDim = dim3(T);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (C > 8) {  // a cluster of 16 where the device has room for one
+    int active = 0;
+    e = cudaOccupancyMaxActiveClusters(&active, kernel, &cfg);
+    if (e != cudaSuccess || active < 1) {
+      (void)cudaGetLastError();
+      return launch_two_means<D, T>(st, N, km_iters, 8, share * 2, s);
+    }
+  }
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return cudaLaunchKernelEx(&cfg, kernel, (const float4*)st.xo, (const int32_t*)st.ord, st.nodes,
+                            (const uint64_t*)st.seeds, km_iters, st.lab, st.vrec, cap, (int)stream);
+}
+
+static vmo_status two_means_clusters(OrderState& st, int N, int64_t max_size, int d, int km_iters, cudaStream_t s,
+                                     bool* done) {
+  *done = max_size <= kClusterNodeMax;
+  if (!*done || N == 0) return VMO_OK;
+  // blocks per node: about 4,096 points each, fewer blocks when there are many nodes
+  int C = 1;
+  while (C < 16 && max_size > (int64_t)C * 4096) C *= 2;
+  while (C > 1 && (int64_t)N * C > 512) C /= 2;
+  while (C < 16 && (max_size + C - 1) / C > (int64_t)kClusterSmem - 16) C *= 2;  // the labels must fit
+  const int share = (int)((max_size + C - 1) / C);
+  cudaError_t e = cudaSuccess;
+  dispatch_d(d, [&](auto DC) {
+    constexpr int D = decltype(DC)::value;
+    e = share > 2048 ? launch_two_means<D, 1024>(st, N, km_iters, C, share, s)
+        : share > 512 ? launch_two_means<D, 512>(st, N, km_iters, C, share, s)
+                      : launch_two_means<D, 128>(st, N, km_iters, C, share, s);
+  });
+  if (e != cudaSuccess) return cuda_fail(e, "two_means (cluster per node)", __FILE__, __LINE__);
+  return VMO_OK;
+}
+
+// The same as a launch sequence over all positions, for nodes that one cluster
+// should not take alone.  The
 // working arrays come from the caller: dval, dpre (n values), cnt (one int),
 // partial (scan_partials_needed(n) values) and, optionally, rep (per-node
 // replicas of the Lloyd sums, N * kRepR * 10 values, zeroed).
@@ -1106,8 +1445,11 @@ static vmo_status two_means_body(OrderState& st, int N, int d, int km_iters, uns
   return stt;
 }
 
-vmo_status two_means(OrderState& st, int N, int d, int km_iters, cudaStream_t s, Scratch& sc) {
+vmo_status two_means(OrderState& st, int N, int64_t max_size, int d, int km_iters, cudaStream_t s, Scratch& sc) {
   const int64_t n = st.n;
+  bool done = false;
+  VMO_TRY(two_means_clusters(st, N, max_size, d, km_iters, s, &done));
+  if (done) return VMO_OK;
   ScratchFrame frame(sc);
   unsigned long long *dval, *dpre, *rep = nullptr;
   uint64_t* partial;
@@ -1120,12 +1462,21 @@ vmo_status two_means(OrderState& st, int N, int d, int km_iters, cudaStream_t s,
     VMO_TRY(sc.alloc(&rep, (size_t)N * kRepR * 10));
     VMO_CUDA(cudaMemsetAsync(rep, 0, (size_t)N * kRepR * 10 * sizeof(unsigned long long), s));
   }
-  return two_means_body(st, N, d, km_iters, dval, dpre, cnt, partial, rep, s);
+  VMO_TRY(two_means_body(st, N, d, km_iters, dval, dpre, cnt, partial, rep, s));
+  if (st.vrec) {
+    dispatch_d(d, [&](auto DC) {
+      launch(k_vertex_state<decltype(DC)::value>, grid_for(n, kBlock), kBlock, 0, s, st.xo, st.ord, st.seg, n, st.nodes,
+             st.lab, st.vrec);
+    });
+    VMO_LAUNCHED("vertex_state");
+  }
+  return VMO_OK;
 }
 
-vmo_status two_means_into(OrderState& st, int N, int d, int km_iters, unsigned long long* dval,
-                          unsigned long long* dpre, int* cnt, uint64_t* partial, cudaStream_t s) {
-  return two_means_body(st, N, d, km_iters, dval, dpre, cnt, partial, nullptr, s);
+vmo_status two_means_one(OrderState& st, int d, int km_iters, cudaStream_t s) {
+  bool done = false;
+  VMO_TRY(two_means_clusters(st, 1, st.n, d, km_iters, s, &done));
+  return done ? VMO_OK : invalid("two_means: too many points for one cluster");
 }
 
 // Separator of every split node of the level by Algorithm 7's loop with the
@@ -1192,16 +1543,12 @@ vmo_status order_levels(OrderState& st, const OrderParams& op, cudaStream_t s, S
   VMO_TRY(sc.alloc(&pk, std::max<int64_t>(n, 1)));
   VMO_TRY(sc.alloc(&pre, std::max<int64_t>(n, 1)));
   VMO_TRY(sc.alloc(&next, st.node_cap));
-  VMO_TRY(sc.alloc(&next_count, 1));
-  VMO_TRY(sc.alloc(&err, 1));
-  VMO_CUDA(cudaMemsetAsync(err, 0, 4, s));
+  VMO_TRY(sc.alloc(&next_count, 3));  // nodes of the next level, their largest size, capacity errors
+  int32_t* next_max = next_count + 1;
+  err = next_count + 2;
+  int64_t max_size = st.max_root;
   while (N > 0) {
-    VMO_TRY(two_means(st, N, op.d, op.km_iters, s, sc));
-    dispatch_d(op.d, [&](auto DC) {
-      constexpr int D = decltype(DC)::value;
-      launch(k_vertex_state<D>, grid_for(n, kBlock), kBlock, 0, s, st.xo, st.ord, st.seg, n, st.nodes, st.lab,
-                                                               st.vrec);
-    });
+    VMO_TRY(two_means(st, N, max_size, op.d, op.km_iters, s, sc));
     if (st.mu && op.mu_order_free) {
       launch(k_pick, grid_for(n, kBlock), kBlock, 0, s, st.ord, st.seg, n, st.adj_ptr, st.adj, st.vrec, st.vpick);
       launch(k_separator_mu, grid_for(n, kBlock), kBlock, 0, s, st.ord, st.seg, n, st.mu, st.vrec, st.vpick, st.nodes,
@@ -1216,10 +1563,10 @@ vmo_status order_levels(OrderState& st, const OrderParams& op, cudaStream_t s, S
     VMO_TRY(scan_inclusive<uint64_t>((const uint64_t*)pk, (uint64_t*)pre, n, s, sc));
     // children first (they number the next level's nodes), then the scatter
     // writes every position's next node
-    VMO_CUDA(cudaMemsetAsync(next_count, 0, 4, s));
+    VMO_CUDA(cudaMemsetAsync(next_count, 0, 3 * sizeof(int32_t), s));
     const int max_depth = op.sep_rec ? std::min(op.max_depth, kSepRecMaxDepth) : op.max_depth;
     launch(k_children, grid_for(N, kBlock), kBlock, 0, s, st.nodes, N, st.pbase, op.min_part, max_depth, op.sbd,
-           op.sep_rec, next, next_count, st.node_cap, st.tree, err);
+           op.sep_rec, next, next_count, next_max, st.node_cap, st.tree, err);
     launch(k_scatter, grid_for(n, kBlock), kBlock, 0, s, st.ord, st.xo, st.seg, labf, n, st.nodes, pre, op.sbd, ord2, xo2,
                                                      seg2, st.vrec);
     VMO_LAUNCHED("partition");
@@ -1227,13 +1574,13 @@ vmo_status order_levels(OrderState& st, const OrderParams& op, cudaStream_t s, S
     std::swap(st.ord, ord2);
     std::swap(st.xo, xo2);
     std::swap(st.seg, seg2);
-    int hN = 0, herr = 0;
-    VMO_CUDA(cudaMemcpyAsync(&hN, next_count, 4, cudaMemcpyDeviceToHost, s));
-    VMO_CUDA(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, s));
+    int32_t h[3] = {0, 0, 0};
+    VMO_CUDA(cudaMemcpyAsync(h, next_count, sizeof(h), cudaMemcpyDeviceToHost, s));
     VMO_CUDA(cudaStreamSynchronize(s));
-    if (herr) return cuda_fail(cudaErrorUnknown, "ordering: node table or tree capacity exceeded", __FILE__, __LINE__);
+    if (h[2]) return cuda_fail(cudaErrorUnknown, "ordering: node table or tree capacity exceeded", __FILE__, __LINE__);
     std::swap(st.nodes, next);
-    N = hN;
+    N = h[0];
+    max_size = h[1];
   }
   return VMO_OK;
 }
@@ -1284,6 +1631,7 @@ vmo_status order_setup(OrderState& st, const float4* x, const std::vector<int64_
   for (int p = 0; p < P; ++p) {
     int64_t k = pbase_host[p + 1] - pbase_host[p];
     if (k > op.min_part && op.max_depth > 0) {
+      st.max_root = std::max(st.max_root, k);
       node_of_prob[p] = (int32_t)ids.size();
       ids.push_back(p);
     }

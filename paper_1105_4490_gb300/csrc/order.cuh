@@ -68,6 +68,7 @@ struct OrderState {
   NodeDev* nodes = nullptr;
   int node_cap = 0;
   int nroots = 0;
+  int64_t max_root = 0;               // points of the largest active root
   TreeDev tree;
 };
 
@@ -76,11 +77,11 @@ struct OrderState {
 vmo_status order_setup(OrderState& st, const float4* x, const std::vector<int64_t>& pbase_host,
                        const std::vector<uint64_t>& seeds, const OrderParams& op, const uint32_t* init_ord,
                        cudaStream_t s, Scratch& sc);
-vmo_status two_means(OrderState& st, int N, int d, int km_iters, cudaStream_t s, Scratch& sc);
-// two_means with every buffer supplied by the caller (allocates nothing):
-// dval, dpre hold st.n values, partial scan_partials_needed(st.n), cnt one int.
-vmo_status two_means_into(OrderState& st, int N, int d, int km_iters, unsigned long long* dval,
-                          unsigned long long* dpre, int* cnt, uint64_t* partial, cudaStream_t s);
+// max_size: points of the largest of the N nodes.
+vmo_status two_means(OrderState& st, int N, int64_t max_size, int d, int km_iters, cudaStream_t s, Scratch& sc);
+// two_means of one node that holds all st.n positions, without any
+// allocation (at most kClusterNodeMax points, 1.8 million).
+vmo_status two_means_one(OrderState& st, int d, int km_iters, cudaStream_t s);
 vmo_status order_levels(OrderState& st, const OrderParams& op, cudaStream_t s, Scratch& sc);
 // Separators stably sorted by b two-bit link numbers (after order_levels).
 vmo_status cut_order_pass(OrderState& st, const OrderParams& op, cudaStream_t s, Scratch& sc);
