@@ -421,7 +421,9 @@ vmo_status vmo_hg_arrays(vmo_hg hg, const int32_t** adj_ptr, const int32_t** adj
 vmo_status vmo_components(vmo_hg hg, int32_t* labels, void* stream) {
   VMO_TRY(ensure_device());
   if (!hg || (!labels && hg->k > 0)) return invalid("null argument");
-  return components(hg, labels, (cudaStream_t)stream);
+  VMO_TRY(components(hg, labels, (cudaStream_t)stream));
+  VMO_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+  return VMO_OK;
 }
 
 vmo_status vmo_init_coords(int32_t k, int32_t d, uint64_t seed, float* coords, void* stream) {

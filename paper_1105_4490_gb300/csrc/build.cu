@@ -117,6 +117,11 @@ __global__ void emit_edges_kernel(const int32_t* __restrict__ adj_ptr, const int
 __global__ void net_ptr_last_kernel(int32_t* net_ptr, const int32_t* nedges) { net_ptr[*nedges] = 2 * *nedges; }
 
 // ----------------------------- components ----------------------------------
+// Union-find on the labels: a root points at itself, every other vertex at a
+// smaller one, so a tree's root is its smallest vertex.  Links are lossless
+// (a compare-and-swap on the larger root, repeated from its new parent when
+// another thread was first), so one pass over the nets finds the components
+// and no round has to be checked on the host.
 __device__ inline int32_t cc_find(const int32_t* p, int32_t v) {
   for (;;) {
     int32_t q = __ldcg(p + v);
@@ -125,9 +130,35 @@ __device__ inline int32_t cc_find(const int32_t* p, int32_t v) {
   }
 }
 
-__global__ void cc_init_kernel(int32_t* p, int32_t k) {
+__device__ inline void cc_link(int32_t u, int32_t v, int32_t* p) {
+  int32_t a = cc_find(p, u), b = cc_find(p, v);
+  while (a != b) {  // the larger of the two falls in every turn
+    const int32_t hi = a > b ? a : b, lo = a > b ? b : a;
+    const int32_t prev = atomicCAS(p + hi, hi, lo);
+    if (prev == hi) return;
+    a = cc_find(p, prev);
+    b = lo;
+  }
+}
+
+// Graph models start from every vertex's smallest neighbour (its own label if
+// that is larger): most vertices then hang below a common root before the pass
+// over the edges, which finds nearly every edge inside a tree (rows ascend, so
+// it is the row's first entry).
+__global__ void cc_init_kernel(const int32_t* __restrict__ adj_ptr, const int32_t* __restrict__ adj,
+                               int32_t* __restrict__ p, int32_t k) {
   int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v < k) p[v] = v;
+  if (v >= k) return;
+  int32_t q = v;
+  if (adj_ptr && adj_ptr[v + 1] > adj_ptr[v]) q = min(v, adj[adj_ptr[v]]);
+  p[v] = q;
+}
+
+// Links every vertex to its largest neighbour.
+__global__ void cc_last_neighbour_kernel(const int32_t* __restrict__ adj_ptr, const int32_t* __restrict__ adj,
+                                         int32_t* p, int32_t k) {
+  int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v < k && adj_ptr[v + 1] > adj_ptr[v]) cc_link(v, adj[adj_ptr[v + 1] - 1], p);
 }
 
 // Marks the last pin of every net (the pins that start no consecutive pair).
@@ -138,16 +169,20 @@ __global__ void cc_last_kernel(const int32_t* __restrict__ net_ptr, int64_t l, u
   if (b > net_ptr[e]) last[b - 1] = 1;
 }
 
-// Hooks the roots of consecutive pins of every net to the smaller root.
-__global__ void cc_hook_kernel(const int32_t* __restrict__ pins, const uint8_t* __restrict__ last, int64_t npins,
-                               int32_t* p, int32_t* changed) {
+// Links the consecutive pins of every net.
+__global__ void cc_pins_kernel(const int32_t* __restrict__ pins, const uint8_t* __restrict__ last, int64_t npins,
+                               int32_t* p) {
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t + 1 >= npins || last[t]) return;  // the last pin of a net pairs with no next pin
-  int32_t a = cc_find(p, pins[t]), b = cc_find(p, pins[t + 1]);
-  if (a == b) return;
-  int32_t hi_ = a > b ? a : b, lo_ = a > b ? b : a;
-  atomicMin(p + hi_, lo_);
-  *changed = 1;
+  cc_link(pins[t], pins[t + 1], p);
+}
+
+// Links the two ends of every edge; most edges already have one label.
+__global__ void cc_edges_kernel(const int2* __restrict__ edge, int64_t l, int32_t* p) {
+  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= l) return;
+  const int2 uv = edge[e];
+  if (__ldcg(p + uv.x) != __ldcg(p + uv.y)) cc_link(uv.x, uv.y, p);
 }
 
 __global__ void cc_compress_kernel(int32_t* p, int32_t k) {
@@ -429,33 +464,26 @@ vmo_status finegrain_coords(const vmo_hg_s* h, const float* xb, float* xf, cudaS
 }
 
 vmo_status components(const vmo_hg_s* h, int32_t* labels, cudaStream_t s) {
-  Scratch sc(s);
-  int32_t* changed;
-  uint8_t* last = nullptr;
-  VMO_TRY(sc.alloc(&changed, 1));
   if (h->k == 0) return VMO_OK;
-  launch(cc_init_kernel, grid_for(h->k, 256), 256, 0, s, labels, h->k);
-  VMO_LAUNCHED("cc_init");
-  if (h->npins > 1) {
+  Scratch sc(s);
+  const bool graph = h->model == VMO_SYMMETRIC || h->model == VMO_BIPARTITE;
+  const unsigned gv = grid_for(h->k, 256);
+  launch(cc_init_kernel, gv, 256, 0, s, graph ? h->adj_ptr.ptr : (const int32_t*)nullptr, h->adj.ptr, labels, h->k);
+  if (graph && h->l > 0) {
+    launch(cc_compress_kernel, gv, 256, 0, s, labels, h->k);
+    launch(cc_last_neighbour_kernel, gv, 256, 0, s, h->adj_ptr.ptr, h->adj.ptr, labels, h->k);
+    launch(cc_compress_kernel, gv, 256, 0, s, labels, h->k);
+    launch(cc_edges_kernel, grid_for(h->l, 256), 256, 0, s, (const int2*)h->pins.ptr, h->l, labels);
+  } else if (!graph && h->npins > 1) {
+    uint8_t* last;
     VMO_TRY(sc.alloc(&last, h->npins));
     VMO_CUDA(cudaMemsetAsync(last, 0, h->npins, s));
     if (h->l > 0) launch(cc_last_kernel, grid_for(h->l, 256), 256, 0, s, h->net_ptr.ptr, h->l, last);
-    VMO_LAUNCHED("cc_last");
+    launch(cc_pins_kernel, grid_for(h->npins, 256), 256, 0, s, h->pins.ptr, last, h->npins, labels);
   }
-  for (int it = 0; it < 64; ++it) {
-    VMO_CUDA(cudaMemsetAsync(changed, 0, 4, s));
-    if (h->npins > 1) {
-      launch(cc_hook_kernel, grid_for(h->npins, 256), 256, 0, s, h->pins.ptr, last, h->npins, labels, changed);
-      VMO_LAUNCHED("cc_hook");
-    }
-    launch(cc_compress_kernel, grid_for(h->k, 256), 256, 0, s, labels, h->k);
-    VMO_LAUNCHED("cc_compress");
-    int32_t hc = 0;
-    VMO_CUDA(cudaMemcpyAsync(&hc, changed, 4, cudaMemcpyDeviceToHost, s));
-    VMO_CUDA(cudaStreamSynchronize(s));
-    if (!hc) return VMO_OK;
-  }
-  return cuda_fail(cudaErrorUnknown, "components did not converge in 64 rounds", __FILE__, __LINE__);
+  launch(cc_compress_kernel, gv, 256, 0, s, labels, h->k);
+  VMO_LAUNCHED("components");
+  return VMO_OK;
 }
 
 vmo_status cut_size(const vmo_hg_s* h, const int32_t* part, int32_t nparts, int64_t* cutnet, int64_t* lambda1,

@@ -542,43 +542,67 @@ __device__ __forceinline__ unsigned long long part_count(uint8_t l) {
 
 // Order-free form of the separator loop of Algorithm 7 (mu = identity):
 // v joins the separator iff a neighbour w in the same node carries the other
-// label and (s(v), v) < (s(w), w).
-__global__ void k_separator(const int32_t* __restrict__ ord, const int32_t* __restrict__ seg, int64_t n,
-                            const int32_t* __restrict__ adj_ptr, const int32_t* __restrict__ adj,
-                            const uint64_t* __restrict__ vrec, NodeDev* __restrict__ nodes,
-                            uint8_t* __restrict__ labf, unsigned long long* __restrict__ pk) {
+// label and (s(v), v) < (s(w), w).  Any neighbour decides, so eight are tested
+// at a time with all their loads issued together; rows of more than
+// kSepLong entries are tested by the whole warp, 32 at a time (a thread with a
+// hub's row held its warp: 155 us for the root of the 400k x 300k bipartite
+// pattern).
+constexpr int kSepLong = 64;
+
+__global__ void __launch_bounds__(kBlock) k_separator(const int32_t* __restrict__ ord, const int32_t* __restrict__ seg,
+                                                      int64_t n, const int32_t* __restrict__ adj_ptr,
+                                                      const int32_t* __restrict__ adj,
+                                                      const uint64_t* __restrict__ vrec, NodeDev* __restrict__ nodes,
+                                                      uint8_t* __restrict__ labf, unsigned long long* __restrict__ pk) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int s = i < n ? seg[i] : -1;
   uint8_t l = 0;
+  int32_t v = 0, t0 = 0, t1 = 0;
+  uint64_t rv = 0;
   if (s >= 0) {
-    const int32_t v = ord[i];
-    const uint64_t rv = vrec[v];
+    v = ord[i];
+    rv = vrec[v];
     l = (uint8_t)vrec_label(rv);
     if (l != 0) {
-      // any neighbour decides, so four are tested at a time with all their
-      // loads issued together
-      const float sv = vrec_s(rv);
-      const uint32_t other = vrec_other(s, l);
-      const int32_t t1 = adj_ptr[v + 1];
-      bool hit = false;
-      for (int32_t t = adj_ptr[v]; t < t1 && !hit; t += 4) {
-        int32_t w[4];
-        uint64_t rw[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) w[u] = t + u < t1 ? adj[t + u] : -1;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) rw[u] = w[u] >= 0 ? vrec[w[u]] : 0ull;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (w[u] < 0 || (uint32_t)(rw[u] >> 32) != other) continue;  // not in this node, or on the same side
-          const float sw = vrec_s(rw[u]);
-          if (sv < sw || (sv == sw && v < w[u])) hit = true;
-        }
-      }
-      if (hit) l = 3;
+      t0 = adj_ptr[v];
+      t1 = adj_ptr[v + 1];
     }
-    labf[i] = l;
   }
+  // does neighbour w (record rw) put vertex u (record ru) into the separator?
+  auto cuts = [](int32_t u, uint64_t ru, int32_t w, uint64_t rw) {
+    if ((uint32_t)(rw >> 32) != ((uint32_t)(ru >> 32) ^ 3u)) return false;  // another node, or the same side
+    const float su = vrec_s(ru), sw = vrec_s(rw);
+    return su < sw || (su == sw && u < w);
+  };
+  bool hit = false;
+  const bool lng = t1 - t0 > kSepLong;
+  if (!lng)
+    for (int32_t t = t0; t < t1 && !hit; t += 8) {
+      int32_t w[8];
+      uint64_t rw[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) w[u] = t + u < t1 ? adj[t + u] : -1;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) rw[u] = w[u] >= 0 ? vrec[w[u]] : 0ull;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) hit = hit || (w[u] >= 0 && cuts(v, rv, w[u], rw[u]));
+    }
+  unsigned todo = __ballot_sync(0xffffffffu, lng);
+  while (todo) {
+    const int src = __ffs(todo) - 1;
+    todo &= todo - 1;
+    const int32_t u = __shfl_sync(0xffffffffu, v, src), a = __shfl_sync(0xffffffffu, t0, src),
+                  b = __shfl_sync(0xffffffffu, t1, src);
+    const uint64_t ru = __shfl_sync(0xffffffffu, (unsigned long long)rv, src);
+    bool any = false;
+    for (int32_t t = a; t < b && !any; t += 32) {
+      const int32_t w = t + (int)lane_id() < b ? adj[t + lane_id()] : -1;
+      any = __any_sync(0xffffffffu, w >= 0 && cuts(u, ru, w, vrec[w >= 0 ? w : 0]));
+    }
+    if ((int)lane_id() == src) hit = any;
+  }
+  if (hit) l = 3;
+  if (s >= 0) labf[i] = l;
   if (i < n) pk[i] = part_count(l);
   count_labels(s, l, nodes);
 }
@@ -1547,7 +1571,9 @@ vmo_status order_levels(OrderState& st, const OrderParams& op, cudaStream_t s, S
   int32_t* next_max = next_count + 1;
   err = next_count + 2;
   int64_t max_size = st.max_root;
+  int levels = 0;  // depth of the deepest record
   while (N > 0) {
+    ++levels;
     VMO_TRY(two_means(st, N, max_size, op.d, op.km_iters, s, sc));
     if (st.mu && op.mu_order_free) {
       launch(k_pick, grid_for(n, kBlock), kBlock, 0, s, st.ord, st.seg, n, st.adj_ptr, st.adj, st.vrec, st.vpick);
@@ -1582,6 +1608,8 @@ vmo_status order_levels(OrderState& st, const OrderParams& op, cudaStream_t s, S
     N = h[0];
     max_size = h[1];
   }
+  // heap numbers of depth t are below 2^(t + 1), with ternary keys below 3^(t + 1) / 2
+  st.heap_bits = std::min(64, op.sep_rec ? (levels + 1) * 8 / 5 + 1 : levels + 1);
   return VMO_OK;
 }
 
@@ -1592,6 +1620,7 @@ vmo_status order_setup(OrderState& st, const float4* x, const std::vector<int64_
   const int P = (int)pbase_host.size() - 1;
   if (n >= (int64_t(1) << 30) - 64) return invalid("ordering: more than 2^30 - 64 vertices");
   st.n = n;
+  st.nprob = P;
   VMO_TRY(sc.alloc(&st.ord, std::max<int64_t>(n, 1)));
   VMO_TRY(sc.alloc(&st.xo, std::max<int64_t>(n, 1)));
   VMO_TRY(sc.alloc(&st.seg, std::max<int64_t>(n, 1)));
@@ -1693,11 +1722,11 @@ vmo_status tree_sorted(OrderState& st, bool by_prob, int32_t* count_out, uint32_
   if (n == 0) { *idx_out = v2; return VMO_OK; }
   launch(k_tree_keys, grid_for(n, kBlock), kBlock, 0, s, st.tree, n, 0, k1, v1);
   VMO_LAUNCHED("tree_keys");
-  VMO_TRY(radix_sort_u64(k1, v1, k2, v2, n, 64, s, sc));
-  if (by_prob) {
+  VMO_TRY(radix_sort_u64(k1, v1, k2, v2, n, st.heap_bits, s, sc));
+  if (by_prob && st.nprob > 1) {
     launch(k_tree_regather, grid_for(n, kBlock), kBlock, 0, s, v2, n, 1, st.tree, k1);
     VMO_LAUNCHED("tree_regather");
-    VMO_TRY(radix_sort_u64(k1, v2, k2, v1, n, 32, s, sc));
+    VMO_TRY(radix_sort_u64(k1, v2, k2, v1, n, bits_for((uint64_t)st.nprob - 1), s, sc));
     *idx_out = v1;
   } else {
     *idx_out = v2;

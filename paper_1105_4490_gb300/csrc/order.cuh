@@ -69,6 +69,8 @@ struct OrderState {
   int node_cap = 0;
   int nroots = 0;
   int64_t max_root = 0;               // points of the largest active root
+  int nprob = 0;                      // problems
+  int heap_bits = 64;                 // bits of the largest heap number (set by order_levels)
   TreeDev tree;
 };
 
