@@ -4,12 +4,13 @@
 // fp32 distances without FMA, ties to the smaller centre, exact fixed-point
 // means on the grid 2^-(30-e)); for m = 2 it is vmo_bisect.
 //
-// Seeding takes m - 1 rounds of (running minimum distance and weights, scan,
-// pick); a Lloyd round is one assignment kernel (centres in shared memory,
-// per-block fixed-point sums in shared memory folded into global int64 sums
-// with atomics, exact and order-free) and one update kernel.
+// Seeding takes m - 1 rounds of (running minimum distance and block sums of
+// the weights, pick); a Lloyd round is one assignment kernel (centres in shared
+// memory, per-block fixed-point sums in shared memory folded into global int64
+// sums with atomics, exact and order-free) and one update kernel.
 #include <algorithm>
 
+#include "blocksort.cuh"
 #include "vmo_internal.cuh"
 
 namespace vmo {
@@ -20,6 +21,7 @@ namespace {
 
 constexpr int kKmBlock = 256;
 constexpr int kKmMaxCentres = 256;
+constexpr int kKmPickBlock = 1024;
 
 struct KmState {
   int e;             // max |x| < 2^e
@@ -56,36 +58,117 @@ __global__ void k_km_seed0(const float4* __restrict__ xo, int64_t n, uint64_t se
   z[0] = xo[scale_draw((uint64_t)n, rand64(seed ^ kTagKmeans, key, 0))];
 }
 
-// Running minimum squared distance to the chosen centres (centre c just
-// picked) and its integer D^2 weight floor(dmin * 2^(34 - 2e)).
-template <int D>
-__global__ void k_km_weights(const float4* __restrict__ xo, int64_t n, const float4* __restrict__ z, int c,
-                             float* __restrict__ dmin, unsigned long long* __restrict__ w,
-                             const KmState* __restrict__ st) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || st->stopped) return;
-  const float dd = sqdist32<D>(xo[i], z[c]);
-  const float dm = c == 0 ? dd : fminf(dmin[i], dd);
-  dmin[i] = dm;
-  w[i] = (unsigned long long)floorf(__fmul_rn(dm, exp2i_f(34 - 2 * st->e)));
+// Seeding of centre c, two launches.  First the running minimum squared
+// distance to the chosen centres (centre c - 1 just picked) and the block's
+// sum of the integer D^2 weights floor(dmin * 2^(34 - 2e)); then the first
+// point whose inclusive prefix of the weights exceeds floor(total * r_c /
+// 2^64) is found from the block sums and, in the one block that holds it, from the
+// weights computed again (a zero total stops the seeding).  The weights and their
+// prefixes are never stored: as five launches with 40 bytes a point a centre
+// took 25 us of a million points, bound by launches and traffic alike.
+constexpr int kKmItems = 8;                        // points per thread
+constexpr int kKmTile = kKmBlock * kKmItems;       // points per block
+static_assert(kKmBlock == 256, "eight warps");
+
+__device__ __forceinline__ unsigned long long km_weight(float dm, int e) {
+  return (unsigned long long)floorf(__fmul_rn(dm, exp2i_f(34 - 2 * e)));
 }
 
-// Centre c: the first point whose inclusive prefix of the weights exceeds
-// floor(total * r_c / 2^64); a zero total stops the seeding.
-__global__ void k_km_pick(const float4* __restrict__ xo, int64_t n, const unsigned long long* __restrict__ w,
-                          const unsigned long long* __restrict__ pre, uint64_t seed, uint64_t key, int c,
-                          float4* __restrict__ z, KmState* __restrict__ st) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || st->stopped) return;
-  const unsigned long long total = pre[n - 1];
+template <int D>
+__global__ void __launch_bounds__(kKmBlock) k_km_weights(const float4* __restrict__ xo, int64_t n,
+                                                         const float4* __restrict__ z, int c, float* __restrict__ dmin,
+                                                         unsigned long long* __restrict__ bsum,
+                                                         const KmState* __restrict__ st) {
+  __shared__ unsigned long long red[kKmBlock / 32];
+  if (st->stopped) return;  // grid-uniform
+  const int e = st->e;
+  const float4 zc = z[c - 1];
+  const int64_t i0 = (int64_t)blockIdx.x * kKmTile + threadIdx.x;
+  float4 p[kKmItems];
+  float old[kKmItems];
+#pragma unroll
+  for (int u = 0; u < kKmItems; ++u) {  // every load in flight together
+    const int64_t i = i0 + u * kKmBlock;
+    p[u] = i < n ? xo[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    old[u] = i < n && c > 1 ? dmin[i] : 0.f;
+  }
+  unsigned long long w = 0;
+#pragma unroll
+  for (int u = 0; u < kKmItems; ++u) {
+    const int64_t i = i0 + u * kKmBlock;
+    if (i >= n) break;
+    const float dd = sqdist32<D>(p[u], zc);
+    const float dm = c == 1 ? dd : fminf(old[u], dd);
+    dmin[i] = dm;
+    w += km_weight(dm, e);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+  if (lane_id() == 0) red[threadIdx.x >> 5] = w;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long sum = 0;
+    for (int q = 0; q < kKmBlock / 32; ++q) sum += red[q];
+    bsum[blockIdx.x] = sum;
+  }
+}
+
+// One block: the block of points that holds the draw, then the point in it.
+__global__ void __launch_bounds__(kKmPickBlock) k_km_pick(const float4* __restrict__ xo, int64_t n,
+                                                          const float* __restrict__ dmin,
+                                                          const unsigned long long* __restrict__ bsum, int nb,
+                                                          uint64_t seed, uint64_t key, int c, float4* __restrict__ z,
+                                                          KmState* __restrict__ st) {
+  __shared__ unsigned long long ws[33];
+  __shared__ unsigned long long s_before;
+  __shared__ int s_block;
+  if (st->stopped) return;
+  // block sums: contiguous parts of the threads, prefixes by a block scan
+  const int per = (nb + kKmPickBlock - 1) / kKmPickBlock;
+  const int a = min((int)threadIdx.x * per, nb), b = min(a + per, nb);
+  unsigned long long sum = 0;
+  for (int q = a; q < b; ++q) sum += bsum[q];
+  unsigned long long total;
+  const unsigned long long ex = block_exclusive<unsigned long long>(sum, ws, &total);
   if (total == 0) {
-    if (i == 0) st->stopped = 1;
+    if (threadIdx.x == 0) st->stopped = 1;
     return;
   }
   const unsigned long long thr = scale_draw(total, rand64(seed ^ kTagKmeans, key, (uint64_t)c));
-  if (pre[i] - w[i] <= thr && thr < pre[i]) {
-    z[c] = xo[i];
-    st->chosen = c + 1;
+  if (threadIdx.x == 0) s_block = -1;
+  __syncthreads();
+  if (thr >= ex && thr - ex < sum) {
+    unsigned long long run = ex;
+    for (int q = a; q < b; ++q) {
+      const unsigned long long w = bsum[q];
+      if (thr - run < w) {
+        s_block = q;
+        s_before = run;
+        break;
+      }
+      run += w;
+    }
+  }
+  __syncthreads();
+  if (s_block < 0) return;
+  const int e = st->e;
+  const int64_t base = (int64_t)s_block * kKmTile;
+  constexpr int kPer = kKmTile / kKmPickBlock;
+  unsigned long long w[kPer], own = 0;
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int64_t i = base + threadIdx.x * kPer + u;
+    w[u] = i < n ? km_weight(dmin[i], e) : 0ull;
+    own += w[u];
+  }
+  unsigned long long run = s_before + block_exclusive<unsigned long long>(own, ws, nullptr);
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    if (run <= thr && thr < run + w[u]) {
+      z[c] = xo[base + threadIdx.x * kPer + u];
+      st->chosen = c + 1;
+    }
+    run += w[u];
   }
 }
 
@@ -95,21 +178,17 @@ __global__ void k_km_fill(float4* __restrict__ z, int m, const KmState* __restri
   if (c < m && c >= st->chosen) z[c] = z[0];
 }
 
-template <int D>
-__device__ __forceinline__ int km_nearest(const float4& p, const float4* zs, int m) {
-  int best = 0;
-  float bd = sqdist32<D>(p, zs[0]);
-  for (int j = 1; j < m; ++j) {
-    const float dj = sqdist32<D>(p, zs[j]);
-    if (dj < bd) {
-      bd = dj;
-      best = j;
-    }
-  }
-  return best;
-}
+// One Lloyd assignment (it >= 0) or the final labelling (it < 0).  Each thread
+// takes kKmAssign points at a time, so that a centre read from shared memory serves
+// all of them, and a block walks over tiles of the points and keeps the
+// clusters' sums in shared memory until its end.  The fixed-point values are
+// added as two 32-bit words (their low 16 bits and the rest): shared memory has
+// native 32-bit additions but adds 64 bits by a compare-and-swap loop, which took most
+// of the 150 us a round of a million points and 64 centres (now 40); a flush into
+// 64-bit sums after kKmFlush points keeps the words from overflowing.
+constexpr int kKmAssign = 4;
+constexpr int kKmFlush = 8192;  // points of a block between flushes: 8192 (2^16 + 2^14) < 2^31
 
-// One Lloyd assignment (it >= 0) or the final labelling (it < 0).
 template <int D>
 __global__ void __launch_bounds__(kKmBlock) k_km_assign(const float4* __restrict__ xo, int64_t n, int m, int it,
                                                         const float4* __restrict__ z, int32_t* __restrict__ lab,
@@ -117,38 +196,88 @@ __global__ void __launch_bounds__(kKmBlock) k_km_assign(const float4* __restrict
                                                         unsigned long long* __restrict__ cnt,
                                                         KmState* __restrict__ st) {
   __shared__ float4 zs[kKmMaxCentres];
-  __shared__ unsigned long long ss[kKmMaxCentres * 4];
-  __shared__ unsigned long long sc[kKmMaxCentres];
+  __shared__ unsigned lo[kKmMaxCentres * D];
+  __shared__ int hi[kKmMaxCentres * D];
+  __shared__ int sc[kKmMaxCentres];
   const bool final_pass = it < 0;
   if (!final_pass && st->converged) return;  // block-uniform
   for (int j = threadIdx.x; j < m; j += blockDim.x) {
     zs[j] = z[j];
     sc[j] = 0;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) ss[j * 4 + q] = 0;
-  }
-  __syncthreads();
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const float fx = exp2i_f(30 - st->e);
-  if (i < n) {
-    const float4 p = xo[i];
-    const int l = km_nearest<D>(p, zs, m);
-    if (!final_pass && it > 0 && lab[i] != l) st->changed = 1;
-    lab[i] = l;
-    atomicAdd(&sc[l], 1ull);
-    if (!final_pass) {
-#pragma unroll
-      for (int q = 0; q < D; ++q)
-        atomicAdd(&ss[l * 4 + q], (unsigned long long)__float2ll_rn(__fmul_rn(comp(p, q), fx)));
+    for (int q = 0; q < D; ++q) {
+      lo[j * D + q] = 0u;
+      hi[j * D + q] = 0;
     }
   }
   __syncthreads();
-  for (int j = threadIdx.x; j < m; j += blockDim.x) {
-    if (sc[j] == 0) continue;
-    atomicAdd(&cnt[j], sc[j]);
-    if (!final_pass)
-      for (int q = 0; q < D; ++q) atomicAdd(&S[j * 4 + q], ss[j * 4 + q]);
+  const float fx = exp2i_f(30 - st->e);
+  bool changed = false;
+  auto flush = [&]() {
+    __syncthreads();
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {
+      if (sc[j] == 0) continue;
+      atomicAdd(&cnt[j], (unsigned long long)sc[j]);
+      sc[j] = 0;
+      if (final_pass) continue;
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        atomicAdd(&S[j * 4 + q], (unsigned long long)(((long long)hi[j * D + q] << 16) + (long long)lo[j * D + q]));
+        lo[j * D + q] = 0u;
+        hi[j * D + q] = 0;
+      }
+    }
+    __syncthreads();
+  };
+  int held = 0;  // points since the last flush
+  constexpr int kTile = kKmBlock * kKmAssign;
+  for (int64_t base = (int64_t)blockIdx.x * kTile; base < n; base += (int64_t)gridDim.x * kTile) {
+    if (held + kTile > kKmFlush) {
+      flush();
+      held = 0;
+    }
+    held += kTile;
+    float4 p[kKmAssign];
+    float bd[kKmAssign];
+    int best[kKmAssign];
+    const int64_t i0 = base + threadIdx.x;
+#pragma unroll
+    for (int u = 0; u < kKmAssign; ++u) {
+      const int64_t i = i0 + u * kKmBlock;
+      p[u] = i < n ? xo[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      bd[u] = sqdist32<D>(p[u], zs[0]);
+      best[u] = 0;
+    }
+    for (int j = 1; j < m; ++j) {
+      const float4 c = zs[j];
+#pragma unroll
+      for (int u = 0; u < kKmAssign; ++u) {
+        const float dj = sqdist32<D>(p[u], c);
+        if (dj < bd[u]) {
+          bd[u] = dj;
+          best[u] = j;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kKmAssign; ++u) {
+      const int64_t i = i0 + u * kKmBlock;
+      if (i >= n) continue;
+      const int l = best[u];
+      if (!final_pass && it > 0 && lab[i] != l) changed = true;
+      lab[i] = l;
+      atomicAdd(&sc[l], 1);
+      if (final_pass) continue;
+#pragma unroll
+      for (int q = 0; q < D; ++q) {  // |value| < 2^30
+        const int v = __float2int_rn(__fmul_rn(comp(p[u], q), fx));
+        atomicAdd(&lo[l * D + q], (unsigned)v & 0xffffu);
+        atomicAdd(&hi[l * D + q], v >> 16);
+      }
+    }
   }
+  flush();
+  if (changed) st->changed = 1;
 }
 
 // Centre update: z = fp32((double(sum) / count) * 2^-(30 - e)) for non-empty
@@ -212,13 +341,13 @@ vmo_status kmeans_m(int32_t d, const float* coords, const int32_t* verts, int32_
   const int64_t n = nverts;
   float4 *xo, *z = reinterpret_cast<float4*>(centres);
   float* dmin;
-  unsigned long long *w, *pre, *S, *cnt;
+  unsigned long long *bsum, *S, *cnt;
   KmState* st;
   int32_t* ne;
   VMO_TRY(sc.alloc(&xo, n));
   VMO_TRY(sc.alloc(&dmin, n));
-  VMO_TRY(sc.alloc(&w, n));
-  VMO_TRY(sc.alloc(&pre, n));
+  const int nt = (int)((n + kKmTile - 1) / kKmTile);  // tiles of the seeding
+  VMO_TRY(sc.alloc(&bsum, nt));
   VMO_TRY(sc.alloc(&S, (size_t)m * 4));
   VMO_TRY(sc.alloc(&cnt, (size_t)m));
   VMO_TRY(sc.alloc(&st, 1));
@@ -227,20 +356,20 @@ vmo_status kmeans_m(int32_t d, const float* coords, const int32_t* verts, int32_
   VMO_CUDA(cudaMemsetAsync(S, 0, (size_t)m * 4 * sizeof(unsigned long long), s));
   VMO_CUDA(cudaMemsetAsync(cnt, 0, (size_t)m * sizeof(unsigned long long), s));
   const unsigned nb = (unsigned)((n + kKmBlock - 1) / kKmBlock);
+  // assignment blocks: one wave, so that the clusters' sums leave a block once
+  const unsigned na = (unsigned)std::min<int64_t>((n + kKmBlock * kKmAssign - 1) / (kKmBlock * kKmAssign), 152 * 6);
   vmo_status stt = VMO_OK;
   km_dispatch(d, [&](auto DC) {
     constexpr int D = decltype(DC)::value;
     launch(k_km_gather<D>, nb, kKmBlock, 0, s, reinterpret_cast<const float4*>(coords), verts, n, xo, st);
     launch(k_km_seed0, 1, 1, 0, s, xo, n, seed, key, z, st);
-    for (int c = 1; c < m && stt == VMO_OK; ++c) {
-      launch(k_km_weights<D>, nb, kKmBlock, 0, s, xo, n, z, c - 1, dmin, w, st);
-      stt = scan_inclusive<uint64_t>((const uint64_t*)w, (uint64_t*)pre, n, s, sc);
-      if (stt == VMO_OK) launch(k_km_pick, nb, kKmBlock, 0, s, xo, n, w, pre, seed, key, c, z, st);
+    for (int c = 1; c < m; ++c) {
+      launch(k_km_weights<D>, (unsigned)nt, kKmBlock, 0, s, xo, n, z, c, dmin, bsum, st);
+      launch(k_km_pick, 1, kKmPickBlock, 0, s, xo, n, dmin, bsum, nt, seed, key, c, z, st);
     }
-    if (stt != VMO_OK) return;
     launch(k_km_fill, 1, kKmMaxCentres, 0, s, z, m, st);
     for (int it = 0; it < km_iters; ++it) {
-      launch(k_km_assign<D>, nb, kKmBlock, 0, s, xo, n, m, it, z, labels, S, cnt, st);
+      launch(k_km_assign<D>, na, kKmBlock, 0, s, xo, n, m, it, z, labels, S, cnt, st);
       launch(k_km_update<D>, 1, kKmMaxCentres, 0, s, z, m, it, S, cnt, st);
       if (it % 4 == 3 && it + 1 < km_iters) {  // stop early once converged
         KmState h;
@@ -254,7 +383,7 @@ vmo_status kmeans_m(int32_t d, const float* coords, const int32_t* verts, int32_
       }
     }
     if (stt != VMO_OK) return;
-    launch(k_km_assign<D>, nb, kKmBlock, 0, s, xo, n, m, -1, z, labels, S, cnt, st);
+    launch(k_km_assign<D>, na, kKmBlock, 0, s, xo, n, m, -1, z, labels, S, cnt, st);
     launch(k_km_nonempty, 1, 1, 0, s, cnt, m, ne);
   });
   VMO_TRY(stt);
