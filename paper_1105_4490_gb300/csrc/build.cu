@@ -1,11 +1,19 @@
 // Hypergraph models of a sparse pattern (Table 1, Sec. 1.1), connected
 // components (Algorithm 1) and cut metrics (Sec. 4.1 footnote, Sec. 5).
 //
-// Every model is built the same way on the device: each nonzero emits 64-bit
-// pair keys (row * ncols + col), a radix sort orders them, a flag/scan pass
-// drops duplicates and the surviving keys become CSR rows whose pointers come
-// from per-row counts and a scan.  Graph models emit both orientations of
-// {u, v} so the result is the symmetric adjacency with ascending neighbours.
+// Any pattern can be built the general way: each nonzero emits 64-bit pair
+// keys (row * ncols + col), a radix sort orders them, a flag/scan pass drops
+// duplicates and the surviving keys become CSR rows whose pointers come from
+// per-row counts and a scan.  Graph models emit both orientations of {u, v} so
+// the result is the symmetric adjacency with ascending neighbours.
+//
+// A pattern whose rows ascend strictly, as matrices are usually stored, needs
+// no such sort (the validation pass finds out): its rows are already the rows of
+// the model, its columns come from one stable sort of 32-bit column keys with the
+// entry numbers (two passes instead of four of 64-bit keys), and a symmetric
+// pattern is its own adjacency, with every entry's mirror found by a binary
+// search in its row.  27-point mesh of 10^6 rows in random numbering, symmetric
+// model with copies of its arrays: 7.6 -> 2.4 ms; 400k x 300k bipartite model: 2.1 -> 1.2 ms.
 #include <algorithm>
 
 #include "vmo_internal.cuh"
@@ -23,17 +31,204 @@ __device__ inline int32_t row_of(const int32_t* __restrict__ rowptr, int32_t m, 
   return lo;
 }
 
-__global__ void validate_csr_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx, int32_t m,
-                                    int32_t n, int64_t nnz, int32_t* __restrict__ bad) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < m) {
-    if (rowptr[t + 1] < rowptr[t]) atomicOr(bad, 1);
+// Error bits: 1 rowptr not monotone, 2 its ends, 4 a column out of range.
+// steps (optional): [0] entries that do not ascend from the entry before them,
+// [1] how many of these start a row; every row ascends strictly iff the two
+// agree (a search of the row at each step took five times the pass).
+__global__ void __launch_bounds__(256) validate_csr_kernel(const int32_t* __restrict__ rowptr,
+                                                           const int32_t* __restrict__ colidx, int32_t m, int32_t n,
+                                                           int64_t nnz, int32_t* __restrict__ bad,
+                                                           int32_t* __restrict__ steps) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int err = 0, down = 0, starts = 0;
+  if (first == 0 && (rowptr[0] != 0 || (int64_t)rowptr[m] != nnz)) err |= 2;
+  for (int64_t r = first; r < m; r += stride) {
+    const int32_t a = rowptr[r], b = rowptr[r + 1];
+    if (b < a) err |= 1;
+    if (steps && a > 0 && a < b && b <= nnz) starts += colidx[a] <= colidx[a - 1];
   }
-  if (t == 0 && (rowptr[0] != 0 || (int64_t)rowptr[m] != nnz)) atomicOr(bad, 2);
-  if (t < nnz) {
-    int32_t c = colidx[t];
-    if (c < 0 || c >= n) atomicOr(bad, 4);
+  for (int64_t t = first; t < nnz; t += 4 * stride) {
+    int32_t c[4], p[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t i = t + u * stride;
+      c[u] = i < nnz ? colidx[i] : 0;
+      p[u] = steps && i < nnz && i > 0 ? colidx[i - 1] : INT32_MIN;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (t + u * stride >= nnz) break;
+      if (c[u] < 0 || c[u] >= n) err |= 4;
+      down += c[u] <= p[u];
+    }
   }
+  err = __reduce_or_sync(0xffffffffu, err);
+  if (lane_id() == 0 && err) atomicOr(bad, err);
+  if (!steps) return;
+  down = __reduce_add_sync(0xffffffffu, down);
+  starts = __reduce_add_sync(0xffffffffu, starts);
+  if (lane_id() == 0) {
+    if (down) atomicAdd(&steps[0], down);
+    if (starts) atomicAdd(&steps[1], starts);
+  }
+}
+
+// ----- models of patterns with strictly ascending rows -----
+constexpr int kRowTile = 2048;  // entries per block
+
+// Row of the entries [t0, t0 + count) of a tile, count <= kRowTile, from the row starts of
+// the tile's rows in shared memory (in global memory when empty rows make them
+// more than fit).
+struct TileRows {
+  int32_t ptr[kRowTile + 2];
+  int32_t r0, r1;  // rows of the tile's first and last entry
+};
+
+__device__ inline void tile_rows_load(TileRows& s, const int32_t* __restrict__ rowptr, int32_t m, int64_t t0,
+                                      int64_t count) {
+  if (threadIdx.x == 0) s.r0 = row_of(rowptr, m, t0);
+  if (threadIdx.x == 32) s.r1 = row_of(rowptr, m, t0 + count - 1);
+  __syncthreads();
+  const int32_t rows = s.r1 - s.r0 + 1;
+  if (rows <= kRowTile + 1)
+    for (int32_t i = threadIdx.x; i < rows; i += blockDim.x) s.ptr[i] = rowptr[s.r0 + i];
+  __syncthreads();
+}
+
+__device__ inline int32_t tile_row(const TileRows& s, const int32_t* __restrict__ rowptr, int64_t t) {
+  const int32_t rows = s.r1 - s.r0 + 1;
+  const int32_t* p = rows <= kRowTile + 1 ? s.ptr : rowptr + s.r0;
+  return s.r0 + row_of(p, rows, t);
+}
+
+// Column keys, entry numbers and rows of the entries (for the column sort).
+__global__ void __launch_bounds__(256) entry_rows_kernel(const int32_t* __restrict__ rowptr,
+                                                         const int32_t* __restrict__ colidx, int32_t m, int64_t nnz,
+                                                         uint32_t* __restrict__ key, uint32_t* __restrict__ val,
+                                                         int32_t* __restrict__ row) {
+  __shared__ TileRows s;
+  const int64_t t0 = (int64_t)blockIdx.x * kRowTile;
+  const int64_t count = min((int64_t)kRowTile, nnz - t0);
+  tile_rows_load(s, rowptr, m, t0, count);
+  for (int64_t t = t0 + threadIdx.x; t < t0 + count; t += blockDim.x) {
+    key[t] = (uint32_t)colidx[t];
+    val[t] = (uint32_t)t;
+    row[t] = tile_row(s, rowptr, t);
+  }
+}
+
+// First sorted entry of every column, and the end.
+__global__ void column_starts_kernel(const uint32_t* __restrict__ key, int64_t nnz, int32_t n, int32_t add,
+                                     int32_t* __restrict__ ptr) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c > n) return;
+  int64_t lo = 0, hi = nnz;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if ((int64_t)key[mid] < c) lo = mid + 1; else hi = mid;
+  }
+  ptr[c] = add + (int32_t)lo;
+}
+
+// The column side of a model: idx[s] (vertex or net of the s-th entry in
+// column order) is its row, or its entry number when row is null.
+__global__ void column_entries_kernel(const uint32_t* __restrict__ val, const int32_t* __restrict__ row, int64_t nnz,
+                                      int32_t* __restrict__ idx, int32_t* __restrict__ entry) {
+  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= nnz) return;
+  const uint32_t t = val[s];
+  if (idx) idx[s] = row[t];
+  if (entry) entry[s] = (int32_t)t;
+}
+
+// The row side of the bipartite model: entry t is net t, of row i and column
+// vertex m + j.
+__global__ void bipartite_rows_kernel(const int32_t* __restrict__ colidx, const int32_t* __restrict__ row, int32_t m,
+                                      int64_t nnz, int32_t* __restrict__ adj, int32_t* __restrict__ vnets,
+                                      int32_t* __restrict__ net_ptr, int2* __restrict__ pins) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t > nnz) return;
+  net_ptr[t] = (int32_t)(2 * t);
+  if (t == nnz) return;
+  const int32_t v = m + colidx[t];
+  adj[t] = v;
+  vnets[t] = (int32_t)t;
+  pins[t] = make_int2(row[t], v);
+}
+
+// Rows of a square pattern: entry on the diagonal (0 or 1) and entries right of it.
+__global__ void row_parts_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx, int32_t m,
+                                 int32_t* __restrict__ diag, int32_t* __restrict__ right) {
+  const int32_t u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u >= m) return;
+  int32_t lo = rowptr[u];
+  const int32_t end = rowptr[u + 1];
+  int32_t hi = end;
+  while (lo < hi) {
+    const int32_t mid = (lo + hi) >> 1;
+    if (colidx[mid] < u) lo = mid + 1; else hi = mid;
+  }
+  const int32_t d = lo < end && colidx[lo] == u ? 1 : 0;
+  diag[u] = d;
+  right[u] = end - lo - d;
+}
+
+// First entry of every row and the diagonal entries before it, side by side (a
+// mirror's row is looked up once per net).
+__global__ void row_heads_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ dpre, int32_t m,
+                                 int2* __restrict__ head) {
+  const int32_t u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u <= m) head[u] = make_int2(rowptr[u], dpre[u]);
+}
+
+// Adjacency of a symmetric pattern: the entries off the diagonal.  Every entry
+// (u, v) right of the diagonal is net number e, and sets the incidence of its
+// mirror (v, u) too; *missing is set when an entry has no mirror.  dpre and rpre:
+// diagonal entries and entries right of the diagonal in the rows before.
+// Bound by the mirrors' scattered sectors (six per net).
+__global__ void __launch_bounds__(256) symmetric_kernel(const int32_t* __restrict__ rowptr,
+                                                        const int32_t* __restrict__ colidx, int32_t m, int64_t nnz,
+                                                        const int2* __restrict__ head,
+                                                        const int32_t* __restrict__ rpre, int32_t* __restrict__ adj,
+                                                        int32_t* __restrict__ vnets, int32_t* __restrict__ net_ptr,
+                                                        int2* __restrict__ pins, int32_t* __restrict__ missing) {
+  __shared__ TileRows s;
+  const int64_t t0 = (int64_t)blockIdx.x * kRowTile;
+  const int64_t count = min((int64_t)kRowTile, nnz - t0);
+  tile_rows_load(s, rowptr, m, t0, count);
+  for (int64_t t = t0 + threadIdx.x; t < t0 + count; t += blockDim.x) {
+    const int32_t v = colidx[t], u = tile_row(s, rowptr, t);
+    if (v == u) continue;
+    if (v < u) {
+      adj[t - head[u].y] = v;
+      continue;
+    }
+    const int2 next = head[u + 1];
+    const int32_t e = rpre[u + 1] - (next.x - (int32_t)t);  // entries right of the diagonal end the row
+    const int32_t place = (int32_t)t - next.y;
+    adj[place] = v;
+    vnets[place] = e;
+    net_ptr[e] = 2 * e;
+    pins[e] = make_int2(u, v);
+    const int2 hv = head[v];
+    const int32_t b1 = head[v + 1].x;
+    int32_t lo = hv.x, hi = b1;
+    while (lo < hi) {
+      const int32_t mid = (lo + hi) >> 1;
+      if (colidx[mid] < u) lo = mid + 1; else hi = mid;
+    }
+    if (lo < b1 && colidx[lo] == u) vnets[lo - hv.y] = e;  // left of the diagonal of row v
+    else *missing = 1;
+  }
+}
+
+__global__ void symmetric_ptr_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ dpre, int32_t m,
+                                     int32_t nets, int32_t* __restrict__ adj_ptr, int32_t* __restrict__ vtx_ptr,
+                                     int32_t* __restrict__ net_ptr) {
+  const int32_t u = blockIdx.x * blockDim.x + threadIdx.x;
+  if (u > m) return;
+  adj_ptr[u] = vtx_ptr[u] = rowptr[u] - dpre[u];
+  if (u == 0) net_ptr[nets] = 2 * nets;
 }
 
 // Pair keys of the graph models: both orientations of every off-diagonal
@@ -225,33 +420,182 @@ __global__ void cut_kernel(const int32_t* __restrict__ net_ptr, const int32_t* _
 
 }  // namespace
 
+static void validate_launch(const vmo_csr* a, int32_t* bad, int32_t* steps, cudaStream_t s) {
+  const int64_t n = std::max<int64_t>(a->m, (a->nnz + 3) / 4);
+  launch(validate_csr_kernel, (unsigned)std::min<int64_t>(grid_for(n + 1, 256), 152 * 8), 256, 0, s, a->rowptr, a->colidx,
+         a->m, a->n, a->nnz, bad, steps);
+}
+
 // Checks one CSR on the device; the error bits are or-ed into *bad.
 vmo_status validate_csr_async(const vmo_csr* a, int32_t* bad, cudaStream_t s) {
   if (!a || a->m < 0 || a->n < 0 || a->nnz < 0) return invalid("csr: negative size or null");
   if (!a->rowptr || (a->nnz > 0 && !a->colidx)) return invalid("csr: null pointer");
   if (a->nnz > INT32_MAX) return unsupported("csr: more than 2^31-1 nonzeros");
-  int64_t n = std::max<int64_t>(a->m, a->nnz);
-  launch(validate_csr_kernel, grid_for(n + 1, 256), 256, 0, s, a->rowptr, a->colidx, a->m, a->n, a->nnz, bad);
+  validate_launch(a, bad, nullptr, s);
   VMO_LAUNCHED("validate_csr");
   return VMO_OK;
 }
 
-vmo_status validate_csr(const vmo_csr* a, cudaStream_t s, Scratch& sc) {
+vmo_status validate_csr(const vmo_csr* a, bool* ascending, cudaStream_t s, Scratch& sc) {
   if (!a || a->m < 0 || a->n < 0 || a->nnz < 0) return invalid("csr: negative size or null");
   if (!a->rowptr || (a->nnz > 0 && !a->colidx)) return invalid("csr: null pointer");
   if (a->nnz > INT32_MAX) return unsupported("csr: more than 2^31-1 nonzeros");
-  int32_t* bad;
-  VMO_TRY(sc.alloc(&bad, 1));
-  VMO_CUDA(cudaMemsetAsync(bad, 0, 4, s));
-  int64_t n = std::max<int64_t>(a->m, a->nnz);
-  launch(validate_csr_kernel, grid_for(n + 1, 256), 256, 0, s, a->rowptr, a->colidx, a->m, a->n, a->nnz, bad);
+  int32_t* bad;  // error bits, steps
+  VMO_TRY(sc.alloc(&bad, 3));
+  VMO_CUDA(cudaMemsetAsync(bad, 0, 12, s));
+  validate_launch(a, bad, bad + 1, s);
   VMO_LAUNCHED("validate_csr");
-  int32_t h = 0;
-  VMO_CUDA(cudaMemcpyAsync(&h, bad, 4, cudaMemcpyDeviceToHost, s));
+  int32_t hb[3] = {0, 0, 0};
+  VMO_CUDA(cudaMemcpyAsync(hb, bad, 12, cudaMemcpyDeviceToHost, s));
   VMO_CUDA(cudaStreamSynchronize(s));
+  const int32_t h = hb[0];
   if (h & 2) return invalid("csr: rowptr[0] != 0 or rowptr[m] != nnz");
   if (h & 1) return invalid("csr: rowptr not monotone");
   if (h & 4) return invalid("csr: column index out of range");
+  *ascending = hb[1] == hb[2];
+  return VMO_OK;
+}
+
+__global__ void fg_vnets_kernel(const int32_t* rptr, const int32_t* cidx, int32_t m, int32_t* vtx_ptr, int32_t* vnets);
+__global__ void fg_nets_kernel(const int32_t* rptr, int32_t m, const int32_t* cptr, const int32_t* cpins, int32_t n,
+                               int64_t u, int32_t* net_ptr, int32_t* pins);
+
+// Entries of a pattern with ascending rows in column order: their entry
+// numbers (order) and rows (by entry number), and the column starts + add in
+// ptr (n + 1).
+static vmo_status column_order(const vmo_csr* a, int32_t add, int32_t* ptr, uint32_t** order, int32_t** row,
+                               cudaStream_t s, Scratch& sc) {
+  const int64_t nnz = a->nnz;
+  uint32_t *k1, *k2, *v1;
+  VMO_TRY(sc.alloc(&k1, (size_t)std::max<int64_t>(nnz, 1)));
+  VMO_TRY(sc.alloc(&k2, (size_t)std::max<int64_t>(nnz, 1)));
+  VMO_TRY(sc.alloc(&v1, (size_t)std::max<int64_t>(nnz, 1)));
+  VMO_TRY(sc.alloc(order, (size_t)std::max<int64_t>(nnz, 1)));
+  VMO_TRY(sc.alloc(row, (size_t)std::max<int64_t>(nnz, 1)));
+  if (nnz > 0) {
+    launch(entry_rows_kernel, grid_for(nnz, kRowTile), 256, 0, s, a->rowptr, a->colidx, a->m, nnz, k1, v1, *row);
+    VMO_LAUNCHED("entry_rows");
+    VMO_TRY(radix_sort_u32(k1, v1, k2, *order, nnz, bits_for((uint64_t)std::max(a->n - 1, 0)), s, sc));
+  }
+  launch(column_starts_kernel, grid_for((int64_t)a->n + 1, 256), 256, 0, s, k2, nnz, a->n, add, ptr);
+  VMO_LAUNCHED("column_starts");
+  return VMO_OK;
+}
+
+// Models of a pattern with strictly ascending rows (see the head of the
+// file); *done is false for a symmetric model of an unsymmetric pattern.
+static vmo_status build_ascending(const vmo_csr* a, vmo_model model, vmo_hg_s* h, bool* done, cudaStream_t s,
+                                  Scratch& sc) {
+  const int32_t m = a->m, n = a->n;
+  const int64_t nnz = a->nnz, cap = std::max<int64_t>(nnz, 1);
+  const unsigned ge = grid_for(nnz, 256);
+  uint32_t* order;
+  int32_t* row;
+  *done = true;
+  if (model == VMO_SYMMETRIC) {
+    int32_t *dpre, *rpre, *missing;
+    VMO_TRY(sc.alloc(&dpre, (size_t)m + 1));
+    VMO_TRY(sc.alloc(&rpre, (size_t)m + 1));
+    VMO_TRY(sc.alloc(&missing, 1));
+    VMO_CUDA(cudaMemsetAsync(missing, 0, 4, s));
+    if (m > 0) {
+      launch(row_parts_kernel, grid_for(m, 256), 256, 0, s, a->rowptr, a->colidx, m, dpre, rpre);
+      VMO_LAUNCHED("row_parts");
+    }
+    VMO_TRY(scan_exclusive<int32_t>(dpre, dpre, m, dpre + m, s, sc));
+    VMO_TRY(scan_exclusive<int32_t>(rpre, rpre, m, rpre + m, s, sc));
+    int32_t diag = 0, right = 0;
+    VMO_CUDA(cudaMemcpyAsync(&diag, dpre + m, 4, cudaMemcpyDeviceToHost, s));
+    VMO_CUDA(cudaMemcpyAsync(&right, rpre + m, 4, cudaMemcpyDeviceToHost, s));
+    VMO_CUDA(cudaStreamSynchronize(s));
+    const int64_t nadj = nnz - diag;
+    if (nadj != 2 * (int64_t)right) {  // more entries on one side of the diagonal
+      *done = false;
+      return VMO_OK;
+    }
+    h->k = m;
+    h->nadj = h->npins = h->nvnets = nadj;
+    h->l = right;
+    VMO_TRY(h->adj_ptr.resize((size_t)m + 1));
+    VMO_TRY(h->vtx_ptr.resize((size_t)m + 1));
+    VMO_TRY(h->adj.resize((size_t)std::max<int64_t>(nadj, 1)));
+    VMO_TRY(h->vnets.resize((size_t)std::max<int64_t>(nadj, 1)));
+    VMO_TRY(h->pins.resize((size_t)std::max<int64_t>(nadj, 1)));
+    VMO_TRY(h->net_ptr.resize((size_t)right + 1));
+    if (nnz > 0) {
+      int2* head;
+      VMO_TRY(sc.alloc(&head, (size_t)m + 1));
+      launch(row_heads_kernel, grid_for((int64_t)m + 1, 256), 256, 0, s, a->rowptr, dpre, m, head);
+      launch(symmetric_kernel, grid_for(nnz, kRowTile), 256, 0, s, a->rowptr, a->colidx, m, nnz, head, rpre,
+             h->adj.ptr, h->vnets.ptr, h->net_ptr.ptr, (int2*)h->pins.ptr, missing);
+      VMO_LAUNCHED("symmetric");
+    }
+    launch(symmetric_ptr_kernel, grid_for((int64_t)m + 1, 256), 256, 0, s, a->rowptr, dpre, m, right, h->adj_ptr.ptr,
+           h->vtx_ptr.ptr, h->net_ptr.ptr);
+    VMO_LAUNCHED("symmetric_ptr");
+    int32_t hm = 0;
+    VMO_CUDA(cudaMemcpyAsync(&hm, missing, 4, cudaMemcpyDeviceToHost, s));
+    VMO_CUDA(cudaStreamSynchronize(s));
+    *done = hm == 0;
+    return VMO_OK;
+  }
+  if (model == VMO_BIPARTITE) {
+    h->k = m + n;
+    h->nadj = h->npins = h->nvnets = 2 * nnz;
+    h->l = nnz;
+    VMO_TRY(h->adj_ptr.resize((size_t)h->k + 1));
+    VMO_TRY(h->vtx_ptr.resize((size_t)h->k + 1));
+    VMO_TRY(h->adj.resize((size_t)2 * cap));
+    VMO_TRY(h->vnets.resize((size_t)2 * cap));
+    VMO_TRY(h->pins.resize((size_t)2 * cap));
+    VMO_TRY(h->net_ptr.resize((size_t)nnz + 1));
+    VMO_TRY(column_order(a, (int32_t)nnz, h->adj_ptr.ptr + m, &order, &row, s, sc));
+    if (m > 0) VMO_CUDA(cudaMemcpyAsync(h->adj_ptr.ptr, a->rowptr, m * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+    VMO_CUDA(cudaMemcpyAsync(h->vtx_ptr.ptr, h->adj_ptr.ptr, ((size_t)h->k + 1) * sizeof(int32_t),
+                             cudaMemcpyDeviceToDevice, s));
+    launch(bipartite_rows_kernel, grid_for(nnz + 1, 256), 256, 0, s, a->colidx, row, m, nnz, h->adj.ptr, h->vnets.ptr,
+           h->net_ptr.ptr, (int2*)h->pins.ptr);
+    if (nnz > 0)
+      launch(column_entries_kernel, ge, 256, 0, s, order, row, nnz, h->adj.ptr + nnz, h->vnets.ptr + nnz);
+    VMO_LAUNCHED("bipartite");
+  } else if (model == VMO_ROWNET || model == VMO_COLNET) {
+    const bool rn = model == VMO_ROWNET;
+    h->k = rn ? n : m;
+    h->l = rn ? m : n;
+    h->npins = h->nvnets = nnz;
+    DevArray<int32_t>&rp = rn ? h->net_ptr : h->vtx_ptr, &ri = rn ? h->pins : h->vnets;
+    DevArray<int32_t>&cp = rn ? h->vtx_ptr : h->net_ptr, &ci = rn ? h->vnets : h->pins;
+    VMO_TRY(rp.resize((size_t)m + 1));
+    VMO_TRY(ri.resize((size_t)cap));
+    VMO_TRY(cp.resize((size_t)n + 1));
+    VMO_TRY(ci.resize((size_t)cap));
+    VMO_TRY(column_order(a, 0, cp.ptr, &order, &row, s, sc));
+    VMO_CUDA(cudaMemcpyAsync(rp.ptr, a->rowptr, ((size_t)m + 1) * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+    if (nnz > 0) {
+      VMO_CUDA(cudaMemcpyAsync(ri.ptr, a->colidx, nnz * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+      launch(column_entries_kernel, ge, 256, 0, s, order, row, nnz, ci.ptr, (int32_t*)nullptr);
+      VMO_LAUNCHED("column_entries");
+    }
+  } else {  // finegrain: vertices are the entries
+    if (2 * nnz > INT32_MAX) return unsupported("too many entries");
+    h->k = (int32_t)nnz;
+    h->l = (int64_t)m + n;
+    h->npins = h->nvnets = 2 * nnz;
+    VMO_TRY(h->vtx_ptr.resize((size_t)nnz + 1));
+    VMO_TRY(h->vnets.resize((size_t)2 * cap));
+    VMO_TRY(h->net_ptr.resize((size_t)m + n + 1));
+    VMO_TRY(h->pins.resize((size_t)2 * cap));
+    int32_t* cptr;
+    VMO_TRY(sc.alloc(&cptr, (size_t)n + 1));
+    VMO_TRY(column_order(a, 0, cptr, &order, &row, s, sc));
+    VMO_CUDA(cudaMemsetAsync(h->vtx_ptr.ptr, 0, sizeof(int32_t), s));
+    if (m > 0) launch(fg_vnets_kernel, grid_for(m, 256), 256, 0, s, a->rowptr, a->colidx, m, h->vtx_ptr.ptr, h->vnets.ptr);
+    const int64_t span = std::max<int64_t>(std::max<int64_t>(nnz, (int64_t)m + 1), (int64_t)n);
+    launch(fg_nets_kernel, grid_for(span, 256), 256, 0, s, a->rowptr, m, cptr, (const int32_t*)order, n, nnz,
+           h->net_ptr.ptr, h->pins.ptr);
+    VMO_LAUNCHED("finegrain");
+  }
+  VMO_CUDA(cudaStreamSynchronize(s));
   return VMO_OK;
 }
 
@@ -326,16 +670,25 @@ __global__ void fg_nets_kernel(const int32_t* __restrict__ rptr, int32_t m, cons
 
 vmo_status build_model(const vmo_csr* a, vmo_model model, vmo_hg_s* h, cudaStream_t s) {
   Scratch sc(s);
-  VMO_TRY(validate_csr(a, s, sc));
+  bool ascending = false;
+  VMO_TRY(validate_csr(a, &ascending, s, sc));
   const int32_t m = a->m, n = a->n;
   const int64_t nnz = a->nnz;
   h->model = model;
   h->m = m;
   h->n = n;
+  if (model == VMO_SYMMETRIC && m != n) return invalid("symmetric model needs a square pattern");
   if (model == VMO_SYMMETRIC || model == VMO_BIPARTITE) {
-    if (model == VMO_SYMMETRIC && m != n) return invalid("symmetric model needs a square pattern");
+    if ((model == VMO_SYMMETRIC ? (int64_t)m : (int64_t)m + n) > INT32_MAX / 2) return unsupported("too many vertices");
+  }
+  if (model == VMO_FINEGRAIN && (int64_t)m + n > INT32_MAX) return unsupported("too many nets");
+  if (ascending && model >= VMO_SYMMETRIC && model <= VMO_FINEGRAIN && (model != VMO_BIPARTITE || 2 * nnz <= INT32_MAX)) {
+    bool done = false;
+    VMO_TRY(build_ascending(a, model, h, &done, s, sc));
+    if (done) return VMO_OK;
+  }
+  if (model == VMO_SYMMETRIC || model == VMO_BIPARTITE) {
     int64_t K = (model == VMO_SYMMETRIC) ? m : (int64_t)m + n;
-    if (K > INT32_MAX / 2) return unsupported("too many vertices");
     h->k = (int32_t)K;
     uint64_t* keys;
     VMO_TRY(sc.alloc(&keys, (size_t)std::max<int64_t>(2 * nnz, 1)));
@@ -403,7 +756,6 @@ vmo_status build_model(const vmo_csr* a, vmo_model model, vmo_hg_s* h, cudaStrea
     return VMO_OK;
   }
   if (model == VMO_FINEGRAIN) {
-    if ((int64_t)m + n > INT32_MAX) return unsupported("too many nets");
     uint64_t* keys;
     VMO_TRY(sc.alloc(&keys, (size_t)std::max<int64_t>(nnz, 1)));
     if (nnz > 0) {
