@@ -13,6 +13,7 @@ namespace vmo {
 static thread_local std::string g_last_error;
 thread_local cudaStream_t g_devarray_stream = nullptr;
 thread_local bool g_devarray_async = false;
+thread_local cudaMemPool_t g_devarray_pool = nullptr;
 thread_local bool g_pdl = false;
 
 void set_error(const std::string& msg) { g_last_error = msg; }
@@ -112,6 +113,8 @@ vmo_status cut_size(const vmo_hg_s* h, const int32_t* part, int32_t nparts, int6
 namespace {
 
 std::once_flag g_pool_once;
+std::mutex g_handle_pool_mu;
+std::vector<std::pair<int, cudaMemPool_t>> g_handle_pools;  // one per device used
 
 // Device present; stream-ordered pool keeps freed scratch for reuse.
 vmo_status ensure_device() {
@@ -181,7 +184,7 @@ vmo_status run_layout(vmo_hg_s* h, const vmo_params* p, float4* x, bool given, c
   if (given || !graph) {
     LevelBatch lb;
     VMO_TRY(single_batch(h, p->d, p->occupancy, lb, s));
-    if (given) return layout_level(lb, o, x, o.iters, -1.0f, nullptr, nullptr, s, sc);
+    if (given) return layout_level(lb, o, x, o.iters, -1.0f, nullptr, nullptr, nullptr, s, sc);
     std::vector<uint64_t> seeds{p->seed};
     return layout_multilevel(lb, o, seeds, p->match_rounds, p->coarse_min, false, x, s, sc);
   }
@@ -249,6 +252,7 @@ vmo_status run_order(vmo_hg_s* h, const float* coords, const vmo_params* p, int 
   if (h->model != VMO_SYMMETRIC && h->model != VMO_BIPARTITE)
     return unsupported("ordering needs a graph model (symmetric or bipartite, Algorithm 7)");
   if (coords && !aligned16(coords)) return invalid("coords must be 16-byte aligned");
+  DevArrayStreamScope scope(s);
   Scratch sc(s);
   const int64_t k = h->k;
   int32_t* mu = nullptr;
@@ -350,6 +354,27 @@ __global__ void k_fill_f32(float* __restrict__ a, int64_t n, float v) {
 
 }  // namespace
 
+cudaMemPool_t handle_pool() {
+  std::lock_guard<std::mutex> lk(g_handle_pool_mu);
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  for (auto& p : g_handle_pools)
+    if (p.first == dev) return p.second;
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t pool = nullptr;
+  uint64_t keep = kHandlePoolKeep;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  g_handle_pools.emplace_back(dev, pool);
+  return pool;
+}
+
 vmo_status ensure_device_public() { return ensure_device(); }
 vmo_status check_params_public(const vmo_params* p) { return check_params(p); }
 
@@ -385,8 +410,11 @@ vmo_status vmo_build_hypergraph(const vmo_csr* a, vmo_model model, const float* 
   VMO_TRY(ensure_device());
   if (model < VMO_SYMMETRIC || model > VMO_FINEGRAIN) return invalid("unknown model");
   cudaStream_t s = (cudaStream_t)stream;
-  std::unique_ptr<vmo_hg_s> h(new vmo_hg_s());
+  // the handle's arrays are freed in vmo_destroy, whatever stream built them
+  std::unique_ptr<vmo_hg_s, void (*)(vmo_hg)> h(new vmo_hg_s(), vmo_destroy);
   cudaGetDevice(&h->device);
+  cudaMemPool_t pool = handle_pool();
+  std::unique_ptr<DevArrayStreamScope> scope(pool ? new DevArrayStreamScope(s, pool) : nullptr);
   VMO_TRY(build_model(a, model, h.get(), s));
   if (vertex_weight) {
     VMO_TRY(h->weight.resize(std::max<int32_t>(h->k, 1)));
@@ -432,6 +460,7 @@ vmo_status vmo_init_coords(int32_t k, int32_t d, uint64_t seed, float* coords, v
   if (d < 2 || d > 4) return unsupported("d must be 2, 3 or 4");
   if (k > 0 && (!coords || !aligned16(coords))) return invalid("coords null or not 16-byte aligned");
   cudaStream_t s = (cudaStream_t)stream;
+  DevArrayStreamScope scope(s);
   LevelBatch lb;
   lb.K = k;
   lb.P = 1;
@@ -453,6 +482,7 @@ vmo_status vmo_layout(vmo_hg hg, const vmo_params* params, float* coords, int32_
   if (!hg) return invalid("handle is null");
   if (hg->k > 0 && (!coords || !aligned16(coords))) return invalid("coords null or not 16-byte aligned");
   cudaStream_t s = (cudaStream_t)stream;
+  DevArrayStreamScope scope(s);
   Scratch sc(s);
   VMO_TRY(run_layout(hg, params, (float4*)coords, use_given_init != 0, s, sc));
   VMO_CUDA(cudaStreamSynchronize(s));
@@ -468,12 +498,13 @@ vmo_status vmo_layout_step(vmo_hg hg, const vmo_params* params, float* coords, f
   if (hg->k > 0 && (!coords || !aligned16(coords))) return invalid("coords null or not 16-byte aligned");
   if (y_out && !aligned16(y_out)) return invalid("y_out must be 16-byte aligned");
   cudaStream_t s = (cudaStream_t)stream;
+  DevArrayStreamScope scope(s);
   Scratch sc(s);
   LevelBatch lb;
   VMO_TRY(single_batch(hg, params->d, params->occupancy, lb, s));
   if (levels_out) *levels_out = lb.L.empty() ? 1 : lb.L[0];
   LayoutOptions o = options_of(params);
-  VMO_TRY(layout_level(lb, o, (float4*)coords, 1, step, (float4*)y_out, keys_out, s, sc));
+  VMO_TRY(layout_level(lb, o, (float4*)coords, 1, step, (float4*)y_out, keys_out, nullptr, s, sc));
   VMO_CUDA(cudaStreamSynchronize(s));
   return VMO_OK;
 }
@@ -485,6 +516,7 @@ vmo_status vmo_coarsen(vmo_hg hg, const vmo_params* params, int32_t* mate, int32
   if (!hg) return invalid("handle is null");
   if (hg->model != VMO_SYMMETRIC && hg->model != VMO_BIPARTITE) return unsupported("coarsening needs a graph model");
   cudaStream_t s = (cudaStream_t)stream;
+  DevArrayStreamScope scope(s);
   Scratch sc(s);
   LevelBatch lb;
   VMO_TRY(single_batch(hg, params->d, params->occupancy, lb, s));
@@ -532,6 +564,7 @@ vmo_status vmo_hierarchy_level(vmo_hg hg, const vmo_params* params, int32_t leve
                                int32_t* adj_ptr, int32_t* adj, float* acost, float* weight, int32_t* pi,
                                void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
+  DevArrayStreamScope scope(s);
   Scratch sc(s);
   LevelBatch lb;
   Hierarchy H;
@@ -561,6 +594,7 @@ vmo_status vmo_hierarchy_level(vmo_hg hg, const vmo_params* params, int32_t leve
 vmo_status vmo_hierarchy_prolong(vmo_hg hg, const vmo_params* params, int32_t level, const float* coarse, float* fine,
                                  void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
+  DevArrayStreamScope scope(s);
   Scratch sc(s);
   LevelBatch lb;
   Hierarchy H;
@@ -577,6 +611,7 @@ vmo_status vmo_hierarchy_prolong(vmo_hg hg, const vmo_params* params, int32_t le
 vmo_status vmo_hierarchy_step(vmo_hg hg, const vmo_params* params, int32_t level, float* coords, float step,
                               float* y_out, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
+  DevArrayStreamScope scope(s);
   Scratch sc(s);
   LevelBatch lb;
   Hierarchy H;
@@ -585,7 +620,7 @@ vmo_status vmo_hierarchy_step(vmo_hg hg, const vmo_params* params, int32_t level
   LevelBatch& L = *H.levels[level];
   if (L.K > 0 && (!coords || !aligned16(coords))) return invalid("coords null or not 16-byte aligned");
   if (y_out && !aligned16(y_out)) return invalid("y_out must be 16-byte aligned");
-  VMO_TRY(layout_level(L, options_of(params), (float4*)coords, 1, step, (float4*)y_out, nullptr, s, sc));
+  VMO_TRY(layout_level(L, options_of(params), (float4*)coords, 1, step, (float4*)y_out, nullptr, nullptr, s, sc));
   VMO_CUDA(cudaStreamSynchronize(s));
   return VMO_OK;
 }
@@ -724,7 +759,20 @@ vmo_status vmo_stats_get(vmo_stats* out) {
   return VMO_OK;
 }
 
-void vmo_destroy(vmo_hg hg) { delete hg; }
+// Waits for the device, as freeing each array with cudaFree would: the arrays
+// may be in use on any stream (vmo_hg_arrays).
+void vmo_destroy(vmo_hg hg) {
+  if (!hg) return;
+  int dev = hg->device;
+  cudaGetDevice(&dev);
+  if (dev != hg->device) cudaSetDevice(hg->device);
+  cudaDeviceSynchronize();
+  for (auto* a : {&hg->adj_ptr, &hg->adj, &hg->net_ptr, &hg->pins, &hg->vtx_ptr, &hg->vnets}) a->astream = nullptr;
+  hg->weight.astream = nullptr;
+  const int own = hg->device;
+  delete hg;
+  if (dev != own) cudaSetDevice(dev);
+}
 
 const char* vmo_status_string(vmo_status s) {
   switch (s) {

@@ -13,7 +13,7 @@
 // entry numbers (two passes instead of four of 64-bit keys), and a symmetric
 // pattern is its own adjacency, with every entry's mirror found by a binary
 // search in its row.  27-point mesh of 10^6 rows in random numbering, symmetric
-// model with copies of its arrays: 7.6 -> 2.4 ms; 400k x 300k bipartite model: 2.1 -> 1.2 ms.
+// model with copies of its arrays: 7.6 -> 1.8 ms; 400k x 300k bipartite model: 2.1 -> 1.2 ms.
 #include <algorithm>
 
 #include "vmo_internal.cuh"
@@ -424,16 +424,6 @@ static void validate_launch(const vmo_csr* a, int32_t* bad, int32_t* steps, cuda
   const int64_t n = std::max<int64_t>(a->m, (a->nnz + 3) / 4);
   launch(validate_csr_kernel, (unsigned)std::min<int64_t>(grid_for(n + 1, 256), 152 * 8), 256, 0, s, a->rowptr, a->colidx,
          a->m, a->n, a->nnz, bad, steps);
-}
-
-// Checks one CSR on the device; the error bits are or-ed into *bad.
-vmo_status validate_csr_async(const vmo_csr* a, int32_t* bad, cudaStream_t s) {
-  if (!a || a->m < 0 || a->n < 0 || a->nnz < 0) return invalid("csr: negative size or null");
-  if (!a->rowptr || (a->nnz > 0 && !a->colidx)) return invalid("csr: null pointer");
-  if (a->nnz > INT32_MAX) return unsupported("csr: more than 2^31-1 nonzeros");
-  validate_launch(a, bad, nullptr, s);
-  VMO_LAUNCHED("validate_csr");
-  return VMO_OK;
 }
 
 vmo_status validate_csr(const vmo_csr* a, bool* ascending, cudaStream_t s, Scratch& sc) {

@@ -1031,19 +1031,21 @@ __global__ void __launch_bounds__(kBlock) k_attract(const int32_t* __restrict__ 
   y[v] = make_float4(0.5f * a[0], 0.5f * a[1], 0.5f * a[2], 0.5f * a[3]);
 }
 
-__global__ void k_degree_class(const int32_t* __restrict__ adj_ptr, int64_t K, int32_t* __restrict__ mid,
-                               int32_t* __restrict__ heavy) {
+// Degree class of every row, counted by one scan: 1 medium, 2^32 heavy.
+__global__ void k_degree_class(const int32_t* __restrict__ adj_ptr, int64_t K, uint64_t* __restrict__ cls) {
   int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= K) return;
-  int32_t deg = adj_ptr[v + 1] - adj_ptr[v];
-  mid[v] = (deg > kLightMax && deg <= kWarpMax) ? 1 : 0;
-  heavy[v] = deg > kWarpMax ? 1 : 0;
+  const int32_t deg = adj_ptr[v + 1] - adj_ptr[v];
+  cls[v] = deg <= kLightMax ? 0ull : (deg <= kWarpMax ? 1ull : 1ull << 32);
 }
 
-__global__ void k_compact_flags(const int32_t* __restrict__ flag, const int32_t* __restrict__ pos, int64_t K,
-                                int32_t* __restrict__ out) {
+__global__ void k_class_lists(const uint64_t* __restrict__ cls, const uint64_t* __restrict__ pos, int64_t K,
+                              int32_t* __restrict__ mid, int32_t* __restrict__ heavy) {
   int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v < K && flag[v]) out[pos[v]] = (int32_t)v;
+  if (v >= K) return;
+  const uint64_t c = cls[v];
+  if (c == 1) mid[(uint32_t)pos[v]] = (int32_t)v;
+  else if (c) heavy[pos[v] >> 32] = (int32_t)v;
 }
 
 // Net centres z_j of general nets (Algorithm 4).
@@ -2247,11 +2249,18 @@ __global__ void k_round_w(const double* __restrict__ wd, int64_t n, float* __res
   if (i < n) w[i] = (float)wd[i];
 }
 
-// Problem of every item of a table whose problems start at base.
-__global__ void k_fill_prob(const int64_t* __restrict__ base, int P, int64_t n, int32_t* __restrict__ out) {
+// Problem of every item of four tables whose problems start at base[t][0..P].
+struct ProbMaps {
+  int32_t* out[4];
+  int64_t n[4];
+};
+
+__global__ void k_fill_prob(const int64_t* __restrict__ base, int P, ProbMaps maps) {
   int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= n) return;
-  out[v] = find_problem(base, P, v);
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    if (v < maps.n[t]) maps.out[t][v] = find_problem(base + (int64_t)t * (P + 1), P, v);
+  }
 }
 
 __global__ void k_set_last(int32_t* ptr, int64_t n, const int32_t* total) { ptr[n] = *total; }
@@ -2291,29 +2300,24 @@ static vmo_status classify_degrees(LevelBatch& lb, cudaStream_t s) {
   lb.n_mid = lb.n_heavy = 0;
   if (!lb.adj_ptr || lb.K == 0) return VMO_OK;
   Scratch sc(s);
-  int32_t *fm, *fh, *pm, *ph, *tm, *th;
-  VMO_TRY(sc.alloc(&fm, lb.K));
-  VMO_TRY(sc.alloc(&fh, lb.K));
-  VMO_TRY(sc.alloc(&pm, lb.K));
-  VMO_TRY(sc.alloc(&ph, lb.K));
-  VMO_TRY(sc.alloc(&tm, 1));
-  VMO_TRY(sc.alloc(&th, 1));
-  launch(k_degree_class, grid_for(lb.K, kBlock), kBlock, 0, s, lb.adj_ptr, lb.K, fm, fh);
+  uint64_t *cls, *pos, *tot;
+  VMO_TRY(sc.alloc(&cls, lb.K));
+  VMO_TRY(sc.alloc(&pos, lb.K));
+  VMO_TRY(sc.alloc(&tot, 1));
+  launch(k_degree_class, grid_for(lb.K, kBlock), kBlock, 0, s, lb.adj_ptr, lb.K, cls);
   VMO_LAUNCHED("degree_class");
-  VMO_TRY(scan_exclusive<int32_t>(fm, pm, lb.K, tm, s, sc));
-  VMO_TRY(scan_exclusive<int32_t>(fh, ph, lb.K, th, s, sc));
-  int32_t h[2] = {0, 0};
-  VMO_CUDA(cudaMemcpyAsync(&h[0], tm, 4, cudaMemcpyDeviceToHost, s));
-  VMO_CUDA(cudaMemcpyAsync(&h[1], th, 4, cudaMemcpyDeviceToHost, s));
-  VMO_CUDA(cudaStreamSynchronize(s));
-  lb.n_mid = h[0];
-  lb.n_heavy = h[1];
+  VMO_TRY(scan_exclusive<uint64_t>(cls, pos, lb.K, tot, s, sc));
+  uint64_t h = 0;
+  VMO_CUDA(cudaMemcpyAsync(&h, tot, 8, cudaMemcpyDeviceToHost, s));
+  VMO_CUDA(cudaStreamSynchronize(s));  // also: the host tables of level_setup have been copied
+  lb.n_mid = (int64_t)(h & 0xffffffffu);
+  lb.n_heavy = (int64_t)(h >> 32);
   VMO_TRY(lb.mid_list.resize(std::max<int64_t>(lb.n_mid, 1)));
   VMO_TRY(lb.heavy_list.resize(std::max<int64_t>(lb.n_heavy, 1)));
-  if (lb.n_mid) launch(k_compact_flags, grid_for(lb.K, kBlock), kBlock, 0, s, fm, pm, lb.K, lb.mid_list.ptr);
-  if (lb.n_heavy) launch(k_compact_flags, grid_for(lb.K, kBlock), kBlock, 0, s, fh, ph, lb.K, lb.heavy_list.ptr);
-  VMO_LAUNCHED("compact_flags");
-  VMO_CUDA(cudaStreamSynchronize(s));
+  if (h) {
+    launch(k_class_lists, grid_for(lb.K, kBlock), kBlock, 0, s, cls, pos, lb.K, lb.mid_list.ptr, lb.heavy_list.ptr);
+    VMO_LAUNCHED("class_lists");
+  }
   return VMO_OK;
 }
 
@@ -2378,17 +2382,15 @@ vmo_status level_setup(LevelBatch& lb, int d, int occ, cudaStream_t s) {
   VMO_CUDA(cudaMallocAsync((void**)&db, base.size() * sizeof(int64_t), s));
   g_device_allocs.fetch_add(1, std::memory_order_relaxed);
   VMO_CUDA(cudaMemcpyAsync(db, base.data(), base.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-  int32_t* maps[4] = {lb.vprob.ptr, lb.wprob.ptr, lb.wprob2.ptr, lb.bprob.ptr};
-  for (int q = 0; q < 4; ++q) {
-    const int64_t n = base[(size_t)q * (P + 1) + P];
-    if (n > 0) launch(k_fill_prob, grid_for(n, kBlock), kBlock, 0, s, db + (size_t)q * (P + 1), P, n, maps[q]);
-  }
+  ProbMaps maps{{lb.vprob.ptr, lb.wprob.ptr, lb.wprob2.ptr, lb.bprob.ptr}, {lb.K, wb[P], wb2[P], bk[P]}};
+  const int64_t items = std::max(std::max(lb.K, wb[P]), std::max(wb2[P], bk[P]));
+  if (items > 0) launch(k_fill_prob, grid_for(items, kBlock), kBlock, 0, s, db, P, maps);
   VMO_LAUNCHED("fill_prob");
   VMO_CUDA(cudaFreeAsync(db, s));
 
-  // host vectors must outlive the copies
-  VMO_CUDA(cudaStreamSynchronize(s));
-  return classify_degrees(lb, s);
+  VMO_TRY(classify_degrees(lb, s));
+  if (!lb.adj_ptr || lb.K == 0) VMO_CUDA(cudaStreamSynchronize(s));  // host tables must outlive the copies
+  return VMO_OK;
 }
 
 vmo_status init_coords_level(LevelBatch& lb, int d, const uint64_t* seeds_dev, float4* x, const int32_t* start_dev,
@@ -2401,10 +2403,11 @@ vmo_status init_coords_level(LevelBatch& lb, int d, const uint64_t* seeds_dev, f
 
 constexpr int kGraphMinIters = 8;
 
-// Streams of one layout call: `side` for the attraction (fork / join events
-// per step) and `main` for the steps when they are replayed from a graph
-// (capture needs a stream of its own: the caller's may be the legacy stream);
-// destroyed in stream order when the call returns.
+// Streams of one layout call, shared by its levels (made for each of 22 levels
+// they cost 2 ms of the 64^3 grid's layout): `side` for the attraction (fork /
+// join events per step) and `main` for the steps when they are replayed from a
+// graph (capture needs a stream of its own: the caller's may be the legacy
+// stream); destroyed in stream order when the call returns.
 struct SideStream {
   cudaStream_t stream = nullptr, main = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr, start = nullptr, done = nullptr;
@@ -2431,6 +2434,21 @@ struct SideStream {
   ~SideStream() { release(); }
 };
 
+struct LayoutContext {
+  SideStream streams;
+  float* scale_tab = nullptr;  // decay^t of the layout's steps
+};
+
+// Step lengths s0 * decay^t: decay^t as the running double product, rounded to
+// fp32 (a table read by the step kernel at the level's step counter, which
+// k_keys advances).
+static vmo_status make_scale_tab(const LayoutOptions& o, int iters, float** tab, cudaStream_t s, Scratch& sc) {
+  VMO_TRY(sc.alloc(tab, std::max(iters, 1)));
+  launch(k_scale_tab, 1, 1, 0, s, iters, (double)o.decay, *tab);
+  VMO_LAUNCHED("scale_tab");
+  return VMO_OK;
+}
+
 // Points a Scratch at another stream for a scope (its allocations and frees
 // then follow that stream's order).
 struct ScratchOnStream {
@@ -2441,7 +2459,7 @@ struct ScratchOnStream {
 };
 
 vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int iters, float step_override,
-                        float4* y_out, uint32_t* keys_out, cudaStream_t s, Scratch& sc) {
+                        float4* y_out, uint32_t* keys_out, LayoutContext* ctx, cudaStream_t s, Scratch& sc) {
   const int64_t K = lb.K;
   const int P = lb.P;
   const int d = o.d;
@@ -2502,20 +2520,17 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   launch(k_bbox_reset, grid_for(16 * P, kBlock), kBlock, 0, s, bb, 16 * P);
   VMO_LAUNCHED("bbox_reset");
   const float kappa = d == 2 ? 1.0f : (float)(d - 2);
-  // step lengths s0 * decay^t: decay^t as the running double product, rounded
-  // to fp32 (a table read by the step kernel at the level's step counter,
-  // which k_keys advances)
-  float* scale_tab;
+  float* scale_tab = ctx ? ctx->scale_tab : nullptr;
   int32_t* tctr;
-  VMO_TRY(sc.alloc(&scale_tab, iters));
+  if (!scale_tab) VMO_TRY(make_scale_tab(o, iters, &scale_tab, s, sc));
   VMO_TRY(sc.alloc(&tctr, 1));
-  launch(k_scale_tab, 1, 1, 0, s, iters, (double)o.decay, scale_tab);
-  VMO_LAUNCHED("scale_tab");
   VMO_CUDA(cudaMemsetAsync(tctr, 0xFF, sizeof(int32_t), s));  // -1: k_keys advances it at every step
   vmo_status st = VMO_OK;
-  SideStream ss;  // attraction stream of this call (none if it cannot be created)
-  cudaStream_t side = ss.stream;
-  cudaEvent_t ev_fork = ss.fork, ev_join = ss.join;
+  // streams: the layout's, the level's own, or none for a few steps (making them
+  // costs more than the overlap of so few gives) or if they cannot be made
+  std::unique_ptr<SideStream> own(!ctx && iters >= kGraphMinIters ? new SideStream : nullptr);
+  SideStream* ss = ctx ? &ctx->streams : own.get();
+  const cudaStream_t side = ss ? ss->stream : nullptr;
   dispatch_d(d, [&](auto DC) {
     constexpr int D = decltype(DC)::value;
     launch(k_bbox<D>, grid_for(K, kBlock), kBlock, 0, s, x, K, lb.vprob.ptr, bb);
@@ -2532,8 +2547,8 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
       // with the binning below, and joins before the step kernel
       cudaStream_t as = side ? side : ms;
       if (side) {
-        cudaEventRecord(ev_fork, ms);
-        cudaStreamWaitEvent(side, ev_fork, 0);
+        cudaEventRecord(ss->fork, ms);
+        cudaStreamWaitEvent(side, ss->fork, 0);
       }
       if (lb.adj_ptr) {
         const int64_t mid_blocks = (lb.n_mid * kMidLanes + kBlock - 1) / kBlock;
@@ -2545,7 +2560,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
       } else {
         cudaMemsetAsync(yatt, 0, K * sizeof(float4), as);
       }
-      if (side) cudaEventRecord(ev_join, side);
+      if (side) cudaEventRecord(ss->join, side);
       if (bin1) {
         launch(k_bin_small<D>, (unsigned)P, kSortThreads, sizeof(BinSmem), ms, x, lb.w, lb.prob.ptr, cur, nxt, tctr,
                keys_out && t == 0 ? keys : nullptr, svals, xs, ws, scell, cst, XP, St, Wt, CP);
@@ -2568,7 +2583,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
           launch(k_cells<D>, (unsigned)lb.bricks, kCellsBlock, 0, ms, lb.bprob.ptr, lb.prob.ptr, xs, ws, cst, St, Wt,
                  CP, done);
       }
-      if (side) cudaStreamWaitEvent(ms, ev_join, 0);
+      if (side) cudaStreamWaitEvent(ms, ss->join, 0);
       const bool timed = stats_timing();
       if (timed) stats_time_begin(ms);
       unsigned long long* icount = stats_interaction_counter();
@@ -2596,14 +2611,14 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
     // Steps are replayed from a CUDA graph of two steps (even and odd parity)
     // when the level runs plain steps; the host then issues one graph launch
     // per two steps instead of ~20 kernel launches per step.
-    const bool graphs = ss.main && iters >= kGraphMinIters && !y_out && !keys_out && step_override <= 0.0f &&
+    const bool graphs = ss && ss->main && iters >= kGraphMinIters && !y_out && !keys_out && step_override <= 0.0f &&
                         !stats_timing() && !stats_interaction_counter();
     int t = 0;
     if (graphs) {
       // the steps run on the call's own stream, joined back to s at the end
-      cudaEventRecord(ss.start, s);
-      cudaStreamWaitEvent(ss.main, ss.start, 0);
-      ms = ss.main;
+      cudaEventRecord(ss->start, s);
+      cudaStreamWaitEvent(ss->main, ss->start, 0);
+      ms = ss->main;
     }
     ScratchOnStream on(sc, ms);  // scratch of a step follows the stream of the step
     if (graphs) {
@@ -2638,8 +2653,8 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
     }
     for (; t < iters && st == VMO_OK; ++t) st = step(t);
     if (ms != s) {
-      cudaEventRecord(ss.done, ms);
-      cudaStreamWaitEvent(s, ss.done, 0);
+      cudaEventRecord(ss->done, ms);
+      cudaStreamWaitEvent(s, ss->done, 0);
     }
   });
   return st;
@@ -2900,13 +2915,15 @@ vmo_status layout_multilevel(LevelBatch& fine, const LayoutOptions& o, const std
   VMO_CUDA(cudaMemcpyAsync(sd_d, seed_all.data(), tb[nl] * 8, cudaMemcpyHostToDevice, s));
   VMO_CUDA(cudaStreamSynchronize(s));  // the host tables must outlive the copies
   // layout from the coarsest level down
+  LayoutContext ctx;
+  if (o.iters > 0) VMO_TRY(make_scale_tab(o, o.iters, &ctx.scale_tab, s, sc));
   float4* xc = nullptr;
   for (int j = nl - 1; j >= 0; --j) {
     LevelBatch& cur = *H.levels[j];
     float4* xj = (j == 0) ? x : nullptr;
     if (!xj) VMO_TRY(sc.alloc(&xj, std::max<int64_t>(cur.K, 1)));
     VMO_TRY(prolong_level_dev(H, j, o.d, xc, xj, st_d + tb[j], fc_d + tb[j], sd_d + tb[j], s));
-    VMO_TRY(layout_level(cur, o, xj, o.iters, -1.0f, nullptr, nullptr, s, sc));
+    VMO_TRY(layout_level(cur, o, xj, o.iters, -1.0f, nullptr, nullptr, &ctx, s, sc));
     xc = xj;
   }
   return VMO_OK;

@@ -76,8 +76,11 @@ vmo_status level_setup(LevelBatch& lb, int d, int occupancy, cudaStream_t s);
 // Runs `iters` steps of Algorithm 4 on a level.  x: device float4[K] in/out.
 // If step_override > 0 it is used as the step length of a single step and
 // y_out / keys_out (vertex order, may be null) receive the gradient and keys.
+// ctx: streams and step-length factors shared by the levels of a layout (null:
+// the level makes its own, and a call of a few steps takes no streams).
+struct LayoutContext;
 vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int iters, float step_override,
-                        float4* y_out, uint32_t* keys_out, cudaStream_t s, Scratch& sc);
+                        float4* y_out, uint32_t* keys_out, LayoutContext* ctx, cudaStream_t s, Scratch& sc);
 
 // Random initial layout of the problems of a level (all, or those with
 // start[p] != 0 when start_dev is given).  seeds_dev: device uint64[P].

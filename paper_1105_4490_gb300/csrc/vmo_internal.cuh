@@ -77,21 +77,31 @@ struct ScratchFrame {
 // DevArray uses cudaMalloc / cudaFree; inside a DevArrayStreamScope it takes
 // its memory from the stream-ordered pool on the scope's stream and returns it
 // on that stream, so threads working on different streams (the request
-// server's slots) never wait for each other in an allocation or a free.
+// server's slots) never wait for each other in an allocation or a free, and a
+// layout's levels cost no device-wide wait each (a dozen arrays a level). A
+// scope may name a pool: a handle's arrays come from one of their own that keeps
+// at most kHandlePoolKeep bytes of what was freed.
 extern std::atomic<uint64_t> g_device_allocs;
 extern thread_local cudaStream_t g_devarray_stream;
 extern thread_local bool g_devarray_async;
+extern thread_local cudaMemPool_t g_devarray_pool;  // null: the device's default pool
+constexpr uint64_t kHandlePoolKeep = uint64_t(1) << 30;
+cudaMemPool_t handle_pool();  // of the current device; null if it cannot be made
 
 struct DevArrayStreamScope {
   cudaStream_t prev_s;
   bool prev_a;
-  explicit DevArrayStreamScope(cudaStream_t s) : prev_s(g_devarray_stream), prev_a(g_devarray_async) {
+  cudaMemPool_t prev_p;
+  explicit DevArrayStreamScope(cudaStream_t s, cudaMemPool_t pool = nullptr)
+      : prev_s(g_devarray_stream), prev_a(g_devarray_async), prev_p(g_devarray_pool) {
     g_devarray_stream = s;
     g_devarray_async = true;
+    g_devarray_pool = pool;
   }
   ~DevArrayStreamScope() {
     g_devarray_stream = prev_s;
     g_devarray_async = prev_a;
+    g_devarray_pool = prev_p;
   }
 };
 
@@ -116,8 +126,10 @@ vmo_status DevArray<T>::resize(size_t n) {
   release();
   if (n == 0) n = 1;
   const bool as = g_devarray_async;
-  cudaError_t e = as ? cudaMallocAsync(reinterpret_cast<void**>(&ptr), n * sizeof(T), g_devarray_stream)
-                     : cudaMalloc(reinterpret_cast<void**>(&ptr), n * sizeof(T));
+  void** pp = reinterpret_cast<void**>(&ptr);
+  cudaError_t e = !as ? cudaMalloc(pp, n * sizeof(T))
+                  : g_devarray_pool ? cudaMallocFromPoolAsync(pp, n * sizeof(T), g_devarray_pool, g_devarray_stream)
+                                    : cudaMallocAsync(pp, n * sizeof(T), g_devarray_stream);
   if (e != cudaSuccess) {
     ptr = nullptr;
     (void)cudaGetLastError();
