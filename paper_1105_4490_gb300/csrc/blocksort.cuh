@@ -1,7 +1,6 @@
-// Block-level pieces shared by the device-wide radix sort (prims.cu) and the
-// one-block binning of small layout levels (layout.cu): warp and block scans,
-// and the stable LSD sort of one tile of at most kSortTile (key, value) pairs
-// held in shared memory.
+// Block-level pieces: warp and block scans (prims.cu, layout.cu, kmeans.cu) and
+// the radix sort's stable LSD sort of one tile of at most kSortTile (key,
+// value) pairs held in shared memory.
 #pragma once
 
 #include "vmo_internal.cuh"

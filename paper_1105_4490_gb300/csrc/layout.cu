@@ -392,15 +392,6 @@ __global__ void __launch_bounds__(kBlock) k_slots(const uint32_t* __restrict__ k
   slot[cst[prob[pb].fbase + pb + keys[v]] + arrival[v]] = (uint32_t)v;
 }
 
-// a[lo..hi) = v, with 16-byte stores over the aligned middle of the range
-// (long runs of empty cells between clusters of the layout).
-__device__ inline void fill_i32(int32_t* __restrict__ a, int64_t lo, int64_t hi, int32_t v) {
-  while (lo < hi && (((uintptr_t)(a + lo)) & 15u)) a[lo++] = v;
-  const int4 v4 = make_int4(v, v, v, v);
-  for (; lo + 4 <= hi; lo += 4) *reinterpret_cast<int4*>(a + lo) = v4;
-  while (lo < hi) a[lo++] = v;
-}
-
 // Sorted positions: the points of a cell by ascending vertex (a point's place
 // is the number of smaller ids in its cell: as many comparisons as the cell
 // has points, against 3^d cells of interactions per point in the step
@@ -736,157 +727,6 @@ __global__ void __launch_bounds__(kCellsBlock) k_cells(const int32_t* __restrict
   }
 }
 
-// One-block binning of a step for levels whose problems all have at most
-// kSortTile points and kBinCells finest cells: one block per problem stages
-// its points in shared memory, computes the keys (as k_keys), sorts (key,
-// local index) stably in shared memory (as the one-tile radix sort), gathers
-// (as k_gather, and writes the sorted vertex ids), sums the finest cells from
-// the staged points (as k_agg_finest: serially up to kCellSerial points, else
-// lane-strided with the xor tree) and every coarser level (agg_cell, a block
-// barrier between levels).  The arithmetic and the order of every sum are
-// those kernels', so the results are bit-identical, from one launch instead
-// of five or more.  The cell charges are read back by other threads of the
-// block after a barrier, so those pointers carry no __restrict__.  keys
-// (optional): the unsorted keys by vertex, as k_keys writes them.
-constexpr int kBinCells = 4096;
-
-struct BinSmem {
-  float4 xin[kSortTile];      // the problem's points by local index
-  float win[kSortTile];       // their weights (1 without weights)
-  int32_t cs[kBinCells + 1];  // cell start table (sorted positions)
-  TileSortSmem sort;
-};
-
-template <int D>
-__global__ void __launch_bounds__(kSortThreads) k_bin_small(
-    const float4* __restrict__ x, const float* __restrict__ w, const ProbDev* __restrict__ prob,
-    const uint32_t* __restrict__ bb, uint32_t* __restrict__ bb_next, int32_t* __restrict__ tctr,
-    uint32_t* __restrict__ keys, uint32_t* __restrict__ svals, float4* __restrict__ xs, float* __restrict__ ws,
-    uint32_t* __restrict__ scell, int32_t* __restrict__ cst, float4* __restrict__ XP, float4* St, float* Wt,
-    float4* CP) {
-  pdl_enter();
-  extern __shared__ __align__(16) unsigned char bin_raw[];
-  BinSmem& sm = *reinterpret_cast<BinSmem*>(bin_raw);
-  const int pb = blockIdx.x;
-  const ProbDev pr = prob[pb];
-  const int k = pr.k;
-  const int64_t vb = pr.vbase;
-  if (pb == 0 && threadIdx.x == 0) ++*tctr;  // the level's step
-  if (threadIdx.x < 8) bb_next[pb * 8 + threadIdx.x] = threadIdx.x < 4 ? 0xFFFFFFFFu : 0u;
-  float lo[D], s;
-  grid_frame<D>(bb, pb, pr.L, lo, &s);
-  {
-    // points, weights and keys by local index; a thread's loads issued first
-    float4 xv[kSortItems];
-    float wv[kSortItems];
-#pragma unroll
-    for (int j = 0; j < kSortItems; ++j) {
-      const int i = threadIdx.x + j * kSortThreads;
-      xv[j] = i < k ? x[vb + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-      wv[j] = (i < k && w) ? w[vb + i] : 1.0f;
-    }
-#pragma unroll
-    for (int j = 0; j < kSortItems; ++j) {
-      const int i = threadIdx.x + j * kSortThreads;
-      if (i < k) {
-        sm.xin[i] = xv[j];
-        sm.win[i] = wv[j];
-        int32_t c[D];
-        cell_of<D>(xv[j], lo, s, pr.L, c);
-        const uint32_t key = (uint32_t)rowmajor<D>(c, 1 << pr.L);
-        sm.sort.key[0][i] = key;
-        sm.sort.val[0][i] = (uint32_t)i;
-        if (keys) keys[vb + i] = key;
-      }
-    }
-  }
-  const int cur = tile_sort_smem(sm.sort, k, D * pr.L);
-  const uint32_t* skey = sm.sort.key[cur];
-  const uint32_t* sloc = sm.sort.val[cur];
-  // gather and cell start table (global for the step kernel, shared here)
-  const int64_t ncell = int64_t(1) << (D * pr.L);
-  const int64_t e = (vb + pb + 1) & ~int64_t(1);
-  int32_t* cs = cst + pr.fbase + pb;
-  for (int i = threadIdx.x; i < k; i += kSortThreads) {
-    const int64_t p = vb + i;
-    const uint32_t li = sloc[i];
-    svals[p] = (uint32_t)(vb + li);
-    const float4 xv = sm.xin[li];
-    const float wv = sm.win[li];
-    xs[p] = xv;
-    if (ws) ws[p] = wv;
-    const float xc[4] = {xv.x, xv.y, xv.z, xv.w};
-    pair_store<D>(XP, e + i, xc, wv);
-    if (i == k - 1 && (k & 1)) {
-      const float zero[4] = {0.f, 0.f, 0.f, 0.f};
-      pair_store<D>(XP, e + k, zero, 0.0f);
-    }
-    int32_t c[D];
-    cell_of<D>(xv, lo, s, pr.L, c);
-    uint32_t packed = 0;
-#pragma unroll
-    for (int m = 0; m < D; ++m) packed |= (uint32_t)c[m] << (m * field_bits(D));
-    scell[p] = packed;
-    const int64_t key = skey[i];
-    const int64_t prev = i == 0 ? -1 : (int64_t)skey[i - 1];
-    for (int64_t q = prev + 1; q <= key; ++q) sm.cs[q] = (int32_t)p;
-    fill_i32(cs, prev + 1, key + 1, (int32_t)p);
-    if (i == k - 1) {
-      for (int64_t q = key + 1; q <= ncell; ++q) sm.cs[q] = (int32_t)(vb + k);
-      fill_i32(cs, key + 1, ncell + 1, (int32_t)(vb + k));
-    }
-  }
-  if (k == 0)
-    for (int64_t c = threadIdx.x; c <= ncell; c += kSortThreads) {
-      cs[c] = (int32_t)vb;
-      sm.cs[c] = (int32_t)vb;
-    }
-  __syncthreads();
-  // finest cells from the staged points, a warp per 32 consecutive cells
-  const int lane = lane_id(), warp = threadIdx.x >> 5;
-  const int64_t cfin = pr.cbase + lvl_off(D, pr.L);
-  for (int64_t c0 = (int64_t)warp * 32; c0 < ncell; c0 += kSortThreads) {
-    const int64_t c = c0 + lane;
-    const bool valid = c < ncell;
-    int q0 = 0, q1 = 0;  // problem-local sorted positions
-    if (valid && k > 0) {
-      q0 = sm.cs[c] - (int)vb;
-      q1 = sm.cs[c + 1] - (int)vb;
-    }
-    const int64_t idx = cfin + c, pidx = idx + pb + 1;
-    const bool big = valid && q1 - q0 > kCellSerial;
-    if (valid && !big) {
-      float S[4] = {0.f, 0.f, 0.f, 0.f};
-      float W = 0.f;
-      for (int q = q0; q < q1; ++q) cell_add<D>(sm.xin[sloc[q]], sm.win[sloc[q]], S, W);
-      store_cell<D>(idx, pidx, S, W, St, Wt, CP);
-    }
-    unsigned todo = __ballot_sync(0xffffffffu, big);
-    while (todo) {
-      const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const int b0 = __shfl_sync(0xffffffffu, q0, src), b1 = __shfl_sync(0xffffffffu, q1, src);
-      float S[4] = {0.f, 0.f, 0.f, 0.f};
-      float W = 0.f;
-      for (int q = b0 + lane; q < b1; q += 32) cell_add<D>(sm.xin[sloc[q]], sm.win[sloc[q]], S, W);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int m = 0; m < D; ++m) S[m] += __shfl_xor_sync(0xffffffffu, S[m], o);
-        W += __shfl_xor_sync(0xffffffffu, W, o);
-      }
-      if (lane == src) store_cell<D>(idx, pidx, S, W, St, Wt, CP);
-    }
-  }
-  __syncthreads();
-  // coarser levels down to 2, each from its children
-  for (int l = pr.L - 1; l >= 2; --l) {
-    const int64_t n = int64_t(1) << (D * l);
-    for (int64_t c = threadIdx.x; c < n; c += kSortThreads) agg_cell<D>(pr, pb, l, c, St, Wt, CP);
-    __syncthreads();
-  }
-}
-
 // Rubber bands of 2-pin nets: y_v = sum_u c_vu (x_v - x_u) / 2.  Rows are
 // split by degree: light rows (<= kLightMax) take one thread, medium rows a
 // quarter warp and heavy rows a block; each class sums in a fixed order (sequential,
@@ -938,38 +778,30 @@ __device__ __forceinline__ void pull_range(float* a, const float4& xv, const int
 constexpr int kMidLanes = 8;
 constexpr int kMidMax = 512;  // entries of a row from which the whole warp takes it
 
-__global__ void __launch_bounds__(kBlock) k_attract(const int32_t* __restrict__ adj_ptr, const int32_t* __restrict__ adj,
-                                                    const float* __restrict__ acost, const float4* __restrict__ x,
-                                                    int64_t K, const int32_t* __restrict__ heavy, int64_t n_heavy,
-                                                    const int32_t* __restrict__ mid, int64_t n_mid, int64_t mid_blocks,
-                                                    float4* __restrict__ y) {
-  pdl_enter();
-  __shared__ float part[kBlock / 32][4];
-  const int lane = lane_id(), warp = threadIdx.x >> 5;
-  int64_t b = blockIdx.x;
-  if (b < n_heavy) {
-    const int32_t v = heavy[b];
-    const float4 xv = x[v];
-    float a[4] = {0.f, 0.f, 0.f, 0.f};
-    pull_range<16>(a, xv, adj, acost, x, adj_ptr[v] + threadIdx.x, adj_ptr[v + 1], blockDim.x);
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) a[m] += __shfl_xor_sync(0xffffffffu, a[m], o);
-    if (lane == 0)
-      for (int m = 0; m < 4; ++m) part[warp][m] = a[m];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float s[4] = {0.f, 0.f, 0.f, 0.f};
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-        for (int m = 0; m < 4; ++m) s[m] += part[w][m];
-      y[v] = make_float4(0.5f * s[0], 0.5f * s[1], 0.5f * s[2], 0.5f * s[3]);
-    }
-    return;
-  }
-  b -= n_heavy;
+struct Attract {
+  const int32_t *adj_ptr, *adj;
+  const float* acost;
+  const float4* x;
+  int64_t K;
+  const int32_t *heavy, *mid;
+  int64_t n_heavy, n_mid, mid_blocks;  // mid_blocks: blocks of T threads for the medium rows
+  float4* y;
+  template <int T>
+  int64_t blocks() const { return n_heavy + mid_blocks + (K + T - 1) / T; }
+};
+
+// The rows of blocks of T threads numbered b, medium and light rows.
+template <int T>
+__device__ __forceinline__ void attract_rows(const Attract& at, int64_t b) {
+  const int32_t *adj_ptr = at.adj_ptr, *adj = at.adj, *mid = at.mid;
+  const float* acost = at.acost;
+  const float4* x = at.x;
+  float4* y = at.y;
+  const int64_t K = at.K, n_mid = at.n_mid, mid_blocks = at.mid_blocks;
+  const int lane = lane_id();
+
   if (b < mid_blocks) {
-    const int64_t i = (b * kBlock + threadIdx.x) / kMidLanes;
+    const int64_t i = (b * T + threadIdx.x) / kMidLanes;
     const int l = threadIdx.x & (kMidLanes - 1);
     const bool in = i < n_mid;
     const int32_t v = in ? mid[i] : 0;
@@ -1021,7 +853,7 @@ __global__ void __launch_bounds__(kBlock) k_attract(const int32_t* __restrict__ 
     }
     return;
   }
-  const int64_t v = (b - mid_blocks) * kBlock + threadIdx.x;
+  const int64_t v = (b - mid_blocks) * T + threadIdx.x;
   if (v >= K) return;
   const int32_t t0 = adj_ptr[v], t1 = adj_ptr[v + 1];
   if (t1 - t0 > kLightMax) return;  // a medium or heavy row
@@ -1029,6 +861,230 @@ __global__ void __launch_bounds__(kBlock) k_attract(const int32_t* __restrict__ 
   float a[4] = {0.f, 0.f, 0.f, 0.f};
   pull_range<4>(a, xv, adj, acost, x, t0, t1, 1);
   y[v] = make_float4(0.5f * a[0], 0.5f * a[1], 0.5f * a[2], 0.5f * a[3]);
+}
+
+__global__ void __launch_bounds__(kBlock) k_attract(Attract at) {
+  pdl_enter();
+  __shared__ float part[kBlock / 32][4];
+  if (blockIdx.x >= at.n_heavy) {
+    attract_rows<kBlock>(at, (int64_t)blockIdx.x - at.n_heavy);
+    return;
+  }
+  const int lane = lane_id(), warp = threadIdx.x >> 5;
+  const float4* x = at.x;
+  float4* y = at.y;
+  const int32_t v = at.heavy[blockIdx.x];
+  const float4 xv = x[v];
+  float a[4] = {0.f, 0.f, 0.f, 0.f};
+  pull_range<16>(a, xv, at.adj, at.acost, x, at.adj_ptr[v] + threadIdx.x, at.adj_ptr[v + 1], blockDim.x);
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a[m] += __shfl_xor_sync(0xffffffffu, a[m], o);
+  if (lane == 0)
+    for (int m = 0; m < 4; ++m) part[warp][m] = a[m];
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+      for (int m = 0; m < 4; ++m) s[m] += part[w][m];
+    y[v] = make_float4(0.5f * s[0], 0.5f * s[1], 0.5f * s[2], 0.5f * s[3]);
+  }
+}
+
+// One-block binning of a step for levels whose problems all have at most
+// kSortTile points and kBinCells finest cells: one block per problem does what
+// the device-wide sequence does, with the counts, the sorted points and the
+// sums of every grid level in shared memory: keys and arrival numbers, scan of
+// the cell counts, vertex order within a cell, sorted copies, sums and charges.
+// The arithmetic and the order of every sum are those kernels', so the results
+// are bit-identical, from one launch instead of five.  The blocks after the
+// problems' do the attraction (no row of such a level is heavy), so that a step
+// is two launches in a row and the level needs no second stream.  As a sort of
+// 8-bit digits with the coarse sums read back through L2, and the attraction on
+// a second stream, a whole step took 12.2 / 17.4 us of 256 / 1,024 points (d =
+// 2) and 15.4 / 24.5 us of 512 / 1,728 (d = 3); now 8.2 / 13.4 and 11.3 / 19.5.
+constexpr int kBinCells = 4096;
+constexpr int kBinBig = kSortTile / (kCellSerial + 1) + 1;  // most large cells of a problem
+
+// Shared memory of a block: sorted points and weights, slots, cell starts, sums.
+struct BinShape {
+  int points, cells, sums;  // capacities: points, finest cells, cells of all levels >= 2
+  size_t bytes(int d) const {
+    return (size_t)points * (sizeof(float4) + sizeof(float) + sizeof(uint32_t)) + (size_t)(cells + 1) * sizeof(int32_t) +
+           (size_t)sums * (d + 1) * sizeof(float);
+  }
+};
+
+template <int D, int T>
+__global__ void __launch_bounds__(T) k_bin_small(
+    const float4* __restrict__ x, const float* __restrict__ w, const ProbDev* __restrict__ prob, int P,
+    const uint32_t* __restrict__ bb, uint32_t* __restrict__ bb_next, int32_t* __restrict__ tctr,
+    uint32_t* __restrict__ keys, uint32_t* __restrict__ svals, float4* __restrict__ xs, float* __restrict__ ws,
+    uint32_t* __restrict__ scell, int32_t* __restrict__ cst, float4* __restrict__ XP, float4* __restrict__ CP,
+    int32_t* __restrict__ cch, int32_t* __restrict__ chunk, BinShape shape, Attract at) {
+  pdl_enter();
+  if ((int)blockIdx.x >= P) {
+    attract_rows<T>(at, (int64_t)blockIdx.x - P);
+    return;
+  }
+  constexpr int ITEMS = 2;  // points per thread: problems of up to 2 T
+  extern __shared__ __align__(16) unsigned char bin_raw[];
+  float4* sx = reinterpret_cast<float4*>(bin_raw);
+  float* sw = reinterpret_cast<float*>(sx + shape.points);
+  uint32_t* slot = reinterpret_cast<uint32_t*>(sw + shape.points);
+  int32_t* cs = reinterpret_cast<int32_t*>(slot + shape.points);
+  float* sS = reinterpret_cast<float*>(cs + shape.cells + 1);  // [D + 1][sums]
+  __shared__ uint64_t scan[33];
+  __shared__ int32_t big[kBinBig];
+  __shared__ int nbig;
+  const int pb = blockIdx.x;
+  const ProbDev pr = prob[pb];
+  const int k = pr.k, L = pr.L;
+  const int64_t vb = pr.vbase;
+  if (pb == 0 && threadIdx.x == 0) ++*tctr;  // the level's step
+  if (threadIdx.x < 8) bb_next[pb * 8 + threadIdx.x] = threadIdx.x < 4 ? 0xFFFFFFFFu : 0u;
+  const int ncell = 1 << (D * L);
+  for (int c = threadIdx.x; c <= ncell; c += T) cs[c] = 0;
+  if (threadIdx.x == 0) nbig = 0;
+  // the thread's points and weights
+  float4 xv[ITEMS];
+  float wv[ITEMS];
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    const int i = threadIdx.x + j * T;
+    xv[j] = i < k ? x[vb + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    wv[j] = (i < k && w) ? w[vb + i] : 1.0f;
+  }
+  float lo[D], s;
+  grid_frame<D>(bb, pb, L, lo, &s);
+  __syncthreads();
+  uint32_t key[ITEMS], arr[ITEMS];
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    const int i = threadIdx.x + j * T;
+    key[j] = arr[j] = 0;
+    if (i < k) {
+      int32_t c[D];
+      cell_of<D>(xv[j], lo, s, L, c);
+      key[j] = min((uint32_t)rowmajor<D>(c, 1 << L), (uint32_t)(ncell - 1));
+      arr[j] = (uint32_t)atomicAdd(&cs[key[j]], 1);
+      if (keys) keys[vb + i] = key[j];
+    }
+  }
+  __syncthreads();
+  {  // cell counts -> starts, and the chunks of two points (see k_cell_scan)
+    const int per = (ncell + T - 1) / T, c0 = min((int)threadIdx.x * per, ncell), c1 = min(c0 + per, ncell);
+    uint64_t sum = 0;
+    for (int c = c0; c < c1; ++c) sum += ((uint64_t)(uint32_t)((cs[c] + 1) >> 1) << 32) | (uint32_t)cs[c];
+    uint64_t total;
+    const uint64_t ex = block_exclusive<uint64_t>(sum, scan, &total);
+    int32_t run = (int32_t)(uint32_t)ex, chk = (int32_t)(ex >> 32);
+    for (int c = c0; c < c1; ++c) {
+      const int32_t n = cs[c];
+      cs[c] = run;
+      cst[pr.fbase + pb + c] = (int32_t)vb + run;
+      if (cch) cch[pr.fbase + pb + c] = (int32_t)vb + chk;  // a problem's chunks are listed from its first point on
+      run += n;
+      chk += (n + 1) >> 1;
+    }
+    if (threadIdx.x == 0) {
+      cs[ncell] = k;
+      cst[pr.fbase + pb + ncell] = (int32_t)vb + k;
+      if (cch) cch[pr.fbase + pb + ncell] = (int32_t)vb + (int32_t)(total >> 32);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    const int i = threadIdx.x + j * T;
+    if (i < k) slot[cs[key[j]] + arr[j]] = (uint32_t)i;
+  }
+  __syncthreads();
+  const int64_t e = (vb + pb + 1) & ~int64_t(1);
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j) {
+    const int i = threadIdx.x + j * T;
+    if (i >= k) continue;
+    const int q0 = cs[key[j]], q1 = cs[key[j] + 1];
+    int less = 0;
+    for (int q = q0; q < q1; ++q) less += slot[q] < (uint32_t)i;
+    const int q = q0 + less;
+    const int64_t p = vb + q;
+    sx[q] = xv[j];
+    sw[q] = wv[j];
+    svals[p] = (uint32_t)(vb + i);
+    xs[p] = xv[j];
+    if (ws) ws[p] = wv[j];
+    const float xc[4] = {xv[j].x, xv[j].y, xv[j].z, xv[j].w};
+    pair_store<D>(XP, e + q, xc, wv[j]);
+    if (q == k - 1 && (k & 1)) {
+      const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+      pair_store<D>(XP, e + k, zero, 0.0f);
+    }
+    uint32_t packed = 0;
+#pragma unroll
+    for (int m = 0; m < D; ++m) packed |= ((key[j] >> (m * L)) & ((1u << L) - 1u)) << (m * field_bits(D));
+    scell[p] = packed;
+    if (cch && !(less & 1)) chunk[cch[pr.fbase + pb + key[j]] + (less >> 1)] = (int32_t)p;
+  }
+  if (L < 2) return;  // no far field
+  __syncthreads();
+  // sums of the finest cells, then of every coarser level from its children
+  auto keep = [&](int l, int at_, int c, const float* S, float W) {
+    float z[4] = {0.f, 0.f, 0.f, 0.f};
+    if (W > 0.0f) {
+      const float iw = 1.0f / W;
+#pragma unroll
+      for (int m = 0; m < D; ++m) z[m] = S[m] * iw;
+    }
+#pragma unroll
+    for (int m = 0; m < D; ++m) sS[m * shape.sums + at_ + c] = S[m];
+    sS[D * shape.sums + at_ + c] = W;
+    pair_store<D>(CP, pr.cbase + lvl_off(D, l) + c + pb + 1, z, W);
+  };
+  for (int c = threadIdx.x; c < ncell; c += T) {
+    const int q0 = cs[c], q1 = cs[c + 1];
+    if (q1 - q0 > kCellSerial) {
+      big[atomicAdd(&nbig, 1)] = c;
+      continue;
+    }
+    float S[4] = {0.f, 0.f, 0.f, 0.f};
+    float W = 0.f;
+    for (int q = q0; q < q1; ++q) cell_add<D>(sx[q], sw[q], S, W);
+    keep(L, 0, c, S, W);
+  }
+  __syncthreads();
+  for (int b0 = 0; b0 < nbig; b0 += T / kCellLanes) {
+    const int b = b0 + threadIdx.x / kCellLanes;
+    const bool mine = b < nbig;
+    float S[4] = {0.f, 0.f, 0.f, 0.f};
+    float W = 0.f;
+    cell_sum_quarter<D>(sx, sw, mine ? cs[big[b]] : 0, mine ? cs[big[b] + 1] : 0, S, W);
+    if (mine && (threadIdx.x & (kCellLanes - 1)) == 0) keep(L, 0, big[b], S, W);
+  }
+  int from = 0, to = ncell;
+  for (int l = L - 1; l >= 2; --l) {
+    __syncthreads();
+    const int n = 1 << (D * l), side = 1 << l;
+    for (int c = threadIdx.x; c < n; c += T) {
+      float S[4] = {0.f, 0.f, 0.f, 0.f};
+      float W = 0.f;
+#pragma unroll
+      for (int ch = 0; ch < (1 << D); ++ch) {
+        int q = 0;
+#pragma unroll
+        for (int m = 0; m < D; ++m)
+          q |= (2 * ((c >> (m * l)) & (side - 1)) + ((ch >> m) & 1)) << (m * (l + 1));
+#pragma unroll
+        for (int m = 0; m < D; ++m) S[m] += sS[m * shape.sums + from + q];
+        W += sS[D * shape.sums + from + q];
+      }
+      keep(l, to, c, S, W);
+    }
+    from = to;
+    to += n;
+  }
 }
 
 // Degree class of every row, counted by one scan: 1 medium, 2^32 heavy.
@@ -2466,8 +2522,8 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   if (K == 0 || iters <= 0) return VMO_OK;
   ScratchFrame frame(sc);
   uint32_t *keys, *arrival = nullptr, *slot = nullptr, *svals, *scell, *bb;
-  float4 *xs, *XP, *yatt, *St, *CP, *z = nullptr;
-  float *ws = nullptr, *Wt, *s0;
+  float4 *xs, *XP, *yatt, *St = nullptr, *CP, *z = nullptr;
+  float *ws = nullptr, *Wt = nullptr, *s0;
   int32_t *cst, *cnt = nullptr, *done = nullptr, *chunk = nullptr, *cch = nullptr;
   uint64_t* tot = nullptr;
   const int64_t ncell = lb.cbase[P], nfine = lb.fbase[P];
@@ -2477,10 +2533,8 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   VMO_TRY(sc.alloc(&xs, K));
   VMO_TRY(sc.alloc(&yatt, K));
   if (lb.w) VMO_TRY(sc.alloc(&ws, K));
-  VMO_TRY(sc.alloc(&St, ncell));
   VMO_TRY(sc.alloc(&CP, (size_t)((ncell + P) / 2 + 1) * (d == 4 ? 3 : 2)));
   VMO_TRY(sc.alloc(&XP, (size_t)((K + P + 1) / 2 + 1) * (d == 4 ? 3 : 2)));
-  VMO_TRY(sc.alloc(&Wt, ncell));
   VMO_TRY(sc.alloc(&cst, nfine + P));
   VMO_TRY(sc.alloc(&bb, (size_t)2 * 8 * P));
   VMO_TRY(sc.alloc(&s0, P));
@@ -2491,29 +2545,36 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   for (int p = 0; p < P; ++p) kmax = std::max(kmax, lb.vbase[p + 1] - lb.vbase[p]);
   bool bin1 = kmax <= std::min<int64_t>(kSortTile, g_tuning.small_bin_points.load(std::memory_order_relaxed));
   for (int p = 0; p < P && bin1; ++p) bin1 = (int64_t(1) << (d * lb.L[p])) <= kBinCells;
-  if (bin1)
+  BinShape shape{(int)std::max<int64_t>((kmax + 3) / 4 * 4, 4), 1 << (d * std::min(lb.maxL, 12 / d)),
+                 (int)(lvl_off(d, std::min(lb.maxL, 12 / d) + 1))};
+  const bool bin_wide = kmax > 512;  // threads of a problem's block: 1,024, else 256, for two points each
+  if (bin1 && shape.bytes(d) > 40 * 1024)  // with the static arrays above the default limit of 48 KB
     dispatch_d(d, [&](auto DC) {
       constexpr int D = decltype(DC)::value;
-      if (cudaFuncSetAttribute(k_bin_small<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BinSmem)) !=
-          cudaSuccess) {
+      if ((bin_wide ? cudaFuncSetAttribute(k_bin_small<D, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)shape.bytes(d))
+                    : cudaFuncSetAttribute(k_bin_small<D, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)shape.bytes(d))) != cudaSuccess) {
         (void)cudaGetLastError();
         bin1 = false;  // the device-wide sequence then
       }
     });
-  const bool pair = !bin1 && lb.threads >= kPairThreadsMin;
+  const bool pair = lb.threads >= kPairThreadsMin;
   const int64_t ncnt = nfine + P;  // entries of the cell start table
+  if (pair) {
+    VMO_TRY(sc.alloc(&chunk, K));
+    VMO_TRY(sc.alloc(&cch, ncnt));
+  }
   const bool one_cluster = ncnt <= kCellScanTile;
   const unsigned scan_blocks = grid_for(ncnt, kCellScanThreads * kCellScanItems);
   if (!bin1) {
+    VMO_TRY(sc.alloc(&St, ncell));
+    VMO_TRY(sc.alloc(&Wt, ncell));
     VMO_TRY(sc.alloc(&arrival, K));
     VMO_TRY(sc.alloc(&slot, K));
     VMO_TRY(sc.alloc(&cnt, ncnt));
     VMO_TRY(sc.alloc(&done, P));
     if (!one_cluster) VMO_TRY(sc.alloc(&tot, scan_blocks));
-    if (pair) {
-      VMO_TRY(sc.alloc(&chunk, std::max<int64_t>(lb.chunks, 1)));
-      VMO_TRY(sc.alloc(&cch, ncnt));
-    }
     VMO_CUDA(cudaMemsetAsync(cnt, 0, ncnt * sizeof(int32_t), s));
     VMO_CUDA(cudaMemsetAsync(done, 0, P * sizeof(int32_t), s));
   }
@@ -2543,27 +2604,37 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
       PdlScope pdl;  // every kernel of a step starts with pdl_wait()
       uint32_t* cur = bb + (t & 1) * 8 * P;
       uint32_t* nxt = bb + ((t + 1) & 1) * 8 * P;
-      // attraction depends only on x: it runs on the side stream, overlapped
-      // with the binning below, and joins before the step kernel
-      cudaStream_t as = side ? side : ms;
-      if (side) {
+      // attraction depends only on x: in the one-block binning's launch, or on
+      // the side stream, overlapped with the binning, joined before the step kernel
+      Attract at{lb.adj_ptr, lb.adj, lb.acost, x, K, lb.heavy_list.ptr, lb.mid_list.ptr, lb.n_heavy, lb.n_mid, 0, yatt};
+      const bool fused = bin1 && lb.adj_ptr && lb.n_heavy == 0;
+      const bool fork = side && !fused;
+      cudaStream_t as = fork ? side : ms;
+      if (fork) {
         cudaEventRecord(ss->fork, ms);
         cudaStreamWaitEvent(side, ss->fork, 0);
       }
-      if (lb.adj_ptr) {
-        const int64_t mid_blocks = (lb.n_mid * kMidLanes + kBlock - 1) / kBlock;
-        launch(k_attract, (unsigned)(lb.n_heavy + mid_blocks + grid_for(K, kBlock)), kBlock, 0, as, lb.adj_ptr, lb.adj,
-               lb.acost, x, K, lb.heavy_list.ptr, lb.n_heavy, lb.mid_list.ptr, lb.n_mid, mid_blocks, yatt);
+      if (fused) {
+      } else if (lb.adj_ptr) {
+        at.mid_blocks = (lb.n_mid * kMidLanes + kBlock - 1) / kBlock;
+        launch(k_attract, (unsigned)at.blocks<kBlock>(), kBlock, 0, as, at);
       } else if (lb.net_ptr) {
         if (lb.nnets > 0) launch(k_net_center, grid_for(lb.nnets, kBlock), kBlock, 0, as, lb.net_ptr, lb.pins, lb.nnets, x, z);
         launch(k_attract_hyper, grid_for(K, kBlock), kBlock, 0, as, lb.vtx_ptr, lb.vnets, x, z, K, yatt);
       } else {
         cudaMemsetAsync(yatt, 0, K * sizeof(float4), as);
       }
-      if (side) cudaEventRecord(ss->join, side);
+      if (fork) cudaEventRecord(ss->join, side);
       if (bin1) {
-        launch(k_bin_small<D>, (unsigned)P, kSortThreads, sizeof(BinSmem), ms, x, lb.w, lb.prob.ptr, cur, nxt, tctr,
-               keys_out && t == 0 ? keys : nullptr, svals, xs, ws, scell, cst, XP, St, Wt, CP);
+        auto bin = [&](auto kernel, auto TC) {
+          constexpr int T = decltype(TC)::value;
+          at.mid_blocks = (lb.n_mid * kMidLanes + T - 1) / T;
+          const unsigned blocks = (unsigned)(P + (fused ? at.blocks<T>() : 0));
+          launch(kernel, blocks, T, shape.bytes(D), ms, x, lb.w, lb.prob.ptr, P, cur, nxt, tctr,
+                 keys_out && t == 0 ? keys : nullptr, svals, xs, ws, scell, cst, XP, CP, cch, chunk, shape, at);
+        };
+        if (bin_wide) bin(k_bin_small<D, 1024>, std::integral_constant<int, 1024>());
+        else bin(k_bin_small<D, 256>, std::integral_constant<int, 256>());
         if (keys_out && t == 0) cudaMemcpyAsync(keys_out, keys, K * 4, cudaMemcpyDeviceToDevice, ms);
       } else {
         auto keys_kernel = K >= kKeyItemsMin ? k_keys<D, 4> : k_keys<D, 1>;
@@ -2583,7 +2654,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
           launch(k_cells<D>, (unsigned)lb.bricks, kCellsBlock, 0, ms, lb.bprob.ptr, lb.prob.ptr, xs, ws, cst, St, Wt,
                  CP, done);
       }
-      if (side) cudaStreamWaitEvent(ms, ss->join, 0);
+      if (fork) cudaStreamWaitEvent(ms, ss->join, 0);
       const bool timed = stats_timing();
       if (timed) stats_time_begin(ms);
       unsigned long long* icount = stats_interaction_counter();
