@@ -35,6 +35,7 @@ struct KmState {
 template <int D>
 __global__ void k_km_gather(const float4* __restrict__ x, const int32_t* __restrict__ verts, int64_t n,
                             float4* __restrict__ xo, KmState* __restrict__ st) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t mx = 0;
   if (i < n) {
@@ -50,6 +51,7 @@ __global__ void k_km_gather(const float4* __restrict__ x, const int32_t* __restr
 // First centre: point floor(n * r0 / 2^64).
 __global__ void k_km_seed0(const float4* __restrict__ xo, int64_t n, uint64_t seed, uint64_t key,
                            float4* __restrict__ z, KmState* __restrict__ st) {
+  pdl_enter();
   st->e = exponent_of(st->maxabs);
   st->chosen = 1;
   st->stopped = 0;
@@ -80,6 +82,7 @@ __global__ void __launch_bounds__(kKmBlock) k_km_weights(const float4* __restric
                                                          unsigned long long* __restrict__ bsum,
                                                          const KmState* __restrict__ st) {
   __shared__ unsigned long long red[kKmBlock / 32];
+  pdl_enter();
   if (st->stopped) return;  // grid-uniform
   const int e = st->e;
   const float4 zc = z[c - 1];
@@ -122,6 +125,7 @@ __global__ void __launch_bounds__(kKmPickBlock) k_km_pick(const float4* __restri
   __shared__ unsigned long long ws[33];
   __shared__ unsigned long long s_before;
   __shared__ int s_block;
+  pdl_enter();
   if (st->stopped) return;
   // block sums: contiguous parts of the threads, prefixes by a block scan
   const int per = (nb + kKmPickBlock - 1) / kKmPickBlock;
@@ -174,6 +178,7 @@ __global__ void __launch_bounds__(kKmPickBlock) k_km_pick(const float4* __restri
 
 // Centres the seeding did not reach are copies of the first (they never win).
 __global__ void k_km_fill(float4* __restrict__ z, int m, const KmState* __restrict__ st) {
+  pdl_enter();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c < m && c >= st->chosen) z[c] = z[0];
 }
@@ -200,6 +205,7 @@ __global__ void __launch_bounds__(kKmBlock) k_km_assign(const float4* __restrict
   __shared__ int hi[kKmMaxCentres * D];
   __shared__ int sc[kKmMaxCentres];
   const bool final_pass = it < 0;
+  pdl_enter();
   if (!final_pass && st->converged) return;  // block-uniform
   for (int j = threadIdx.x; j < m; j += blockDim.x) {
     zs[j] = z[j];
@@ -286,6 +292,7 @@ template <int D>
 __global__ void k_km_update(float4* __restrict__ z, int m, int it, unsigned long long* __restrict__ S,
                             unsigned long long* __restrict__ cnt, KmState* __restrict__ st) {
   const int j = threadIdx.x;  // one block of at least m threads
+  pdl_enter();
   const bool done = st->converged || (it > 0 && !st->changed);
   __syncthreads();
   if (j < m) {
@@ -309,6 +316,7 @@ __global__ void k_km_update(float4* __restrict__ z, int m, int it, unsigned long
 }
 
 __global__ void k_km_nonempty(const unsigned long long* __restrict__ cnt, int m, int32_t* __restrict__ out) {
+  pdl_enter();
   int c = 0;
   for (int j = 0; j < m; ++j) c += cnt[j] > 0;
   *out = c;
@@ -359,6 +367,7 @@ vmo_status kmeans_m(int32_t d, const float* coords, const int32_t* verts, int32_
   // assignment blocks: one wave, so that the clusters' sums leave a block once
   const unsigned na = (unsigned)std::min<int64_t>((n + kKmBlock * kKmAssign - 1) / (kKmBlock * kKmAssign), 152 * 6);
   vmo_status stt = VMO_OK;
+  PdlScope pdl;  // every kernel below starts with pdl_enter()
   km_dispatch(d, [&](auto DC) {
     constexpr int D = decltype(DC)::value;
     launch(k_km_gather<D>, nb, kKmBlock, 0, s, reinterpret_cast<const float4*>(coords), verts, n, xo, st);

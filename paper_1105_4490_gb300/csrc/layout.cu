@@ -900,11 +900,12 @@ __global__ void __launch_bounds__(kBlock) k_attract(Attract at) {
 // The arithmetic and the order of every sum are those kernels', so the results
 // are bit-identical, from one launch instead of five.  The blocks after the
 // problems' do the attraction (no row of such a level is heavy), so that a step
-// is two launches in a row and the level needs no second stream.  As a sort of
+// of few problems is two launches in a row without a second stream.  As a sort of
 // 8-bit digits with the coarse sums read back through L2, and the attraction on
 // a second stream, a whole step took 12.2 / 17.4 us of 256 / 1,024 points (d =
 // 2) and 15.4 / 24.5 us of 512 / 1,728 (d = 3); now 8.2 / 13.4 and 11.3 / 19.5.
 constexpr int kBinCells = 4096;
+constexpr int kFusedProblems = 64;  // most problems of a level whose binning launch does the attraction
 constexpr int kBinBig = kSortTile / (kCellSerial + 1) + 1;  // most large cells of a problem
 
 // Shared memory of a block: sorted points and weights, slots, cell starts, sums.
@@ -2583,7 +2584,8 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   const float kappa = d == 2 ? 1.0f : (float)(d - 2);
   float* scale_tab = ctx ? ctx->scale_tab : nullptr;
   int32_t* tctr;
-  if (!scale_tab) VMO_TRY(make_scale_tab(o, iters, &scale_tab, s, sc));
+  const bool own_step = step_override <= 0.0f;  // the step length comes from the box, not from the caller
+  if (!scale_tab && own_step) VMO_TRY(make_scale_tab(o, iters, &scale_tab, s, sc));
   VMO_TRY(sc.alloc(&tctr, 1));
   VMO_CUDA(cudaMemsetAsync(tctr, 0xFF, sizeof(int32_t), s));  // -1: k_keys advances it at every step
   vmo_status st = VMO_OK;
@@ -2595,7 +2597,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   dispatch_d(d, [&](auto DC) {
     constexpr int D = decltype(DC)::value;
     launch(k_bbox<D>, grid_for(K, kBlock), kBlock, 0, s, x, K, lb.vprob.ptr, bb);
-    launch(k_step0<D>, grid_for(P, kBlock), kBlock, 0, s, bb, lb.prob.ptr, P, o.sigma, s0);
+    if (own_step) launch(k_step0<D>, grid_for(P, kBlock), kBlock, 0, s, bb, lb.prob.ptr, P, o.sigma, s0);
     cudaStream_t ms = s;  // stream of the steps
     // one step t of Algorithm 4 for every problem (only the parity of t and
     // whether it is the first step matter to the launches)
@@ -2607,7 +2609,9 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
       // attraction depends only on x: in the one-block binning's launch, or on
       // the side stream, overlapped with the binning, joined before the step kernel
       Attract at{lb.adj_ptr, lb.adj, lb.acost, x, K, lb.heavy_list.ptr, lb.mid_list.ptr, lb.n_heavy, lb.n_mid, 0, yatt};
-      const bool fused = bin1 && lb.adj_ptr && lb.n_heavy == 0;
+      // (with many problems the wide blocks of the binning fill the SMs and the
+      // attraction would wait for them)
+      const bool fused = bin1 && lb.adj_ptr && lb.n_heavy == 0 && P <= kFusedProblems;
       const bool fork = side && !fused;
       cudaStream_t as = fork ? side : ms;
       if (fork) {

@@ -554,6 +554,7 @@ __global__ void __launch_bounds__(kBlock) k_separator(const int32_t* __restrict_
                                                       const int32_t* __restrict__ adj,
                                                       const uint64_t* __restrict__ vrec, NodeDev* __restrict__ nodes,
                                                       uint8_t* __restrict__ labf, unsigned long long* __restrict__ pk) {
+  pdl_enter();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int s = i < n ? seg[i] : -1;
   uint8_t l = 0;
@@ -824,6 +825,7 @@ __global__ void k_scatter(const int32_t* __restrict__ ord, const float4* __restr
                           const NodeDev* __restrict__ nodes, const unsigned long long* __restrict__ pre, int sbd,
                           int32_t* __restrict__ ord2, float4* __restrict__ xo2, int32_t* __restrict__ seg2,
                           uint64_t* __restrict__ vrec) {
+  pdl_enter();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int s = seg[i];
@@ -862,6 +864,7 @@ __global__ void k_children(NodeDev* __restrict__ nodes, int N, const int64_t* __
                            int max_depth, int sbd, int sep_rec, NodeDev* __restrict__ next,
                            int* __restrict__ next_count, int* __restrict__ next_max, int next_cap, TreeDev tree,
                            int* __restrict__ err) {
+  pdl_enter();
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= N) return;
   NodeDev& nd = nodes[s];
@@ -1098,6 +1101,7 @@ __global__ void __launch_bounds__(T) k_two_means(const float4* __restrict__ xo, 
                                                  NodeDev* __restrict__ nodes, const uint64_t* __restrict__ seeds,
                                                  int km_iters, uint8_t* __restrict__ lab, uint64_t* __restrict__ vrec,
                                                  int cap, int stream) {
+  pdl_enter();
   namespace cg = cooperative_groups;
   constexpr int W = T / 32;
   extern __shared__ __align__(16) unsigned char tm_raw[];
@@ -1373,12 +1377,14 @@ static cudaError_t launch_two_means(const OrderState& st, int N, int km_iters, i
   cfg.blockDim = dim3(T);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)C;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   if (C > 8) {  // a cluster of 16 where the device has room for one
     int active = 0;
     e = cudaOccupancyMaxActiveClusters(&active, kernel, &cfg);
@@ -1582,10 +1588,12 @@ vmo_status order_levels(OrderState& st, const OrderParams& op, cudaStream_t s, S
     } else if (st.mu) {
       VMO_TRY(mu_loop_separator(st, n, labf, pk, s, sc));
     } else {
+      PdlScope pdl;
       launch(k_separator, grid_for(n, kBlock), kBlock, 0, s, st.ord, st.seg, n, st.adj_ptr, st.adj, st.vrec, st.nodes,
              labf, pk);
     }
     VMO_LAUNCHED("separator");
+    PdlScope pdl;  // every kernel from here to the scatter starts with pdl_enter()
     VMO_TRY(scan_inclusive<uint64_t>((const uint64_t*)pk, (uint64_t*)pre, n, s, sc));
     // children first (they number the next level's nodes), then the scatter
     // writes every position's next node

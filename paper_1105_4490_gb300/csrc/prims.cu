@@ -27,6 +27,7 @@ constexpr int kScanTile = kScanThreads * kScanItems;
 template <class T>
 __global__ void scan_reduce_kernel(const T* __restrict__ in, int64_t n, T* __restrict__ partial) {
   __shared__ T ws[33];
+  pdl_enter();
   int64_t base = (int64_t)blockIdx.x * kScanTile;
   T acc = 0;
   for (int i = threadIdx.x; i < kScanTile; i += kScanThreads) {
@@ -41,6 +42,7 @@ __global__ void scan_reduce_kernel(const T* __restrict__ in, int64_t n, T* __res
 template <class T>
 __global__ void scan_partials_kernel(T* partial, int64_t ntiles, T* total) {
   __shared__ T ws[33];
+  pdl_enter();
   T carry = 0;
   for (int64_t b = 0; b < ntiles; b += blockDim.x) {
     int64_t i = b + threadIdx.x;
@@ -62,6 +64,7 @@ __global__ void scan_tile_kernel(const T* __restrict__ in, T* __restrict__ out, 
                                  const T* __restrict__ partial, T* __restrict__ total) {
   __shared__ T tile[kScanTile];
   __shared__ T ws[33];
+  pdl_enter();
   int64_t base = (int64_t)blockIdx.x * kScanTile;
   for (int i = threadIdx.x; i < kScanTile; i += kScanThreads) {
     int64_t g = base + i;
