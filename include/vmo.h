@@ -448,8 +448,9 @@ vmo_status vmo_finegrain_coords(vmo_hg hg, const float* bipartite_coords, float*
  *     8 (default 4; fewer are used when the blocks would not fill the GPU);
  *   small_bin_points: a layout level whose problems all have at most this
  *     many vertices (0 ... 2,048) is binned by one block per problem (keys,
- *     sort, gather and cell charges in one launch) instead of the device-wide
- *     sequence; 0 turns it off (default 2,048).
+ *     sorted copies and cell charges in one launch) instead of the device-wide
+ *     sequence; 0 turns it off (default 2,048, which also takes levels of at
+ *     most 64 problems of up to 4,096 vertices for d = 2).
  * The setting is process-wide and read at every launch.
  * ------------------------------------------------------------------------ */
 typedef struct {

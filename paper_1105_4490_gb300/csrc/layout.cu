@@ -229,7 +229,10 @@ __global__ void __launch_bounds__(kBlock) k_keys(const float4* __restrict__ x, i
                                                  int32_t* __restrict__ tctr) {
   pdl_enter();
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gt == 0) ++*tctr;  // the level's step (read by the step kernel of this step)
+  if (gt == 0) {
+    ++tctr[0];    // the level's step (read by the step kernel of this step)
+    tctr[1] = 0;  // set by the scan of the counts if a cell is crowded
+  }
   const int64_t nreset = 8 * (int64_t)P;
   for (int64_t r = gt; r < nreset; r += (int64_t)gridDim.x * blockDim.x) bb_next[r] = ((r & 7) < 4) ? 0xFFFFFFFFu : 0u;
   const int64_t v0 = (int64_t)blockIdx.x * blockDim.x * U + threadIdx.x;
@@ -244,7 +247,8 @@ __global__ void __launch_bounds__(kBlock) k_keys(const float4* __restrict__ x, i
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int64_t v = v0 + (int64_t)u * blockDim.x;
-    if (v >= K) break;
+    const unsigned in = __ballot_sync(0xffffffffu, v < K);
+    if (v >= K) continue;
     const int L = prob[pb[u]].L;
     float lo[D], s;
     grid_frame<D>(bb, pb[u], L, lo, &s);
@@ -253,7 +257,23 @@ __global__ void __launch_bounds__(kBlock) k_keys(const float4* __restrict__ x, i
     // the key indexes the count table: kept inside it whatever the coordinates are
     const uint32_t key = min((uint32_t)rowmajor<D>(c, 1 << L), (uint32_t)((int64_t(1) << (D * L)) - 1));
     keys[v] = key;
-    arrival[v] = (uint32_t)atomicAdd(&cnt[prob[pb[u]].fbase + pb[u] + key], 1);
+    // One atomic for the warp's points of the first cell that two neighbouring
+    // lanes share: the points of a crowded cell would take their numbers one by
+    // one (99,000 of 100,000 points in one cell, d = 2: 67 us, now 6.3 us).
+    const int64_t slot = prob[pb[u]].fbase + pb[u] + key;
+    const int64_t next = __shfl_down_sync(in, slot, 1);
+    const unsigned shared = __ballot_sync(in, lane_id() < 31 && ((in >> (lane_id() + 1)) & 1u) && slot == next);
+    unsigned same = 0;
+    if (shared) same = __ballot_sync(in, slot == __shfl_sync(in, slot, __ffs(shared) - 1));
+    const bool joined = (same >> lane_id()) & 1u;
+    const unsigned below = same & ((1u << lane_id()) - 1u);
+    uint32_t number = 0;
+    if (!joined || !below) number = (uint32_t)atomicAdd(&cnt[slot], joined ? __popc(same) : 1);
+    if (shared) {
+      const uint32_t first = __shfl_sync(in, number, __ffs(same) - 1);
+      if (joined) number = first + __popc(below);
+    }
+    arrival[v] = number;
   }
 }
 
@@ -306,9 +326,17 @@ __device__ __forceinline__ uint64_t items_sum(const int32_t* v) {
   return s;
 }
 
-// The starts of a thread's items from the sums before it.
-__device__ __forceinline__ void store_starts(int32_t* __restrict__ cst, int32_t* __restrict__ cch, int64_t i0, int64_t n,
-                                             const int32_t* v, uint64_t before) {
+// The starts of a thread's items from the sums before it, and whether one of
+// them is a crowded cell (see rank_large).
+constexpr int kRankBlock = 1024;  // points of a cell from which a block places them together
+
+__device__ __forceinline__ void store_starts(int32_t* __restrict__ cst, int32_t* __restrict__ cch,
+                                             int32_t* __restrict__ crowded, int64_t i0, int64_t n, const int32_t* v,
+                                             uint64_t before) {
+  int32_t most = 0;
+#pragma unroll
+  for (int j = 0; j < kCellScanItems; ++j) most = max(most, v[j]);
+  if (most > kRankBlock) *crowded = 1;
   int32_t e[kCellScanItems];
   int32_t run = (int32_t)(uint32_t)before;
 #pragma unroll
@@ -328,7 +356,8 @@ __device__ __forceinline__ void store_starts(int32_t* __restrict__ cst, int32_t*
 }
 
 __global__ void __cluster_dims__(kCellScanCtas, 1, 1) __launch_bounds__(kCellScanThreads)
-    k_cell_scan(const int32_t* __restrict__ cnt, int32_t* __restrict__ cst, int32_t* __restrict__ cch, int64_t n) {
+    k_cell_scan(const int32_t* __restrict__ cnt, int32_t* __restrict__ cst, int32_t* __restrict__ cch,
+                int32_t* __restrict__ crowded, int64_t n) {
   pdl_enter();
   __shared__ uint64_t ws[33];
   __shared__ uint64_t tot;
@@ -347,7 +376,7 @@ __global__ void __cluster_dims__(kCellScanCtas, 1, 1) __launch_bounds__(kCellSca
   uint64_t before = ex;
 #pragma unroll
   for (unsigned q = 0; q < kCellScanCtas; ++q) before += q < r ? peer[q] : 0;
-  store_starts(cst, cch, i0, n, v, before);
+  store_starts(cst, cch, crowded, i0, n, v, before);
 }
 
 // The same scan for larger tables in two launches: block totals, then every
@@ -366,7 +395,8 @@ __global__ void __launch_bounds__(kCellScanThreads) k_cell_totals(const int32_t*
 
 __global__ void __launch_bounds__(kCellScanThreads) k_cell_starts(const int32_t* __restrict__ cnt, int64_t n,
                                                                   const uint64_t* __restrict__ tot,
-                                                                  int32_t* __restrict__ cst, int32_t* __restrict__ cch) {
+                                                                  int32_t* __restrict__ cst, int32_t* __restrict__ cch,
+                                                                  int32_t* __restrict__ crowded) {
   pdl_enter();
   __shared__ uint64_t ws[33];
   int32_t v[kCellScanItems];
@@ -377,7 +407,7 @@ __global__ void __launch_bounds__(kCellScanThreads) k_cell_starts(const int32_t*
   uint64_t before;
   block_exclusive<uint64_t>(part, ws, &before);
   const uint64_t ex = block_exclusive<uint64_t>(items_sum(v), ws, nullptr);
-  store_starts(cst, cch, i0, n, v, before + ex);
+  store_starts(cst, cch, crowded, i0, n, v, before + ex);
 }
 
 // Vertex ids to their cells, in arrival order.
@@ -392,40 +422,119 @@ __global__ void __launch_bounds__(kBlock) k_slots(const uint32_t* __restrict__ k
   slot[cst[prob[pb].fbase + pb + keys[v]] + arrival[v]] = (uint32_t)v;
 }
 
-// Sorted positions: the points of a cell by ascending vertex (a point's place
-// is the number of smaller ids in its cell: as many comparisons as the cell
-// has points, against 3^d cells of interactions per point in the step
-// kernel), coordinates and weights in sorted order (plain and in the paired
-// table XP) and the packed cell of every point.  The counts are cleared for
-// the next step.
-template <int D>
-__global__ void __launch_bounds__(kBlock) k_place(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ keys,
-                                                  int64_t K, const float4* __restrict__ x, const float* __restrict__ w,
-                                                  const int32_t* __restrict__ vprob, const ProbDev* __restrict__ prob,
-                                                  const int32_t* __restrict__ cst, int32_t* __restrict__ cnt,
-                                                  int64_t ncnt, const int32_t* __restrict__ cch,
-                                                  int32_t* __restrict__ chunk, uint32_t* __restrict__ svals,
-                                                  float4* __restrict__ xs, float* __restrict__ ws,
-                                                  uint32_t* __restrict__ scell, float4* __restrict__ XP) {
-  pdl_enter();
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (int64_t i = t; i < ncnt; i += (int64_t)gridDim.x * blockDim.x) cnt[i] = 0;
-  if (t >= K) return;
-  const uint32_t v = slot[t];
-  const int pb = vprob[v];
-  const ProbDev pr = prob[pb];
-  const float4 xv = x[v];
-  const uint32_t key = keys[v];
-  const int32_t* cs = cst + pr.fbase + pb;
-  const int32_t q0 = cs[key], q1 = cs[key + 1];
-  int32_t less = 0;
-  int32_t q = q0;
-  for (; q < q1 && (q & 3); ++q) less += slot[q] < v;
-  for (; q + 8 <= q1; q += 8) {  // 16-byte reads, two in flight
-    const uint4 a = *reinterpret_cast<const uint4*>(slot + q), b = *reinterpret_cast<const uint4*>(slot + q + 4);
-    less += (a.x < v) + (a.y < v) + (a.z < v) + (a.w < v) + (b.x < v) + (b.y < v) + (b.z < v) + (b.w < v);
+// Places of a block's points in cells of more than kRankBlock points.  The block
+// holds up to kBlock points of the cell (those of consecutive slots): it sorts
+// their ids, then reads the cell's ids once, finds for each by binary search the
+// first of its own that is larger, and counts there; the prefix sums of the
+// counts are the places.  A thread that compared its point with the whole cell
+// took kBlock / 8 times the operations (99,000 of 100,000 points in one cell, d = 2:
+// 2,280 us, now 180 us; 50,000, d = 3: 1,140 and 83 us).  kRankBlock > kBlock, so only
+// the cells of the block's first and last point can be large.  Every thread of the
+// block calls it; `in` marks those with a point.
+struct RankShared {
+  uint32_t ids[kBlock], sorted[kBlock];
+  int32_t count[kBlock], place[kBlock];
+  int32_t seg[2][2];
+  uint64_t scan[33];
+};
+
+__device__ __noinline__ void rank_large(const uint32_t* __restrict__ slot, bool in, bool last, uint32_t v, int32_t q0,
+                                           int32_t q1, RankShared& sh) {
+  const int tid = threadIdx.x;
+  const int32_t b0 = (int32_t)(blockIdx.x * kBlock);
+  const bool large = in && q1 - q0 > kRankBlock;
+  if (tid == 0 || last) {
+    const int e = last ? 1 : 0;
+    sh.seg[e][0] = large ? q0 : 0;
+    sh.seg[e][1] = large ? q1 : 0;
+    if (tid == 0 && last) sh.seg[0][0] = sh.seg[0][1] = 0;  // one point: handled as the last
   }
-  for (; q < q1; ++q) less += slot[q] < v;
+  __syncthreads();
+  for (int e = 0; e < 2; ++e) {
+    const int32_t c0 = sh.seg[e][0], c1 = sh.seg[e][1];
+    if (c0 == c1 || (e == 0 && c0 == sh.seg[1][0] && c1 == sh.seg[1][1])) continue;
+    const bool mine = large && q0 == c0;
+    const int a = max(c0 - b0, 0), m = min(c1 - b0, kBlock) - a;  // the block's points of the cell
+    if (mine) sh.ids[tid - a] = v;
+    sh.count[tid] = 0;
+    __syncthreads();
+    int r = 0;
+    if (mine) {
+      for (int i = 0; i < m; ++i) r += sh.ids[i] < v;
+      sh.sorted[r] = v;
+    }
+    __syncthreads();
+    const uint32_t lo = sh.sorted[0], hi = sh.sorted[m - 1];
+    int below = 0;
+    for (int64_t i = c0 + tid; i < c1; i += 8 * kBlock) {
+      uint32_t u[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) u[j] = i + j * kBlock < c1 ? slot[i + j * kBlock] : 0xFFFFFFFFu;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        below += u[j] < lo;
+        if (u[j] < lo || u[j] >= hi) continue;
+        int x0 = 0, x1 = m - 1;  // sorted[x0] <= u < sorted[x1]
+        while (x1 - x0 > 1) {
+          const int mid = (x0 + x1) >> 1;
+          if (sh.sorted[mid] <= u[j]) x0 = mid;
+          else x1 = mid;
+        }
+        atomicAdd(&sh.count[x1], 1);
+      }
+    }
+    below = __reduce_add_sync(0xffffffffu, below);
+    if (lane_id() == 0 && below) atomicAdd(&sh.count[0], below);
+    __syncthreads();
+    const int own = sh.count[tid];
+    const uint64_t before = block_exclusive<uint64_t>((uint64_t)(uint32_t)own, sh.scan, nullptr);
+    sh.count[tid] = (int32_t)before + own;
+    __syncthreads();
+    if (mine) sh.place[tid] = sh.count[r];
+    __syncthreads();
+  }
+}
+
+// Sorted positions: the points of a cell by ascending vertex (a point's place
+// is the number of smaller ids in its cell), coordinates and weights in
+// sorted order (plain and in the paired table XP) and the packed cell of every
+// point.  v is the vertex in the thread's slot (0 beyond the last).
+template <int D, bool CROWDED>
+__device__ __forceinline__ void place_points(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ keys,
+                                             uint32_t v, int64_t K, const float4* __restrict__ x, const float* __restrict__ w,
+                                             const int32_t* __restrict__ vprob, const ProbDev* __restrict__ prob,
+                                             const int32_t* __restrict__ cst, const int32_t* __restrict__ cch,
+                                             int32_t* __restrict__ chunk, uint32_t* __restrict__ svals,
+                                             float4* __restrict__ xs, float* __restrict__ ws,
+                                             uint32_t* __restrict__ scell, float4* __restrict__ XP) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool in = t < K;
+  if (!CROWDED && !in) return;
+  const int pb = vprob[v];
+  const uint32_t key = keys[v];
+  const float4 xv = x[v];
+  const int32_t* cs = cst + prob[pb].fbase + pb;
+  const int32_t q0 = cs[key], q1 = cs[key + 1];
+  const bool large = CROWDED && q1 - q0 > kRankBlock;
+  __shared__ RankShared rank;
+  if (CROWDED) {
+    if (__syncthreads_or(large && in))
+      rank_large(slot, in, in && (t == K - 1 || threadIdx.x == kBlock - 1), v, q0, q1, rank);
+    if (!in) return;
+  }
+  const ProbDev pr = prob[pb];
+  int32_t less = 0;
+  if (large) {
+    less = rank.place[threadIdx.x];
+  } else {
+    int32_t q = q0;
+    for (; q < q1 && (q & 3); ++q) less += slot[q] < v;
+    for (; q + 8 <= q1; q += 8) {  // 16-byte reads, two in flight
+      const uint4 a = *reinterpret_cast<const uint4*>(slot + q), b = *reinterpret_cast<const uint4*>(slot + q + 4);
+      less += (a.x < v) + (a.y < v) + (a.z < v) + (a.w < v) + (b.x < v) + (b.y < v) + (b.z < v) + (b.w < v);
+    }
+    for (; q < q1; ++q) less += slot[q] < v;
+  }
   const int64_t p = (int64_t)q0 + less;
   if (cch && !(less & 1)) chunk[cch[pr.fbase + pb + key] + (less >> 1)] = (int32_t)p;
   svals[p] = v;
@@ -445,6 +554,44 @@ __global__ void __launch_bounds__(kBlock) k_place(const uint32_t* __restrict__ s
 #pragma unroll
   for (int m = 0; m < D; ++m) packed |= ((key >> (m * pr.L)) & ((1u << pr.L) - 1u)) << (m * field_bits(D));
   scell[p] = packed;
+}
+
+// The launches of a level without a crowded cell (a flag of the scan) do without
+// the barrier and the registers of the other path: with them in the same body the
+// launch took 20.2 us at 500,000 points, without 16.5 us.
+template <int D>
+__device__ __noinline__ void place_crowded(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ keys,
+                                          uint32_t v, int64_t K, const float4* __restrict__ x, const float* __restrict__ w,
+                                          const int32_t* __restrict__ vprob, const ProbDev* __restrict__ prob,
+                                          const int32_t* __restrict__ cst, const int32_t* __restrict__ cch,
+                                          int32_t* __restrict__ chunk, uint32_t* __restrict__ svals,
+                                          float4* __restrict__ xs, float* __restrict__ ws,
+                                          uint32_t* __restrict__ scell, float4* __restrict__ XP) {
+  place_points<D, true>(slot, keys, v, K, x, w, vprob, prob, cst, cch, chunk, svals, xs, ws, scell, XP);
+}
+
+// Places of all points; the counts are cleared for the next step.
+template <int D>
+__global__ void __launch_bounds__(kBlock, 6) k_place(const uint32_t* __restrict__ slot,
+                                                      const uint32_t* __restrict__ keys, int64_t K,
+                                                      const float4* __restrict__ x, const float* __restrict__ w,
+                                                      const int32_t* __restrict__ vprob,
+                                                      const ProbDev* __restrict__ prob,
+                                                      const int32_t* __restrict__ cst, int32_t* __restrict__ cnt,
+                                                      int64_t ncnt, const int32_t* __restrict__ crowded,
+                                                      const int32_t* __restrict__ cch, int32_t* __restrict__ chunk,
+                                                      uint32_t* __restrict__ svals, float4* __restrict__ xs,
+                                                      float* __restrict__ ws, uint32_t* __restrict__ scell,
+                                                      float4* __restrict__ XP) {
+  pdl_enter();
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t v = t < K ? slot[t] : 0u;  // in flight together with the flag
+  const int32_t any = *crowded;
+  for (int64_t i = t; i < ncnt; i += (int64_t)gridDim.x * blockDim.x) cnt[i] = 0;
+  if (any)
+    place_crowded<D>(slot, keys, v, K, x, w, vprob, prob, cst, cch, chunk, svals, xs, ws, scell, XP);
+  else
+    place_points<D, false>(slot, keys, v, K, x, w, vprob, prob, cst, cch, chunk, svals, xs, ws, scell, XP);
 }
 
 // Cell sums (St, Wt) at cell index idx, and the cell's charge (weighted mean
@@ -903,10 +1050,16 @@ __global__ void __launch_bounds__(kBlock) k_attract(Attract at) {
 // of few problems is two launches in a row without a second stream.  As a sort of
 // 8-bit digits with the coarse sums read back through L2, and the attraction on
 // a second stream, a whole step took 12.2 / 17.4 us of 256 / 1,024 points (d =
-// 2) and 15.4 / 24.5 us of 512 / 1,728 (d = 3); now 8.2 / 13.4 and 11.3 / 19.5.
+// 2) and 15.4 / 24.5 us of 512 / 1,728 (d = 3); now 8.2 / 12.3 and 11.3 / 19.5.
+// With four points per thread a problem may have 2 kSortTile points where the
+// level has few problems and d = 2 (a whole layout of 4,096 points 16.3 -> 15.7
+// ms); for d = 3 the block's one pass over the cells made that slower (24 us
+// for the launch, 17 for the device-wide sequence with its launches overlapped).
 constexpr int kBinCells = 4096;
 constexpr int kFusedProblems = 64;  // most problems of a level whose binning launch does the attraction
-constexpr int kBinBig = kSortTile / (kCellSerial + 1) + 1;  // most large cells of a problem
+constexpr int kBinWide = 2 * kSortTile;  // most points of a problem of a level of at most kFusedProblems
+constexpr int kBinSorted = 64;  // points of a cell from which its ids are sorted (problems of over kSortTile points)
+constexpr int kBinBig = kBinWide / (kCellSerial + 1) + 1;  // most large cells of a problem
 
 // Shared memory of a block: sorted points and weights, slots, cell starts, sums.
 struct BinShape {
@@ -917,7 +1070,7 @@ struct BinShape {
   }
 };
 
-template <int D, int T>
+template <int D, int T, int ITEMS>  // up to ITEMS points per thread
 __global__ void __launch_bounds__(T) k_bin_small(
     const float4* __restrict__ x, const float* __restrict__ w, const ProbDev* __restrict__ prob, int P,
     const uint32_t* __restrict__ bb, uint32_t* __restrict__ bb_next, int32_t* __restrict__ tctr,
@@ -929,7 +1082,7 @@ __global__ void __launch_bounds__(T) k_bin_small(
     attract_rows<T>(at, (int64_t)blockIdx.x - P);
     return;
   }
-  constexpr int ITEMS = 2;  // points per thread: problems of up to 2 T
+  constexpr bool SORT = ITEMS * T > kSortTile;
   extern __shared__ __align__(16) unsigned char bin_raw[];
   float4* sx = reinterpret_cast<float4*>(bin_raw);
   float* sw = reinterpret_cast<float*>(sx + shape.points);
@@ -984,6 +1137,7 @@ __global__ void __launch_bounds__(T) k_bin_small(
     for (int c = c0; c < c1; ++c) {
       const int32_t n = cs[c];
       cs[c] = run;
+      if (SORT && n > kBinSorted) big[atomicAdd(&nbig, 1)] = c;
       cst[pr.fbase + pb + c] = (int32_t)vb + run;
       if (cch) cch[pr.fbase + pb + c] = (int32_t)vb + chk;  // a problem's chunks are listed from its first point on
       run += n;
@@ -1002,6 +1156,30 @@ __global__ void __launch_bounds__(T) k_bin_small(
     if (i < k) slot[cs[key[j]] + arr[j]] = (uint32_t)i;
   }
   __syncthreads();
+  if (SORT && nbig > 0) {
+    // the ids of a crowded cell in order, a warp per cell: a bit per point of the
+    // problem, set for the cell's, the prefix sums of the set bits, and the bits
+    // read off (4,000 points, 99 % of them in one cell: 32 us of the launch, 311 us
+    // when every two points of a cell were compared)
+    uint32_t* bits = reinterpret_cast<uint32_t*>(sx) + (threadIdx.x >> 5) * ((k + 31) / 32);
+    const int lane = lane_id(), words = (k + 31) / 32, per = (words + 31) / 32;
+    for (int b = threadIdx.x >> 5; b < nbig; b += T / 32) {
+      const int q0 = cs[big[b]], q1 = cs[big[b] + 1];
+      for (int i = lane; i < words; i += 32) bits[i] = 0;
+      __syncwarp();
+      for (int q = q0 + lane; q < q1; q += 32) atomicOr(&bits[slot[q] >> 5], 1u << (slot[q] & 31));
+      __syncwarp();
+      const int i0 = min(lane * per, words), i1 = min(i0 + per, words);
+      int own = 0;
+      for (int i = i0; i < i1; ++i) own += __popc(bits[i]);
+      int q = q0 + warp_inclusive(own) - own;
+      for (int i = i0; i < i1; ++i)
+        for (uint32_t m = bits[i]; m; m &= m - 1) slot[q++] = (uint32_t)(32 * i + __ffs(m) - 1);
+      __syncwarp();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) nbig = 0;
+  }
   const int64_t e = (vb + pb + 1) & ~int64_t(1);
 #pragma unroll
   for (int j = 0; j < ITEMS; ++j) {
@@ -1009,7 +1187,16 @@ __global__ void __launch_bounds__(T) k_bin_small(
     if (i >= k) continue;
     const int q0 = cs[key[j]], q1 = cs[key[j] + 1];
     int less = 0;
-    for (int q = q0; q < q1; ++q) less += slot[q] < (uint32_t)i;
+    if (!SORT || q1 - q0 <= kBinSorted) {
+      for (int q = q0; q < q1; ++q) less += slot[q] < (uint32_t)i;
+    } else {  // the first of the sorted ids that is not smaller
+      for (int n = q1 - q0; n > 0;) {
+        const int half = n >> 1;
+        const bool up = slot[q0 + less + half] < (uint32_t)i;
+        less += up ? half + 1 : 0;
+        n = up ? n - half - 1 : half;
+      }
+    }
     const int q = q0 + less;
     const int64_t p = vb + q;
     sx[q] = xv[j];
@@ -1432,8 +1619,18 @@ __device__ __forceinline__ void near_trip(const float4* __restrict__ xp, int j, 
   float4 Q[U][N];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    if (!GUARD || u == 0 || 2 * (j + u * G) < qb) pair_load<D>(xp, j + u * G, Q[u]);
-    else pair_zero<D>(Q[u]);
+    if (!GUARD || u == 0 || 2 * (j + u * G) < qb) {
+      // the coordinates alone, half the bytes through the load unit (99,000 of 100,000
+      // points in one cell: 4.86 -> 3.70 ms a step)
+      if (D == 2 && UNIT) {
+        Q[u][0] = xp[(int64_t)(j + u * G) * N];
+        Q[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      } else {
+        pair_load<D>(xp, j + u * G, Q[u]);
+      }
+    } else {
+      pair_zero<D>(Q[u]);
+    }
   }
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -2544,18 +2741,31 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   // problem (k_bin_small) when the tuning allows it
   int64_t kmax = 0;
   for (int p = 0; p < P; ++p) kmax = std::max(kmax, lb.vbase[p + 1] - lb.vbase[p]);
-  bool bin1 = kmax <= std::min<int64_t>(kSortTile, g_tuning.small_bin_points.load(std::memory_order_relaxed));
+  const int64_t bin_points = g_tuning.small_bin_points.load(std::memory_order_relaxed);
+  bool bin1 = kmax <= (bin_points >= kSortTile && P <= kFusedProblems && d == 2 ? kBinWide : bin_points);
   for (int p = 0; p < P && bin1; ++p) bin1 = (int64_t(1) << (d * lb.L[p])) <= kBinCells;
   BinShape shape{(int)std::max<int64_t>((kmax + 3) / 4 * 4, 4), 1 << (d * std::min(lb.maxL, 12 / d)),
                  (int)(lvl_off(d, std::min(lb.maxL, 12 / d) + 1))};
-  const bool bin_wide = kmax > 512;  // threads of a problem's block: 1,024, else 256, for two points each
+  // (512 threads up to 1,024 points: 13.4 -> 12.3 us a step of one problem for d = 2, the launch of
+  // 168 problems 10.9 -> 9.0 us; one problem of d = 3 9.2 -> 9.8 us, so that keeps 1,024)
+  const int64_t mid = d == 2 || P > kFusedProblems ? 1024 : 512;
+  const auto bin_size = [&](auto DC, auto&& f) {  // threads of a problem's block and points of a thread
+    using std::integral_constant;
+    if (kmax > kSortTile) {
+      if constexpr (decltype(DC)::value == 2) f(integral_constant<int, 1024>(), integral_constant<int, 4>());
+    } else if (kmax > mid) f(integral_constant<int, 1024>(), integral_constant<int, 2>());
+    else if (kmax > 512) f(integral_constant<int, 512>(), integral_constant<int, 1024 / 512>());
+    else f(integral_constant<int, 256>(), integral_constant<int, 2>());
+  };
   if (bin1 && shape.bytes(d) > 40 * 1024)  // with the static arrays above the default limit of 48 KB
     dispatch_d(d, [&](auto DC) {
       constexpr int D = decltype(DC)::value;
-      if ((bin_wide ? cudaFuncSetAttribute(k_bin_small<D, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)shape.bytes(d))
-                    : cudaFuncSetAttribute(k_bin_small<D, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)shape.bytes(d))) != cudaSuccess) {
+      cudaError_t err = cudaSuccess;
+      bin_size(DC, [&](auto TC, auto IC) {
+        err = cudaFuncSetAttribute(k_bin_small<D, decltype(TC)::value, decltype(IC)::value>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shape.bytes(d));
+      });
+      if (err != cudaSuccess) {
         (void)cudaGetLastError();
         bin1 = false;  // the device-wide sequence then
       }
@@ -2586,7 +2796,8 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   int32_t* tctr;
   const bool own_step = step_override <= 0.0f;  // the step length comes from the box, not from the caller
   if (!scale_tab && own_step) VMO_TRY(make_scale_tab(o, iters, &scale_tab, s, sc));
-  VMO_TRY(sc.alloc(&tctr, 1));
+  VMO_TRY(sc.alloc(&tctr, 2));
+  int32_t* crowded = tctr + 1;
   VMO_CUDA(cudaMemsetAsync(tctr, 0xFF, sizeof(int32_t), s));  // -1: k_keys advances it at every step
   vmo_status st = VMO_OK;
   // streams: the layout's, the level's own, or none for a few steps (making them
@@ -2630,15 +2841,13 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
       }
       if (fork) cudaEventRecord(ss->join, side);
       if (bin1) {
-        auto bin = [&](auto kernel, auto TC) {
+        bin_size(DC, [&](auto TC, auto IC) {
           constexpr int T = decltype(TC)::value;
           at.mid_blocks = (lb.n_mid * kMidLanes + T - 1) / T;
           const unsigned blocks = (unsigned)(P + (fused ? at.blocks<T>() : 0));
-          launch(kernel, blocks, T, shape.bytes(D), ms, x, lb.w, lb.prob.ptr, P, cur, nxt, tctr,
-                 keys_out && t == 0 ? keys : nullptr, svals, xs, ws, scell, cst, XP, CP, cch, chunk, shape, at);
-        };
-        if (bin_wide) bin(k_bin_small<D, 1024>, std::integral_constant<int, 1024>());
-        else bin(k_bin_small<D, 256>, std::integral_constant<int, 256>());
+          launch(k_bin_small<D, T, decltype(IC)::value>, blocks, T, shape.bytes(D), ms, x, lb.w, lb.prob.ptr, P, cur, nxt,
+                 tctr, keys_out && t == 0 ? keys : nullptr, svals, xs, ws, scell, cst, XP, CP, cch, chunk, shape, at);
+        });
         if (keys_out && t == 0) cudaMemcpyAsync(keys_out, keys, K * 4, cudaMemcpyDeviceToDevice, ms);
       } else {
         auto keys_kernel = K >= kKeyItemsMin ? k_keys<D, 4> : k_keys<D, 1>;
@@ -2646,14 +2855,15 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
                lb.prob.ptr, cur, keys, arrival, cnt, P, nxt, tctr);
         if (keys_out && t == 0) cudaMemcpyAsync(keys_out, keys, K * 4, cudaMemcpyDeviceToDevice, ms);
         if (one_cluster) {
-          launch(k_cell_scan, kCellScanCtas, kCellScanThreads, 0, ms, cnt, cst, cch, ncnt);
+          launch(k_cell_scan, kCellScanCtas, kCellScanThreads, 0, ms, cnt, cst, cch, crowded, ncnt);
         } else {
           launch(k_cell_totals, scan_blocks, kCellScanThreads, 0, ms, cnt, ncnt, tot);
-          launch(k_cell_starts, scan_blocks, kCellScanThreads, 0, ms, cnt, ncnt, tot, cst, cch);
+          launch(k_cell_starts, scan_blocks, kCellScanThreads, 0, ms, cnt, ncnt, tot, cst, cch,
+                 crowded);
         }
         launch(k_slots, grid_for(K, kBlock), kBlock, 0, ms, keys, arrival, K, lb.vprob.ptr, lb.prob.ptr, cst, slot);
         launch(k_place<D>, grid_for(K, kBlock), kBlock, 0, ms, slot, keys, K, x, lb.w, lb.vprob.ptr, lb.prob.ptr, cst,
-               cnt, ncnt, cch, chunk, svals, xs, ws, scell, XP);
+               cnt, ncnt, crowded, cch, chunk, svals, xs, ws, scell, XP);
         if (lb.bricks > 0)
           launch(k_cells<D>, (unsigned)lb.bricks, kCellsBlock, 0, ms, lb.bprob.ptr, lb.prob.ptr, xs, ws, cst, St, Wt,
                  CP, done);

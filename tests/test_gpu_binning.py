@@ -75,3 +75,38 @@ def test_device_wide_binning_many_problems(V):
             V.set_tuning(19456, 10, 4, small)
             out.append(V.batch_layout(mats, V.Params(d=d, iters=9, seed=4))[0].cpu().numpy())
         assert np.array_equal(out[0].view(np.uint32), out[1].view(np.uint32))
+
+
+@pytest.mark.parametrize("d,k,sizes", [
+    (2, 2100, (65, 64)), (2, 3000, (1024, 1025)), (2, 4096, (4096,)), (2, 4095, (2000, 2000)), (2, 4097, (4097,)),
+    (2, 9000, (1025, 1100, 4000)), (3, 5000, (2500, 2499)), (3, 2049, (1025,)), (4, 6000, (3000, 1024))])
+def test_crowded_cells(V, O, d, k, sizes):
+    """Cells of hundreds and thousands of points, side by side in the sorted order:
+    the vertex order within them shows in the bits of the sums, so the step is
+    compared with the oracle's and, where a problem fits one block, with that
+    binning bit by bit."""
+    A = W.random_symmetric(k, 6, seed=k)
+    hg, ref = V.Hypergraph.from_matrix(A), O.build_from_matrix("symmetric", A)
+    rng = np.random.default_rng(k + d)
+    side = float(k) ** (1.0 / d)
+    x = np.zeros((k, 4), dtype=np.float32)
+    x[:, :d] = rng.random((k, d)) * side
+    n = 0
+    for i, size in enumerate(sizes):
+        x[n:n + size, :d] = side * (0.3 + 0.2 * i) + 1e-3 * rng.standard_normal((size, d))
+        n += size
+    x = x[rng.permutation(k)]
+    p = V.Params(d=d)
+    V.set_tuning(19456, 10, 4, 0)
+    xg, yg, kg, L = hg.layout_step(torch.as_tensor(x).cuda(), 0.25, p)
+    xo, yo, ko, Lo = O.layout_step(ref, d, x.astype(np.float64), 0.25)
+    assert L == Lo and np.array_equal(kg.cpu().numpy().view(np.uint32), ko)
+    yn = yg.cpu().numpy().astype(np.float64)
+    # (TOL is for clouds about their own width from the origin; where the cloud is the
+    # cluster itself, 1e-3 wide at 20, single-precision cell centres alone are 1e-3 off)
+    if sum(sizes) < k:
+        assert np.linalg.norm(yn[:, :d] - yo[:, :d]) <= TOL * np.linalg.norm(yo[:, :d])
+    V.set_tuning(19456, 10, 4, 2048)
+    xs, ys, ks, _ = hg.layout_step(torch.as_tensor(x).cuda(), 0.25, p)
+    assert torch.equal(ys.view(torch.int32), yg.view(torch.int32))
+    assert torch.equal(xs.view(torch.int32), xg.view(torch.int32)) and torch.equal(ks, kg)
