@@ -259,7 +259,7 @@ vmo_status vmo_bisect(vmo_hg hg, int32_t d, const float* coords, const int32_t* 
  * counterpart: this is a deployment variant of vmo_bisect, without the handle.
  * Same arguments, results and rules as vmo_bisect (verts must be valid rows of
  * coords), but every intermediate lives in one fixed device array that the
- * library reserves on each GPU that loads it (about 5.3 MB, kept until the
+ * library reserves on each GPU that loads it (about 2.75 MB, kept until the
  * process exits) instead of in freshly allocated memory; no cudaMalloc or
  * other allocation is made.  Limit: nverts <= 131072, larger inputs return
  * VMO_ERR_INVALID.  Every call looks up the array's device address
@@ -444,8 +444,9 @@ vmo_status vmo_finegrain_coords(vmo_hg hg, const float* bipartite_coords, float*
  *     warps per SM);
  *   radix_max_bits: widest digit of the LSD radix sorts, 8, 9 or
  *     10 (default 10: fewest passes);
- *   assign_items: positions per thread of the Lloyd assignment, 1, 2, 4 or
- *     8 (default 4; fewer are used when the blocks would not fill the GPU);
+ *   assign_items: positions per thread of the Lloyd assignment of nodes of
+ *     more than 1.8 M points, 1, 2, 4 or 8 (default 4; fewer are used when
+ *     the blocks would not fill the GPU);
  *   small_bin_points: a layout level whose problems all have at most this
  *     many vertices (0 ... 2,048) is binned by one block per problem (keys,
  *     sorted copies and cell charges in one launch) instead of the device-wide
