@@ -5,7 +5,7 @@
 // model of the joined pattern is built once, and every connected component of
 // every matrix becomes one problem of the layout batch and one root of the
 // level-synchronous recursion.  All per-problem arithmetic (grid, group size,
-// sort segment, step length, k-means++ draws keyed by heap number) depends on
+// sorted order, step length, k-means++ draws keyed by heap number) depends on
 // the problem alone, so each matrix's permutation is the one it gets when
 // ordered by itself.
 #include <algorithm>

@@ -4,9 +4,9 @@
 // One step of a level, for every problem of a batch at once:
 //   keys      cell of every point on a uniform grid over the bounding cube
 //             (fp32, no FMA), row-major key of the finest cell
-//   sort      stable segmented radix sort of (key, vertex)
-//   gather    points copied in key order; first point of every finest cell
-//             recorded in a dense table
+//   sort      counting sort by cell, the points of a cell by vertex; first
+//             point of every finest cell recorded in a dense table, points
+//             copied in that order
 //   aggregate per cell weight and weighted mean: finest cells from their
 //             points, coarser cells from their 2^d children (fixed order)
 //   attract   y_n = sum_j c_j (x_n - z_j) (2-pin nets: c/2 (x_n - x_u))
