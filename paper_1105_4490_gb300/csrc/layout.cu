@@ -1064,11 +1064,25 @@ constexpr int kBinBig = kBinWide / (kCellSerial + 1) + 1;  // most large cells o
 // Shared memory of a block: sorted points and weights, slots, cell starts, sums.
 struct BinShape {
   int points, cells, sums;  // capacities: points, finest cells, cells of all levels >= 2
-  size_t bytes(int d) const {
+  constexpr size_t bytes(int d) const {
     return (size_t)points * (sizeof(float4) + sizeof(float) + sizeof(uint32_t)) + (size_t)(cells + 1) * sizeof(int32_t) +
            (size_t)sums * (d + 1) * sizeof(float);
   }
 };
+
+// Shared-memory limit of the kernel for blocks of T threads with ITEMS points
+// each: its largest shape.  The limit belongs to the function, for all host
+// threads, and a smaller one set by one of them would have another's larger
+// launch refused, so it is this constant whatever shape a level has.
+template <int D, int T, int ITEMS>
+constexpr size_t bin_limit() {
+  constexpr int L = 12 / D;  // finest level of at most kBinCells cells
+  static_assert((1 << (D * L)) <= kBinCells, "cells of the finest level");
+  return BinShape{T * ITEMS, 1 << (D * L), ((1 << (D * (L + 1))) - 1) / ((1 << D) - 1)}.bytes(D);
+}
+static_assert(bin_limit<2, 1024, 4>() <= 220 * 1024 && bin_limit<3, 1024, 2>() <= 220 * 1024 &&
+                  bin_limit<4, 1024, 2>() <= 220 * 1024,
+              "a block's shared memory, with room for the static arrays");
 
 template <int D, int T, int ITEMS>  // up to ITEMS points per thread
 __global__ void __launch_bounds__(T) k_bin_small(
@@ -2762,8 +2776,9 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
       constexpr int D = decltype(DC)::value;
       cudaError_t err = cudaSuccess;
       bin_size(DC, [&](auto TC, auto IC) {
-        err = cudaFuncSetAttribute(k_bin_small<D, decltype(TC)::value, decltype(IC)::value>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shape.bytes(d));
+        constexpr int T = decltype(TC)::value, ITEMS = decltype(IC)::value;
+        err = cudaFuncSetAttribute(k_bin_small<D, T, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)bin_limit<D, T, ITEMS>());
       });
       if (err != cudaSuccess) {
         (void)cudaGetLastError();
