@@ -19,6 +19,7 @@ thread_local bool g_pdl = false;
 void set_error(const std::string& msg) { g_last_error = msg; }
 
 vmo_status cuda_fail(cudaError_t e, const char* what, const char* file, int line) {
+  (void)cudaGetLastError();  // collected: the next call starts without it
   char buf[512];
   snprintf(buf, sizeof(buf), "%s: %s (%s:%d)", what, cudaGetErrorString(e), file, line);
   set_error(buf);

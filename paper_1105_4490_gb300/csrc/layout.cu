@@ -120,6 +120,14 @@ __device__ inline int64_t rowmajor(const int32_t* c, int side) {
 
 __host__ __device__ constexpr int field_bits(int D) { return D == 4 ? 8 : 30 / D; }
 
+// Coordinate m of a packed cell, kept inside the grid whatever the word holds
+// (the ranges around a cell outside it would be empty or negative, and the
+// loops over them would not end).
+template <int D>
+__device__ __forceinline__ int32_t cell_field(uint32_t packed, int m, int side) {
+  return min((int32_t)((packed >> (m * field_bits(D))) & ((1u << field_bits(D)) - 1)), side - 1);
+}
+
 // Block-level bounding-box accumulation into ordered-uint min/max slots.
 // uniform: every valid thread of the block belongs to problem pblock (the
 // block result is then published once for pblock); otherwise each valid
@@ -1810,7 +1818,7 @@ __global__ void __launch_bounds__(kStepBlock, step_min_blocks(MODE)) k_repulse_u
       for (int m = 0; m < D; ++m) g.nx[t][m] = make_float2(-comp(xn[t], m), -comp(xn[t], m));
     int32_t c[D];
 #pragma unroll
-    for (int m = 0; m < D; ++m) c[m] = (int32_t)((packed >> (m * field_bits(D))) & ((1u << field_bits(D)) - 1));
+    for (int m = 0; m < D; ++m) c[m] = cell_field<D>(packed, m, side);
     // near field: rows of 3 cells along coordinate 0 around the target's cell
     const int32_t* cs = cst + pr.fbase + pb;
     const float4* xp = XP + ((pr.vbase + pb + 1) >> 1) * N;  // the problem's first pair
@@ -2039,7 +2047,7 @@ __global__ void __launch_bounds__(kSplitBlock, 4) k_repulse_split(
   }
   int32_t c[D];
 #pragma unroll
-  for (int m = 0; m < D; ++m) c[m] = (int32_t)((packed >> (m * field_bits(D))) & ((1u << field_bits(D)) - 1));
+  for (int m = 0; m < D; ++m) c[m] = cell_field<D>(packed, m, side);
   if (threadIdx.x < 2) rounds[threadIdx.x] = 0;
   if (producer) {  // near field: the lane's pairs of the 3^(d-1) rows as one sequence
     for (int o = r; o < NR; o += R) {

@@ -1393,6 +1393,7 @@ static cudaError_t launch_two_means(const OrderState& st, int N, int km_iters, i
       return launch_two_means<D, T>(st, N, km_iters, 8, share * 2, s);
     }
   }
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;  // as launch(): nothing after a refused one
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaLaunchKernelEx(&cfg, kernel, (const float4*)st.xo, (const int32_t*)st.ord, st.nodes,
                             (const uint64_t*)st.seeds, km_iters, st.lab, st.vrec, cap, (int)stream);

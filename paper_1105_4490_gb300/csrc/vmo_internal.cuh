@@ -255,8 +255,13 @@ __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// A kernel of a sequence reads what the ones before it wrote, so after a refused
+// launch (or copy) nothing more is launched until the error has been collected
+// by VMO_LAUNCHED: kernels on unwritten tables would read out of range or loop
+// on what they find there.
 template <class... KArgs, class... Args>
 inline void launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
+  if (cudaPeekAtLastError() != cudaSuccess) return;
   g_launches.fetch_add(1, std::memory_order_relaxed);
   if (g_pdl) {
     cudaLaunchConfig_t cfg = {};
