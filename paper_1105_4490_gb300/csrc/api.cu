@@ -372,6 +372,10 @@ cudaMemPool_t handle_pool() {
     (void)cudaGetLastError();
     return nullptr;
   }
+  // Kept for good: the fences of the handles (vmo_hg_s) are then parts of its
+  // 2 MB block, which a fence alone would map and unmap (180 us a handle).
+  void* anchor = nullptr;
+  if (cudaMalloc(&anchor, 16) != cudaSuccess) (void)cudaGetLastError();
   g_handle_pools.emplace_back(dev, pool);
   return pool;
 }
@@ -414,6 +418,8 @@ vmo_status vmo_build_hypergraph(const vmo_csr* a, vmo_model model, const float* 
   // the handle's arrays are freed in vmo_destroy, whatever stream built them
   std::unique_ptr<vmo_hg_s, void (*)(vmo_hg)> h(new vmo_hg_s(), vmo_destroy);
   cudaGetDevice(&h->device);
+  VMO_CUDA(cudaMalloc(&h->fence, 16));
+  g_device_allocs.fetch_add(1, std::memory_order_relaxed);
   cudaMemPool_t pool = handle_pool();
   std::unique_ptr<DevArrayStreamScope> scope(pool ? new DevArrayStreamScope(s, pool) : nullptr);
   VMO_TRY(build_model(a, model, h.get(), s));
@@ -760,16 +766,19 @@ vmo_status vmo_stats_get(vmo_stats* out) {
   return VMO_OK;
 }
 
-// Waits for the device, as freeing each array with cudaFree would: the arrays
-// may be in use on any stream (vmo_hg_arrays).
+// The arrays may be in use on any stream (vmo_hg_arrays).  Freeing the fence, a
+// plain allocation, waits for all work on the device; the pool's memory is then
+// given back without an order of its own.  (cudaDeviceSynchronize would be
+// invalid while any thread captures a stream, as every layout does for its
+// steps: it ends the capture and returns without having waited.)
 void vmo_destroy(vmo_hg hg) {
   if (!hg) return;
   int dev = hg->device;
   cudaGetDevice(&dev);
   if (dev != hg->device) cudaSetDevice(hg->device);
-  cudaDeviceSynchronize();
-  for (auto* a : {&hg->adj_ptr, &hg->adj, &hg->net_ptr, &hg->pins, &hg->vtx_ptr, &hg->vnets}) a->astream = nullptr;
-  hg->weight.astream = nullptr;
+  cudaFree(hg->fence);
+  for (auto* a : {&hg->adj_ptr, &hg->adj, &hg->net_ptr, &hg->pins, &hg->vtx_ptr, &hg->vnets}) a->async = false;
+  hg->weight.async = false;
   const int own = hg->device;
   delete hg;
   if (dev != own) cudaSetDevice(dev);

@@ -2938,7 +2938,11 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
       if (ok) {
         cst0 = step(0);
         if (cst0 == VMO_OK) cst0 = step(1);
-        ok = cudaStreamEndCapture(ms, &g) == cudaSuccess && cst0 == VMO_OK;
+        // a capture that another thread has ended (by a device-wide wait) says
+        // nothing about the steps: they are launched directly then
+        const cudaError_t ended = cudaStreamEndCapture(ms, &g);
+        if (ended == cudaErrorStreamCaptureInvalidated) cst0 = VMO_OK;
+        ok = ended == cudaSuccess && cst0 == VMO_OK;
       }
       if (ok) ok = cudaGraphInstantiate(&ge, g, 0) == cudaSuccess;
       const uint64_t per_graph = g_launches.load() - before;

@@ -181,6 +181,7 @@ struct vmo_hg_s {
   int64_t nadj = 0, npins = 0, nvnets = 0;
   bool has_weight = false;
   int device = 0;
+  void* fence = nullptr;  // of a user's handle: freeing it waits for the device (vmo_destroy)
 };
 
 namespace vmo {
