@@ -2010,6 +2010,13 @@ __device__ __forceinline__ void pair_terms(const float4* P, const float2* nx, fl
   }
 }
 
+// The end of a round, where the producer warps and the adding warp arrive from
+// different code: a barrier of its own number, which counts the block's
+// threads wherever they come from (__syncthreads() wants one place for all).
+__device__ __forceinline__ void split_round_barrier() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kSplitBlock) : "memory");
+}
+
 template <int D>
 __global__ void __launch_bounds__(kSplitBlock, 4) k_repulse_split(
     const float4* __restrict__ xs, const float* __restrict__ ws, const float4* __restrict__ XP,
@@ -2180,7 +2187,7 @@ __global__ void __launch_bounds__(kSplitBlock, 4) k_repulse_split(
         }
         if (t + 1 < all) load_far();
       }
-      __syncthreads();
+      split_round_barrier();
     }
     return;
   }
@@ -2205,7 +2212,7 @@ __global__ void __launch_bounds__(kSplitBlock, 4) k_repulse_split(
   };
   for (int t = 0; t < all; ++t) {
     if (t > 0) add_round(t - 1);
-    __syncthreads();
+    split_round_barrier();
   }
   if (all > 0) add_round(all - 1);
   // even + odd sources, then the G lanes of the target with the same xor tree
