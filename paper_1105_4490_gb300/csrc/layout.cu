@@ -1905,6 +1905,10 @@ constexpr int kSplitS = 4 * kSplitR;                // pairs of a round
 constexpr int kSplitWarps = 4;                      // producer warps
 constexpr int kSplitLanes = kSplitWarps * 32 / kSplitR;  // target lanes of a block: 16, two threads each of the last warp
 constexpr int kSplitBlock = 32 * (kSplitWarps + 1);
+static_assert(32 % kSplitLanes == 0 && kSplitLanes % kGroupMax == 0, "a block's lanes: whole targets of one problem");
+// Pair indices fit 32 bits: two targets per thread take over at kPairThreadsMin, so a
+// level has fewer points than that, and a grid less than 2^4 cells a point.
+static_assert(kPairThreadsMin * 16 * 2 < INT32_MAX, "pairs of a level's cell tables");
 constexpr int kSplitPitch = kSplitS + 1;            // terms between two halves: 16-byte reads of 8 threads miss no bank twice
 
 // Far-field rows of a target lane as one sequence over the levels (the rows
@@ -2574,7 +2578,7 @@ int group_size(int64_t k) {
   // GPU, that cost is all that remains (measured: 4 / 2 lanes for <= 512 /
   // 4,096 vertices order the 4,096-matrix batch 17% faster than 16 / 4, a
   // single small matrix 3% slower).
-  if (k <= 512) return 4;
+  if (k <= 512) return kGroupMax;
   if (k <= 4096) return 2;
   return 1;
 }

@@ -7,6 +7,8 @@
 
 namespace vmo {
 
+constexpr int kGroupMax = 4;  // most lanes per target of the step kernels
+
 // Per-problem constants of one level of a batch (device copy in LevelBatch).
 struct ProbDev {
   int64_t vbase;   // first vertex of the problem in the level
@@ -18,7 +20,7 @@ struct ProbDev {
   int32_t k;       // vertices
   int32_t L;       // finest grid level
   int32_t side;    // side of the random initial box
-  int32_t group;   // lanes per target in the step kernel (power of two <= 32)
+  int32_t group;   // lanes per target in the step kernel (power of two <= kGroupMax)
 };
 
 // One level of the multilevel hierarchy for a batch of independent problems
