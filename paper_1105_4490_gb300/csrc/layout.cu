@@ -1907,7 +1907,7 @@ constexpr int kSplitLanes = kSplitWarps * 32 / kSplitR;  // target lanes of a bl
 constexpr int kSplitBlock = 32 * (kSplitWarps + 1);
 static_assert(32 % kSplitLanes == 0 && kSplitLanes % kGroupMax == 0, "a block's lanes: whole targets of one problem");
 // Pair indices fit 32 bits: two targets per thread take over at kPairThreadsMin, so a
-// level has fewer points than that, and a grid less than 2^4 cells a point.
+// level has fewer points than that, and its grids at most 17 cells a point (d = 4).
 static_assert(kPairThreadsMin * 16 * 2 < INT32_MAX, "pairs of a level's cell tables");
 constexpr int kSplitPitch = kSplitS + 1;            // terms between two halves: 16-byte reads of 8 threads miss no bank twice
 
@@ -2002,8 +2002,8 @@ __device__ __forceinline__ void pair_terms(const float4* P, const float2* nx, fl
   float2 dx[4];
   dx[0] = __fadd2_rn(make_float2(P[0].x, P[0].y), nx[0]);
   dx[1] = __fadd2_rn(make_float2(P[0].z, P[0].w), nx[1]);
-  dx[2] = dx[3] = make_float2(0.f, 0.f);
-  if (D > 2) dx[2] = __fadd2_rn(make_float2(P[1].x, P[1].y), nx[D > 2 ? 2 : 0]);
+  dx[2] = __fadd2_rn(make_float2(P[1].x, P[1].y), nx[2]);
+  dx[3] = make_float2(0.f, 0.f);
   if (D > 3) dx[3] = __fadd2_rn(make_float2(P[1].z, P[1].w), nx[D > 3 ? 3 : 0]);
   const float2 g = pair_factor<D, UNIT>(dx, w);
   terms[at] = make_float4(g.x, dx[0].x, dx[1].x, dx[2].x);
@@ -2031,7 +2031,8 @@ __global__ void __launch_bounds__(kSplitBlock, 4) k_repulse_split(
     float4* __restrict__ x, float4* __restrict__ y_out, uint32_t* __restrict__ bb_next) {
   pdl_enter();
   constexpr int N = Pair<D>::N, R = kSplitR, S = kSplitS, PITCH = kSplitPitch, LN = kSplitLanes;
-  constexpr int NR = D == 2 ? 3 : (D == 3 ? 9 : 27);  // near-field rows
+  static_assert(D > 2, "the sums of d = 2 are too short");
+  constexpr int NR = D == 3 ? 9 : 27;  // near-field rows
   __shared__ float4 terms[2][LN * 2 * PITCH];
   __shared__ float terms3[2][D > 3 ? LN * 2 * PITCH : 1];
   __shared__ int32_t rq[LN][NR][2];     // near rows: [qa, qb)
@@ -2206,7 +2207,7 @@ __global__ void __launch_bounds__(kSplitBlock, 4) k_repulse_split(
       const float4 v = in[half + f];
       F[0] = __fmaf_rn(v.x, v.y, F[0]);
       F[1] = __fmaf_rn(v.x, v.z, F[1]);
-      if (D > 2) F[D > 2 ? 2 : 0] = __fmaf_rn(v.x, v.w, F[D > 2 ? 2 : 0]);
+      F[2] = __fmaf_rn(v.x, v.w, F[2]);
       if (D > 3) F[D > 3 ? 3 : 0] = __fmaf_rn(v.x, in3[half + f], F[D > 3 ? 3 : 0]);
     }
   };
@@ -2911,17 +2912,19 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
         launch(kernel, grid_for(nth, kStepBlock), kStepBlock, 0, ms, xs, ws, XP, svals, scell, cst, CP, yatt, wprob,
                lb.prob.ptr, nth, chunk, cch, kappa, s0, scale_tab, tctr, step_override, x, y_out, nxt, icount);
       };
-      if (icount)
+      if (icount) {
         step_launch(k_repulse_update<D, true, kStepPlain>, lb.threads, lb.wprob.ptr);
-      else if (pair)
+      } else if (pair) {
         step_launch(k_repulse_update<D, false, kStepPair>, lb.threads2, lb.wprob2.ptr);
-      else if (D > 2 && lb.threads <= small / 8 * 5)
-        launch(k_repulse_split<D>, (unsigned)(lb.threads / kSplitLanes), kSplitBlock, 0, ms, xs, ws, XP, svals, scell,
-               cst, CP, yatt, lb.wprob.ptr, lb.prob.ptr, kappa, s0, scale_tab, tctr, step_override, x, y_out, nxt);
-      else if (D == 2 && lb.threads <= small)
-        step_launch(k_repulse_update<2, false, kStepPipe>, lb.threads, lb.wprob.ptr);
-      else
+      } else if (lb.threads <= (D > 2 ? small / 8 * 5 : small)) {
+        if constexpr (D > 2)
+          launch(k_repulse_split<D>, (unsigned)(lb.threads / kSplitLanes), kSplitBlock, 0, ms, xs, ws, XP, svals, scell,
+                 cst, CP, yatt, lb.wprob.ptr, lb.prob.ptr, kappa, s0, scale_tab, tctr, step_override, x, y_out, nxt);
+        else
+          step_launch(k_repulse_update<D, false, kStepPipe>, lb.threads, lb.wprob.ptr);
+      } else {
         step_launch(k_repulse_update<D, false, kStepPlain>, lb.threads, lb.wprob.ptr);
+      }
       if (timed) stats_time_end(ms, (uint64_t)K);
       cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return cuda_fail(e, "layout step", __FILE__, __LINE__);

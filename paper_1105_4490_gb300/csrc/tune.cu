@@ -1,7 +1,8 @@
 // Autotuner of the launch shapes that never change a result: the largest
-// step launch that takes the two-rows-in-flight variant of the step kernel,
-// the widest radix digit, the positions per thread of
-// the Lloyd assignment, and the largest problem whose level is binned by one
+// step launch that takes the step kernel of small levels (two rows in flight
+// for d = 2; split terms, up to five eighths of it, for d = 3 and 4), the
+// widest radix digit, the positions per thread of the Lloyd assignment of
+// nodes beyond a cluster, and the largest problem whose level is binned by one
 // block per problem.  Every candidate orders the caller's matrices
 // through vmo_batch_order; the fastest (median of the repetitions, CUDA
 // events on the caller's stream) becomes the process-wide setting.  The

@@ -230,9 +230,11 @@ void stats_time_end(cudaStream_t s, uint64_t points);
 // was launched without the attribute).
 extern thread_local bool g_pdl;
 
-// Launch-shape choices that never change a result (tune.cu): the largest
-// step launch that takes the variant with two far-field rows in flight, the
-// widest radix digit, and the positions per thread of the Lloyd assignment.
+// Launch-shape choices that never change a result (tune.cu): the largest step
+// launch that takes the step kernel of small levels (two far-field rows in
+// flight for d = 2, split terms up to five eighths of it for d = 3 and 4), the
+// widest radix digit, the positions per thread of the Lloyd assignment of nodes
+// beyond a cluster, and the largest problem binned by one block.
 // Process-wide; set by vmo_set_tuning / vmo_autotune.
 struct Tuning {
   std::atomic<int64_t> small_step_threads{152 * 4 * 32};
