@@ -68,3 +68,43 @@ def test_separator_row_lengths(V, O, deg):
     want, tree_o = O.order(ref, 2, x, seed=2, min_part=16)
     assert np.array_equal(perm.cpu().numpy(), want)
     assert np.array_equal(tree["nsep"].cpu().numpy(), tree_o["nsep"])
+
+
+def _chains(n):
+    a = np.arange(n - 1)
+    yield "ascending", _sym(n, a, a + 1)
+    yield "descending", _sym(n, n - 1 - a, n - 2 - a)
+    yield "comb", _sym(n, np.concatenate([a[::2], a[:-2:2]]), np.concatenate([a[::2] + 1, a[:-2:2] + 2]))
+    yield "grid", _sym(n, np.concatenate([a, a[:-99]]), np.concatenate([a + 1, a[:-99] + 100]))
+
+
+@pytest.mark.parametrize("model", ("symmetric", "bipartite", "rownet", "colnet", "finegrain"))
+def test_components_of_chains(V, O, model):
+    for name, A in _chains(20000):
+        B = W.csr_from_coo(A.m, A.n, np.concatenate([np.repeat(np.arange(A.m), np.diff(A.rowptr)), np.arange(A.m)]),
+                           np.concatenate([A.colidx, np.arange(A.m)]), "diag")
+        hg, ref = V.Hypergraph.from_matrix(B, model), O.build_from_matrix(model, B)
+        assert np.array_equal(hg.components().cpu().numpy(), O.components(ref)), name
+
+
+def test_chains_take_no_longer_than_other_patterns(V):
+    """A tridiagonal pattern, whose edges all link at once, costs about what a
+    random one of the same size does (it took 30 times as long)."""
+    n = 1_000_000
+    a = np.arange(n - 1)
+    d = np.arange(n)
+    best = []
+    for p, q in ((a, a + 1), (np.random.default_rng(1).integers(0, n, n - 1), np.random.default_rng(2).integers(0, n, n - 1))):
+        A = W.csr_from_coo(n, n, np.concatenate([p, q, d]), np.concatenate([q, p, d]), "chain")
+        hg = V.Hypergraph.from_matrix(A, "bipartite")
+        t = []
+        for _ in range(5):
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            torch.cuda.synchronize()
+            ev[0].record()
+            hg.components()
+            ev[1].record()
+            torch.cuda.synchronize()
+            t.append(ev[0].elapsed_time(ev[1]))
+        best.append(min(t))
+    assert best[0] < 5 * best[1], best
