@@ -445,8 +445,8 @@ vmo_status vmo_finegrain_coords(vmo_hg hg, const float* bipartite_coords, float*
  *   radix_max_bits: widest digit of the LSD radix sorts, 8, 9 or
  *     10 (default 10: fewest passes);
  *   assign_items: positions per thread of the Lloyd assignment of nodes of
- *     more than 1.8 M points, 1, 2, 4 or 8 (default 4; fewer are used when
- *     the blocks would not fill the GPU);
+ *     more than 1.8 M (d = 2), 1.6 M (d = 3) or 1.25 M points (d = 4), 1, 2, 4
+ *     or 8 (default 4; fewer are used when the blocks would not fill the GPU);
  *   small_bin_points: a layout level whose problems all have at most this
  *     many vertices (0 ... 2,048) is binned by one block per problem (keys,
  *     sorted copies and cell charges in one launch) instead of the device-wide

@@ -1355,12 +1355,17 @@ __global__ void __launch_bounds__(T) k_two_means(const float4* __restrict__ xo, 
 // 2-means of every node of the table (Algorithm 5), leaving the final labels
 // in lab (position order), the node fields z1, z2, n1, n2, state and, when
 // st.vrec is set, the vertex records of the separator phase.  One cluster per
-// node; false: a node of more than kClusterNodeMax points (max_size is the
-// largest; a cluster of 8 holds the labels of that many), to be done by the
-// launch sequence below.  At that size a round of one cluster streams 28 MB
-// from L2 through 16 SMs, about what the launch sequence needs for it.
+// node; false: a node of more than cluster_node_max points (max_size is the
+// largest), to be done by the launch sequence below.
 constexpr int kClusterSmem = 220 * 1024;
-constexpr int64_t kClusterNodeMax = 8 * (int64_t)(kClusterSmem - 16);
+constexpr int64_t kClusterNodeMax = 8 * (int64_t)(kClusterSmem - 16);  // a cluster of 8 holds their labels
+
+// Where one cluster streams a node it is bound by the arithmetic of its 16 SMs,
+// which grows with d, the launch sequence by its launches and passes.  Bisection
+// of 1.4 / 1.6 / 1.75 M points by a cluster: d = 3 0.82 / 0.90 / 0.97 ms (sequence
+// 0.88 / 0.90 / 0.90), d = 4 0.99 / 1.10 / 1.17 (0.94 / 1.00 / 1.00), d = 2 0.70 / 0.76 /
+// 0.86 (1.00 / 1.24 / 1.26), so that takes as many as fit.
+static int64_t cluster_node_max(int d) { return d == 2 ? kClusterNodeMax : d == 3 ? 1600000 : 1250000; }
 
 template <int D, int T>
 static cudaError_t launch_two_means(const OrderState& st, int N, int km_iters, int C, int share, cudaStream_t s) {
@@ -1401,7 +1406,7 @@ static cudaError_t launch_two_means(const OrderState& st, int N, int km_iters, i
 
 static vmo_status two_means_clusters(OrderState& st, int N, int64_t max_size, int d, int km_iters, cudaStream_t s,
                                      bool* done) {
-  *done = max_size <= kClusterNodeMax;
+  *done = max_size <= cluster_node_max(d);
   if (!*done || N == 0) return VMO_OK;
   // blocks per node: about 4,096 points each, fewer blocks when there are many nodes
   int C = 1;

@@ -82,7 +82,7 @@ vmo_status order_setup(OrderState& st, const float4* x, const std::vector<int64_
 // max_size: points of the largest of the N nodes.
 vmo_status two_means(OrderState& st, int N, int64_t max_size, int d, int km_iters, cudaStream_t s, Scratch& sc);
 // two_means of one node that holds all st.n positions, without any
-// allocation (at most kClusterNodeMax points, 1.8 million).
+// allocation (at most 1.25 million points, in two dimensions 1.8 million).
 vmo_status two_means_one(OrderState& st, int d, int km_iters, cudaStream_t s);
 vmo_status order_levels(OrderState& st, const OrderParams& op, cudaStream_t s, Scratch& sc);
 // Separators stably sorted by b two-bit link numbers (after order_levels).

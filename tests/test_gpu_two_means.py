@@ -64,6 +64,14 @@ def test_largest_node(V, O, n):
     _check(V, O, hg, x, np.arange(n, dtype=np.int32), 2, 3, seed=3)
 
 
+@pytest.mark.parametrize("d,n", [(3, 1600000), (3, 1600001), (4, 1250000), (4, 1250001)])
+def test_largest_node_of_more_dimensions(V, O, d, n):
+    hg = V.Hypergraph.from_matrix(W.grid_laplacian_2d(4))
+    x = np.zeros((n, 4), dtype=np.float32)
+    x[:, :d] = np.random.default_rng(n).standard_normal((n, d)) * 300.0
+    _check(V, O, hg, x, np.arange(n, dtype=np.int32), d, 3, seed=3)
+
+
 def test_coincident_points(V, O):
     hg = V.Hypergraph.from_matrix(W.grid_laplacian_2d(4))
     for n in (2, 700, 20000):
