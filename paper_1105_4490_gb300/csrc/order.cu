@@ -1096,11 +1096,13 @@ struct TwoMeansSums {           // one block's sums of a round, read by the clus
   unsigned long long v[6];      // S1[0..3], n1 | labels changed << 40, weights
 };
 
-template <int D, int T>
+// LIST: the node of cluster i is list[i], else i (an instance of its own: with a
+// branch for both the others were 4% slower for d = 3).
+template <int D, int T, bool LIST>
 __global__ void __launch_bounds__(T) k_two_means(const float4* __restrict__ xo, const int32_t* __restrict__ ord,
                                                  NodeDev* __restrict__ nodes, const uint64_t* __restrict__ seeds,
                                                  int km_iters, uint8_t* __restrict__ lab, uint64_t* __restrict__ vrec,
-                                                 int cap, int stream) {
+                                                 int cap, int stream, const int32_t* __restrict__ list) {
   pdl_enter();
   namespace cg = cooperative_groups;
   constexpr int W = T / 32;
@@ -1113,7 +1115,7 @@ __global__ void __launch_bounds__(T) k_two_means(const float4* __restrict__ xo, 
   __shared__ int s_flag;
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-  const int s = blockIdx.x / C;
+  const int s = LIST ? list[blockIdx.x / C] : blockIdx.x / C;
   NodeDev& nd = nodes[s];
   const int64_t off = nd.off;
   const int size = nd.size;
@@ -1367,9 +1369,10 @@ constexpr int64_t kClusterNodeMax = 8 * (int64_t)(kClusterSmem - 16);  // a clus
 // 0.86 (1.00 / 1.24 / 1.26), so that takes as many as fit.
 static int64_t cluster_node_max(int d) { return d == 2 ? kClusterNodeMax : d == 3 ? 1600000 : 1250000; }
 
-template <int D, int T>
-static cudaError_t launch_two_means(const OrderState& st, int N, int km_iters, int C, int share, cudaStream_t s) {
-  auto kernel = k_two_means<D, T>;
+template <int D, int T, bool LIST>
+static cudaError_t launch_two_means(const OrderState& st, int N, int km_iters, int C, int share, const int32_t* list,
+                                    cudaStream_t s) {
+  auto kernel = k_two_means<D, T, LIST>;
   const int cap = (share + 15) / 16 * 16;
   const bool stream = (size_t)cap * (4 * D + 1) > (size_t)kClusterSmem;
   const size_t smem = (size_t)cap * (stream ? 1 : 4 * D + 1);
@@ -1395,34 +1398,86 @@ static cudaError_t launch_two_means(const OrderState& st, int N, int km_iters, i
     e = cudaOccupancyMaxActiveClusters(&active, kernel, &cfg);
     if (e != cudaSuccess || active < 1) {
       (void)cudaGetLastError();
-      return launch_two_means<D, T>(st, N, km_iters, 8, share * 2, s);
+      return launch_two_means<D, T, LIST>(st, N, km_iters, 8, share * 2, list, s);
     }
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;  // as launch(): nothing after a refused one
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaLaunchKernelEx(&cfg, kernel, (const float4*)st.xo, (const int32_t*)st.ord, st.nodes,
-                            (const uint64_t*)st.seeds, km_iters, st.lab, st.vrec, cap, (int)stream);
+                            (const uint64_t*)st.seeds, km_iters, st.lab, st.vrec, cap, (int)stream, list);
 }
 
-static vmo_status two_means_clusters(OrderState& st, int N, int64_t max_size, int d, int km_iters, cudaStream_t s,
-                                     bool* done) {
-  *done = max_size <= cluster_node_max(d);
-  if (!*done || N == 0) return VMO_OK;
-  // blocks per node: about 4,096 points each, fewer blocks when there are many nodes
+// Blocks of a node's cluster: about 4,096 points each, fewer blocks when there
+// are many nodes.
+static int cluster_blocks(int N, int64_t max_size) {
   int C = 1;
   while (C < 16 && max_size > (int64_t)C * 4096) C *= 2;
   while (C > 1 && (int64_t)N * C > 512) C /= 2;
   while (C < 16 && (max_size + C - 1) / C > (int64_t)kClusterSmem - 16) C *= 2;  // the labels must fit
+  return C;
+}
+
+// One launch for N nodes of at most max_size points (those of the list, or the
+// table's first N).
+static vmo_status two_means_launch(OrderState& st, int N, int64_t max_size, const int32_t* list, int d, int km_iters,
+                                   cudaStream_t s) {
+  const int C = cluster_blocks(N, max_size);
   const int share = (int)((max_size + C - 1) / C);
   cudaError_t e = cudaSuccess;
   dispatch_d(d, [&](auto DC) {
     constexpr int D = decltype(DC)::value;
-    e = share > 2048 ? launch_two_means<D, 1024>(st, N, km_iters, C, share, s)
-        : share > 512 ? launch_two_means<D, 512>(st, N, km_iters, C, share, s)
-                      : launch_two_means<D, 128>(st, N, km_iters, C, share, s);
+    auto blocks_of = [&](auto T) {
+      return list ? launch_two_means<D, decltype(T)::value, true>(st, N, km_iters, C, share, list, s)
+                  : launch_two_means<D, decltype(T)::value, false>(st, N, km_iters, C, share, list, s);
+    };
+    using std::integral_constant;
+    e = share > 2048 ? blocks_of(integral_constant<int, 1024>())
+        : share > 512 ? blocks_of(integral_constant<int, 512>())
+                      : blocks_of(integral_constant<int, 128>());
   });
   if (e != cudaSuccess) return cuda_fail(e, "two_means (cluster per node)", __FILE__, __LINE__);
   return VMO_OK;
+}
+
+// Nodes of more than `most` points from the front of the list, the others from
+// its end.
+__global__ void k_large_nodes(const NodeDev* __restrict__ nodes, int N, int most, int32_t* __restrict__ list,
+                              int32_t* __restrict__ count) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= N) return;
+  if (nodes[s].size > most) list[atomicAdd(&count[0], 1)] = s;
+  else list[N - 1 - atomicAdd(&count[1], 1)] = s;
+}
+
+// A level of many nodes gives each one block; a few large nodes among them would
+// then pass through one SM each.  They get a launch of their own, with as many
+// blocks as they would have alone, where a block's share is more than it holds in
+// shared memory (sc: null where nothing may be allocated, a single node then).
+// 600 nodes of 70 points and one of 200,000, one level: 3.5 -> 2.1 ms for the
+// call; 20,000 and one of 1.5 million: 76 -> 48 ms.
+constexpr int kLargeNode = 16384;
+
+static vmo_status two_means_clusters(OrderState& st, int N, int64_t max_size, int d, int km_iters, cudaStream_t s,
+                                     Scratch* sc, bool* done) {
+  *done = max_size <= cluster_node_max(d);
+  if (!*done || N == 0) return VMO_OK;
+  const int C = cluster_blocks(N, max_size);
+  if (sc && C < cluster_blocks(1, max_size) && max_size > (int64_t)C * kLargeNode) {
+    ScratchFrame frame(*sc);
+    int32_t *list, *count, large = 0;
+    VMO_TRY(sc->alloc(&list, N));
+    VMO_TRY(sc->alloc(&count, 2));
+    VMO_CUDA(cudaMemsetAsync(count, 0, 2 * sizeof(int32_t), s));
+    launch(k_large_nodes, grid_for(N, kBlock), kBlock, 0, s, st.nodes, N, kLargeNode, list, count);
+    VMO_LAUNCHED("large_nodes");
+    VMO_CUDA(cudaMemcpyAsync(&large, count, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    VMO_CUDA(cudaStreamSynchronize(s));
+    if (large < N) {
+      VMO_TRY(two_means_launch(st, large, max_size, list, d, km_iters, s));
+      return two_means_launch(st, N - large, kLargeNode, list + large, d, km_iters, s);
+    }
+  }
+  return two_means_launch(st, N, max_size, nullptr, d, km_iters, s);
 }
 
 // The same as a launch sequence over all positions, for nodes that one cluster
@@ -1484,7 +1539,7 @@ static vmo_status two_means_body(OrderState& st, int N, int d, int km_iters, uns
 vmo_status two_means(OrderState& st, int N, int64_t max_size, int d, int km_iters, cudaStream_t s, Scratch& sc) {
   const int64_t n = st.n;
   bool done = false;
-  VMO_TRY(two_means_clusters(st, N, max_size, d, km_iters, s, &done));
+  VMO_TRY(two_means_clusters(st, N, max_size, d, km_iters, s, &sc, &done));
   if (done) return VMO_OK;
   ScratchFrame frame(sc);
   unsigned long long *dval, *dpre, *rep = nullptr;
@@ -1511,7 +1566,7 @@ vmo_status two_means(OrderState& st, int N, int64_t max_size, int d, int km_iter
 
 vmo_status two_means_one(OrderState& st, int d, int km_iters, cudaStream_t s) {
   bool done = false;
-  VMO_TRY(two_means_clusters(st, 1, st.n, d, km_iters, s, &done));
+  VMO_TRY(two_means_clusters(st, 1, st.n, d, km_iters, s, nullptr, &done));
   return done ? VMO_OK : invalid("two_means: too many points for one cluster");
 }
 

@@ -97,3 +97,22 @@ def test_uneven_nodes(V, O):
         ref = O.build_from_matrix("symmetric", mats[i])
         want, _ = O.order(ref, 3, xs[i], seed=6, min_part=8)
         assert np.array_equal(perm[offs[i]:offs[i + 1]], want), i
+
+
+@pytest.mark.parametrize("d", [2, 3, 4])
+def test_large_nodes_among_many(V, O, d):
+    """Levels of more than 512 nodes with a few of more than 16,384 points, which
+    have a launch of their own."""
+    mats = [W.random_symmetric(n, 4, n) for n in (70000, 16384, 16385, 40000)] + \
+        [W.random_symmetric(70 + i % 9, 4, i) for i in range(540)]
+    rng = np.random.default_rng(d)
+    xs = [np.zeros((A.m, 4), dtype=np.float32) for A in mats]
+    for x in xs:
+        x[:, :d] = rng.standard_normal((len(x), d)) * 10
+    perm, offs = V.batch_order(mats, V.Params(d=d, min_part=60, max_depth=3, seed=6),
+                               coords=torch.as_tensor(np.concatenate(xs)).cuda())
+    perm = perm.cpu().numpy()
+    for i in (0, 1, 2, 3, 4, 100, 543):
+        ref = O.build_from_matrix("symmetric", mats[i])
+        want, _ = O.order(ref, d, xs[i], seed=6, min_part=60, max_depth=3)
+        assert np.array_equal(perm[offs[i]:offs[i + 1]], want), i
