@@ -635,7 +635,41 @@ __device__ __forceinline__ void cell_add(const float4& p, float wq, float* S, fl
 }
 
 // Points q0, q0 + stride, ... < q1 added in that order; U loads issued before
-// their additions (the last of them guarded).
+// their additions, those of the last, incomplete trip guarded.  The whole trips of a
+// large cell go without guards, with which two loads' times passed per trip: the
+// first step of 19,800 points in a cell, d = 2, 118 -> 88 us, the layout of the
+// 64^3 grid 1.3% shorter (16 loads instead of 8: 53 us, but twice the registers,
+// and a batch of 256 matrices 1% longer).
+template <int D, int U>
+__device__ __forceinline__ void cell_sum_long(const float4* xs, const float* ws, int64_t q0, int64_t q1, int64_t stride,
+                                              float* S, float& W) {
+  int64_t q = q0;
+  for (; q + (U - 1) * stride < q1; q += U * stride) {
+    float4 p[U];
+    float wq[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      p[u] = xs[q + u * stride];
+      wq[u] = ws ? ws[q + u * stride] : 1.0f;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) cell_add<D>(p[u], wq[u], S, W);
+  }
+  if (q >= q1) return;
+  float4 p[U];
+  float wq[U];
+#pragma unroll
+  for (int u = 0; u + 1 < U; ++u) {
+    const bool in = q + u * stride < q1;
+    p[u] = in ? xs[q + u * stride] : make_float4(0.f, 0.f, 0.f, 0.f);
+    wq[u] = in && ws ? ws[q + u * stride] : 1.0f;
+  }
+#pragma unroll
+  for (int u = 0; u + 1 < U; ++u)
+    if (q + u * stride < q1) cell_add<D>(p[u], wq[u], S, W);
+}
+
+// The same for cells of a few points, every load guarded.
 template <int D, int U>
 __device__ __forceinline__ void cell_sum(const float4* xs, const float* ws, int64_t q0, int64_t q1, int64_t stride,
                                          float* S, float& W) {
@@ -659,7 +693,7 @@ __device__ __forceinline__ void cell_sum(const float4* xs, const float* ws, int6
 template <int D>
 __device__ __forceinline__ void cell_sum_warp(const float4* xs, const float* ws, int64_t q0, int64_t q1, float* S,
                                               float& W) {
-  cell_sum<D, 8>(xs, ws, q0 + lane_id(), q1, 32, S, W);
+  cell_sum_long<D, 8>(xs, ws, q0 + lane_id(), q1, 32, S, W);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
