@@ -110,3 +110,26 @@ def test_crowded_cells(V, O, d, k, sizes):
     xs, ys, ks, _ = hg.layout_step(torch.as_tensor(x).cuda(), 0.25, p)
     assert torch.equal(ys.view(torch.int32), yg.view(torch.int32))
     assert torch.equal(xs.view(torch.int32), xg.view(torch.int32)) and torch.equal(ks, kg)
+
+
+@pytest.mark.parametrize("d,k,sizes", [(2, 1025, (64, 65)), (2, 2048, (2048,)), (2, 2000, (1000, 66, 900)),
+                                       (3, 2048, (1200, 700)), (3, 1500, (1024, 65)), (4, 2000, (1999,))])
+def test_crowded_cells_of_one_block(V, d, k, sizes):
+    """Problems of 1,025 to 2,048 points, whose crowded cells one block sorts by
+    bits: steps from the crowded cloud and a few after it, as device-wide."""
+    hg = V.Hypergraph.from_matrix(W.random_symmetric(k, 6, seed=k))
+    rng = np.random.default_rng(k + d)
+    side = float(k) ** (1.0 / d)
+    x = np.zeros((k, 4), dtype=np.float32)
+    x[:, :d] = rng.random((k, d)) * side
+    n = 0
+    for i, size in enumerate(sizes):
+        x[n:n + size, :d] = side * (0.3 + 0.2 * i) + 1e-3 * rng.standard_normal((size, d))
+        n += size
+    x = torch.as_tensor(x[rng.permutation(k)]).cuda()
+    runs = []
+    for small in (0, 2048):
+        V.set_tuning(19456, 10, 4, small)
+        runs.append((hg.layout_step(x, 0.25, V.Params(d=d))[:3], hg.layout(V.Params(d=d, iters=9), x.clone())))
+    for a, b in zip(runs[0][0] + (runs[0][1],), runs[1][0] + (runs[1][1],)):
+        assert torch.equal(a.view(torch.int32), b.view(torch.int32))
