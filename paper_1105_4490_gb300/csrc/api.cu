@@ -82,7 +82,10 @@ void stats_time_end(cudaStream_t s, uint64_t points) {
   g_timed.back().points = points;
 }
 
-Scratch::~Scratch() { release_to(0); }
+Scratch::~Scratch() {
+  held.clear();
+  release_to(0);
+}
 
 vmo_status Scratch::alloc_bytes(void** p, size_t bytes) {
   if (bytes < 16) bytes = 16;

@@ -2729,7 +2729,7 @@ constexpr int kGraphMinIters = 8;
 // they cost 2 ms of the 64^3 grid's layout): `side` for the attraction (fork /
 // join events per step) and `main` for the steps when they are replayed from a
 // graph (capture needs a stream of its own: the caller's may be the legacy
-// stream); destroyed in stream order when the call returns.
+// stream).
 struct SideStream {
   cudaStream_t stream = nullptr, main = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr, start = nullptr, done = nullptr;
@@ -2756,9 +2756,48 @@ struct SideStream {
   ~SideStream() { release(); }
 };
 
+// Streams, step-length factors and graphs of one layout call.  A graph is
+// destroyed and the streams are closed only when nothing of them is queued any
+// more: destroyed behind their last launch, as the levels are queued far ahead
+// of the device, they left the request server's slots (four host threads)
+// standing after some 100,000 steps, kernels not started and hosts inside the
+// driver.  The graphs go level by level while the last level runs; the rest is
+// held by the call's Scratch to its end, so that the host does not wait for the
+// last level here (1% of a 64 x 64 ordering).
 struct LayoutContext {
+  struct Replay {
+    cudaGraphExec_t graph;
+    cudaEvent_t done;  // behind its last launch (null if it could not be made)
+  };
   SideStream streams;
   float* scale_tab = nullptr;  // decay^t of the layout's steps
+  std::vector<Replay> replays;
+  void keep(cudaGraphExec_t graph) {
+    Replay r{graph, nullptr};
+    if (cudaEventCreateWithFlags(&r.done, cudaEventDisableTiming) != cudaSuccess) {
+      (void)cudaGetLastError();
+      r.done = nullptr;
+    } else {
+      cudaEventRecord(r.done, streams.main);
+    }
+    replays.push_back(r);
+  }
+  void destroy_all_but(size_t last) {
+    size_t n = 0;
+    for (; n + last < replays.size(); ++n) {
+      const Replay& r = replays[n];
+      if (r.done) cudaEventSynchronize(r.done);
+      else cudaStreamSynchronize(streams.main);
+      cudaGraphExecDestroy(r.graph);
+      if (r.done) cudaEventDestroy(r.done);
+    }
+    replays.erase(replays.begin(), replays.begin() + n);
+  }
+  ~LayoutContext() {
+    destroy_all_but(0);
+    for (cudaStream_t st : {streams.main, streams.stream})
+      if (st) cudaStreamSynchronize(st);
+  }
 };
 
 // Step lengths s0 * decay^t: decay^t as the running double product, rounded to
@@ -2871,8 +2910,12 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
   vmo_status st = VMO_OK;
   // streams: the layout's, the level's own, or none for a few steps (making them
   // costs more than the overlap of so few gives) or if they cannot be made
-  std::unique_ptr<SideStream> own(!ctx && iters >= kGraphMinIters ? new SideStream : nullptr);
-  SideStream* ss = ctx ? &ctx->streams : own.get();
+  if (!ctx && iters >= kGraphMinIters) {
+    auto own = std::make_shared<LayoutContext>();
+    ctx = own.get();
+    sc.held.push_back(own);
+  }
+  SideStream* ss = ctx ? &ctx->streams : nullptr;
   const cudaStream_t side = ss ? ss->stream : nullptr;
   dispatch_d(d, [&](auto DC) {
     constexpr int D = decltype(DC)::value;
@@ -3008,7 +3051,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
         (void)cudaGetLastError();  // fall back to direct launches
         if (cst0 != VMO_OK) st = cst0;
       }
-      if (ge) cudaGraphExecDestroy(ge);
+      if (ge) ctx->keep(ge);
       if (g) cudaGraphDestroy(g);
     }
     for (; t < iters && st == VMO_OK; ++t) st = step(t);
@@ -3275,17 +3318,19 @@ vmo_status layout_multilevel(LevelBatch& fine, const LayoutOptions& o, const std
   VMO_CUDA(cudaMemcpyAsync(sd_d, seed_all.data(), tb[nl] * 8, cudaMemcpyHostToDevice, s));
   VMO_CUDA(cudaStreamSynchronize(s));  // the host tables must outlive the copies
   // layout from the coarsest level down
-  LayoutContext ctx;
-  if (o.iters > 0) VMO_TRY(make_scale_tab(o, o.iters, &ctx.scale_tab, s, sc));
+  auto ctx = std::make_shared<LayoutContext>();
+  sc.held.push_back(ctx);
+  if (o.iters > 0) VMO_TRY(make_scale_tab(o, o.iters, &ctx->scale_tab, s, sc));
   float4* xc = nullptr;
   for (int j = nl - 1; j >= 0; --j) {
     LevelBatch& cur = *H.levels[j];
     float4* xj = (j == 0) ? x : nullptr;
     if (!xj) VMO_TRY(sc.alloc(&xj, std::max<int64_t>(cur.K, 1)));
     VMO_TRY(prolong_level_dev(H, j, o.d, xc, xj, st_d + tb[j], fc_d + tb[j], sd_d + tb[j], s));
-    VMO_TRY(layout_level(cur, o, xj, o.iters, -1.0f, nullptr, nullptr, &ctx, s, sc));
+    VMO_TRY(layout_level(cur, o, xj, o.iters, -1.0f, nullptr, nullptr, ctx.get(), s, sc));
     xc = xj;
   }
+  ctx->destroy_all_but(1);
   return VMO_OK;
 }
 

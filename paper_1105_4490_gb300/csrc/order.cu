@@ -1665,6 +1665,7 @@ vmo_status order_levels(OrderState& st, const OrderParams& op, cudaStream_t s, S
     launch(k_scatter, grid_for(n, kBlock), kBlock, 0, s, st.ord, st.xo, st.seg, labf, n, st.nodes, pre, op.sbd, ord2, xo2,
                                                      seg2, st.vrec);
     VMO_LAUNCHED("partition");
+    sc.held.clear();  // of the layout, which order_setup has waited for: closed while this level runs
     // the scattered arrays become the current ones
     std::swap(st.ord, ord2);
     std::swap(st.xo, xo2);

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <memory>
 #include <string>
 #include <utility>
 #include <vector>
@@ -54,6 +55,7 @@ vmo_status unsupported(const std::string& msg);
 struct Scratch {
   cudaStream_t stream = nullptr;
   std::vector<void*> ptrs;
+  std::vector<std::shared_ptr<void>> held;  // what must outlive the call's queued work, destroyed first
   explicit Scratch(cudaStream_t s) : stream(s) {}
   ~Scratch();
   template <class T>

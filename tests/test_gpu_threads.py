@@ -3,6 +3,7 @@ every result is the one of the same call alone, bit for bit.  The problems'
 sizes differ, so that the threads' levels take launches of different shared
 memory from the same kernels."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -88,3 +89,23 @@ def test_two_server_slots(V, d, sizes):
             info = srv.wait(r, 60.0)
             assert info["state"] == "done", info
             assert np.array_equal(srv.result(r), want)
+
+
+def test_four_server_slots_under_load(V):
+    """Four slots that take requests of the small mix as they come, each a layout of
+    ten levels whose steps are queued far ahead: they all finish, with the plain
+    ordering's permutations."""
+    mats = W.batch_mix(180, 5)
+    with V.Server(V.Params(d=3, seed=1), slots=4) as srv:
+        for rnd in range(3):
+            ids = []
+            for i, A in enumerate(mats):
+                ids.append(srv.submit_matrix(A))
+                if i % 4 == 3:
+                    time.sleep(0.02)
+            for r in ids:
+                assert srv.wait(r, 60.0)["state"] == "done"
+            got = {i: srv.result(ids[i]).copy() for i in range(rnd, len(ids), 23)}
+    for i, perm in got.items():
+        rp, _, _ = V.Hypergraph.from_matrix(mats[i]).order(V.Params(d=3, seed=1), None, sbd=False, with_tree=False)
+        assert np.array_equal(perm, rp.cpu().numpy()), i
