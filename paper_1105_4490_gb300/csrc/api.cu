@@ -13,7 +13,7 @@ namespace vmo {
 static thread_local std::string g_last_error;
 thread_local cudaStream_t g_devarray_stream = nullptr;
 thread_local bool g_devarray_async = false;
-thread_local cudaMemPool_t g_devarray_pool = nullptr;
+thread_local PoolKind g_devarray_pool = kDefaultPool;
 thread_local bool g_pdl = false;
 
 void set_error(const std::string& msg) { g_last_error = msg; }
@@ -117,8 +117,8 @@ vmo_status cut_size(const vmo_hg_s* h, const int32_t* part, int32_t nparts, int6
 namespace {
 
 std::once_flag g_pool_once;
-std::mutex g_handle_pool_mu;
-std::vector<std::pair<int, cudaMemPool_t>> g_handle_pools;  // one per device used
+std::mutex g_library_pool_mu;
+std::vector<std::pair<int, cudaMemPool_t>> g_library_pools[3];  // per kind: one per device used
 
 // Device present; stream-ordered pool keeps freed scratch for reuse.
 vmo_status ensure_device() {
@@ -256,7 +256,7 @@ vmo_status run_order(vmo_hg_s* h, const float* coords, const vmo_params* p, int 
   if (h->model != VMO_SYMMETRIC && h->model != VMO_BIPARTITE)
     return unsupported("ordering needs a graph model (symmetric or bipartite, Algorithm 7)");
   if (coords && !aligned16(coords)) return invalid("coords must be 16-byte aligned");
-  DevArrayStreamScope scope(s);
+  DevArrayStreamScope scope(s, kLevelPool);
   Scratch sc(s);
   const int64_t k = h->k;
   int32_t* mu = nullptr;
@@ -358,28 +358,30 @@ __global__ void k_fill_f32(float* __restrict__ a, int64_t n, float v) {
 
 }  // namespace
 
-cudaMemPool_t handle_pool() {
-  std::lock_guard<std::mutex> lk(g_handle_pool_mu);
+cudaMemPool_t library_pool(PoolKind kind) {
+  std::lock_guard<std::mutex> lk(g_library_pool_mu);
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-  for (auto& p : g_handle_pools)
+  for (auto& p : g_library_pools[kind])
     if (p.first == dev) return p.second;
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = dev;
   cudaMemPool_t pool = nullptr;
-  uint64_t keep = kHandlePoolKeep;
+  uint64_t keep = kPoolKeep;
   if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
       cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
     (void)cudaGetLastError();
     return nullptr;
   }
-  // Kept for good: the fences of the handles (vmo_hg_s) are then parts of its
-  // 2 MB block, which a fence alone would map and unmap (180 us a handle).
-  void* anchor = nullptr;
-  if (cudaMalloc(&anchor, 16) != cudaSuccess) (void)cudaGetLastError();
-  g_handle_pools.emplace_back(dev, pool);
+  if (kind == kHandlePool) {
+    // Kept for good: the fences of the handles (vmo_hg_s) are then parts of its
+    // 2 MB block, which a fence alone would map and unmap (180 us a handle).
+    void* anchor = nullptr;
+    if (cudaMalloc(&anchor, 16) != cudaSuccess) (void)cudaGetLastError();
+  }
+  g_library_pools[kind].emplace_back(dev, pool);
   return pool;
 }
 
@@ -423,8 +425,7 @@ vmo_status vmo_build_hypergraph(const vmo_csr* a, vmo_model model, const float* 
   cudaGetDevice(&h->device);
   VMO_CUDA(cudaMalloc(&h->fence, 16));
   g_device_allocs.fetch_add(1, std::memory_order_relaxed);
-  cudaMemPool_t pool = handle_pool();
-  std::unique_ptr<DevArrayStreamScope> scope(pool ? new DevArrayStreamScope(s, pool) : nullptr);
+  std::unique_ptr<DevArrayStreamScope> scope(library_pool(kHandlePool) ? new DevArrayStreamScope(s, kHandlePool) : nullptr);
   VMO_TRY(build_model(a, model, h.get(), s));
   if (vertex_weight) {
     VMO_TRY(h->weight.resize(std::max<int32_t>(h->k, 1)));
@@ -470,7 +471,7 @@ vmo_status vmo_init_coords(int32_t k, int32_t d, uint64_t seed, float* coords, v
   if (d < 2 || d > 4) return unsupported("d must be 2, 3 or 4");
   if (k > 0 && (!coords || !aligned16(coords))) return invalid("coords null or not 16-byte aligned");
   cudaStream_t s = (cudaStream_t)stream;
-  DevArrayStreamScope scope(s);
+  DevArrayStreamScope scope(s, kLevelPool);
   LevelBatch lb;
   lb.K = k;
   lb.P = 1;
@@ -492,7 +493,7 @@ vmo_status vmo_layout(vmo_hg hg, const vmo_params* params, float* coords, int32_
   if (!hg) return invalid("handle is null");
   if (hg->k > 0 && (!coords || !aligned16(coords))) return invalid("coords null or not 16-byte aligned");
   cudaStream_t s = (cudaStream_t)stream;
-  DevArrayStreamScope scope(s);
+  DevArrayStreamScope scope(s, kLevelPool);
   Scratch sc(s);
   VMO_TRY(run_layout(hg, params, (float4*)coords, use_given_init != 0, s, sc));
   VMO_CUDA(cudaStreamSynchronize(s));
@@ -508,7 +509,7 @@ vmo_status vmo_layout_step(vmo_hg hg, const vmo_params* params, float* coords, f
   if (hg->k > 0 && (!coords || !aligned16(coords))) return invalid("coords null or not 16-byte aligned");
   if (y_out && !aligned16(y_out)) return invalid("y_out must be 16-byte aligned");
   cudaStream_t s = (cudaStream_t)stream;
-  DevArrayStreamScope scope(s);
+  DevArrayStreamScope scope(s, kLevelPool);
   Scratch sc(s);
   LevelBatch lb;
   VMO_TRY(single_batch(hg, params->d, params->occupancy, lb, s));
@@ -526,7 +527,7 @@ vmo_status vmo_coarsen(vmo_hg hg, const vmo_params* params, int32_t* mate, int32
   if (!hg) return invalid("handle is null");
   if (hg->model != VMO_SYMMETRIC && hg->model != VMO_BIPARTITE) return unsupported("coarsening needs a graph model");
   cudaStream_t s = (cudaStream_t)stream;
-  DevArrayStreamScope scope(s);
+  DevArrayStreamScope scope(s, kLevelPool);
   Scratch sc(s);
   LevelBatch lb;
   VMO_TRY(single_batch(hg, params->d, params->occupancy, lb, s));
@@ -574,7 +575,7 @@ vmo_status vmo_hierarchy_level(vmo_hg hg, const vmo_params* params, int32_t leve
                                int32_t* adj_ptr, int32_t* adj, float* acost, float* weight, int32_t* pi,
                                void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
-  DevArrayStreamScope scope(s);
+  DevArrayStreamScope scope(s, kLevelPool);
   Scratch sc(s);
   LevelBatch lb;
   Hierarchy H;
@@ -604,7 +605,7 @@ vmo_status vmo_hierarchy_level(vmo_hg hg, const vmo_params* params, int32_t leve
 vmo_status vmo_hierarchy_prolong(vmo_hg hg, const vmo_params* params, int32_t level, const float* coarse, float* fine,
                                  void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
-  DevArrayStreamScope scope(s);
+  DevArrayStreamScope scope(s, kLevelPool);
   Scratch sc(s);
   LevelBatch lb;
   Hierarchy H;
@@ -621,7 +622,7 @@ vmo_status vmo_hierarchy_prolong(vmo_hg hg, const vmo_params* params, int32_t le
 vmo_status vmo_hierarchy_step(vmo_hg hg, const vmo_params* params, int32_t level, float* coords, float step,
                               float* y_out, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
-  DevArrayStreamScope scope(s);
+  DevArrayStreamScope scope(s, kLevelPool);
   Scratch sc(s);
   LevelBatch lb;
   Hierarchy H;

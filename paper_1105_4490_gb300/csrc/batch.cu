@@ -128,7 +128,7 @@ static vmo_status join_and_build(const vmo_csr* mats, int32_t count, vmo_hg_s& h
 
 vmo_status batch_order(const vmo_csr* mats, int32_t count, const float* coords, const vmo_params* p, int32_t sbd,
                        int32_t* perm, cudaStream_t s) {
-  DevArrayStreamScope scope(s);
+  DevArrayStreamScope scope(s, kLevelPool);
   Scratch sc(s);
   vmo_hg_s h;
   Joined J;
@@ -152,7 +152,7 @@ vmo_status batch_order(const vmo_csr* mats, int32_t count, const float* coords, 
 }
 
 vmo_status batch_layout(const vmo_csr* mats, int32_t count, const vmo_params* p, float* coords, cudaStream_t s) {
-  DevArrayStreamScope scope(s);
+  DevArrayStreamScope scope(s, kLevelPool);
   Scratch sc(s);
   vmo_hg_s h;
   Joined J;

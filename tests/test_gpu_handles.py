@@ -58,3 +58,18 @@ def test_destroy_beside_layouts_of_another_thread(V):
     torch.cuda.synchronize()
     assert not errors, errors
     assert all(np.array_equal(ref, x.cpu().numpy()) for x in got)
+
+
+def test_level_arrays_are_given_back(V):
+    """A layout's level arrays of more than 1 GiB return to the device with the
+    call's end, as far as they exceed what the library keeps."""
+    n = 20000  # a full pattern: 1.6 GB of adjacency, next to nothing per vertex
+    rowptr = torch.arange(n + 1, dtype=torch.int32, device="cuda") * n
+    colidx = torch.arange(n, dtype=torch.int32, device="cuda").repeat(n)
+    hg = V.Hypergraph(rowptr, colidx, n, n)
+    del colidx
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    hg.layout(V.Params(d=3, iters=0, multilevel=False))
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] <= (1 << 30) + (256 << 20)
