@@ -423,7 +423,11 @@ vmo_status vmo_build_hypergraph(const vmo_csr* a, vmo_model model, const float* 
   // the handle's arrays are freed in vmo_destroy, whatever stream built them
   std::unique_ptr<vmo_hg_s, void (*)(vmo_hg)> h(new vmo_hg_s(), vmo_destroy);
   cudaGetDevice(&h->device);
-  VMO_CUDA(cudaMalloc(&h->fence, 16));
+  if (cudaMalloc(&h->fence, 16) != cudaSuccess) {
+    (void)cudaGetLastError();
+    set_error("device allocation of 16 bytes failed");
+    return VMO_ERR_OOM;
+  }
   g_device_allocs.fetch_add(1, std::memory_order_relaxed);
   std::unique_ptr<DevArrayStreamScope> scope(library_pool(kHandlePool) ? new DevArrayStreamScope(s, kHandlePool) : nullptr);
   VMO_TRY(build_model(a, model, h.get(), s));
