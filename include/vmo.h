@@ -472,7 +472,8 @@ vmo_status vmo_set_tuning(const vmo_tuning* tuning);
 /* Timed search for the setting that orders the given matrices fastest: from
  * the current setting, each choice in turn over its candidates
  * (small_step_threads 0 ... 155,648; radix_max_bits 8, 9, 10; assign_items
- * 1, 2, 4, 8; small_bin_points 0, 512, 2,048), every candidate timed as the median of `reps` calls of
+ * 1, 2, 4, 8 if a matrix has more rows than the sizes above, else left as it
+ * is; small_bin_points 0, 512, 2,048), every candidate timed as the median of `reps` calls of
  * vmo_batch_order(mats, count, NULL, params, BBD) after one untimed call, with
  * CUDA events on `stream`.  The fastest becomes the process-wide setting.
  * mats: host array of `count` vmo_csr (device pointers inside), as for

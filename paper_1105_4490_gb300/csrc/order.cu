@@ -1367,7 +1367,7 @@ constexpr int64_t kClusterNodeMax = 8 * (int64_t)(kClusterSmem - 16);  // a clus
 // of 1.4 / 1.6 / 1.75 M points by a cluster: d = 3 0.82 / 0.90 / 0.97 ms (sequence
 // 0.88 / 0.90 / 0.90), d = 4 0.99 / 1.10 / 1.17 (0.94 / 1.00 / 1.00), d = 2 0.70 / 0.76 /
 // 0.86 (1.00 / 1.24 / 1.26), so that takes as many as fit.
-static int64_t cluster_node_max(int d) { return d == 2 ? kClusterNodeMax : d == 3 ? 1600000 : 1250000; }
+int64_t cluster_node_max(int d) { return d == 2 ? kClusterNodeMax : d == 3 ? 1600000 : 1250000; }
 
 template <int D, int T, bool LIST>
 static cudaError_t launch_two_means(const OrderState& st, int N, int km_iters, int C, int share, const int32_t* list,

@@ -81,6 +81,8 @@ vmo_status order_setup(OrderState& st, const float4* x, const std::vector<int64_
                        cudaStream_t s, Scratch& sc);
 // max_size: points of the largest of the N nodes.
 vmo_status two_means(OrderState& st, int N, int64_t max_size, int d, int km_iters, cudaStream_t s, Scratch& sc);
+// Points of the largest node that one cluster takes.
+int64_t cluster_node_max(int d);
 // two_means of one node that holds all st.n positions, without any
 // allocation (at most 1.25 million points, in two dimensions 1.8 million).
 vmo_status two_means_one(OrderState& st, int d, int km_iters, cudaStream_t s);

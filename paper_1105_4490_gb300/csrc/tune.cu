@@ -10,7 +10,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "vmo_internal.cuh"
+#include "order.cuh"
 
 namespace vmo {
 
@@ -107,7 +107,13 @@ extern "C" vmo_status vmo_autotune(const vmo_csr* mats, int32_t count, const vmo
   const std::vector<int> bits = {8, 9, 10};
   const std::vector<int> items = {1, 2, 4, 8};
   const std::vector<int> bins = {0, 512, kSortTile};
+  // assign_items shapes the Lloyd rounds of nodes beyond one cluster only: without
+  // such a matrix its candidates would differ by noise, and the choice would stand
+  // for later calls that have one
+  bool lloyd = false;
+  for (int32_t i = 0; i < count && st == VMO_OK; ++i) lloyd = lloyd || mats[i].m > cluster_node_max(params->d);
   for (int knob = 0; knob < 4 && st == VMO_OK; ++knob) {
+    if (knob == 2 && !lloyd) continue;
     const size_t nc = knob == 0 ? steps.size() : knob == 1 ? bits.size() : knob == 2 ? items.size() : bins.size();
     for (size_t c = 0; c < nc && st == VMO_OK; ++c) {
       vmo_tuning t = bt;

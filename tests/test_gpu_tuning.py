@@ -102,3 +102,17 @@ def test_small_bin_equals_device_wide(V):
         V.set_tuning(**t0)
     for a, b in zip(*runs):
         assert np.array_equal(a, b)
+
+
+def test_autotune_leaves_what_its_matrices_do_not_use(V):
+    """assign_items matters for nodes of more than 1.25 million points only: with
+    smaller matrices it stays as it was."""
+    t0 = V.get_tuning()
+    mats = W.batch_mix(4, 45, nmin=500, nmax=2000)
+    try:
+        for items in (1, 8):
+            V.set_tuning(t0["small_step_threads"], t0["radix_max_bits"], items, t0["small_bin_points"])
+            best, _, _ = V.autotune(mats, V.Params(d=3, seed=1), reps=1)
+            assert best["assign_items"] == items
+    finally:
+        V.set_tuning(**t0)
