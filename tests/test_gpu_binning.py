@@ -133,3 +133,27 @@ def test_crowded_cells_of_one_block(V, d, k, sizes):
         runs.append((hg.layout_step(x, 0.25, V.Params(d=d))[:3], hg.layout(V.Params(d=d, iters=9), x.clone())))
     for a, b in zip(runs[0][0] + (runs[0][1],), runs[1][0] + (runs[1][1],)):
         assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+
+
+@pytest.mark.parametrize("d", [2, 3])
+def test_one_block_binning_with_two_targets_per_thread(V, d):
+    """A batch whose problems each fit one block and whose levels have more than
+    196,608 step threads, so that the blocks number their problems' chunks of two
+    points: as the device-wide binning, and as with one target per thread (the
+    counting kernel), bit for bit."""
+    rng = np.random.default_rng(d)
+    mats = [W.random_symmetric(int(n), 6, seed=i) for i, n in enumerate(rng.integers(500, 2049, 220))]
+    p = V.Params(d=d, seed=3, iters=12)
+    try:
+        runs = []
+        for small in (2048, 0):
+            V.set_tuning(19456, 10, 4, small)
+            runs.append(V.batch_layout(mats, p)[0])
+        V.set_tuning(19456, 10, 4, 2048)
+        V.stats_reset(time_step_kernel=False, count_interactions=True)
+        runs.append(V.batch_layout(mats, p)[0])
+        assert V.stats()["step_interactions"] > 0
+    finally:
+        V.stats_reset(time_step_kernel=False, count_interactions=False)
+    for x in runs[1:]:
+        assert torch.equal(x.view(torch.int32), runs[0].view(torch.int32))
