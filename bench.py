@@ -294,7 +294,8 @@ def step_roofline(V, torch, run_once, d: int, steps: int, peak: dict) -> dict:
     flops_per_launch = counted["step_interactions"] * FLOPS_PER_INTERACTION[d] / launches
     avg_ms = st["step_ms"] / max(st["step_launches"], 1)
     achieved = flops_per_launch / (avg_ms / 1e3) / 1e12
-    return {"bound": "alu", "kernel": f"k_repulse_update<{d}> (layout step)", "achieved": achieved,
+    kernels = f"k_repulse_update<{d}>" + (f", k_repulse_split<{d}>" if d > 2 else "")
+    return {"bound": "alu", "kernel": f"{kernels} (layout step)", "achieved": achieved,
             "peak": peak["ffma2_tflops"], "unit": "TFLOP/s", "frac": achieved / peak["ffma2_tflops"],
             "peak_source": f"measured in this run (vmo_measure_alu_peaks): packed FP32 fma2 on all "
                            f"{peak['sms']} SMs, {peak['ffma2_tflops']:.1f} TFLOP/s (scalar fma "
@@ -705,12 +706,12 @@ def main():
     flops_per_launch = inter_per_step * FLOPS_PER_INTERACTION[d] / launches_per_step
     avg_ms = st["step_ms"] / max(st["step_launches"], 1)
     achieved = flops_per_launch / (avg_ms / 1e3) / 1e12
-    roofline = {"bound": "alu", "kernel": "k_repulse_update<3> (layout step)", "achieved": achieved,
+    roofline = {"bound": "alu", "kernel": "k_repulse_update<3>, k_repulse_split<3> (layout step)", "achieved": achieved,
                 "peak": peak["ffma2_tflops"], "unit": "TFLOP/s", "frac": achieved / peak["ffma2_tflops"],
                 "traffic": None,
                 "traffic_note": "the per-launch mean over a step's 3,000 launches is not captured for the "
                                 "current kernel (ncu captures are kept to single launches); one finest-level "
-                                "launch of the 500k power-law read 31.9 MB from DRAM",
+                                "launch of the 500k power-law read 33.2 MB from DRAM",
                 "peak_source": f"measured in this run (vmo_measure_alu_peaks): packed FP32 fma2 on all "
                                f"{peak['sms']} SMs, {peak['ffma2_tflops']:.1f} TFLOP/s (scalar fma "
                                f"{peak['ffma_tflops']:.1f}, rsqrt {peak['rsqrt_tops']:.2f} T/s); nominal "

@@ -13,7 +13,7 @@
 // entry numbers (two passes instead of four of 64-bit keys), and a symmetric
 // pattern is its own adjacency, with every entry's mirror found by a binary
 // search in its row.  27-point mesh of 10^6 rows in random numbering, symmetric
-// model with copies of its arrays: 7.6 -> 1.8 ms; 400k x 300k bipartite model: 2.1 -> 1.2 ms.
+// model with copies of its arrays: 7.6 -> 1.05 ms; 400k x 300k bipartite model: 2.1 -> 0.61 ms.
 #include <algorithm>
 
 #include "vmo_internal.cuh"

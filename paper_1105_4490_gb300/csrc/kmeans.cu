@@ -189,7 +189,7 @@ __global__ void k_km_fill(float4* __restrict__ z, int m, const KmState* __restri
 // clusters' sums in shared memory until its end.  The fixed-point values are
 // added as two 32-bit words (their low 16 bits and the rest): shared memory has
 // native 32-bit additions but adds 64 bits by a compare-and-swap loop, which took most
-// of the 150 us a round of a million points and 64 centres (now 40); a flush into
+// of the 150 us a round of a million points and 64 centres (now 35); a flush into
 // 64-bit sums after kKmFlush points keeps the words from overflowing.
 constexpr int kKmAssign = 4;
 constexpr int kKmFlush = 8192;  // points of a block between flushes: 8192 (2^16 + 2^14) < 2^31

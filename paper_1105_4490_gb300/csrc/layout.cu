@@ -827,7 +827,7 @@ __global__ void __launch_bounds__(kCellsBlock) k_cells(const int32_t* __restrict
     }
     pair_store<D>(CP, pr.cbase + lvl_off(D, l) + c + pb + 1, z, W);
   };
-  const int nc = 1 << (D * lb);  // at most kCellsBlock
+  const int nc = 1 << (D * lb);  // at most NC: 64, for d = 4 256
   const int32_t* cs = cst + pr.fbase + pb;
   for (int i = threadIdx.x; i < nc; i += kCellsBlock) {
     const int64_t c = cell_index(i, 0);

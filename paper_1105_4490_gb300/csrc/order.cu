@@ -1090,8 +1090,8 @@ __global__ void k_cut_scatter(const uint64_t* __restrict__ keys, const uint32_t*
 // integers, so the results are the same to the bit.  As a launch sequence a
 // level took up to 45 launches and five host waits, about 0.45 ms whatever
 // its size; here a round is three block barriers and one cluster barrier.
-// Ordering of given coordinates: 64^3 grid to depth 10 5.8 -> 2.0 ms, 400k x
-// 300k bipartite pattern to 64 parts 6.9 -> 3.3 ms.
+// Ordering of given coordinates: 64^3 grid to depth 10 5.9 -> 1.6 ms, 400k x
+// 300k bipartite pattern to 64 parts 6.9 -> 1.7 ms.
 struct TwoMeansSums {           // one block's sums of a round, read by the cluster
   unsigned long long v[6];      // S1[0..3], n1 | labels changed << 40, weights
 };
