@@ -549,7 +549,7 @@ typedef struct {
   int64_t batches;
   int64_t nnz_completed;
   int64_t budget_bytes, bytes_in_use, bytes_peak;  /* by estimate */
-  int64_t pool_peak_bytes;  /* high-water mark of the device pool (measured) */
+  int64_t pool_peak_bytes;  /* high-water marks of the device pool and the levels' pool, added (measured) */
 } vmo_server_stats;
 
 /* Fills the defaults shown above (params = vmo_default_params()). */

@@ -385,6 +385,17 @@ cudaMemPool_t library_pool(PoolKind kind) {
   return pool;
 }
 
+uint64_t level_pool_peak(int device) {
+  std::lock_guard<std::mutex> lk(g_library_pool_mu);
+  uint64_t hi = 0;
+  for (auto& p : g_library_pools[kLevelPool])
+    if (p.first == device && cudaMemPoolGetAttribute(p.second, cudaMemPoolAttrUsedMemHigh, &hi) != cudaSuccess) {
+      (void)cudaGetLastError();
+      hi = 0;
+    }
+  return hi;
+}
+
 vmo_status ensure_device_public() { return ensure_device(); }
 vmo_status check_params_public(const vmo_params* p) { return check_params(p); }
 

@@ -450,7 +450,7 @@ vmo_status vmo_server_get_stats(vmo_server srv, vmo_server_stats* out) {
   uint64_t hi = 0;
   if (cudaDeviceGetDefaultMemPool(&pool, S.device) == cudaSuccess &&
       cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &hi) == cudaSuccess)
-    out->pool_peak_bytes = (int64_t)hi;
+    out->pool_peak_bytes = (int64_t)(hi + level_pool_peak(S.device));
   else
     (void)cudaGetLastError();
   return VMO_OK;

@@ -94,6 +94,7 @@ extern thread_local PoolKind g_devarray_pool;
 constexpr uint64_t kPoolKeep = uint64_t(1) << 30;
 constexpr size_t kLevelPoolMin = size_t(16) << 20;  // bytes of an array from which a level takes it there
 cudaMemPool_t library_pool(PoolKind kind);  // of the current device; null if it cannot be made
+uint64_t level_pool_peak(int device);       // most bytes of its level pool in use at once (0: none made)
 
 struct DevArrayStreamScope {
   cudaStream_t prev_s;
