@@ -3,6 +3,9 @@ that matrix alone (bit-exact: the permutation is integer work), whether the
 request ran alone or mixed into batches with others that arrived while
 earlier ones were on the device; admission stays within the memory budget;
 cancellation and rejection behave as documented."""
+import os
+import subprocess
+import sys
 import time
 
 import numpy as np
@@ -130,18 +133,28 @@ def test_cancel_running_stays_running_until_batch_ends(V):
         assert srv.release(r2) is True
 
 
+PEAK = """
+import numpy as np
+import paper_1105_4490_gb300 as V
+before = None
+for n in (3000, 6000):  # full patterns: 36 and 144 MB of adjacency
+    rowptr = (np.arange(n + 1, dtype=np.int64) * n).astype(np.int32)
+    colidx = np.tile(np.arange(n, dtype=np.int32), n)
+    with V.Server(V.Params(d=3, seed=1, iters=0, multilevel=False), slots=1) as srv:
+        rid = srv.submit(rowptr, colidx)
+        assert srv.wait(rid, 120.0)["state"] == "done"
+        peak = srv.stats()["pool_peak_bytes"]
+    if before is not None:
+        assert peak - before >= 5 * (6000 * 6000 - 3000 * 3000) * 4, (before, peak)
+    before = peak
+"""
+
+
 def test_pool_peak_counts_large_level_arrays(V):
     """The server's peak covers the arrays of a level that have a pool of their
     own: a request with more edges has a higher one, by the copy of its pattern, the
-    joined one, and the model's and the level's arrays (four at least of its size)."""
-    before = None
-    for n in (3000, 6000):  # full patterns: 36 and 144 MB of adjacency
-        rowptr = (np.arange(n + 1, dtype=np.int64) * n).astype(np.int32)
-        colidx = np.tile(np.arange(n, dtype=np.int32), n)
-        with V.Server(V.Params(d=3, seed=1, iters=0, multilevel=False), slots=1) as srv:
-            rid = srv.submit(rowptr, colidx)
-            assert srv.wait(rid, 120.0)["state"] == "done"
-            peak = srv.stats()["pool_peak_bytes"]
-        if before is not None:
-            assert peak - before >= 5 * (6000 * 6000 - 3000 * 3000) * 4
-        before = peak
+    joined one, and the model's and the level's arrays (four at least of its size).
+    In a process of its own, since the marks are the process's."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", PEAK], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
