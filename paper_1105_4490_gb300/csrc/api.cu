@@ -15,11 +15,12 @@ thread_local cudaStream_t g_devarray_stream = nullptr;
 thread_local bool g_devarray_async = false;
 thread_local PoolKind g_devarray_pool = kDefaultPool;
 thread_local bool g_pdl = false;
+thread_local cudaError_t g_refused = cudaSuccess;
 
 void set_error(const std::string& msg) { g_last_error = msg; }
 
 vmo_status cuda_fail(cudaError_t e, const char* what, const char* file, int line) {
-  (void)cudaGetLastError();  // collected: the next call starts without it
+  (void)launch_status();  // collected: the next call starts without it
   char buf[512];
   snprintf(buf, sizeof(buf), "%s: %s (%s:%d)", what, cudaGetErrorString(e), file, line);
   set_error(buf);
@@ -138,6 +139,7 @@ vmo_status ensure_device() {
       cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
     }
   });
+  begin_launches();
   return VMO_OK;
 }
 

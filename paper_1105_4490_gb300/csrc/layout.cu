@@ -2981,6 +2981,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
                  CP, done);
       }
       if (fork) cudaStreamWaitEvent(ms, ss->join, 0);
+      if (g_refused == cudaSuccess) begin_launches();  // also of the events and copies so far
       const bool timed = stats_timing();
       if (timed) stats_time_begin(ms);
       unsigned long long* icount = stats_interaction_counter();
@@ -3003,7 +3004,7 @@ vmo_status layout_level(LevelBatch& lb, const LayoutOptions& o, float4* x, int i
         step_launch(k_repulse_update<D, false, kStepPlain>, lb.threads, lb.wprob.ptr);
       }
       if (timed) stats_time_end(ms, (uint64_t)K);
-      cudaError_t e = cudaGetLastError();
+      const cudaError_t e = launch_status();
       if (e != cudaSuccess) return cuda_fail(e, "layout step", __FILE__, __LINE__);
       return VMO_OK;
     };

@@ -53,6 +53,7 @@ vmo_status bisect_noalloc(int32_t d, const float* coords, const int32_t* verts, 
                    std::to_string(kNoAllocMaxPoints) + " points (use vmo_bisect)");
   if (nverts > 0 && (!coords || !verts || !labels || ((uintptr_t)coords & 15u)))
     return invalid("null or unaligned argument");
+  begin_launches();
   unsigned char* base;
   VMO_TRY(scratch_address(&base));
   float zh[8] = {0, 0, 0, 0, 0, 0, 0, 0};

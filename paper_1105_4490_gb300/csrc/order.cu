@@ -1401,7 +1401,7 @@ static cudaError_t launch_two_means(const OrderState& st, int N, int km_iters, i
       return launch_two_means<D, T, LIST>(st, N, km_iters, 8, share * 2, list, s);
     }
   }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;  // as launch(): nothing after a refused one
+  if ((e = launch_status()) != cudaSuccess) return e;  // as launch(): nothing after a refused one
   g_launches.fetch_add(1, std::memory_order_relaxed);
   return cudaLaunchKernelEx(&cfg, kernel, (const float4*)st.xo, (const int32_t*)st.ord, st.nodes,
                             (const uint64_t*)st.seeds, km_iters, st.lab, st.vrec, cap, (int)stream, list);
@@ -1530,7 +1530,7 @@ static vmo_status two_means_body(OrderState& st, int N, int d, int km_iters, uns
     launch(k_clear_counts, grid_for(N, kBlock), kBlock, 0, s, st.nodes, N);
     launch_assign<D>(n, s, st.xo, st.seg, 0, st.nodes, st.lab, 1, rep);
     if (rep) launch(k_fold_reps, grid_for(N * 10, kBlock), kBlock, 0, s, st.nodes, N, rep);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_status();
     if (e != cudaSuccess) stt = cuda_fail(e, "two_means", __FILE__, __LINE__);
   });
   return stt;

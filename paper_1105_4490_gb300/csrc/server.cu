@@ -148,6 +148,7 @@ void ServerImpl::run_batch(int slot, const std::vector<uint64_t>& ids, cudaStrea
     for (uint64_t id : ids) rs.push_back(&reqs[id]);
   }
   const int count = (int)rs.size();
+  begin_launches();
   int64_t rows = 0, ents = 0;
   for (Req* r : rs) {
     rows += r->n + 1;
